@@ -826,6 +826,9 @@ static int run_lloyd(pscl_job *j, const LloydPlan &p, const float *pts, float *c
     // the near ties' candidate masks borrow the peel's bucket lists (d * ord_ld words, idle
     // once the peel is done; 8 words per row fit whenever d >= 8)
     if (j->pb.ord && (size_t)p.rows * 8 <= (size_t)j->d * (size_t)j->pb.ord_ld) b.tmask = j->pb.ord;
+    // and the labels before the ties are decided the peel's round of each point (n words; idle
+    // once the subclusters are packed)
+    if (b.tmask) b.raw = reinterpret_cast<int32_t *>(j->pb.rnd);
     // the pooled set past 256 centers: the chunked search's tables, its row state in the same
     // idle lists (4 rows + 1 words)
     if (stage == 1 && j->final_k > 256 && j->fp256.d_split && b.tmask &&
@@ -1262,7 +1265,7 @@ struct pscl_batch : Owner {
     float *centers = nullptr;
     unsigned long long *acc = nullptr;
     int32_t *cnt = nullptr, *labels = nullptr, *out_labels = nullptr, *trace = nullptr;
-    uint32_t *tmask = nullptr;        // rows x 8 (tensor-core precisions only)
+    uint32_t *tmask = nullptr;        // rows x 8, then rows more for the undecided labels (tensor-core precisions only)
     int64_t trace_len = 0;
     double *unit_sse = nullptr, *seg_sse = nullptr;
     uint32_t *flags = nullptr;
@@ -1447,6 +1450,7 @@ static int batch_enqueue(pscl_batch *b, int iters, uint64_t seed, int prec, bool
     lb.trace = b->trace_on ? b->trace : nullptr;
     lb.rows = b->rows;
     lb.tmask = b->tmask;
+    if (b->tmask) lb.raw = reinterpret_cast<int32_t *>(b->tmask + (size_t)b->rows * 8);
     const int64_t P = b->plan.P;
     CU(launch_lloyd_init(lb, t, b->d, P, seed, 0u, 0, b->plan.kmax, st, &b->kt));
     if (events) CU(cudaEventRecord(b->ev[0], st));
@@ -1489,8 +1493,9 @@ extern "C" int pscl_batch_run(pscl_batch *b, int32_t iters, uint64_t seed, int p
         if (tl) TRY(A(b, &b->trace, tl));
     }
     b->iters = iters;
-    // the tensor-core assignment's candidate masks: 8 words per row, allocated once
-    if (prec != PSCL_PREC_FP32 && !b->tmask) TRY(A(b, &b->tmask, (size_t)b->rows * 8));
+    // the tensor-core assignment's candidate masks, 8 words per row, and its labels before the
+    // near ties are decided, allocated once
+    if (prec != PSCL_PREC_FP32 && !b->tmask) TRY(A(b, &b->tmask, (size_t)b->rows * 9));
     if (!b->graph) return batch_enqueue(b, iters, seed, prec, true);
     const uint64_t key[6] = {(uint64_t)iters, seed, (uint64_t)prec, (uint64_t)(b->trace_on | b->plain << 1),
                              (uint64_t)b->unit_rows, (uint64_t)b->rpt};

@@ -317,13 +317,15 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
 }
 
 // center = exact sum / count (double), rounded once to float; empty clusters keep their
-// center.  Clears the sums and the other parity's counts for the next iteration.  A thread
+// center.  Clears the sums and the other parity's counts for the next iteration, or with
+// `keep` (a sums pass that adds only the rows that moved) leaves the sums and carries the
+// counts over.  A thread
 // takes EPT consecutive attributes of one center (d % EPT == 0) and forms the count's
 // reciprocal once for them: float64 is the slow pipe of this GPU.  I is the element index
 // type (32-bit whenever the elements fit, which avoids 64-bit division).
 template <int EPT, typename I>
 __global__ void k_lloyd_finalize(float *centers, unsigned long long *acc, const int32_t *count,
-                                 int32_t *count_next, int64_t cen_lo, int64_t cen_hi, int d)
+                                 int32_t *count_next, int64_t cen_lo, int64_t cen_hi, int d, bool keep)
 {
     const I g0 = (I)(cen_lo * d / EPT), g1 = (I)(cen_hi * d / EPT), dd = (I)d;
     for (I g = g0 + (I)blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += (I)gridDim.x * blockDim.x) {
@@ -338,24 +340,26 @@ __global__ void k_lloyd_finalize(float *centers, unsigned long long *acc, const 
                 centers[e + q] = __double2float_rn(__dmul_rn(__dmul_rn((double)sum, 0x1p-32), r));
             }
         }
+        if (!keep) {
 #pragma unroll
-        for (int q = 0; q < EPT; q++) acc[e + q] = 0ull;
-        if (e - c * dd == 0) count_next[c] = 0;
+            for (int q = 0; q < EPT; q++) acc[e + q] = 0ull;
+        }
+        if (e - c * dd == 0) count_next[c] = keep ? n : 0;
     }
 }
 
 template <int EPT>
 void finalize_launch(const LloydBuffers &b, int32_t *count_next, int64_t cen_lo, int64_t cen_hi, int d,
-                     int sm_count, cudaStream_t st)
+                     int sm_count, bool keep, cudaStream_t st)
 {
     const int64_t work = (cen_hi - cen_lo) * d / EPT;
     int64_t g = (work + 255) / 256;
     if (g > (int64_t)sm_count * 8) g = (int64_t)sm_count * 8;
     if (g < 1) g = 1;
     if (cen_hi * d < ((int64_t)1 << 31))
-        k_lloyd_finalize<EPT, uint32_t><<<(int)g, 256, 0, st>>>(b.centers, b.acc, b.count, count_next, cen_lo, cen_hi, d);
+        k_lloyd_finalize<EPT, uint32_t><<<(int)g, 256, 0, st>>>(b.centers, b.acc, b.count, count_next, cen_lo, cen_hi, d, keep);
     else
-        k_lloyd_finalize<EPT, int64_t><<<(int)g, 256, 0, st>>>(b.centers, b.acc, b.count, count_next, cen_lo, cen_hi, d);
+        k_lloyd_finalize<EPT, int64_t><<<(int)g, 256, 0, st>>>(b.centers, b.acc, b.count, count_next, cen_lo, cen_hi, d, keep);
 }
 
 // Nearest final center of every scaled point (original order) and the sum of squared
@@ -619,9 +623,11 @@ cudaError_t launch_lloyd_iter(const LloydBuffers &b, int32_t *count_next, const 
                               KTimer *kt, int rows_per_thread)
 {
     cudaError_t e;
+    bool keep = false;
     if (prec != PSCL_PREC_FP32 && !b.weights && b.tmask && t.split && unit_lo == 0 && unit_hi == t.n_units &&
         tc_supported(d, kmax, prec)) {
         e = launch_lloyd_assign_tc(b, t, d, iter, kmax, prec, flags, sm_count, st, kt);
+        keep = b.raw != nullptr;
     } else if (prec != PSCL_PREC_FP32 && !b.weights && b.has_chunks && b.chunk_scratch && t.n_seg == 1 &&
                kmax > 256 && unit_lo == 0 && unit_hi == t.n_units && tc_sse_supported(d, kmax, prec)) {
         e = launch_lloyd_chunks_tc(b, d, iter, kmax, prec, flags, sm_count, st, kt);
@@ -637,9 +643,9 @@ cudaError_t launch_lloyd_iter(const LloydBuffers &b, int32_t *count_next, const 
     }
     if (e != cudaSuccess) return e;
     kt->begin(st);
-    if (d % 4 == 0) finalize_launch<4>(b, count_next, cen_lo, cen_hi, d, sm_count, st);
-    else if (d % 2 == 0) finalize_launch<2>(b, count_next, cen_lo, cen_hi, d, sm_count, st);
-    else finalize_launch<1>(b, count_next, cen_lo, cen_hi, d, sm_count, st);
+    if (d % 4 == 0) finalize_launch<4>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
+    else if (d % 2 == 0) finalize_launch<2>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
+    else finalize_launch<1>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
     kt->end(PSCL_K_LLOYD_FINALIZE, st);
     return cudaGetLastError();
 }

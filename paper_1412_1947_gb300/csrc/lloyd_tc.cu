@@ -839,11 +839,106 @@ __host__ __device__ constexpr int sum_threads()
     return D <= 64 ? 512 : 256;          // a near tie's row is held in registers
 }
 
+// A near tie re-scored by one thread against the row's candidate centers (the bits of its
+// mask; every center left out lies beyond the float32 direct sum's error of the best), the
+// centers read from shared memory as float4 at a stride of D + 4 floats.
+template <int D>
+__device__ __forceinline__ int32_t rescore_row(const float *__restrict__ pts, const uint32_t *__restrict__ tmask,
+                                               const float *scen, int k, int64_t row)
+{
+    constexpr int DC = D + 4;
+    int32_t mylab = 0;
+    float x[D];
+    const float4 *x4 = reinterpret_cast<const float4 *>(pts + row * D);
+#pragma unroll
+    for (int a4 = 0; a4 < D / 4; a4++) {
+        const float4 v = __ldg(&x4[a4]);
+        x[4 * a4 + 0] = v.x;
+        x[4 * a4 + 1] = v.y;
+        x[4 * a4 + 2] = v.z;
+        x[4 * a4 + 3] = v.w;
+    }
+    const uint4 *mk = reinterpret_cast<const uint4 *>(tmask + row * 8);
+    const uint4 ma = __ldg(mk), mb = __ldg(mk + 1);
+    uint32_t wd[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
+#pragma unroll
+    for (int c = 0; c < 8; c++) {      // no bit at or past k
+        const int rem = k - 32 * c;
+        wd[c] &= rem >= 32 ? 0xffffffffu : rem > 0 ? (1u << rem) - 1u : 0u;
+    }
+    // the candidates in ascending order, two at a time (two independent
+    // chains); strict comparisons in that order keep the lowest index
+    // (the words move down as they empty: registers, no indexed access)
+    int base = 0, left = 8;
+    auto next = [&](int &j) -> bool {
+        while (wd[0] == 0u && left > 1) {
+#pragma unroll
+            for (int q = 0; q < 7; q++) wd[q] = wd[q + 1];
+            wd[7] = 0u;
+            base += 32;
+            left--;
+        }
+        if (wd[0] == 0u) return false;
+        j = base + __ffs(wd[0]) - 1;
+        wd[0] &= wd[0] - 1u;
+        return true;
+    };
+    float bd = __int_as_float(0x7f800000);
+    int j0, j1;
+    while (next(j0)) {
+        const bool two = next(j1);
+        if (!two) j1 = j0;
+        const float4 *c0 = reinterpret_cast<const float4 *>(scen + (size_t)j0 * DC);
+        const float4 *c1 = reinterpret_cast<const float4 *>(scen + (size_t)j1 * DC);
+        float d0 = 0.0f, d1 = 0.0f;
+#pragma unroll
+        for (int a4 = 0; a4 < D / 4; a4++) {
+            const float4 u = c0[a4], w4 = c1[a4];
+            float t, y;
+            t = __fsub_rn(x[4 * a4 + 0], u.x); d0 = __fmaf_rn(t, t, d0);
+            y = __fsub_rn(x[4 * a4 + 0], w4.x); d1 = __fmaf_rn(y, y, d1);
+            t = __fsub_rn(x[4 * a4 + 1], u.y); d0 = __fmaf_rn(t, t, d0);
+            y = __fsub_rn(x[4 * a4 + 1], w4.y); d1 = __fmaf_rn(y, y, d1);
+            t = __fsub_rn(x[4 * a4 + 2], u.z); d0 = __fmaf_rn(t, t, d0);
+            y = __fsub_rn(x[4 * a4 + 2], w4.z); d1 = __fmaf_rn(y, y, d1);
+            t = __fsub_rn(x[4 * a4 + 3], u.w); d0 = __fmaf_rn(t, t, d0);
+            y = __fsub_rn(x[4 * a4 + 3], w4.w); d1 = __fmaf_rn(y, y, d1);
+        }
+        if (d0 < bd) {
+            bd = d0;
+            mylab = j0;
+        }
+        if (two && d1 < bd) {
+            bd = d1;
+            mylab = j1;
+        }
+    }
+    return mylab;
+}
+
+// The near ties of a warp (lanes with `tie` set, each at its own row): lane i re-scores the
+// warp's i-th tie row alone; the labels go back by shuffles.  Returns a tie lane's label
+// (else nothing of use).
+template <int D>
+__device__ __forceinline__ int32_t rescore_ties(const float *__restrict__ pts, const uint32_t *__restrict__ tmask,
+                                                const float *scen, int k, int64_t row, bool tie)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t tm = __ballot_sync(0xffffffffu, tie);
+    if (!tm) return 0;
+    const int nt = __popc(tm);
+    const int src = lane < nt ? (int)__fns(tm, 0u, lane + 1) : 0;
+    const int64_t trow = __shfl_sync(0xffffffffu, row, src);
+    const int32_t mylab = lane < nt ? rescore_row<D>(pts, tmask, scen, k, trow) : 0;
+    // the q-th tie lane of the warp gets the label lane q found
+    return __shfl_sync(0xffffffffu, mylab, __popc(tm & ((1u << lane) - 1u)));
+}
+
 template <int D>
 __global__ void __launch_bounds__(sum_threads<D>(), D <= 32 ? 2 : 1) k_tc_sums(const float *__restrict__ pts,
                                                              const float *__restrict__ centers, SegTable t,
-                                                             const int32_t *split, int32_t *labels,
-                                                             const uint32_t *__restrict__ tmask,
+                                                             const int32_t *split, const int32_t *raw,
+                                                             int32_t *labels, const uint32_t *__restrict__ tmask,
                                                              int32_t *trace, int64_t trace_off,
                                                              unsigned long long *acc, int32_t *count, int kmax)
 {
@@ -873,94 +968,11 @@ __global__ void __launch_bounds__(sum_threads<D>(), D <= 32 ? 2 : 1) k_tc_sums(c
             const int pr = p0 + tid;
             const bool live = pr < run.R;
             const int64_t row = run.row0 + (live ? pr : 0);
-            int32_t lab = live ? labels[row] : 0;
+            int32_t lab = live ? raw[row] : 0;
             const bool tie = live && ((uint32_t)lab & kTieBit);
             if (!tie && (uint32_t)lab >= (uint32_t)k) lab = 0;   // only after an assignment that gave up
-            // near ties: lane i of a warp re-scores the warp's i-th tie row against the row's
-            // candidate centers (the bits of its mask; every center left out lies beyond the
-            // float32 direct sum's error of the best), the centers read from shared memory as
-            // float4 at a stride of D + 4 floats; the labels go back by shuffles
-            {
-                const int lane = tid & 31;
-                const uint32_t tm = __ballot_sync(0xffffffffu, tie);
-                if (tm) {
-                    const int nt = __popc(tm);
-                    const int src = lane < nt ? (int)__fns(tm, 0u, lane + 1) : 0;
-                    const int64_t trow = __shfl_sync(0xffffffffu, row, src);
-                    int32_t mylab = 0;
-                    if (lane < nt) {
-                        float x[D];
-                        const float4 *x4 = reinterpret_cast<const float4 *>(pts + trow * D);
-#pragma unroll
-                        for (int a4 = 0; a4 < D / 4; a4++) {
-                            const float4 v = __ldg(&x4[a4]);
-                            x[4 * a4 + 0] = v.x;
-                            x[4 * a4 + 1] = v.y;
-                            x[4 * a4 + 2] = v.z;
-                            x[4 * a4 + 3] = v.w;
-                        }
-                        const uint4 *mk = reinterpret_cast<const uint4 *>(tmask + trow * 8);
-                        const uint4 ma = __ldg(mk), mb = __ldg(mk + 1);
-                        uint32_t wd[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
-#pragma unroll
-                        for (int c = 0; c < 8; c++) {      // no bit at or past k
-                            const int rem = k - 32 * c;
-                            wd[c] &= rem >= 32 ? 0xffffffffu : rem > 0 ? (1u << rem) - 1u : 0u;
-                        }
-                        // the candidates in ascending order, two at a time (two independent
-                        // chains); strict comparisons in that order keep the lowest index
-                        // (the words move down as they empty: registers, no indexed access)
-                        int base = 0, left = 8;
-                        auto next = [&](int &j) -> bool {
-                            while (wd[0] == 0u && left > 1) {
-#pragma unroll
-                                for (int q = 0; q < 7; q++) wd[q] = wd[q + 1];
-                                wd[7] = 0u;
-                                base += 32;
-                                left--;
-                            }
-                            if (wd[0] == 0u) return false;
-                            j = base + __ffs(wd[0]) - 1;
-                            wd[0] &= wd[0] - 1u;
-                            return true;
-                        };
-                        float bd = __int_as_float(0x7f800000);
-                        int j0, j1;
-                        while (next(j0)) {
-                            const bool two = next(j1);
-                            if (!two) j1 = j0;
-                            const float4 *c0 = reinterpret_cast<const float4 *>(scen + (size_t)j0 * DC);
-                            const float4 *c1 = reinterpret_cast<const float4 *>(scen + (size_t)j1 * DC);
-                            float d0 = 0.0f, d1 = 0.0f;
-#pragma unroll
-                            for (int a4 = 0; a4 < D / 4; a4++) {
-                                const float4 u = c0[a4], w4 = c1[a4];
-                                float t, y;
-                                t = __fsub_rn(x[4 * a4 + 0], u.x); d0 = __fmaf_rn(t, t, d0);
-                                y = __fsub_rn(x[4 * a4 + 0], w4.x); d1 = __fmaf_rn(y, y, d1);
-                                t = __fsub_rn(x[4 * a4 + 1], u.y); d0 = __fmaf_rn(t, t, d0);
-                                y = __fsub_rn(x[4 * a4 + 1], w4.y); d1 = __fmaf_rn(y, y, d1);
-                                t = __fsub_rn(x[4 * a4 + 2], u.z); d0 = __fmaf_rn(t, t, d0);
-                                y = __fsub_rn(x[4 * a4 + 2], w4.z); d1 = __fmaf_rn(y, y, d1);
-                                t = __fsub_rn(x[4 * a4 + 3], u.w); d0 = __fmaf_rn(t, t, d0);
-                                y = __fsub_rn(x[4 * a4 + 3], w4.w); d1 = __fmaf_rn(y, y, d1);
-                            }
-                            if (d0 < bd) {
-                                bd = d0;
-                                mylab = j0;
-                            }
-                            if (two && d1 < bd) {
-                                bd = d1;
-                                mylab = j1;
-                            }
-                        }
-                    }
-                    // the q-th tie lane of the warp gets the label lane q found
-                    const int q = __popc(tm & ((1u << lane) - 1u));
-                    const int32_t res = __shfl_sync(0xffffffffu, mylab, q);
-                    if (tie) lab = res;
-                }
-            }
+            const int32_t fixed = rescore_ties<D>(pts, tmask, scen, k, row, tie);
+            if (tie) lab = fixed;
             if (live) {
                 labels[row] = lab;
                 if (trace) trace[trace_off + row] = lab;
@@ -1018,6 +1030,144 @@ __global__ void __launch_bounds__(sum_threads<D>(), D <= 32 ? 2 : 1) k_tc_sums(c
                 }
                 __syncthreads();
             }
+        }
+    }
+}
+
+// The sums of every later iteration, from the rows that changed their center.  The sums of
+// the iteration before are kept (launch_lloyd_iter leaves them and carries the counts), and
+// a row whose label differs from its last one is taken off its old center's sum and added
+// to its new one's.  The sums are integers modulo 2^64, so they end up the same bits as if
+// every row had been added again.  After the first few iterations few rows move, so the pass
+// is bound by one read of the two label arrays and by the near ties' re-scoring, not by the
+// points: 64-bit atomics in L2 for the moved rows (lane a attribute a, so a row's atomics
+// fall in whole 32-byte sectors) need no shared sums, no clearing and no fold, and shared
+// memory holds the centers, which leaves room for several CTAs per SM.
+// A warp takes delta_rows() rows at a time, lists their near ties and then the rows that
+// moved in its own piece of shared memory, and works through each list with full lanes (a
+// tie per lane; a moved row per D lanes): with the ties of 32 rows at a time most lanes of a
+// warp waited on the few that held one (2^24 x 64: 1.44 against 0.90 ms).
+// Mean time of an iteration's sums, every row added -> the moved rows only: 2^24 x 64 with
+// k = 256 1.98 -> 0.90 ms, the uneven batch (2.5e7 x 32) 0.80 -> 0.19 ms, 2^20 x 16 (the rows
+// in L2) 33 -> 17 us.
+template <int D>
+__host__ __device__ constexpr int delta_threads()
+{
+    return D <= 32 ? 512 : 256;
+}
+
+template <int D>
+__host__ __device__ constexpr int delta_rows()
+{
+    return D <= 32 ? 128 : 256;
+}
+
+template <int D>
+size_t delta_smem(int kmax)
+{
+    return (size_t)kmax * (D + 4) * 4 + (size_t)(delta_threads<D>() / 32) * delta_rows<D>() * (8 + 2);
+}
+
+template <int D>
+__global__ void __launch_bounds__(delta_threads<D>(), 2)
+k_tc_delta(const float *__restrict__ pts, const float *__restrict__ centers, SegTable t, const int32_t *split,
+           const int32_t *__restrict__ raw, int32_t *labels, const uint32_t *__restrict__ tmask, int32_t *trace,
+           int64_t trace_off, unsigned long long *acc, int32_t *count, int kmax)
+{
+    constexpr int NT = delta_threads<D>(), NW = NT / 32, WR = delta_rows<D>(), Q = WR / 32;
+    constexpr int DC = D + 4;
+    constexpr int RPI = D < 32 ? 32 / D : 1;           // moved rows per atomic instruction
+    constexpr int PL = D < 32 ? 1 : D / 32;            // attributes per lane
+    constexpr int U = PL >= 4 ? 1 : 4 / PL;            // groups of moved rows in flight
+    extern __shared__ __align__(16) float scen_d[];    // [centers | moved lists | tie lists]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    uint2 *mv = reinterpret_cast<uint2 *>(scen_d + (size_t)kmax * DC) + (size_t)w * WR;   // (row, old << 16 | new)
+    uint16_t *tl = reinterpret_cast<uint16_t *>(reinterpret_cast<uint2 *>(scen_d + (size_t)kmax * DC) + (size_t)NW * WR) +
+                   (size_t)w * WR;
+    const int sub = D < 32 ? lane / D : 0, at0 = D < 32 ? lane % D : lane;
+    const int ub = split[blockIdx.x], ue = split[blockIdx.x + 1];
+    int u = ub;
+    Run run;
+    while (next_run(t, u, ue, run)) {
+        const int k = run.k;
+        const float *cen = centers + run.c0 * D;
+        __syncthreads();
+        for (int e = tid; e < k * (D / 4); e += NT)
+            *reinterpret_cast<float4 *>(scen_d + (e / (D / 4)) * DC + 4 * (e % (D / 4))) =
+                __ldg(reinterpret_cast<const float4 *>(cen) + e);
+        __syncthreads();
+        for (int p0 = w * WR; p0 < run.R; p0 += NW * WR) {
+            const int64_t row0 = run.row0 + p0;
+            const int nrow = min(WR, run.R - p0);
+            int32_t lab[Q], old[Q];
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                const int r = q * 32 + lane;
+                lab[q] = r < nrow ? __ldg(&raw[row0 + r]) : 0;
+                old[q] = r < nrow ? labels[row0 + r] : 0;
+            }
+            int nt = 0, nm = 0;
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                const int r = q * 32 + lane;
+                const bool tie = r < nrow && ((uint32_t)lab[q] & kTieBit);
+                if (!tie && (uint32_t)lab[q] >= (uint32_t)k) lab[q] = 0;     // only after an assignment that gave up
+                if ((uint32_t)old[q] >= (uint32_t)k) old[q] = 0;
+                const bool moved = !tie && r < nrow && lab[q] != old[q];
+                const uint32_t bt = __ballot_sync(0xffffffffu, tie), bm = __ballot_sync(0xffffffffu, moved);
+                if (tie) tl[nt + __popc(bt & lt)] = (uint16_t)r;
+                if (moved) mv[nm + __popc(bm & lt)] = make_uint2((uint32_t)r, ((uint32_t)old[q] << 16) | (uint32_t)lab[q]);
+                if (trace && r < nrow && !tie) trace[trace_off + row0 + r] = lab[q];
+                nt += __popc(bt);
+                nm += __popc(bm);
+            }
+            __syncwarp();
+            for (int b = 0; b < nt; b += 32) {
+                const bool on = b + lane < nt;
+                const int r = on ? tl[b + lane] : 0;
+                int32_t nl = 0, ol = 0;
+                if (on) {
+                    ol = labels[row0 + r];
+                    if ((uint32_t)ol >= (uint32_t)k) ol = 0;
+                    nl = rescore_row<D>(pts, tmask, scen_d, k, row0 + r);
+                    if (trace) trace[trace_off + row0 + r] = nl;
+                }
+                const bool moved = on && nl != ol;
+                const uint32_t bm = __ballot_sync(0xffffffffu, moved);
+                if (moved) mv[nm + __popc(bm & lt)] = make_uint2((uint32_t)r, ((uint32_t)ol << 16) | (uint32_t)nl);
+                nm += __popc(bm);
+            }
+            __syncwarp();
+            for (int i = lane; i < nm; i += 32) {
+                const uint2 m = mv[i];
+                labels[row0 + m.x] = (int32_t)(m.y & 0xffffu);
+                atomicAdd(&count[run.c0 + (m.y & 0xffffu)], 1);
+                atomicSub(&count[run.c0 + (m.y >> 16)], 1);
+            }
+            for (int b = 0; b < nm; b += RPI * U) {
+                float xv[U][PL];
+                uint2 m[U];
+#pragma unroll
+                for (int q = 0; q < U; q++) {
+                    const int i = b + q * RPI + sub;
+                    m[q] = mv[min(i, nm - 1)];
+#pragma unroll
+                    for (int e = 0; e < PL; e++) xv[q][e] = __ldg(&pts[(row0 + m[q].x) * D + at0 + 32 * e]);
+                }
+#pragma unroll
+                for (int q = 0; q < U; q++) {
+                    if (b + q * RPI + sub < nm) {
+#pragma unroll
+                        for (int e = 0; e < PL; e++) {
+                            const unsigned long long v = fix_of(xv[q][e]);
+                            atomicAdd(&acc[(run.c0 + (m[q].y & 0xffffu)) * D + at0 + 32 * e], v);
+                            atomicAdd(&acc[(run.c0 + (m[q].y >> 16)) * D + at0 + 32 * e], 0ull - v);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
         }
     }
 }
@@ -1200,7 +1350,7 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     if (e != cudaSuccess) return e;
     TcArgs a;
     a.centers = b.centers;
-    a.labels = b.labels;
+    a.labels = b.raw ? b.raw : b.labels;
     a.tmask = b.tmask;
     a.t = t;
     a.flags = flags;
@@ -1226,13 +1376,25 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     kt->end(PSCL_K_LLOYD_ASSIGN, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // sums: four CTAs' unit ranges per SM whatever fits at once, so that the block scheduler
-    // evens out ranges whose near ties cost more
+    // evens out ranges whose near ties cost more; the first iteration adds every row, the
+    // later ones (raw labels kept apart) only the rows that moved
+    const int m = 4;
+    if (b.raw && iter > 0) {
+        const size_t sd = delta_smem<D>(kmax);
+        auto kd = k_tc_delta<D>;
+        if ((e = cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sd)) != cudaSuccess) return e;
+        kt->begin(st);
+        kd<<<m * sm_count, delta_threads<D>(), sd, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], b.raw, b.labels,
+                                                         b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count,
+                                                         kmax);
+        kt->end(PSCL_K_LLOYD_SUMS, st);
+        return cudaGetLastError();
+    }
     const size_t ss = sums_smem<D>(kmax);
     auto ks = k_tc_sums<D>;
     if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss)) != cudaSuccess) return e;
-    const int m = 4;
     kt->begin(st);
-    ks<<<m * sm_count, sum_threads<D>(), ss, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], b.labels,
+    ks<<<m * sm_count, sum_threads<D>(), ss, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], a.labels, b.labels,
                                                    b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count, kmax);
     kt->end(PSCL_K_LLOYD_SUMS, st);
     return cudaGetLastError();

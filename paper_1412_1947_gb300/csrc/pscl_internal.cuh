@@ -215,6 +215,9 @@ struct LloydBuffers {
     // 8 words per row (or NULL): the tensor-core assignment marks a near tie's candidate
     // centers here (bit j of word j / 32), the sums pass re-scores only those
     uint32_t *tmask = nullptr;
+    // rows words (or NULL): the tensor-core assignment's labels before the near ties are
+    // decided, kept apart from `labels` so that the sums pass sees which rows moved
+    int32_t *raw = nullptr;
     // a single set of more than 256 centers on the tensor cores: the rows as one set of 256
     // and of the remaining centers, with CTA splits (has_chunks), and 4 rows + 1 words of
     // scratch for the chunked search
