@@ -62,9 +62,10 @@ typedef enum { PSCL_F32 = 0, PSCL_BF16 = 1 } pscl_dtype;
  *      contraction (far fewer near ties to re-decide).
  *  PSCL_PREC_TC: per point set, TF32X3 where its operands fit one CTA's shared memory,
  *      else BF16X3 (the split mode that serves the shape; the result is the same).
- *  The contraction covers d in {16, 32, 64, 128} and at most 256 centers per point set
- *  whose operand tiles fit one CTA's shared memory (d = 128 only in BF16 with 16
- *  centers, d = 64 in TF32X3 only with 16); other shapes use the float32 direct sum.
+ *  The contraction covers d in {16, 32, 64} with at most 256 centers per point set and
+ *  d = 128 with at most 128, where the operand tiles fit one CTA's shared memory (d = 64
+ *  in TF32X3 only with 16 centers; d = 128 not in TF32X3, and in TF32 and BF16X3 with 16
+ *  centers or fewer only from 20480 rows on); other shapes use the float32 direct sum.
  *  The near-tie bound is rigorous, so every mode assigns exactly as PSCL_PREC_FP32 does.
  *  Every mode yields the same partition into subclusters; the update step is the same
  *  exact fixed-point mean in all modes. */

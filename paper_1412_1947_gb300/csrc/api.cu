@@ -133,10 +133,10 @@ struct pscl_job : Owner {
     int final_k = 0, fiters = 0, fprec = 0;
     uint64_t fseed = 0;
     LloydPlan fp;
-    // the SSE pass's row tables: all n rows as one set of 256 centers (final_k > 256) and of
-    // the remaining final_k mod 256 centers (final_k itself when it is at most 256)
+    // the SSE pass's row tables: all n rows as one set of a chunk of tc_chunk(d) centers
+    // (final_k above that) and of the last chunk's (final_k itself when one chunk holds it)
     LloydPlan sp256, sprem;
-    // the final Lloyd's row tables for the same chunked search (final_k > 256 only)
+    // the final Lloyd's row tables for the same chunked search (final_k > tc_chunk(d) only)
     LloydPlan fp256, fprem;
     float *cf = nullptr;
     unsigned long long *acc_f = nullptr;
@@ -673,7 +673,7 @@ static int plan_cluster(pscl_job *j, int32_t final_k, int32_t iters, uint64_t se
         j->acc_f = nullptr;
         j->cnt_f = nullptr;
         j->lab_f = nullptr;
-        // the SSE pass's tables for a search in chunks of 256 centers (tensor-core modes)
+        // the SSE pass's tables for a search in chunks of tc_chunk(d) centers (tensor-core modes)
         {
             for (LloydPlan *q : {&j->sp256, &j->sprem, &j->fp256, &j->fprem}) {
                 job_free(j, q->d_seg_start);
@@ -685,12 +685,12 @@ static int plan_cluster(pscl_job *j, int32_t final_k, int32_t iters, uint64_t se
             }
             std::vector<int64_t> s0(1, 0);
             std::vector<int32_t> sn(1, (int32_t)j->n);
-            const int32_t rem = final_k % 256;
-            if (final_k > 256) TRY(build_lloyd_plan(j, j->sp256, s0, sn, std::vector<int32_t>(1, 256)));
-            if (final_k <= 256 || rem) TRY(build_lloyd_plan(j, j->sprem, s0, sn, std::vector<int32_t>(1, final_k <= 256 ? final_k : rem)));
-            if (final_k > 256) {
+            const int32_t cw = tc_chunk(d), rem = final_k % cw;
+            if (final_k > cw) TRY(build_lloyd_plan(j, j->sp256, s0, sn, std::vector<int32_t>(1, cw)));
+            if (final_k <= cw || rem) TRY(build_lloyd_plan(j, j->sprem, s0, sn, std::vector<int32_t>(1, final_k <= cw ? final_k : rem)));
+            if (final_k > cw) {
                 std::vector<int32_t> sp(1, (int32_t)j->P);
-                TRY(build_lloyd_plan(j, j->fp256, s0, sp, std::vector<int32_t>(1, 256)));
+                TRY(build_lloyd_plan(j, j->fp256, s0, sp, std::vector<int32_t>(1, cw)));
                 if (rem) TRY(build_lloyd_plan(j, j->fprem, s0, sp, std::vector<int32_t>(1, rem)));
             }
         }
@@ -761,10 +761,11 @@ static size_t job_footprint(int64_t n, int d, int64_t N, int local_k, int final_
     {   // the SSE pass's row tables (one set of n rows; one or two of them)
         const int64_t tn = unit_target(n, sm, 0);
         const int64_t un = (n + unit_size(n, tn) - 1) / unit_size(n, tn);
-        const int tables = (final_k > 256 ? 1 : 0) + (final_k <= 256 || final_k % 256 ? 1 : 0);
+        const int cw = tc_chunk(d);
+        const int tables = (final_k > cw ? 1 : 0) + (final_k <= cw || final_k % cw ? 1 : 0);
         b += (size_t)tables * (r256(8) + r256((4 + 3 * (size_t)un + 1) * 4) + r256(split * 4));
-        if (final_k > 256) {   // the final Lloyd's, over the P pooled rows
-            const int ftables = 1 + (final_k % 256 ? 1 : 0);
+        if (final_k > cw) {    // the final Lloyd's, over the P pooled rows
+            const int ftables = 1 + (final_k % cw ? 1 : 0);
             const int64_t tp = unit_target(P, sm, 0);
             const int64_t up = (P + unit_size(P, tp) - 1) / unit_size(P, tp);
             b += (size_t)ftables * (r256(8) + r256((4 + 3 * (size_t)up + 1) * 4) + r256(split * 4));
@@ -829,12 +830,13 @@ static int run_lloyd(pscl_job *j, const LloydPlan &p, const float *pts, float *c
     // and the labels before the ties are decided the peel's round of each point (n words; idle
     // once the subclusters are packed)
     if (b.tmask) b.raw = reinterpret_cast<int32_t *>(j->pb.rnd);
-    // the pooled set past 256 centers: the chunked search's tables, its row state in the same
+    // the pooled set past tc_chunk(d) centers: the chunked search's tables, its row state in the same
     // idle lists (4 rows + 1 words)
-    if (stage == 1 && j->final_k > 256 && j->fp256.d_split && b.tmask &&
+    const int cw = tc_chunk(j->d);
+    if (stage == 1 && j->final_k > cw && j->fp256.d_split && b.tmask &&
         (size_t)4 * p.rows + 1 <= (size_t)j->d * (size_t)j->pb.ord_ld) {
         b.chunk256 = j->fp256.table();
-        b.chunkrem = (j->final_k % 256 ? j->fprem : j->fp256).table();
+        b.chunkrem = (j->final_k % cw ? j->fprem : j->fp256).table();
         b.has_chunks = true;
         b.chunk_scratch = j->pb.ord;
     }
@@ -905,12 +907,13 @@ static int enqueue_cluster(pscl_job *j, bool events)
     TRY(run_lloyd(j, j->fp, j->cl, j->cf, j->acc_f, j->cnt_f, j->lab_f, j->trace_f, j->fiters, j->fseed, 1u,
                   false, j->fprec, w));
     if (events) CU(cudaEventRecord(j->ev[4], st));
-    // the SSE pass: on the tensor cores in chunks of 256 centers where the mode and the shape
+    // the SSE pass: on the tensor cores in chunks of tc_chunk(d) centers where the mode and the shape
     // allow (its row state borrows the peel's bucket lists, idle by now), else float32
-    if (j->fprec != PSCL_PREC_FP32 && j->pb.ord && tc_sse_supported(j->d, j->final_k, j->fprec) &&
+    if (j->fprec != PSCL_PREC_FP32 && j->pb.ord && tc_sse_supported(j->d, j->final_k, j->fprec, j->n) &&
         (size_t)4 * j->n + 1 <= (size_t)j->d * (size_t)j->pb.ord_ld && j->n < ((int64_t)1 << 31)) {
-        const SegTable t256 = (j->final_k > 256 ? j->sp256 : j->sprem).table();
-        const SegTable trem = (j->final_k <= 256 || j->final_k % 256 ? j->sprem : j->sp256).table();
+        const int cw = tc_chunk(j->d);
+        const SegTable t256 = (j->final_k > cw ? j->sp256 : j->sprem).table();
+        const SegTable trem = (j->final_k <= cw || j->final_k % cw ? j->sprem : j->sp256).table();
         CU(launch_final_sse_tc(j->x, j->n, j->d, j->cf, j->final_k, t256, trem, j->pb.ord, j->labels, j->blk_sse,
                                j->sse, j->tickets + 1, j->fprec, j->flags, j->wait_limit, j->ctx->sm_count, st,
                                &j->kt));

@@ -50,8 +50,8 @@ constexpr int kCvtWarp0 = 8;              // converter warps 8..11
 constexpr int kProdWarp = 12;
 constexpr int kMmaWarp = 13;
 constexpr int kTcThreads = 14 * 32;
-constexpr int kXStages = 2;               // float32 point tiles in flight (deeper rings measured no faster)
-constexpr int kAStages = 2;               // operand A buffers
+constexpr int kXMax = 4;                  // slots of the point ring, at most
+constexpr int kAMax = 2;                  // operand A buffers, at most
 constexpr int kMeta = 8;                  // per-tile metadata ring (tiles in flight < kMeta)
 constexpr unsigned kDefaultWait = 1u << 26;
 constexpr size_t kTcSmemMax = 220 * 1024;
@@ -235,7 +235,11 @@ struct TcLayout {
     static constexpr int kXBoxCols = D < 32 ? D : 32;          // attributes per TMA box
     static constexpr int kXBoxes = D / kXBoxCols;
     static constexpr uint32_t kXBoxBytes = kTileRows * kXBoxCols * 4;
-    static constexpr uint32_t kXBytes = kXBoxes * kXBoxBytes;
+    // A slot of the point ring holds a whole tile (two slots: deeper rings measured no
+    // faster), or for d = 128, whose tile would be 64 KB, one of its four boxes.
+    static constexpr int kXPer = D == 128 ? 1 : kXBoxes;           // boxes per slot
+    static constexpr int kXTile = kXBoxes / kXPer;                 // slots per tile
+    static constexpr uint32_t kXBytes = kXPer * kXBoxBytes;
     // bank swizzle of the boxes: its span equals the box row (bytes), 16 .. 128
     static constexpr int kSwzMask = kXBoxCols * 4 == 128 ? 7 : kXBoxCols * 4 == 64 ? 3 : kXBoxCols * 4 == 32 ? 1 : 0;
 };
@@ -308,6 +312,7 @@ struct TcArgs {
     unsigned wait_limit;
     int stall;                   // test hook: wait once on a barrier nothing completes
     int npmax;                   // operand B rows (centers rounded up to 16)
+    int xslots, astages;         // point ring slots, operand A buffers (both 2 for d < 128)
     uint32_t ncols;              // TMEM columns of one accumulator
     // Search of a whole set in chunks of centers (ref_centers != NULL): the launch covers
     // one chunk (centers, the set of its runs); the reference point and the error bound's
@@ -359,11 +364,11 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
     // boundary (the bank swizzle of the point boxes repeats every 8 rows of 128 bytes)
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     unsigned char *sx = smem;
-    constexpr int XS = kXStages;
+    const uint32_t XS = D == 128 ? (uint32_t)p.xslots : 2u, AS = D == 128 ? (uint32_t)p.astages : 2u;
     unsigned char *sa = sx + (size_t)XS * L::kXBytes;
-    unsigned char *sb = sa + kAStages * L::kABytes;
+    unsigned char *sb = sa + (size_t)AS * L::kABytes;
     TileMeta *meta = reinterpret_cast<TileMeta *>(sb + (size_t)(p.npmax / 8) * L::kGroup);
-    __shared__ __align__(8) uint64_t bars[2 * kXStages + 2 * kAStages + 4 + 2 * kMeta + 1];
+    __shared__ __align__(8) uint64_t bars[2 * kXMax + 2 * kAMax + 4 + 2 * kMeta + 1];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     __shared__ float s_ref[D];
@@ -372,14 +377,14 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
     __shared__ uint32_t s_stat[2];
     const uint32_t b0 = smem_u32(bars);
     auto XFULL = [&](int s) { return b0 + 8u * (uint32_t)s; };
-    auto XEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(kXStages + s); };
-    auto AFULL = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXStages + s); };
-    auto AEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXStages + kAStages + s); };
-    auto TFULL = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXStages + 2 * kAStages + s); };
-    auto TEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXStages + 2 * kAStages + 2 + s); };
-    auto MFULL = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXStages + 2 * kAStages + 4 + s); };
-    auto MEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXStages + 2 * kAStages + 4 + kMeta + s); };
-    const uint32_t STALL = b0 + 8u * (uint32_t)(2 * kXStages + 2 * kAStages + 4 + 2 * kMeta);
+    auto XEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(kXMax + s); };
+    auto AFULL = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXMax + s); };
+    auto AEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXMax + kAMax + s); };
+    auto TFULL = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXMax + 2 * kAMax + s); };
+    auto TEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXMax + 2 * kAMax + 2 + s); };
+    auto MFULL = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXMax + 2 * kAMax + 4 + s); };
+    auto MEMPTY = [&](int s) { return b0 + 8u * (uint32_t)(2 * kXMax + 2 * kAMax + 4 + kMeta + s); };
+    const uint32_t STALL = b0 + 8u * (uint32_t)(2 * kXMax + 2 * kAMax + 4 + 2 * kMeta);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ub = p.split[blockIdx.x], ue = p.split[blockIdx.x + 1];
@@ -390,11 +395,11 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
         s_abort = 0;
         s_stat[0] = 0u;
         s_stat[1] = 0u;
-        for (int s = 0; s < XS; s++) {
+        for (int s = 0; s < kXMax; s++) {
             mbar_init(XFULL(s), 1);
             mbar_init(XEMPTY(s), 4);
         }
-        for (int s = 0; s < kAStages; s++) {
+        for (int s = 0; s < kAMax; s++) {
             mbar_init(AFULL(s), 4);
             mbar_init(AEMPTY(s), 1);
         }
@@ -430,26 +435,29 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
         if (lane == 0 && !*abort) {
             int u = ub;
             Run run;
-            uint32_t i = 0;
+            uint32_t j = 0;                              // slots filled so far
             bool ok = true;
             while (ok && next_run(p.t, u, ue, run)) {
-                for (int tt = 0; tt < run.ntiles; tt++, i++) {
-                    const int s = (int)(i % (uint32_t)XS);
-                    const uint32_t use = i / (uint32_t)XS;
-                    if (use > 0 && !mbar_wait(XEMPTY(s), (use - 1) & 1u, lim, abort)) {
-                        ok = false;
-                        break;
+                for (int tt = 0; tt < run.ntiles && ok; tt++) {
+                    for (int part = 0; part < L::kXTile; part++, j++) {
+                        const int s = (int)(j % XS);
+                        const uint32_t use = j / XS;
+                        if (use > 0 && !mbar_wait(XEMPTY(s), (use - 1) & 1u, lim, abort)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_expect_tx(XFULL(s), L::kXBytes);
+                        for (int bx = 0; bx < L::kXPer; bx++)
+                            tma_load_2d(smem_u32(sx + (size_t)s * L::kXBytes + (size_t)bx * L::kXBoxBytes), &xmap,
+                                        (part * L::kXPer + bx) * L::kXBoxCols,
+                                        (int)(run.row0 + (int64_t)tt * kTileRows), XFULL(s));
+                        issued = j + 1;
                     }
-                    mbar_expect_tx(XFULL(s), L::kXBytes);
-                    for (int bx = 0; bx < L::kXBoxes; bx++)
-                        tma_load_2d(smem_u32(sx + (size_t)s * L::kXBytes + (size_t)bx * L::kXBoxBytes), &xmap,
-                                    bx * L::kXBoxCols, (int)(run.row0 + (int64_t)tt * kTileRows), XFULL(s));
-                    issued = i + 1;
                 }
             }
             if (*abort)   // copies still in flight land before the CTA leaves
-                for (uint32_t j = issued > (uint32_t)XS ? issued - (uint32_t)XS : 0u; j < issued; j++)
-                    mbar_drain(XFULL((int)(j % (uint32_t)XS)), (j / (uint32_t)XS) & 1u, lim);
+                for (uint32_t q = issued > XS ? issued - XS : 0u; q < issued; q++)
+                    mbar_drain(XFULL((int)(q % XS)), (q / XS) & 1u, lim);
         }
     } else if (warp == kMmaWarp) {
         // ---- MMA issue: one thread
@@ -462,8 +470,8 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                 const int np = (run.k + 15) & ~15;
                 const uint32_t idesc = O::idesc(np);
                 for (int tt = 0; tt < run.ntiles; tt++, i++) {
-                    const int a = (int)(i % kAStages), bfr = (int)(i & 1u);
-                    if (!mbar_wait(AFULL(a), (i / kAStages) & 1u, lim, abort) ||
+                    const int a = (int)(i % AS), bfr = (int)(i & 1u);
+                    if (!mbar_wait(AFULL(a), (i / AS) & 1u, lim, abort) ||
                         (i >= 2 && !mbar_wait(TEMPTY(bfr), ((i >> 1) - 1) & 1u, lim, abort))) {
                         ok = false;
                         break;
@@ -519,8 +527,8 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
         // end, and after a failed wait only the bookkeeping goes on
         while (next_run(p.t, u, ue, run)) {
             // the earlier tiles' MMAs must be done before operand B and s_ref change
-            for (uint32_t j = i > kAStages ? i - kAStages : 0u; ok && j < i; j++)
-                ok = mbar_wait(AEMPTY((int)(j % kAStages)), (j / kAStages) & 1u, lim, abort);
+            for (uint32_t j = i > AS ? i - AS : 0u; ok && j < i; j++)
+                ok = mbar_wait(AEMPTY((int)(j % AS)), (j / AS) & 1u, lim, abort);
             ok = cvt_bar_and(ok && !*abort);
             if (!ok) {
                 i += (uint32_t)run.ntiles;
@@ -594,50 +602,58 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
             asm volatile("bar.sync 1, 128;" ::: "memory");
             const float cmax = sqrtf(s_cmax2);
             for (int tt = 0; tt < run.ntiles; tt++, i++) {
-                const int xs = (int)(i % (uint32_t)XS), a = (int)(i % kAStages), m = (int)(i % kMeta);
+                const int a = (int)(i % AS), m = (int)(i % kMeta);
                 if (ok)
-                    ok = mbar_wait(XFULL(xs), (i / (uint32_t)XS) & 1u, lim, abort) &&
-                         (i < kAStages || mbar_wait(AEMPTY(a), (i / kAStages - 1) & 1u, lim, abort)) &&
+                    ok = (i < AS || mbar_wait(AEMPTY(a), (i / AS - 1) & 1u, lim, abort)) &&
                          (i < kMeta || mbar_wait(MEMPTY(m), (i / kMeta - 1) & 1u, lim, abort));
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) continue;
                 const bool live = tt * kTileRows + r < run.R;
-                const unsigned char *xt = sx + (size_t)xs * L::kXBytes;
                 unsigned char *at = sa + (size_t)a * L::kABytes;
                 float xn2 = 0.0f;
+                for (int part = 0; part < L::kXTile; part++) {
+                    const uint32_t j = i * (uint32_t)L::kXTile + (uint32_t)part;       // the slot's use
+                    const int xs = (int)(j % XS);
+                    if (ok) ok = mbar_wait(XFULL(xs), (j / XS) & 1u, lim, abort);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const unsigned char *xt = sx + (size_t)xs * L::kXBytes;
 #pragma unroll 4
-                for (int a4 = 0; a4 < D / 4; a4++) {
-                    const int bx = (4 * a4) / L::kXBoxCols, c = ((4 * a4) % L::kXBoxCols) / 4;
-                    const float4 v = *reinterpret_cast<const float4 *>(xt + (size_t)bx * L::kXBoxBytes +
-                                                                       xbox_off<D, MODE>(r, c));
-                    float xv[4] = {v.x, v.y, v.z, v.w}, xc[4];
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        xc[q] = live ? __fsub_rn(xv[q], s_ref[4 * a4 + q]) : 0.0f;
-                        xn2 = __fmaf_rn(xc[q], xc[q], xn2);
-                    }
-                    if constexpr (O::kBf16) {
-                        // pairs rounded to bfloat16 in one conversion each, written as they are
-                        const __nv_bfloat162 h01 = __floats2bfloat162_rn(xc[0], xc[1]);
-                        const __nv_bfloat162 h23 = __floats2bfloat162_rn(xc[2], xc[3]);
-                        put4_bits<D, MODE>(at, r, 4 * a4, bf2_bits(h01), bf2_bits(h23));
-                        if (O::kSplit) {
-                            const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
-                            const __nv_bfloat162 l01 = __floats2bfloat162_rn(__fsub_rn(xc[0], f01.x), __fsub_rn(xc[1], f01.y));
-                            const __nv_bfloat162 l23 = __floats2bfloat162_rn(__fsub_rn(xc[2], f23.x), __fsub_rn(xc[3], f23.y));
-                            put4_bits<D, MODE>(at, r, D + 4 * a4, bf2_bits(l01), bf2_bits(l23));
-                        }
-                    } else {
-                        float h[4], lo[4];
+                    for (int b4 = 0; b4 < L::kXPer * L::kXBoxCols / 4; b4++) {
+                        const int a4 = part * (L::kXPer * L::kXBoxCols / 4) + b4;
+                        const int bx = (4 * b4) / L::kXBoxCols, c = ((4 * b4) % L::kXBoxCols) / 4;
+                        const float4 v = *reinterpret_cast<const float4 *>(xt + (size_t)bx * L::kXBoxBytes +
+                                                                           xbox_off<D, MODE>(r, c));
+                        float xv[4] = {v.x, v.y, v.z, v.w}, xc[4];
 #pragma unroll
                         for (int q = 0; q < 4; q++) {
-                            h[q] = O::rnd(xc[q]);
-                            lo[q] = O::rnd(__fsub_rn(xc[q], h[q]));
+                            xc[q] = live ? __fsub_rn(xv[q], s_ref[4 * a4 + q]) : 0.0f;
+                            xn2 = __fmaf_rn(xc[q], xc[q], xn2);
                         }
-                        put4<D, MODE>(at, r, 4 * a4, h[0], h[1], h[2], h[3]);
-                        if (O::kSplit) put4<D, MODE>(at, r, D + 4 * a4, lo[0], lo[1], lo[2], lo[3]);
+                        if constexpr (O::kBf16) {
+                            // pairs rounded to bfloat16 in one conversion each, written as they are
+                            const __nv_bfloat162 h01 = __floats2bfloat162_rn(xc[0], xc[1]);
+                            const __nv_bfloat162 h23 = __floats2bfloat162_rn(xc[2], xc[3]);
+                            put4_bits<D, MODE>(at, r, 4 * a4, bf2_bits(h01), bf2_bits(h23));
+                            if (O::kSplit) {
+                                const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+                                const __nv_bfloat162 l01 = __floats2bfloat162_rn(__fsub_rn(xc[0], f01.x), __fsub_rn(xc[1], f01.y));
+                                const __nv_bfloat162 l23 = __floats2bfloat162_rn(__fsub_rn(xc[2], f23.x), __fsub_rn(xc[3], f23.y));
+                                put4_bits<D, MODE>(at, r, D + 4 * a4, bf2_bits(l01), bf2_bits(l23));
+                            }
+                        } else {
+                            float h[4], lo[4];
+#pragma unroll
+                            for (int q = 0; q < 4; q++) {
+                                h[q] = O::rnd(xc[q]);
+                                lo[q] = O::rnd(__fsub_rn(xc[q], h[q]));
+                            }
+                            put4<D, MODE>(at, r, 4 * a4, h[0], h[1], h[2], h[3]);
+                            if (O::kSplit) put4<D, MODE>(at, r, D + 4 * a4, lo[0], lo[1], lo[2], lo[3]);
+                        }
                     }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(XEMPTY(xs));
                 }
+                if (!ok) continue;
                 const float one = live ? 1.0f : 0.0f;
                 put4<D, MODE>(at, r, L::kParts * D, one, one, O::kNormParts > 2 ? one : 0.0f, 0.0f);
 #pragma unroll
@@ -652,7 +668,6 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(XEMPTY(xs));
                     mbar_arrive(AFULL(a));
                     mbar_arrive(MFULL(m));
                 }
@@ -1069,7 +1084,7 @@ size_t delta_smem(int kmax)
 }
 
 template <int D>
-__global__ void __launch_bounds__(delta_threads<D>(), 2)
+__global__ void __launch_bounds__(delta_threads<D>(), D <= 64 ? 2 : 1)
 k_tc_delta(const float *__restrict__ pts, const float *__restrict__ centers, SegTable t, const int32_t *split,
            const int32_t *__restrict__ raw, int32_t *labels, const uint32_t *__restrict__ tmask, int32_t *trace,
            int64_t trace_off, unsigned long long *acc, int32_t *count, int kmax)
@@ -1326,13 +1341,25 @@ cudaError_t make_xmap(const float *pts, int64_t rows, CUtensorMap *map)
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Shared memory of the assignment kernel for sets of up to kmax centers.  d < 128: two whole
+// point tiles and two operand A buffers.  d = 128: as many box slots and A buffers as fit,
+// two A buffers before four slots (the conversion of a tile then overlaps the MMAs of the
+// one before; with one buffer they alternate).
 template <int D, int MODE>
-size_t assign_smem(int kmax)
+size_t assign_smem(int kmax, int *xslots = nullptr, int *astages = nullptr)
 {
     using L = TcLayout<D, MODE>;
     const int np = (kmax + 15) & ~15;
-    return 1024 + (size_t)kXStages * L::kXBytes + (size_t)kAStages * L::kABytes + (size_t)(np / 8) * L::kGroup +
-           (size_t)kMeta * sizeof(TileMeta);
+    const size_t fixed = 1024 + (size_t)(np / 8) * L::kGroup + (size_t)kMeta * sizeof(TileMeta);
+    static const int opt[4][2] = {{4, 2}, {2, 2}, {4, 1}, {2, 1}};
+    size_t b = 0;
+    for (int o = D == 128 ? 0 : 1; o < (D == 128 ? 4 : 2); o++) {
+        b = fixed + (size_t)opt[o][0] * L::kXBytes + (size_t)opt[o][1] * L::kABytes;
+        if (xslots) *xslots = opt[o][0];
+        if (astages) *astages = opt[o][1];
+        if (b <= kTcSmemMax) break;
+    }
+    return b;
 }
 
 template <int D>
@@ -1358,7 +1385,7 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     a.stall = b.tc_stall;
     a.npmax = (kmax + 15) & ~15;
     a.ncols = tmem_cols(a.npmax);
-    const size_t smem = assign_smem<D, MODE>(kmax);
+    const size_t smem = assign_smem<D, MODE>(kmax, &a.xslots, &a.astages);
     auto ka = k_tc_assign<D, MODE>;
     if ((e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     // as many CTAs per SM as registers, shared memory and the 512 TMEM columns allow (<= 4):
@@ -1400,7 +1427,7 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     return cudaGetLastError();
 }
 
-// A whole-set search on the tensor cores: the k centers in chunks of up to 256, one
+// A whole-set search on the tensor cores: the k centers in chunks of up to tc_chunk(D), one
 // assignment launch per chunk (rows keep their running state), then the undecided rows
 // re-scored in float32.  Leaves every row's float32 direct label in labels.
 template <int D, int MODE>
@@ -1417,12 +1444,13 @@ cudaError_t chunk_search(const float *x, int64_t n, const float *centers, int k,
     uint32_t *ties = reinterpret_cast<uint32_t *>(c1 + n);
     if ((e = cudaMemsetAsync(ties, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
     auto ka = k_tc_assign<D, MODE>;
-    const int nch = (k + 255) / 256;
+    const int cw = tc_chunk(D);
+    const int nch = (k + cw - 1) / cw;
     for (int c = 0; c < nch; c++) {
-        const int kc = std::min(256, k - 256 * c);
-        const SegTable &t = kc == 256 ? t256 : trem;
+        const int kc = std::min(cw, k - cw * c);
+        const SegTable &t = kc == cw ? t256 : trem;
         TcArgs a;
-        a.centers = centers + (size_t)256 * c * D;
+        a.centers = centers + (size_t)cw * c * D;
         a.labels = labels;
         a.tmask = nullptr;
         a.t = t;
@@ -1433,14 +1461,14 @@ cudaError_t chunk_search(const float *x, int64_t n, const float *centers, int k,
         a.ncols = tmem_cols(a.npmax);
         a.ref_centers = centers;
         a.ref_k = k;
-        a.chunk_first = 256 * c;
+        a.chunk_first = cw * c;
         a.first_chunk = c == 0;
         a.last_chunk = c == nch - 1;
         a.st_m1 = m1;
         a.st_m2 = m2;
         a.st_c1 = c1;
         a.ties = ties;
-        const size_t smem = assign_smem<D, MODE>(kc);
+        const size_t smem = assign_smem<D, MODE>(kc, &a.xslots, &a.astages);
         if ((e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
             return e;
         int occ = 1;
@@ -1560,9 +1588,17 @@ cudaError_t tc_by_d(const LloydBuffers &b, const SegTable &t, int d, int iter, i
     }
 }
 
+// d = 128: BF16 at any size that fits; TF32 and BF16X3 above 16 centers, or with rows for a
+// tile per SM (with fewer of both the float32 kernel is level: 10000 rows, k = 16, 24.7 us an
+// iteration against 23.9; 20480 rows 39.0 against 33.6; 100000 rows 88 against 63, and with
+// k = 64 180 against 75; 300000 rows, k = 64, 365 against 138); TF32X3's 135 KB of operand A
+// per tile would leave one buffer and no overlap.
+constexpr int64_t kWideRows = 160 * kTileRows;
+
 template <int MODE>
-bool fits_by_d(int d, int kmax)
+bool fits_by_d(int d, int kmax, int64_t rows)
 {
+    if (d == 128 && (MODE == kModeTf32x3 || (MODE != kModeBf16 && kmax <= 16 && rows < kWideRows))) return false;
     switch (d) {
     case 16: return assign_smem<16, MODE>(kmax) <= kTcSmemMax && sums_smem<16>(kmax) <= kTcSmemMax;
     case 32: return assign_smem<32, MODE>(kmax) <= kTcSmemMax && sums_smem<32>(kmax) <= kTcSmemMax;
@@ -1583,38 +1619,41 @@ int mode_of(int prec)
 }
 
 // PSCL_PREC_TC: TF32x3 where its operands fit, else BF16x3.
-int resolve_prec(int d, int kmax, int prec)
+int resolve_prec(int d, int kmax, int prec, int64_t rows)
 {
     if (prec != PSCL_PREC_TC) return prec;
-    return fits_by_d<kModeTf32x3>(d, kmax) ? PSCL_PREC_TF32X3 : PSCL_PREC_BF16X3;
+    return fits_by_d<kModeTf32x3>(d, kmax, rows) ? PSCL_PREC_TF32X3 : PSCL_PREC_BF16X3;
 }
 
 }  // namespace
 
-// The tensor-core assignment serves d in {16, 32, 64, 128} and at most 256 centers per
+// Centers per launch of a whole-set search, and the most centers of a set: for d = 128 the
+// operand rows are 544 bytes and 128 of them share shared memory with one A buffer.
+int tc_chunk(int d) { return d == 128 ? 128 : 256; }
+
+// The tensor-core assignment serves d in {16, 32, 64, 128} and at most tc_chunk(d) centers per
 // set whose operands, point tiles and sums fit in shared memory; every other case takes
 // the float32 direct kernel (same labels).
-bool tc_supported(int d, int kmax, int prec)
+bool tc_supported(int d, int kmax, int prec, int64_t rows)
 {
-    if (kmax < 1 || kmax > 256 || !encode_tiled()) return false;
-    switch (mode_of(resolve_prec(d, kmax, prec))) {
-    case kModeBf16: return fits_by_d<kModeBf16>(d, kmax);
-    case kModeTf32x3: return fits_by_d<kModeTf32x3>(d, kmax);
-    case kModeBf16x3: return fits_by_d<kModeBf16x3>(d, kmax);
-    default: return fits_by_d<kModeTf32>(d, kmax);
+    if (kmax < 1 || kmax > tc_chunk(d) || !encode_tiled()) return false;
+    switch (mode_of(resolve_prec(d, kmax, prec, rows))) {
+    case kModeBf16: return fits_by_d<kModeBf16>(d, kmax, rows);
+    case kModeTf32x3: return fits_by_d<kModeTf32x3>(d, kmax, rows);
+    case kModeBf16x3: return fits_by_d<kModeBf16x3>(d, kmax, rows);
+    default: return fits_by_d<kModeTf32>(d, kmax, rows);
     }
 }
 
-bool tc_sse_supported(int d, int k, int prec)
+bool tc_sse_supported(int d, int k, int prec, int64_t rows)
 {
-    return k >= 1 && tc_supported(d, std::min(k, 256), prec) &&
-           (k <= 256 || tc_supported(d, 256, prec));
+    return k >= 1 && tc_supported(d, std::min(k, tc_chunk(d)), prec, rows);
 }
 
 cudaError_t launch_lloyd_chunks_tc(const LloydBuffers &b, int d, int iter, int k, int prec, uint32_t *flags,
                                    int sm_count, cudaStream_t st, KTimer *kt)
 {
-    switch (mode_of(resolve_prec(d, 256, prec))) {
+    switch (mode_of(resolve_prec(d, tc_chunk(d), prec, b.rows))) {
     case kModeBf16: return lloyd_chunks_by_d<kModeBf16>(d, b, iter, k, flags, sm_count, st, kt);
     case kModeTf32x3: return lloyd_chunks_by_d<kModeTf32x3>(d, b, iter, k, flags, sm_count, st, kt);
     case kModeBf16x3: return lloyd_chunks_by_d<kModeBf16x3>(d, b, iter, k, flags, sm_count, st, kt);
@@ -1627,8 +1666,8 @@ cudaError_t launch_final_sse_tc(const float *x, int64_t n, int d, const float *c
                                 double *sse, uint32_t *ticket, int prec, uint32_t *flags, unsigned wait_limit,
                                 int sm_count, cudaStream_t st, KTimer *kt)
 {
-    const int ck = std::min(k, 256);
-    switch (mode_of(resolve_prec(d, ck, prec))) {
+    const int ck = std::min(k, tc_chunk(d));
+    switch (mode_of(resolve_prec(d, ck, prec, n))) {
     case kModeBf16: return sse_tc_by_d<kModeBf16>(d, x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
     case kModeTf32x3: return sse_tc_by_d<kModeTf32x3>(d, x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
     case kModeBf16x3: return sse_tc_by_d<kModeBf16x3>(d, x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
@@ -1640,7 +1679,7 @@ cudaError_t launch_lloyd_assign_tc(const LloydBuffers &b, const SegTable &t, int
                                    uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt)
 {
     if (!t.split) return cudaErrorInvalidValue;
-    switch (mode_of(resolve_prec(d, kmax, prec))) {
+    switch (mode_of(resolve_prec(d, kmax, prec, b.rows))) {
     case kModeBf16: return tc_by_d<kModeBf16>(b, t, d, iter, kmax, flags, sm_count, st, kt);
     case kModeTf32x3: return tc_by_d<kModeTf32x3>(b, t, d, iter, kmax, flags, sm_count, st, kt);
     case kModeBf16x3: return tc_by_d<kModeBf16x3>(b, t, d, iter, kmax, flags, sm_count, st, kt);

@@ -218,7 +218,7 @@ struct LloydBuffers {
     // rows words (or NULL): the tensor-core assignment's labels before the near ties are
     // decided, kept apart from `labels` so that the sums pass sees which rows moved
     int32_t *raw = nullptr;
-    // a single set of more than 256 centers on the tensor cores: the rows as one set of 256
+    // a single set of more than tc_chunk(d) centers on the tensor cores: the rows as one set of tc_chunk(d)
     // and of the remaining centers, with CTA splits (has_chunks), and 4 rows + 1 words of
     // scratch for the chunked search
     SegTable chunk256{}, chunkrem{};
@@ -243,13 +243,15 @@ cudaError_t launch_seg_sse(const float *pts, const SegTable &t, const int32_t *s
                            cudaStream_t st, KTimer *kt);
 
 // lloyd_tc.cu
-bool tc_supported(int d, int kmax, int prec);
+bool tc_supported(int d, int kmax, int prec, int64_t rows);
+// Most centers of one launch: a set's, or a chunk's of a whole-set search (256; 128 for d = 128).
+int tc_chunk(int d);
 // The SSE pass (labels and sum as launch_final_sse gives them) on the tensor cores for k
-// centers in chunks of up to 256.  t256 / trem: the n rows as one set of 256 centers and of
-// the k mod 256 remaining ones (k itself when k <= 256), with CTA splits; scratch: 4 n + 1
+// centers in chunks of up to tc_chunk(d).  t256 / trem: the n rows as one set of tc_chunk(d) centers and of
+// the remaining ones of the last chunk (k itself when it is the only one), with CTA splits; scratch: 4 n + 1
 // words (row state and the list of rows re-scored in float32).
-bool tc_sse_supported(int d, int k, int prec);
-// One Lloyd iteration of a single set of k > 256 centers on the tensor cores (b.has_chunks):
+bool tc_sse_supported(int d, int k, int prec, int64_t rows);
+// One Lloyd iteration of a single set of k > tc_chunk(d) centers on the tensor cores (b.has_chunks):
 // labels by the chunked search, then the exact sums; the update is launched separately.
 cudaError_t launch_lloyd_chunks_tc(const LloydBuffers &b, int d, int iter, int k, int prec, uint32_t *flags,
                                    int sm_count, cudaStream_t st, KTimer *kt);
