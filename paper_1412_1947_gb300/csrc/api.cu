@@ -122,6 +122,7 @@ struct pscl_job : Owner {
     std::vector<int64_t> seg_off;
     PeelBuffers pb{};
     bool peel_alloc = false;
+    uint32_t *scratch = nullptr;      // tensor-core stages: candidate masks, chunk state (scratch_words)
     LloydPlan lp;
     float *cl = nullptr;              // P x d local centers
     unsigned long long *acc_l = nullptr;
@@ -573,6 +574,11 @@ static int plan_subcluster(pscl_job *j, int64_t N, int32_t local_k, int32_t iter
     return plan_trace(j, iters);
 }
 
+// Words of a job's tensor-core scratch: 8 per row for the near ties' candidate masks, at least
+// the 4 per row + 1 of a chunked search's row state (none for widths the contraction leaves
+// to the float32 kernels).
+static size_t scratch_words(int64_t n, int d) { return d >= 16 ? 8 * (size_t)n + 8 : 0; }
+
 // The subcluster buffers every scheme uses (allocated once per job).
 static int alloc_subcluster_buffers(pscl_job *j)
 {
@@ -581,13 +587,9 @@ static int alloc_subcluster_buffers(pscl_job *j)
     if (!j->peel_alloc) {
         PeelBuffers &b = j->pb;
         b.x = j->x;
-        b.ord_ld = (n + 3) & ~(int64_t)3;
-        b.nbuckets = peel_buckets(n);
         TRY(A(j, &b.rnd, n));
         TRY(A(j, &b.pflag, 2 * (size_t)n));
-        TRY(A(j, &b.ord, (size_t)d * b.ord_ld));
-        TRY(A(j, &b.bcnt, (size_t)d * b.nbuckets));
-        TRY(A(j, &b.bcs, (size_t)d * b.nbuckets));
+        if (scratch_words(n, d)) TRY(A(j, &j->scratch, scratch_words(n, d)));
         TRY(A(j, &b.lidx, 2 * (size_t)n));
         TRY(A(j, &b.kpos, 2 * (size_t)n));
         TRY(A(j, &b.band_k32, n));
@@ -731,12 +733,10 @@ static size_t job_footprint(int64_t n, int d, int64_t N, int local_k, int final_
     } else if (host_input) {
         b += r256((size_t)n * d * 4);
     }
-    const int64_t ord_ld = (n + 3) & ~(int64_t)3;
-    const size_t nbk = peel_buckets(n);
-    // rnd, pflag, ord, bcnt, bcs, lidx, kpos, band_k32, band_pos, gkey, gpos, akey, apos, pcnt,
+    // rnd, pflag, the tensor-core scratch, lidx, kpos, band_k32, band_pos, gkey, gpos, akey, apos, pcnt,
     // perm, then xseg and the local labels
-    b += r256((size_t)n * 4) + r256(2 * (size_t)n) + r256((size_t)d * ord_ld * 4) + r256((size_t)d * nbk * 4) +
-         r256((size_t)d * nbk * 16) + 2 * r256(2 * (size_t)n * 4) + 2 * r256((size_t)n * 4) +
+    b += r256((size_t)n * 4) + r256(2 * (size_t)n) + (scratch_words(n, d) ? r256(scratch_words(n, d) * 4) : 0) +
+         2 * r256(2 * (size_t)n * 4) + 2 * r256((size_t)n * 4) +
          r256((size_t)n * 8) + r256((size_t)n * 4) + r256((size_t)n * 8) + r256((size_t)n * 4) +
          r256(256 * (size_t)perm_grid(n, sm) * 4) + r256((size_t)n * 4) +
          r256((size_t)n * d * 4) + r256((size_t)n * 4);
@@ -824,21 +824,18 @@ static int run_lloyd(pscl_job *j, const LloydPlan &p, const float *pts, float *c
     b.trace = trace;
     b.rows = p.rows;
     b.weights = weights;
-    // the near ties' candidate masks borrow the peel's bucket lists (d * ord_ld words, idle
-    // once the peel is done; 8 words per row fit whenever d >= 8)
-    if (j->pb.ord && (size_t)p.rows * 8 <= (size_t)j->d * (size_t)j->pb.ord_ld) b.tmask = j->pb.ord;
-    // and the labels before the ties are decided the peel's round of each point (n words; idle
+    b.tmask = j->scratch;            // the near ties' candidate masks
+    // the labels before the ties are decided the peel's round of each point (n words; idle
     // once the subclusters are packed)
     if (b.tmask) b.raw = reinterpret_cast<int32_t *>(j->pb.rnd);
-    // the pooled set past tc_chunk(d) centers: the chunked search's tables, its row state in the same
-    // idle lists (4 rows + 1 words)
+    // the pooled set past tc_chunk(d) centers: the chunked search's tables, its row state in the
+    // same scratch
     const int cw = tc_chunk(j->d);
-    if (stage == 1 && j->final_k > cw && j->fp256.d_split && b.tmask &&
-        (size_t)4 * p.rows + 1 <= (size_t)j->d * (size_t)j->pb.ord_ld) {
+    if (stage == 1 && j->final_k > cw && j->fp256.d_split && b.tmask) {
         b.chunk256 = j->fp256.table();
         b.chunkrem = (j->final_k % cw ? j->fprem : j->fp256).table();
         b.has_chunks = true;
-        b.chunk_scratch = j->pb.ord;
+        b.chunk_scratch = j->scratch;
     }
     b.wait_limit = j->wait_limit;
     b.tc_stall = j->test_stall == 2;
@@ -908,13 +905,12 @@ static int enqueue_cluster(pscl_job *j, bool events)
                   false, j->fprec, w));
     if (events) CU(cudaEventRecord(j->ev[4], st));
     // the SSE pass: on the tensor cores in chunks of tc_chunk(d) centers where the mode and the shape
-    // allow (its row state borrows the peel's bucket lists, idle by now), else float32
-    if (j->fprec != PSCL_PREC_FP32 && j->pb.ord && tc_sse_supported(j->d, j->final_k, j->fprec, j->n) &&
-        (size_t)4 * j->n + 1 <= (size_t)j->d * (size_t)j->pb.ord_ld && j->n < ((int64_t)1 << 31)) {
+    // allow (its row state in the scratch, idle by now), else float32
+    if (j->fprec != PSCL_PREC_FP32 && j->scratch && tc_sse_supported(j->d, j->final_k, j->fprec, j->n)) {
         const int cw = tc_chunk(j->d);
         const SegTable t256 = (j->final_k > cw ? j->sp256 : j->sprem).table();
         const SegTable trem = (j->final_k <= cw || j->final_k % cw ? j->sprem : j->sp256).table();
-        CU(launch_final_sse_tc(j->x, j->n, j->d, j->cf, j->final_k, t256, trem, j->pb.ord, j->labels, j->blk_sse,
+        CU(launch_final_sse_tc(j->x, j->n, j->d, j->cf, j->final_k, t256, trem, j->scratch, j->labels, j->blk_sse,
                                j->sse, j->tickets + 1, j->fprec, j->flags, j->wait_limit, j->ctx->sm_count, st,
                                &j->kt));
     } else {

@@ -25,11 +25,12 @@
 // boundaries:
 //   A. delta32_i in float32 (FMA chains, a row's pieces summed across the lanes that read
 //      it), kept as its bit pattern (order-preserving for non-negative floats), and a
-//      2048-bin histogram of key bits 31..21.  Points equal to L in an attribute are
-//      counted per attribute and flagged (the holders);
+//      2048-bin histogram of the keys, the bins fitted to the range the keys can lie in
+//      (DigitMap).  Points equal to L in an attribute are counted per attribute and flagged
+//      (the holders);
 //   B. per boundary, the first-digit bin holding its rank, and 2048-bin histograms of
-//      bits 20..10 inside those bins: each boundary's float32 key lies in a 22-bit prefix
-//      [A, B];
+//      the keys inside those bins: each boundary's float32 key lies in a range [A, B] of a
+//      few units in the last place;
 //   C. |delta32 - delta64| <= eps*delta32 + ea with eps = (d+4)*2^-23, ea = 2^-120, so the
 //      boundary's delta64 lies in [A(1-eps)-ea, B(1+eps)+ea]: a point whose bound lies
 //      below that interval is certainly before the boundary, one above it certainly
@@ -58,17 +59,19 @@
 // Points never move: CTA c owns the index slice [c n/G, (c+1) n/G) and keeps the ids of its
 // points left in a list, in ascending order, with their keys by list position.  Every
 // point gets its round in rnd[]; after the launch a stable counting sort by round packs
-// the subclusters (ascending index inside each).  The next landmark needs no pass over
-// the rows: before the first epoch a counting sort lists, per attribute, the point ids by
-// value bucket (buckets are monotone in the value); the minimum over the points left is
-// the smallest value left in the first bucket that still has a point left, and one bucket
-// pointer per attribute only moves forward (the buckets it passes hold no point left, and
-// points never come back), so each bucket emptied by removals is read once more in all.
+// the subclusters (ascending index inside each).  The next landmark differs from the last
+// one only in the attributes that lost their last holder (the commit knows them), usually
+// one to three: the compaction that drops the committed points is followed by a minimum of
+// those attributes over the points it kept, the same columns the key update reads next.
+// (Sorted bucket lists per attribute, built before the first epoch and walked from their low
+// end, took 27-34 ms of atomics at 2^24 x 64, 1 ms at 400000 x 128, and 42 us an epoch of
+// dependent loads on clustered 2-D data.)
 //
 // All epochs run in one persistent cooperative launch, the phases separated by grid
 // barriers.  Every barrier wait is bounded; a CTA that gives up sets the abort flag, every
 // other CTA then leaves at its next wait, and the host sees PSCL_ETIMEOUT.
 #include <algorithm>
+#include <cstddef>
 
 #include "pscl_internal.cuh"
 
@@ -80,8 +83,6 @@ constexpr int kW = kThreads / 32;
 constexpr uint32_t kInfBits = 0x7f800000u;
 constexpr uint32_t kGone = 0xFFFFFFFFu;       // key past the end of a list
 constexpr uint32_t kNone = 0xFFFFFFFFu;       // round of a point not assigned (yet)
-constexpr int kBkGroup = 16;                   // attributes per sweep of the bucket build
-constexpr int kBkUnroll = 4;                   // (point, attribute) pairs per thread at a time
 constexpr int kIncMax = 8;                     // moved attributes a pass may update keys for
 constexpr int kKeyCache = 4096;               // keys and ids of a slice kept in shared memory, if it fits
 constexpr int kSelBins = 2048;
@@ -104,7 +105,6 @@ constexpr uint8_t kFlBand = 0x7E;
 constexpr uint8_t kFlNone = 0x7F;
 constexpr uint32_t kPosMask = 0x7FFFFFFFu;    // a band entry's id; bit 31 carries its hold flag
 constexpr int kDefaultRounds = 32;            // rounds per distance pass by default
-constexpr int kSlotsSmem = kScrWords / kHistBins;   // second-digit histograms counted in shared memory
 constexpr unsigned kDefaultSpin = 1u << 25;   // ~1-2 s of polling per barrier at most
 
 // ------------------------------------------------------------------ block helpers
@@ -328,16 +328,56 @@ __device__ __forceinline__ uint64_t dff_key(const float *__restrict__ row, const
     return (uint64_t)__double_as_longlong(v);
 }
 
-// Cut-offs of phase C from the 22-bit key prefix [A, B] of a boundary's float32 key.
+// The digits of the keys in one pass.  Every key left lies in [base, top] (the range's
+// derivation: see its assignment in the kernel; a key below base only widens a band), cut
+// into bins of 2^sh values (bin 0: the keys below base) and a bin into sub-bins of 2^ss (2^s0
+// for bin 0).  With the range spread over the whole first digit (before, its bits were the
+// key's top 11: two bits of mantissa, a few bins holding most points), the second digit
+// reaches down to single keys or nearly, so the bands shrink to the float32 error, and few
+// points share a boundary's bin: phase B counts 2000 keys instead of half of them.
+struct DigitMap {
+    uint32_t base;
+    int sh, ss, s0;
+    __device__ __forceinline__ uint32_t bin(uint32_t k) const
+    {
+        return k < base ? 0u : min((uint32_t)kHistBins - 1u, 1u + ((k - base) >> sh));
+    }
+    __device__ __forceinline__ uint32_t low(uint32_t b) const { return b ? base + ((b - 1u) << sh) : 0u; }
+    __device__ __forceinline__ uint32_t sub(uint32_t k, uint32_t b) const
+    {
+        return min((uint32_t)kHistBins - 1u, (k - low(b)) >> (b ? ss : s0));
+    }
+    // the keys of a sub-bin: [A, B]
+    __device__ __forceinline__ void range(uint32_t b, uint32_t sb, uint32_t &A, uint32_t &B) const
+    {
+        const int s = b ? ss : s0;
+        A = low(b) + (sb << s);
+        B = A + ((1u << s) - 1u);
+        if (sb == (uint32_t)kHistBins - 1u) B = b == (uint32_t)kHistBins - 1u ? kInfBits - 1u : max(B, low(b + 1u) - 1u);
+    }
+};
+
+__device__ __forceinline__ DigitMap digit_map(uint32_t base, uint32_t top)
+{
+    DigitMap m;
+    m.base = base;
+    const uint32_t span = top > base ? top - base : 0u;
+    m.sh = max(0, 21 - __clz(span | 1u));                // span >> sh <= 2047 - 1
+    if ((span >> m.sh) > (uint32_t)kHistBins - 3u) m.sh++;
+    m.ss = max(0, m.sh - 11);
+    m.s0 = max(0, 21 - __clz(base | 1u));
+    return m;
+}
+
+// Cut-offs of phase C from the range [kA, kB] of a boundary's float32 key.
 // With |delta32 - delta64| <= eps delta32 + ea (eps <= 1/3) the boundary's delta64 lies in
 // [A(1-eps) - ea, B(1+eps) + ea]; a point is certainly before it if delta32 (1+eps) + ea
 // is below that interval, which holds for delta32 < A(1-2eps) - 2ea, and certainly after
 // it if delta32 (1-eps) - ea is above it, which holds for delta32 > B(1+3eps) + 3ea.  Both
 // cut-offs are evaluated in float32 rounded towards the safe side.
-__device__ void band_cutoffs(uint32_t b0, uint32_t b1, float eps, float ea, uint32_t &in_key, uint32_t &out_key)
+__device__ void band_cutoffs(uint32_t kA, uint32_t kB, float eps, float ea, uint32_t &in_key, uint32_t &out_key)
 {
-    const uint32_t lo = (b0 << 21) | (b1 << 10), hi = lo | 0x3FFu;
-    const float A = __uint_as_float(lo), B = __uint_as_float(hi);
+    const float A = __uint_as_float(kA), B = __uint_as_float(kB);
     const float in_thr = __fsub_rd(__fmul_rd(A, __fsub_rd(1.0f, 2.0f * eps)), 2.0f * ea);
     const float out_thr = __fadd_ru(__fmul_ru(B, __fadd_ru(1.0f, __fmul_ru(3.0f, eps))), __fmul_ru(3.0f, ea));
     in_key = in_thr > 0.0f ? __float_as_uint(in_thr) : 0u;
@@ -530,15 +570,6 @@ __device__ void select_kth(KeyAt key_at, PosAt pos_at, uint32_t nb, uint32_t nee
     if (!select_fast(key_at, pos_at, nb, need, scratch, K, Pp)) select_radix(key_at, pos_at, nb, need, K, Pp);
 }
 
-// ------------------------------------------------------------------ buckets
-// Bucket of a scaled value (in [0, 1]) among nb equal buckets: monotone in the value.
-__device__ __forceinline__ uint32_t bucket_of(float v, uint32_t nb)
-{
-    v = fminf(fmaxf(v, 0.0f), 1.0f);
-    const uint32_t b = __float2uint_rz(v * (float)nb);
-    return b < nb ? b : nb - 1u;
-}
-
 // ------------------------------------------------------------------ the kernel
 struct PeelArgs {
     const float *x;
@@ -547,13 +578,8 @@ struct PeelArgs {
     int64_t n, N, S;
     uint32_t *rnd;
     uint8_t *pflag;              // 2 x n: the state byte of each list position
-    uint32_t *ord;               // d x ord_ld: point ids by value bucket, per attribute
-    uint32_t *bcnt;              // d x nbk: bucket counts, then cursors (zeroed before)
-    uint4 *bcs;                  // d x nbk: (points left, first entry, end entry, 0)
     uint32_t *lidx;              // 2 x n: per CTA slice, the ids of its points left (not kc; two lists)
     uint32_t *kpos;              // 2 x n: their keys by list position
-    int64_t ord_ld;
-    uint32_t nbk;
     uint32_t *band_k32;
     uint32_t *band_pos;
     uint64_t *gkey;
@@ -566,6 +592,8 @@ struct PeelArgs {
     uint32_t kmax;               // rounds per distance pass
     uint32_t spin;               // polls of a barrier wait before it gives up
     uint32_t stall;              // test hook: the first barrier awaits one arrival too many
+    int transpose;               // the launch writes xt itself (xt_out)
+    float *xt_out;
 };
 
 // rows a thread keeps in flight at once (64 floats of rows at most)
@@ -617,27 +645,26 @@ __device__ __forceinline__ void note_holder(const float *__restrict__ row, const
 }
 
 // Phase A: every live point's float32 key, stored by list position (shared memory when
-// kc, else kpos: the slice's keys) and counted in the first-digit histogram sh; holders
+// kc, else kpos: the slice's keys) and counted in the first-digit histogram sh (but in the
+// first epoch); holders
 // counted per attribute of jm and flagged in their position's state byte (pfl: the
 // slice's, by list position).  Out of line, so that the register allocation of the
 // kernel's other phases does not carry its loads in flight.
 template <int D>
 __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float *Ls, int d, uint32_t n_live,
                                         uint32_t s0, bool first, bool kc, const uint32_t *sid, const uint32_t *glin,
-                                        uint32_t *skey, uint32_t *kpos, uint32_t *sh, uint8_t *pfl, uint32_t *chold,
-                                        const uint32_t *jm)
+                                        uint32_t *skey, uint32_t *kpos, uint32_t *sh, const DigitMap *dm,
+                                        uint8_t *pfl, uint32_t *chold, const uint32_t *jm)
 {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const DigitMap mp = *dm;
     auto LID = [&](uint32_t q) -> uint32_t { return first ? s0 + q : kc ? sid[q] : __ldcg(&glin[q]); };
     auto key_out = [&](bool live, uint32_t pos, uint32_t k) {
         if (live) {
             if (kc) skey[pos] = k;
             else kpos[pos] = k;
+            if (!first) atomicAdd(&sh[mp.bin(k)], 1u);       // the first epoch fits the bins to its keys
         }
-        // the keys of a pass crowd into a few bins: one shared atomic per bin and warp
-        const uint32_t b = live ? (k >> 21) : kGone;
-        const uint32_t peers = __match_any_sync(0xffffffffu, b);
-        if (live && lane == __ffs(peers) - 1) atomicAdd(&sh[b], (uint32_t)__popc(peers));
     };
     if constexpr (kCoopRows<D>()) {
         constexpr int P = kCoopLanes<D>();                 // lanes per row
@@ -770,13 +797,16 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
 template <int D>
 __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float *__restrict__ xt, uint32_t n, int d,
                                        uint32_t n_live, bool kc, const uint32_t *sid, const uint32_t *glin,
-                                       uint32_t *skey, uint32_t *kpos, uint32_t *sh, uint8_t *pfl, uint32_t *chold,
-                                       uint32_t nj, const int *jj, const float *jo, const float *jl)
+                                       uint32_t *skey, uint32_t *kpos, uint32_t *sh, const DigitMap *dm,
+                                       uint8_t *pfl, uint32_t *chold, uint32_t nj, const int *jj, const float *jo,
+                                       const float *jl)
 {
     constexpr int U = 4;                                   // list positions per thread in flight
-    const int t = threadIdx.x, lane = t & 31;
+    const int t = threadIdx.x;
+    const DigitMap mp = *dm;
     // attribute j of point i at src[i * ps + j * as]: the by-attribute copy (a CTA's ids
-    // ascend, so a warp's loads fall close together) or the rows
+    // ascend, so a warp's loads fall close together) or the rows; read through L2, since this
+    // launch may have written the copy
     const float *src = xt ? xt : x;
     const size_t ps = xt ? 1 : (size_t)(D > 0 ? D : d), as = xt ? (size_t)n : 1;
     for (uint32_t q0 = 0; q0 < n_live; q0 += U * kThreads) {          // block-uniform bound
@@ -795,7 +825,7 @@ __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float 
             const float ln = jl[i], c = __fsub_rn(ln, jo[i]), sm = __fadd_rn(ln, jo[i]);
             float v[U];
 #pragma unroll
-            for (int u = 0; u < U; u++) v[u] = id[u] != kGone ? __ldg(&src[(size_t)id[u] * ps + (size_t)j * as]) : ln;
+            for (int u = 0; u < U; u++) v[u] = id[u] != kGone ? __ldcg(&src[(size_t)id[u] * ps + (size_t)j * as]) : ln;
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 acc[u] = __fmaf_rn(c, __fmaf_rn(-2.0f, v[u], sm), acc[u]);
@@ -815,10 +845,8 @@ __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float 
                 if (kc) skey[qi] = k;
                 else kpos[qi] = k;
                 if ((hold >> u) & 1u) pfl[qi] |= kFlHold;
+                atomicAdd(&sh[mp.bin(k)], 1u);
             }
-            const uint32_t b = live ? (k >> 21) : kGone;
-            const uint32_t peers = __match_any_sync(0xffffffffu, b);
-            if (live && lane == __ffs(peers) - 1) atomicAdd(&sh[b], (uint32_t)__popc(peers));
         }
     }
 }
@@ -991,114 +1019,55 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
     if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
 }
 
-// The next landmark (attributes j_first, j_first + j_step, ...): in each attribute the
-// smallest value among the points left (rnd >= live_from), found from the bucket order:
-// from the attribute's bucket pointer on, the first bucket whose entries include a point
-// left holds it.  A point taken stays taken (live_from only grows), so each bucket's start
-// is moved past the entries found gone and a bucket whose start reaches its end is passed
-// for good: every entry is found gone at most once per run.  Buckets are examined kThreads
-// at a time, a thread peeking at the next kPeek entries of its bucket (their loads issued
-// together); a bucket that still has entries after those, and the first bucket with a
-// point left, are scanned by the whole CTA.
-constexpr int kPeek = 16;
+// The next landmark: in each attribute that lost its last holder (lost[0 .. nl)), the smallest
+// value among the points left, here those of one CTA's list, kMinAttrs attributes and
+// kMinBatch points per thread at a time (their loads issued together), added to the grid's
+// minimum (values lie in [0, 1], so their bits order like them).
+constexpr int kMinAttrs = 4;
+constexpr int kMinBatch = 4;
 
-__device__ __noinline__ void find_landmark(const PeelArgs &a, int j_first, int j_step, uint32_t live_from)
+__device__ __noinline__ void lost_minima(const float *__restrict__ x, const float *__restrict__ xt, uint32_t n, int d,
+                                         uint32_t n_live, bool kc, const uint32_t *sid, const uint32_t *glist,
+                                         const uint32_t *lost, uint32_t nl, uint32_t *Lbits)
 {
-    PeelCtl *ctl = a.ctl;
-    const int d = a.d;
-    const uint32_t nbk = a.nbk;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    __shared__ uint32_t red_a[kW], red_u[kW], red_b[kW], red_p[kW];
-    __shared__ uint32_t s_st, s_en;
-    for (int j = j_first; j >= 0 && j < d; j += j_step) {
-        uint4 *bj = a.bcs + (size_t)j * nbk;
-        const uint32_t *oj = a.ord + (size_t)j * a.ord_ld;
-        uint32_t b = __ldcg(&ctl->lptr[j]);       // the buckets before b hold no point left
-        uint32_t mnb = kGone;
-        while (b < nbk) {
-            // bucket b + t: 1 = a point left among its next kPeek entries, 2 = entries left
-            // to look at after those, 0 = nothing left
-            const uint32_t bb = b + (uint32_t)t;
-            uint4 e = bb < nbk ? __ldcg(&bj[bb]) : make_uint4(0u, 0u, 0u, 0u);
-            int state = 0;
-            if (e.y < e.z) {
-                uint32_t ids[kPeek];
+    __shared__ uint32_t s_min[kMinAttrs];
+    const int t = threadIdx.x, lane = t & 31;
+    const float *src = xt ? xt : x;
+    const size_t ps = xt ? 1 : (size_t)d, as = xt ? (size_t)n : 1;
+    for (uint32_t l0 = 0; l0 < nl; l0 += kMinAttrs) {
+        const float *col[kMinAttrs];
+        uint32_t mn[kMinAttrs];
 #pragma unroll
-                for (int i = 0; i < kPeek; i++) ids[i] = e.y + i < e.z ? __ldcg(&oj[e.y + i]) : kGone;
-                uint32_t first = kPeek;
-#pragma unroll
-                for (int i = kPeek - 1; i >= 0; i--)
-                    if (ids[i] != kGone && __ldcg(&a.rnd[ids[i]]) >= live_from) first = (uint32_t)i;
-                const uint32_t adv = first < kPeek ? first : min((uint32_t)kPeek, e.z - e.y);
-                if (adv) {
-                    e.y += adv;
-                    reinterpret_cast<uint32_t *>(&bj[bb])[1] = e.y;     // entries before e.y are gone
-                }
-                state = first < kPeek ? 1 : (e.y < e.z ? 2 : 0);
-            }
-            uint32_t fa = warp_min(state == 1 ? bb : kGone), fu = warp_min(state == 2 ? bb : kGone);
-            if (lane == 0) {
-                red_a[w] = fa;
-                red_u[w] = fu;
-            }
-            __syncthreads();
-            fa = red_a[0];
-            fu = red_u[0];
-#pragma unroll
-            for (int q = 1; q < kW; q++) {
-                fa = min(fa, red_a[q]);
-                fu = min(fu, red_u[q]);
-            }
-            const uint32_t fb = min(fa, fu);
-            if (bb == fb) {
-                s_st = e.y;
-                s_en = e.z;
-            }
-            __syncthreads();
-            if (fb == kGone) {                     // kThreads buckets with nothing left
-                b += kThreads;
-                continue;
-            }
-            // bucket fb, the whole CTA: the smallest value among its entries left and the
-            // first of them (its start moves there, or to its end)
-            const uint32_t st = s_st, en = s_en;
-            uint32_t lm = kGone, fp = en;
-            for (uint32_t q = st + t; q < en; q += kThreads) {
-                const uint32_t id = __ldcg(&oj[q]);
-                if (__ldcg(&a.rnd[id]) >= live_from) {
-                    lm = min(lm, __float_as_uint(__ldg(&a.x[(size_t)id * d + j])));
-                    fp = min(fp, q);
-                }
-            }
-            lm = warp_min(lm);
-            fp = warp_min(fp);
-            if (lane == 0) {
-                red_b[w] = lm;
-                red_p[w] = fp;
-            }
-            __syncthreads();
-            lm = red_b[0];
-            fp = red_p[0];
-#pragma unroll
-            for (int q = 1; q < kW; q++) {
-                lm = min(lm, red_b[q]);
-                fp = min(fp, red_p[q]);
-            }
-            if (t == 0 && fp > st) reinterpret_cast<uint32_t *>(&bj[fb])[1] = fp;
-            __syncthreads();
-            if (lm != kGone) {
-                mnb = lm;
-                b = fb;
-                break;
-            }
-            b = fb + 1;                            // every entry of fb is gone
+        for (int i = 0; i < kMinAttrs; i++) {       // past the last one, the first of the group again
+            const uint32_t j = __ldcg(&lost[l0 + i < nl ? l0 + i : l0]);
+            col[i] = src + (size_t)j * as;
+            mn[i] = kInfBits;
         }
-        if (t == 0) {
-            const uint32_t nb = mnb == kGone ? kInfBits : mnb;
-            ctl->lptr[j] = b;
-            if (nb != __ldcg(&ctl->Lbits[j])) ctl->chold[j] = 0;    // a new value: its holders are counted again
-            ctl->Lbits[j] = nb;
+        if (t < kMinAttrs) s_min[t] = kInfBits;
+        __syncthreads();
+        const uint32_t na = min((uint32_t)kMinAttrs, nl - l0);
+        for (uint32_t q0 = 0; q0 < n_live; q0 += kMinBatch * kThreads) {
+            uint32_t id[kMinBatch];
+#pragma unroll
+            for (int u = 0; u < kMinBatch; u++) {
+                const uint32_t qi = min(q0 + u * kThreads + t, n_live - 1u);
+                id[u] = kc ? sid[qi] : __ldcg(&glist[qi]);
+            }
+#pragma unroll
+            for (int i = 0; i < kMinAttrs; i++)
+                if (i < (int)na) {
+#pragma unroll
+                    for (int u = 0; u < kMinBatch; u++)
+                        mn[i] = min(mn[i], __float_as_uint(__ldcg(&col[i][(size_t)id[u] * ps])));
+                }
         }
+#pragma unroll
+        for (int i = 0; i < kMinAttrs; i++) {
+            const uint32_t m = __reduce_min_sync(0xffffffffu, mn[i]);
+            if (lane == 0 && i < (int)na) atomicMin(&s_min[i], m);
+        }
+        __syncthreads();
+        if (t < (int)na && s_min[t] != kInfBits) atomicMin(&Lbits[__ldcg(&lost[l0 + t])], s_min[t]);
     }
 }
 
@@ -1108,11 +1077,12 @@ __device__ __noinline__ void find_landmark(const PeelArgs &a, int j_first, int j
 // second-digit bins [64 i, 64 i + 64) in two halves, a warp scan finds the lane holding
 // the rank, and that lane walks the half holding it (its loads issued together).
 __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t Kb, uint32_t N, int d, float keps, float kabs,
-                                             const uint32_t *sb, const uint32_t *sr, const uint32_t *sslot,
-                                             const uint32_t *sbin, uint32_t nslot)
+                                             const DigitMap *dm, const uint32_t *sb, const uint32_t *sr,
+                                             const uint32_t *sslot, const uint32_t *sbin, uint32_t nslot)
 {
     __shared__ uint32_t s_b1[kMaxEpoch];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const DigitMap mp = *dm;
     if (t < kMaxEpoch) s_b1[t] = 0;
     // the rounds this landmark can serve: up to the one in which the last holder of some
     // attribute's landmark value leaves (the landmark changes after it).  That holder's key
@@ -1123,7 +1093,7 @@ __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t Kb, uint32_t
     uint32_t m = kGone;
     for (int j = t; j < d; j += kThreads) m = min(m, __ldcg(&ctl->hmax[j]));
     m = block_min(m);
-    const uint32_t mb0 = m >> 21, mb1 = (m >> 10) & (kHistBins - 1);
+    const uint32_t mb0 = mp.bin(m), mb1 = mp.sub(m, mb0);
     int slot = -1;
     for (uint32_t q = 0; q < nslot; q++)
         if (sbin[q] == mb0) slot = (int)q;
@@ -1170,29 +1140,34 @@ __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t Kb, uint32_t
         }
     }
     __syncthreads();
-    if (t == 0) {
-        uint32_t ng = 0, gi = 0, go = 0;
-        for (uint32_t q = 0; q < K; q++) {
-            uint32_t ik, ok;
-            band_cutoffs(sb[q], s_b1[q], keps, kabs, ik, ok);
-            if (ng > 0 && ik <= go) {
-                go = max(go, ok);
-                ctl->g_out[ng - 1] = go;
-                ctl->g_q2[ng - 1] = q;
-            } else {
-                gi = ik;
-                go = ok;
-                ctl->g_in[ng] = gi;
-                ctl->g_out[ng] = go;
-                ctl->g_q1[ng] = q;
-                ctl->g_q2[ng] = q;
-                ng++;
+    static_assert(kMaxEpoch <= 32, "a lane per boundary");
+    if (w == 0) {
+        // lane q: boundary q's cut-offs, ascending with q; a boundary whose band starts past
+        // the one before it ends opens a group
+        uint32_t A = 0, B = 0, ik = 0, ok = 0;
+        if (lane < (int)K) {
+            mp.range(sb[lane], s_b1[lane], A, B);
+            band_cutoffs(A, B, keps, kabs, ik, ok);
+        }
+        const uint32_t pk = __shfl_up_sync(0xffffffffu, ok, 1);
+        const uint32_t open = __ballot_sync(0xffffffffu, lane < (int)K && (lane == 0 || ik > pk));
+        if (lane < (int)K) {
+            const uint32_t g = (uint32_t)__popc(open & ((2u << lane) - 1u)) - 1u;
+            if ((open >> lane) & 1u) {
+                ctl->g_in[g] = ik;
+                ctl->g_q1[g] = (uint32_t)lane;
+            }
+            if (lane == (int)K - 1 || ((open >> (lane + 1)) & 1u)) {
+                ctl->g_out[g] = ok;
+                ctl->g_q2[g] = (uint32_t)lane;
             }
         }
-        ctl->n_groups = ng;
-        ctl->n_slots = nslot;
-        ctl->k_eff = K;
-        ctl->kref = __uint_as_float(sb[0] << 21);
+        if (lane == 0) {
+            ctl->n_groups = (uint32_t)__popc(open);
+            ctl->n_slots = nslot;
+            ctl->k_eff = K;
+            ctl->kref = __uint_as_float(A);
+        }
     }
 }
 
@@ -1225,14 +1200,24 @@ __device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, ui
     qs = block_min(qs);
     const uint32_t kc_ = qs < K ? qs + 1u : K;
     const bool changed = qs < K;
-    // the holders that leave with the committed rounds (an attribute whose landmark value
-    // changes has its count cleared by find_landmark and counted again by the next pass)
+    // the holders that leave with the committed rounds; an attribute that has none left gets
+    // a new landmark value (the minimum over the points left, taken next) and its holders are
+    // counted by the next pass
+    __shared__ uint32_t s_nl;
+    if (t == 0) s_nl = 0;
+    __syncthreads();
     for (int j = t; j < d; j += kThreads) {
         uint32_t gone = 0;
 #pragma unroll
         for (int r = 0; r < kMaxEpoch; r++) gone += r < (int)kc_ ? __ldcg(&ctl->hcnt[j][r]) : 0u;
-        ctl->chold[j] = __ldcg(&ctl->chold[j]) - gone;
+        const uint32_t left = __ldcg(&ctl->chold[j]) - gone;
+        ctl->chold[j] = left;
+        if (left == 0u) {
+            ctl->lost[atomicAdd(&s_nl, 1u)] = (uint32_t)j;
+            ctl->Lbits[j] = kInfBits;
+        }
     }
+    __syncthreads();
     if (t < (int)K && __ldcg(&ctl->cert[t]) + __ldcg(&ctl->bnd[t]) != N) atomicOr(&a.flags[1], 1u);
     if (changed) {
         for (int b = t; b < kHistBins; b += kThreads) ctl->h0[b] = 0;
@@ -1244,9 +1229,53 @@ __device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, ui
     if (t == 0) {
         ctl->k_commit = kc_;
         ctl->l_changed = changed ? 1u : 0u;
+        ctl->n_lost = s_nl;
+        // every point left lies at or past the start of the last committed boundary's band
+        const uint32_t ng = __ldcg(&ctl->n_groups);
+        uint32_t g = 0;
+        while (g + 1 < ng && __ldcg(&ctl->g_q2[g]) < kc_ - 1u) g++;
+        ctl->klast = __ldcg(&ctl->g_in[g]);
         ctl->epochs += 1;
         ctl->passes += need_keys ? 1u : 0u;
     }
+}
+
+// ------------------------------------------------------------------ the points by attribute
+// x (n x d, by point) into xt (d x n, by attribute) for the landmark's minima and the key
+// updates: 32 x 32 tiles through shared memory, so that both the reads (32 attributes of a
+// point) and the writes (32 points of an attribute) are coalesced.  The peel's own launch
+// makes it for small sets, whose few tiles per CTA cost less than another launch; larger ones
+// take a launch of their own before it, at full occupancy (2^20 x 16: 240 us inside the
+// peel's launch, 25 us outside).
+constexpr size_t kTransposeBytes = size_t(1) << 20;
+
+__device__ __forceinline__ void transpose_tiles(const float *__restrict__ x, int64_t n, int d, float *__restrict__ xt,
+                                                float (*tile)[33])
+{
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t tiles_c = (d + 31) / 32;
+    const int64_t tiles = (n + 31) / 32 * tiles_c;
+    for (int64_t tt = blockIdx.x; tt < tiles; tt += gridDim.x) {
+        const int64_t r0 = tt / tiles_c * 32;
+        const int c0 = (int)(tt % tiles_c) * 32;
+        for (int k = ty; k < 32; k += kThreads / 32) {
+            const int64_t r = r0 + k;
+            if (r < n && c0 + tx < d) tile[k][tx] = __ldg(&x[r * d + c0 + tx]);
+        }
+        __syncthreads();
+        for (int k = ty; k < 32; k += kThreads / 32) {
+            const int64_t r = r0 + tx;
+            if (r < n && c0 + k < d) xt[(size_t)(c0 + k) * (size_t)n + (size_t)r] = tile[tx][k];
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) k_transpose(const float *__restrict__ x, int64_t n, int d,
+                                                        float *__restrict__ xt)
+{
+    __shared__ float tile[32][33];
+    transpose_tiles(x, n, d, xt, tile);
 }
 
 // A CTA's list of points left, by list position: ids, float32 keys and state bytes; in
@@ -1340,11 +1369,12 @@ __device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L,
 // lies before live_from leave it; dropped assignments are reset; with the landmark kept,
 // the committed keys leave the first-digit histogram.  Returns the points left.
 __device__ __noinline__ uint32_t compact_shared(const PeelArgs &a, const ListView &L, uint32_t n_live, uint32_t r0,
-                                                uint32_t live_from, bool changed, uint32_t *scr)
+                                                uint32_t live_from, bool changed, const DigitMap *dmp, uint32_t *scr)
 {
     PeelCtl *ctl = a.ctl;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
+    const DigitMap dm = *dmp;
     uint8_t *pfl = L.sfl;
     if (!changed)
         for (int b = t; b < kHistBins; b += kThreads) scr[b] = 0;
@@ -1411,7 +1441,7 @@ __device__ __noinline__ uint32_t compact_shared(const PeelArgs &a, const ListVie
                 if (rv[q] != kNone) a.rnd[ids[q]] = kNone;       // an assignment dropped
             } else if (valid && !changed) {
                 // the next epoch keeps these keys: the committed ones leave the histogram
-                atomicAdd(&scr[keys[q] >> 21], 1u);
+                atomicAdd(&scr[dm.bin(keys[q])], 1u);
             }
         }
         done += woff[kQT * kW];
@@ -1432,11 +1462,12 @@ __device__ __noinline__ uint32_t compact_shared(const PeelArgs &a, const ListVie
 // subclusters are packed by a counting sort over rnd afterwards), claiming slots with one
 // shared atomic per 32 positions; no block barrier inside.  Returns the points left.
 __device__ __noinline__ uint32_t compact_global(const PeelArgs &a, const ListView &L, uint32_t n_live, uint32_t r0,
-                                                uint32_t live_from, bool changed, uint32_t *scr)
+                                                uint32_t live_from, bool changed, const DigitMap *dmp, uint32_t *scr)
 {
     PeelCtl *ctl = a.ctl;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
+    const DigitMap dm = *dmp;
     __shared__ uint32_t s_out;
     if (!changed)
         for (int b = t; b < kHistBins; b += kThreads) scr[b] = 0;
@@ -1475,7 +1506,7 @@ __device__ __noinline__ uint32_t compact_global(const PeelArgs &a, const ListVie
                 L.gfl2[o] = (uint8_t)((fls[q] & kFlHold) | kFlNone);
                 if (rvs[q] != kNone) a.rnd[ids[q]] = kNone;          // an assignment dropped
             } else if (valid && !changed) {
-                atomicAdd(&scr[keys[q] >> 21], 1u);
+                atomicAdd(&scr[dm.bin(keys[q])], 1u);
             }
             ob += __popc(bk[q]);
         }
@@ -1505,7 +1536,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     __shared__ uint32_t s_gin[kMaxEpoch], s_gout[kMaxEpoch], s_gq2[kMaxEpoch];
     __shared__ uint32_t s_cc[kMaxEpoch], s_gc[kMaxEpoch];
     __shared__ uint32_t s_nslot, s_glast;
-    __shared__ uint8_t s_map[kHistBins];
+    __shared__ __align__(4) uint8_t s_map[kHistBins];
     // the previous epoch's landmark; the attributes whose landmark value is new (mask) and,
     // for an update of the keys, those attributes with their old and new values
     __shared__ float Lold[D > 0 ? D : kMaxD];
@@ -1515,20 +1546,15 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     __shared__ uint32_t s_nj;
     __shared__ int s_inc;
     __shared__ float s_keps, s_kabs;
+    __shared__ DigitMap s_dm;
     PeelCtl *ctl = a.ctl;
     const int d = a.d;
     const uint32_t n = (uint32_t)a.n, N = (uint32_t)a.N;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const unsigned G = gridDim.x, c = blockIdx.x;
     const unsigned lim = a.spin;
-    // With 16 CTAs or more, the last Gl CTAs own no points and only build landmarks, which
-    // then overlaps with the others' compaction; otherwise every CTA does both.
-    const int Gl = G >= 16 ? min(d, (int)(G / 8)) : 0;
-    const unsigned Gs = G - (unsigned)Gl;
-    const uint32_t s0 = c < Gs ? (uint32_t)((uint64_t)c * n / Gs) : n;
-    const uint32_t s1 = c < Gs ? (uint32_t)((uint64_t)(c + 1) * n / Gs) : n;
-    const int lm_first = Gl ? (int)c - (int)Gs : (int)(G - 1 - c);
-    const int lm_step = Gl ? Gl : (int)G;
+    const uint32_t s0 = (uint32_t)((uint64_t)c * n / G);
+    const uint32_t s1 = (uint32_t)((uint64_t)(c + 1) * n / G);
     uint32_t n_live = s1 - s0;           // points of the slice left
     const bool kc = s1 - s0 <= (uint32_t)kKeyCache;   // the list and its keys stay in shared memory
     // slices beyond the key cache alternate between two lists in global memory
@@ -1537,91 +1563,20 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     uint8_t *gfl = a.pflag + s0, *gfl2 = a.pflag + n + s0;
     uint8_t *pfl = kc ? sfl : gfl;                      // the slice's state bytes by list position
     unsigned gen = 0;
-    if (kc)
-        for (uint32_t q = t; q < s1 - s0; q += kThreads) sfl[q] = kFlNone;
-
-    // ---- before the first epoch: per attribute, the point ids by value bucket (counting sort)
-    // The attributes go in groups of kBkGroup, each group one grid-stride sweep over its
-    // (point, attribute) pairs, kBkUnroll pairs per thread at a time (their loads, then
-    // their atomics, then their stores, so that each thread keeps several of each in
-    // flight).  A sweep writes the lists through kBkGroup x nbk cursors, few enough that
-    // the partly written sectors at the cursors stay in L2 until they fill.
+    // ---- before the first epoch: the control block (but for its first words, cleared by the
+    // host) and the slice's state; then the points by attribute where the launch makes them
     {
-        const uint32_t nbk = a.nbk;
-        const uint32_t stride = G * (uint32_t)kThreads;
-        const uint32_t e0 = c * (uint32_t)kThreads + (uint32_t)t;
-        for (int pass = 0; pass < 2; pass++) {
-            for (int j0 = 0; j0 < d; j0 += kBkGroup) {
-                const uint32_t w = (uint32_t)min(kBkGroup, d - j0);
-                const uint32_t si = stride / w, sj = stride % w;
-                uint32_t i = e0 / w, j = e0 % w;
-                while (i < n) {
-                    uint32_t pi[kBkUnroll], pj[kBkUnroll], pb[kBkUnroll];
-#pragma unroll
-                    for (int u = 0; u < kBkUnroll; u++) {
-                        pi[u] = i;
-                        pj[u] = (uint32_t)j0 + j;
-                        pb[u] = i < n ? bucket_of(__ldg(&a.x[(size_t)i * d + j0 + j]), nbk) : 0u;
-                        i += si;
-                        j += sj;
-                        if (j >= w) {
-                            j -= w;
-                            i++;
-                        }
-                    }
-                    if (pass == 0) {
-#pragma unroll
-                        for (int u = 0; u < kBkUnroll; u++)
-                            if (pi[u] < n) atomicAdd(&a.bcnt[(size_t)pj[u] * nbk + pb[u]], 1u);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < kBkUnroll; u++)
-                            if (pi[u] < n) pb[u] = atomicAdd(&a.bcnt[(size_t)pj[u] * nbk + pb[u]], 1u);
-#pragma unroll
-                        for (int u = 0; u < kBkUnroll; u++)
-                            if (pi[u] < n) a.ord[(size_t)pj[u] * a.ord_ld + pb[u]] = pi[u];
-                    }
-                }
-            }
-            if (!grid_sync(ctl, a.flags, gen, lim, pass == 0 ? a.stall : 0u)) return;
-            if (pass == 1) break;
-            // exclusive scan of each attribute's counts in place: they become the cursors
-            for (int jj = (int)c; jj < d; jj += (int)G) {
-                uint32_t *cj = a.bcnt + (size_t)jj * nbk;
-                uint32_t run = 0;
-                for (uint32_t b0 = 0; b0 < nbk; b0 += 16 * kThreads) {
-                    uint4 *p4 = reinterpret_cast<uint4 *>(cj + b0 + 16 * t);
-                    uint32_t v[16];
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        const uint4 u = __ldcg(p4 + q);
-                        v[4 * q + 0] = u.x;
-                        v[4 * q + 1] = u.y;
-                        v[4 * q + 2] = u.z;
-                        v[4 * q + 3] = u.w;
-                    }
-                    uint32_t s = 0;
-#pragma unroll
-                    for (int q = 0; q < 16; q++) s += v[q];
-                    uint32_t tot;
-                    uint32_t acc = run + block_excl_scan(s, tot);
-                    uint4 *bs = a.bcs + (size_t)jj * nbk + b0 + 16 * t;
-#pragma unroll
-                    for (int q = 0; q < 16; q++) {
-                        const uint32_t cur = v[q];
-                        bs[q] = make_uint4(cur, acc, acc + cur, 0u);
-                        v[q] = acc;
-                        acc += cur;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; q++) p4[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                    run += tot;
-                }
-            }
-            if (!grid_sync(ctl, a.flags, gen, lim)) return;
+        uint32_t *cw = &ctl->h0[0];
+        constexpr uint32_t words = (uint32_t)(sizeof(PeelCtl) - offsetof(PeelCtl, h0)) / 4u;
+        for (uint32_t b = c * kThreads + t; b < words; b += G * kThreads) cw[b] = 0;
+        for (uint32_t q = t; q < s1 - s0; q += kThreads) {
+            a.rnd[s0 + q] = kNone;
+            pfl[q] = kFlNone;
         }
     }
-
+    if (!grid_sync(ctl, a.flags, gen, lim, a.stall)) return;
+    if (a.transpose) transpose_tiles(a.x, a.n, d, a.xt_out, reinterpret_cast<float(*)[33]>(scr));
+    if (!grid_sync(ctl, a.flags, gen, lim)) return;
     bool first = true;           // the first epoch: a slice's list is the slice itself
     bool need_keys = true;       // the landmark changed: the keys must be computed
     uint32_t r0 = 0;             // the epoch's first round
@@ -1702,14 +1657,42 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 if (inc && c == 0) ctl->key_updates += 1;
                 s_keps = __double2float_ru(k_eps);
                 s_kabs = __double2float_ru(k_abs);
+                // the range of the new keys: none was below klast, the landmark's move takes
+                // at most 2 cs off a distance (c (2 x - l - o) <= 2 c per attribute, x <= 1) and
+                // adds nothing (x >= l for every point left), so none is above the first
+                // epoch's largest; a margin of 2^-12 for the roundings
+                if (!first) {
+                    const float lo = __uint_as_float(__ldcg(&ctl->klast)) * (1.0f - 0x1p-12f) - (float)cs * (2.0f + 0x1p-12f);
+                    s_dm = digit_map(lo > 0.0f ? __float_as_uint(lo) : 0u, __ldcg(&ctl->kmax) + 4096u);
+                }
             }
             __syncthreads();
             if (s_inc)
-                phase_inc<D>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, pfl, ctl->chold, s_nj, s_ij, s_io,
-                             s_il);
+                phase_inc<D>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, ctl->chold, s_nj, s_ij,
+                             s_io, s_il);
             else
-                phase_keys<D>(a.x, Ls, d, n_live, s0, first, kc, sid, gid, skey, gkp, scr, pfl, ctl->chold, s_jm);
+                phase_keys<D>(a.x, Ls, d, n_live, s0, first, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, ctl->chold, s_jm);
             __syncthreads();
+            if (first) {
+                // the first epoch's bins, from its own keys
+                uint32_t mn = kGone, mx = 0;
+                for (uint32_t q = t; q < n_live; q += kThreads) {
+                    const uint32_t k = LKEY(q);
+                    mn = min(mn, k);
+                    mx = max(mx, k);
+                }
+                mn = __reduce_min_sync(0xffffffffu, mn);
+                mx = __reduce_max_sync(0xffffffffu, mx);
+                if (lane == 0 && n_live) {
+                    atomicMax(&ctl->kmin, ~mn);
+                    atomicMax(&ctl->kmax, mx);
+                }
+                if (!grid_sync(ctl, a.flags, gen, lim)) return;
+                if (t == 0) s_dm = digit_map(~__ldcg(&ctl->kmin), __ldcg(&ctl->kmax) + 4096u);
+                __syncthreads();
+                for (uint32_t q = t; q < n_live; q += kThreads) atomicAdd(&scr[s_dm.bin(LKEY(q))], 1u);
+                __syncthreads();
+            }
             // each attribute's largest holder key (the holders are the flagged points left)
             for (uint32_t q0 = 0; q0 < n_live; q0 += kHoldBatch * kThreads) {
                 uint8_t f[kHoldBatch];
@@ -1743,62 +1726,67 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             for (int q = 0; q < per; q++) s += l0[q];
             uint32_t tot;
             const uint32_t e0 = block_excl_scan(s, tot);
-            for (uint32_t q = 0; q < Kb; q++) {
+            // boundary q's rank is (q + 1) N - 1: the boundaries inside this thread's bins
+            for (uint32_t q = e0 / N; q < Kb && (q + 1) * N - 1u < e0 + s; q++) {
                 const uint32_t target = (q + 1) * N - 1u;
-                if (target >= e0 && target < e0 + s) {
-                    uint32_t cc = e0;
+                uint32_t cc = e0;
 #pragma unroll
-                    for (int i = 0; i < per; i++) {
-                        if (target >= cc && target < cc + l0[i]) {
-                            s_b[q] = (uint32_t)(t * per + i);
-                            s_r[q] = target - cc;
-                        }
-                        cc += l0[i];
+                for (int i = 0; i < per; i++) {
+                    if (target >= cc && target < cc + l0[i]) {
+                        s_b[q] = (uint32_t)(t * per + i);
+                        s_r[q] = target - cc;
+                    }
+                    cc += l0[i];
+                }
+            }
+            for (int b = t; b < kHistBins / 4; b += kThreads) reinterpret_cast<uint32_t *>(s_map)[b] = 0xFFFFFFFFu;
+            __syncthreads();
+            if (w == 0) {
+                const bool v = lane < (int)Kb;
+                const uint32_t b = v ? s_b[lane] : 0u;
+                const uint32_t pb = __shfl_up_sync(0xffffffffu, b, 1);
+                const uint32_t open = __ballot_sync(0xffffffffu, v && (lane == 0 || b != pb));
+                if (v) {
+                    const uint32_t sl = (uint32_t)__popc(open & ((2u << lane) - 1u)) - 1u;
+                    s_slot[lane] = sl;
+                    if ((open >> lane) & 1u) {
+                        s_sbin[sl] = b;
+                        s_map[b] = (uint8_t)sl;
                     }
                 }
-            }
-            for (int b = t; b < kHistBins; b += kThreads) s_map[b] = 0xFF;
-            __syncthreads();
-            if (t == 0) {
-                uint32_t ns = 0;
-                for (uint32_t q = 0; q < Kb; q++) {
-                    if (q == 0 || s_b[q] != s_b[q - 1]) s_sbin[ns++] = s_b[q];
-                    s_slot[q] = ns - 1;
+                if (lane == 0) {
+                    s_nslot = (uint32_t)__popc(open);
+                    if (tot != nl_tot) atomicOr(&a.flags[1], 1u);
                 }
-                s_nslot = ns;
-                if (tot != nl_tot) atomicOr(&a.flags[1], 1u);
             }
             __syncthreads();
-            if (t < (int)s_nslot) s_map[s_sbin[t]] = (uint8_t)t;
-            __syncthreads();
-            // in shared memory for the first kSlotsSmem bins (the others straight to global),
-            // then the non-zero bins added to the grid's histograms
-            const uint32_t nss = min(s_nslot, (uint32_t)kSlotsSmem);
-            for (uint32_t b = t; b < nss * kHistBins; b += kThreads) scr[b] = 0;
-            __syncthreads();
-            for (uint32_t q0 = t; q0 < n_live; q0 += 4 * kThreads) {
+            // the keys in those bins, straight to the grid's histograms: few of them, but one
+            // atomic per warp for the equal ones (tied data crowds them into one)
+            const DigitMap mp = s_dm;
+            for (uint32_t q0 = t - lane; q0 < n_live; q0 += 4 * kThreads) {       // warp-uniform bound
                 uint32_t k4[4];
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    const uint32_t qi = q0 + q * kThreads;
+                    const uint32_t qi = q0 + lane + q * kThreads;
                     k4[q] = qi < n_live ? LKEY(qi) : kGone;
                 }
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    const uint32_t sl = k4[q] == kGone ? 0xFFu : s_map[k4[q] >> 21];
-                    const uint32_t sub = (k4[q] >> 10) & (kHistBins - 1);
-                    if (sl < nss) atomicAdd(&scr[sl * kHistBins + sub], 1u);
-                    else if (sl != 0xFFu) atomicAdd(&ctl->h1[sl][sub], 1u);
+                    const uint32_t b = mp.bin(k4[q]);
+                    const uint32_t sl = k4[q] == kGone ? 0xFFu : s_map[b];
+                    const uint32_t hit = __ballot_sync(0xffffffffu, sl != 0xFFu);
+                    if (!hit) continue;
+                    const uint32_t at = sl != 0xFFu ? sl * kHistBins + mp.sub(k4[q], b) : kGone;
+                    const uint32_t peers = __match_any_sync(0xffffffffu, at);
+                    if (at != kGone && lane == __ffs(peers) - 1)
+                        atomicAdd(&ctl->h1[0][0] + at, (uint32_t)__popc(peers));
                 }
             }
-            __syncthreads();
-            for (uint32_t b = t; b < nss * kHistBins; b += kThreads)
-                if (scr[b]) atomicAdd(&ctl->h1[b / kHistBins][b % kHistBins], scr[b]);
         }
         // the last CTA to arrive turns each boundary's bins into its band cut-offs, and
         // merges boundaries whose bands overlap into groups
         if (!grid_sync_last(ctl, a.flags, gen, lim, [&]() {
-                resolve_cutoffs(ctl, Kb, N, d, s_keps, s_kabs, s_b, s_r, s_slot, s_sbin, s_nslot);
+                resolve_cutoffs(ctl, Kb, N, d, s_keps, s_kabs, &s_dm, s_b, s_r, s_slot, s_sbin, s_nslot);
             }))
             return;
         const uint32_t K = __ldcg(&ctl->k_eff);       // boundaries of the epoch
@@ -1869,8 +1857,8 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         }
         const bool changed = __ldcg(&ctl->l_changed) != 0;
         const uint32_t live_from = r0 + kcm;
-        n_live = kc ? compact_shared(a, LV, n_live, r0, live_from, changed, scr)
-                    : compact_global(a, LV, n_live, r0, live_from, changed, scr);
+        n_live = kc ? compact_shared(a, LV, n_live, r0, live_from, changed, &s_dm, scr)
+                    : compact_global(a, LV, n_live, r0, live_from, changed, &s_dm, scr);
         if (!kc) {
             uint32_t *ti = gid; gid = gid2; gid2 = ti;
             uint32_t *tk = gkp; gkp = gkp2; gkp2 = tk;
@@ -1892,7 +1880,8 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             }
             if (c == 0 && t == 0) ctl->band_cnt = 0;
         }
-        if (changed) find_landmark(a, lm_first, lm_step, live_from);
+        if (changed && n_live)
+            lost_minima(a.x, a.xt, n, d, n_live, kc, sid, gid, ctl->lost, __ldcg(&ctl->n_lost), ctl->Lbits);
         first = false;
         need_keys = changed;
         r0 += kcm;
@@ -1911,36 +1900,6 @@ __global__ void __launch_bounds__(kThreads) k_barrier_bench(PeelCtl *ctl, uint32
     unsigned gen = 0;
     for (int r = 0; r < rounds; r++)
         if (!grid_sync(ctl, flags, gen, lim)) return;
-}
-
-// ------------------------------------------------------------------ the points by attribute
-// x (n x d, by point) into xt (d x n, by attribute) for the peel's key updates: 32 x 32
-// tiles through shared memory, so that both the reads (32 attributes of a point) and the
-// writes (32 points of an attribute) are coalesced.
-constexpr int kTrThreads = 256;
-constexpr size_t kTransposeBytes = size_t(96) << 20;
-
-__global__ void __launch_bounds__(kTrThreads) k_transpose(const float *__restrict__ x, int64_t n, int d,
-                                                          float *__restrict__ xt)
-{
-    __shared__ float tile[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int64_t tiles_c = (d + 31) / 32;
-    const int64_t tiles = (n + 31) / 32 * tiles_c;
-    for (int64_t tt = blockIdx.x; tt < tiles; tt += gridDim.x) {
-        const int64_t r0 = tt / tiles_c * 32;
-        const int c0 = (int)(tt % tiles_c) * 32;
-        for (int k = ty; k < 32; k += kTrThreads / 32) {
-            const int64_t r = r0 + k;
-            if (r < n && c0 + tx < d) tile[k][tx] = __ldg(&x[r * d + c0 + tx]);
-        }
-        __syncthreads();
-        for (int k = ty; k < 32; k += kTrThreads / 32) {
-            const int64_t r = r0 + tx;
-            if (r < n && c0 + k < d) xt[(size_t)(c0 + k) * (size_t)n + (size_t)r] = tile[tx][k];
-        }
-        __syncthreads();
-    }
 }
 
 // ------------------------------------------------------------------ packing by round
@@ -2070,15 +2029,9 @@ cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int s
                         cudaStream_t st, KTimer *kt)
 {
     const int64_t S = (n + N - 1) / N;
-    // all control state starts cleared; the first landmark is the origin (the scaled
-    // minimum of every attribute is exactly 0); no point has a round yet
-    cudaError_t e = cudaMemsetAsync(b.ctl, 0, sizeof(PeelCtl), st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(b.bcnt, 0, (size_t)d * b.nbuckets * sizeof(uint32_t), st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(b.rnd, 0xFF, (size_t)n * sizeof(uint32_t), st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(b.pflag, kFlNone, (size_t)n, st);
+    // all control state starts cleared (the launch clears the rest); the first landmark is
+    // the origin (the scaled minimum of every attribute is exactly 0)
+    cudaError_t e = cudaMemsetAsync(b.ctl, 0, offsetof(PeelCtl, h0), st);
     if (e != cudaSuccess) return e;
     const size_t smem = kPeelDynWords * sizeof(uint32_t);
     e = cudaFuncSetAttribute(k_peel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2094,23 +2047,20 @@ cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int s
     if (b.max_grid > 0 && grid > b.max_grid) grid = b.max_grid;
     PeelArgs a;
     a.x = b.x;
-    // the points by attribute for the key updates, in xseg (idle until the subclusters are
-    // gathered after the launch), where the rows do not fit in L2: an update then reads 4
-    // bytes of each point left instead of a 32-byte sector of its row
-    a.xt = (size_t)n * d * sizeof(float) > kTransposeBytes ? b.xseg : nullptr;
+    // the points by attribute for the landmark's minima and the key updates, in xseg (idle
+    // until the subclusters are gathered after the launch): they then read 4 bytes of each
+    // point left instead of a 32-byte sector of its row
+    a.xt = d >= 4 ? b.xseg : nullptr;
+    a.xt_out = b.xseg;
+    a.transpose = a.xt && (size_t)n * d * sizeof(float) <= kTransposeBytes;
     a.d = d;
     a.n = n;
     a.N = N;
     a.S = S;
     a.rnd = b.rnd;
     a.pflag = b.pflag;
-    a.ord = b.ord;
-    a.bcnt = b.bcnt;
-    a.bcs = b.bcs;
     a.lidx = b.lidx;
     a.kpos = b.kpos;
-    a.ord_ld = b.ord_ld;
-    a.nbk = b.nbuckets;
     a.band_k32 = b.band_k32;
     a.band_pos = b.band_pos;
     a.gkey = b.gkey;
@@ -2134,8 +2084,8 @@ cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     kt->begin(st);
-    if (a.xt) {                  // timed and counted with the peel it serves
-        k_transpose<<<sm_count * 8, kTrThreads, 0, st>>>(b.x, n, d, b.xseg);
+    if (a.xt && !a.transpose) {  // timed and counted with the peel it serves
+        k_transpose<<<sm_count * 8, kThreads, 0, st>>>(b.x, n, d, b.xseg);
         kt->launches[PSCL_K_PEEL]++;
     }
     e = cudaLaunchKernelEx(&cfg, k_peel<D>, a);
@@ -2232,13 +2182,6 @@ cudaError_t measure_grid_barrier(int sm_count, double *us, bool *timed_out)
     *timed_out = hf[1] != 0u;
     *us = 1e3 * (double)best / kRounds;
     return cudaSuccess;
-}
-
-uint32_t peel_buckets(int64_t n)
-{
-    uint32_t nb = 4096;
-    while (nb < 65536u && (int64_t)nb * 16 < n) nb <<= 1;
-    return nb;
 }
 
 int perm_grid(int64_t n, int sm_count)

@@ -21,12 +21,20 @@ constexpr int kMaxPeelGrid = 2048;   // CTAs of the persistent peel launch
 // Rounds one peel epoch may select from one set of distances (boundaries per epoch).
 constexpr int kMaxEpoch = 32;
 
-// Device-resident control block of one persistent peel launch (cleared before it).
+// Device-resident control block of one persistent peel launch.  The host clears the words
+// before h0 before the launch, the launch itself the rest.
 struct PeelCtl {
-    uint32_t h0[kHistBins];              // first digit (key bits 31..21) of the live keys
-    uint32_t h1[kMaxEpoch][kHistBins];   // second digit (bits 20..10) inside each boundary's bin
+    uint32_t bar_count;                  // grid barrier: arrivals since the launch
+    uint32_t abort;                      // set when a barrier wait gave up
+    uint32_t epochs;                     // statistics: epochs run,
+    uint32_t passes;                     //   distance passes over the points left,
+    uint32_t key_updates;                //   of which updates of the keys in a few attributes,
+    uint32_t barriers;                   //   grid-wide barriers passed
+    uint32_t kmin, kmax;                 // smallest and largest key of the first epoch (kmin: ~key)
+    uint32_t h0[kHistBins];              // first digit of the live keys
+    uint32_t h1[kMaxEpoch][kHistBins];   // second digit inside each boundary's bin
     uint32_t Lbits[kMaxD];               // landmark of the current epoch (float bits)
-    uint32_t lptr[kMaxD];                // per attribute: buckets in front of it hold no remaining point
+    uint32_t lost[kMaxD];                // attributes whose last holder left with the last commit
     uint32_t chold[kMaxD];               // live points whose attribute j equals L_j
     uint32_t hmax[kMaxD];                // the largest key among them (since the last pass)
     uint32_t hcnt[kMaxD][kMaxEpoch];     // of those, the ones assigned to each round of the epoch
@@ -36,19 +44,15 @@ struct PeelCtl {
     uint32_t gfill[kMaxEpoch];           // of those, regrouped into the group's region so far
     uint32_t g_in[kMaxEpoch], g_out[kMaxEpoch];   // a group's band: keys in [g_in, g_out]
     uint32_t g_q1[kMaxEpoch], g_q2[kMaxEpoch];    // a group's first and last boundary
-    float kref;                          // lower end of the first boundary's key bin, last epoch
+    float kref;                          // lower end of the first boundary's key range, last epoch
+    uint32_t klast;                      // no point left has a smaller key (before the landmark moved)
+    uint32_t n_lost;
     uint32_t n_slots;                    // first-digit bins with a second-digit histogram
     uint32_t n_groups;
     uint32_t band_cnt;                   // band entries listed this epoch
     uint32_t k_eff;                      // boundaries the epoch resolves (rounds it can commit)
     uint32_t k_commit;                   // rounds the epoch commits
     uint32_t l_changed;                  // the landmark changes after them
-    uint32_t bar_count;                  // grid barrier: arrivals since the launch
-    uint32_t abort;                      // set when a barrier wait gave up
-    uint32_t epochs;                     // statistics: epochs run,
-    uint32_t passes;                     //   distance passes over the points left,
-    uint32_t key_updates;                //   of which updates of the keys in a few attributes,
-    uint32_t barriers;                   //   grid-wide barriers passed
 };
 
 // v (a scaled coordinate, in [0, 1]) times 2^32 rounded to the nearest integer, ties to
@@ -146,13 +150,8 @@ struct PeelBuffers {
     const float *x;                  // n x d scaled points
     uint32_t *rnd;                   // n: round (subcluster) of each point, all ones while unassigned
     uint8_t *pflag;                  // 2 x n: per CTA slice, a state byte per list position
-    uint32_t *ord;                   // d x ord_ld: point ids of each attribute in bucket order
-    uint32_t *bcnt;                  // d x nbuckets: bucket counts, then scatter cursors
-    uint4 *bcs;                      // d x nbuckets: (points left, first entry, end entry, 0)
     uint32_t *lidx;                  // 2 x n: per CTA slice, the ids of its points left (two lists)
     uint32_t *kpos;                  // 2 x n: per CTA slice, the keys of its points left by list position
-    int64_t ord_ld;                  // n rounded up to a multiple of 4
-    uint32_t nbuckets;               // power of two, 4096 .. 65536
     uint32_t *band_k32;              // n: float32 keys of the epoch's band entries
     uint32_t *band_pos;              // n: their point ids
     uint64_t *gkey;                  // n: band entries regrouped by group (compensated distances)
@@ -173,8 +172,6 @@ struct PeelBuffers {
 // Time per grid-wide barrier of the peel's own implementation, in the peel's launch shape
 // (pscl_measure_grid_barrier).
 cudaError_t measure_grid_barrier(int sm_count, double *us, bool *timed_out);
-// Buckets of the per-attribute orders the peel builds for n points.
-uint32_t peel_buckets(int64_t n);
 // CTAs of the counting sort that packs the subclusters after the peel (pcnt: 256 x this).
 int perm_grid(int64_t n, int sm_count);
 // Rows of x in the order of perm, packed into xseg (the gather after any subclustering).
