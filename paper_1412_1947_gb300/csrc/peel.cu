@@ -31,7 +31,7 @@
 //   B. per boundary, the first-digit bin holding its rank, and 2048-bin histograms of
 //      the keys inside those bins: each boundary's float32 key lies in a range [A, B] of a
 //      few units in the last place;
-//   C. |delta32 - delta64| <= eps*delta32 + ea with eps = (d+4)*2^-23, ea = 2^-120, so the
+//   C. |delta32 - delta64| <= eps*delta32 + ea with eps = key_roundings*2^-23, ea = 2^-120, so the
 //      boundary's delta64 lies in [A(1-eps)-ea, B(1+eps)+ea]: a point whose bound lies
 //      below that interval is certainly before the boundary, one above it certainly
 //      after; the few in between form the boundary's band (boundaries whose bands overlap
@@ -47,12 +47,12 @@
 //     sum_{j in J} (l_j - o_j)(l_j + o_j - 2 x_j),
 // which is added to every live key in float32.  The keys' error bound then takes the form
 // |delta32 - delta64| <= eps*delta32 + ea with eps and ea carried from pass to pass: a
-// full pass sets (eps0, ea0) = ((d+4) 2^-23, 2^-120), and an update with C = sum_J (l_j - o_j)
+// full pass sets (eps0, ea0) = (key_roundings 2^-23, 2^-120), and an update with C = sum_J (l_j - o_j)
 // gives eps' = eps + 2^-23 and ea' = ea + (5 eps + (16 + 4|J|) 2^-24) C (the update's own
 // rounding, the old key's error carried to the new key, and the float64 definition's;
 // scaled values lie in [0, 1]).  Phase C uses the carried bound; a full pass is taken
 // instead when J spans many 32-byte sectors of a row, when more than kIncMax attributes
-// moved, or when eps would pass 1.5 eps0 or ea an eighth of eps0 times the last epoch's
+// moved, or when eps would pass 1.5 (d+4) 2^-23 or ea an eighth of (d+4) 2^-23 times the last epoch's
 // first boundary key (the landmark sits at the corner of the minima, so the boundary keys
 // are large and ea stays a small share of the bands' width).
 //
@@ -317,15 +317,54 @@ __device__ __forceinline__ float eps_ff(int d)
     return (float)((double)d * d + 8.0 * d + 1.0) * 0x1p-47f;
 }
 
+// The same by 8 lanes of a warp (sub = lane & 7, every lane of the warp taking part): lane sub
+// sums the attributes sub, sub + 8, ..., then the partial sums are added pairwise, the high
+// parts error-free.  Fewer roundings per term than the one chain the bound allows.
+__device__ __forceinline__ void dist_ff8(const float *__restrict__ row, const float *Ls, int d, int sub, float &h,
+                                         float &l)
+{
+    float hi = 0.0f, lo = 0.0f;
+#pragma unroll 4
+    for (int j = sub; j < d; j += 8) {
+        const float a = __ldg(&row[j]), b = Ls[j];
+        const float s = __fsub_rn(a, b);
+        const float bb = __fsub_rn(s, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(-b, bb));
+        const float p = __fmul_rn(s, s);
+        const float q = __fmaf_rn(__fmul_rn(2.0f, s), e, __fmaf_rn(s, s, -p));
+        const float t = __fadd_rn(hi, p);
+        const float bv = __fsub_rn(t, hi);
+        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bv)), __fsub_rn(p, bv));
+        hi = t;
+        lo = __fadd_rn(lo, __fadd_rn(err, q));
+    }
+#pragma unroll
+    for (int o = 4; o; o >>= 1) {
+        const float p = __shfl_xor_sync(0xffffffffu, hi, o), pl = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float t = __fadd_rn(hi, p);
+        const float bv = __fsub_rn(t, hi);
+        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bv)), __fsub_rn(p, bv));
+        hi = t;
+        lo = __fadd_rn(__fadd_rn(lo, pl), err);
+    }
+    h = __fadd_rn(hi, lo);
+    l = __fsub_rn(lo, __fsub_rn(h, hi));
+}
+
+__device__ __forceinline__ uint64_t ff_key(float h, float l)
+{
+    double v = __dadd_rn((double)h, (double)l);
+    if (!(v > 0.0)) v = 0.0;
+    return (uint64_t)__double_as_longlong(v);
+}
+
 // The compensated distance h + l rounded once to float64 (its bit pattern orders like
 // the value), the key a group's entries are ranked by.
 __device__ __forceinline__ uint64_t dff_key(const float *__restrict__ row, const float *Ls, int d)
 {
     float h, l;
     dist_ff(row, Ls, d, h, l);
-    double v = __dadd_rn((double)h, (double)l);
-    if (!(v > 0.0)) v = 0.0;
-    return (uint64_t)__double_as_longlong(v);
+    return ff_key(h, l);
 }
 
 // The digits of the keys in one pass.  Every key left lies in [base, top] (the range's
@@ -628,6 +667,17 @@ __host__ __device__ constexpr int kCoopBatch()
     return 16 / (D / 4) >= 4 ? 4 : (16 / (D / 4) >= 1 ? 16 / (D / 4) : 1);
 }
 
+// The key's error bound in units of 2^-23: the roundings a term passes through (its own
+// difference's twice, the chain's, the butterfly's), with a factor two of margin.
+template <int D>
+__host__ __device__ constexpr int key_roundings(int d)
+{
+    if (!kCoopRows<D>()) return d + 4;
+    int lg = 0;
+    for (int p = kCoopLanes<D>(); p > 1; p >>= 1) lg++;
+    return D / kCoopLanes<D>() + lg + 4;
+}
+
 __device__ __forceinline__ bool in_mask(const uint32_t *jm, int j)
 {
     return (jm[j >> 5] >> (j & 31)) & 1u;
@@ -851,23 +901,35 @@ __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float 
     }
 }
 
-// A holder's key, as the candidate largest key of each attribute whose landmark value it
-// holds.
-__device__ __forceinline__ void note_hold_key(const float *__restrict__ row, const float *Ls, int d, uint32_t key,
-                                              uint32_t *hmax)
+// The holders among a warp's 32 points (lanes with `hold` set; ids by lane), one at a time by
+// the whole warp: f(j, v) for every attribute j in which the point equals the landmark, v its
+// lane's val.  A row is read in one coalesced load per 32 attributes, where a thread walking
+// it alone held its warp for d loads (400000 x 128: 15 us of an epoch's key pass).
+template <class F>
+__device__ __forceinline__ void for_held(const float *__restrict__ x, const float *Ls, int d, bool hold, uint32_t id,
+                                         uint32_t val, F f)
 {
-    for (int j = 0; j < d; j++)
-        if (__ldg(&row[j]) == Ls[j]) atomicMax(&hmax[j], key);
-}
-
-// A holder of some attribute's landmark value assigned to round rr of the epoch: counted
-// per attribute it holds.
-__device__ __forceinline__ void count_holder(const float *__restrict__ x, const float *Ls, int d, uint32_t id,
-                                             uint32_t rr, PeelCtl *ctl)
-{
-    const float *row = x + (size_t)id * d;
-    for (int j = 0; j < d; j++)
-        if (__ldg(&row[j]) == Ls[j]) atomicAdd(&ctl->hcnt[j][rr], 1u);
+    const int lane = threadIdx.x & 31;
+    uint32_t m = __ballot_sync(0xffffffffu, hold);
+    while (m) {
+        const int q = __ffs(m) - 1;
+        m &= m - 1u;
+        const float *row = x + (size_t)__shfl_sync(0xffffffffu, id, q) * d;
+        const uint32_t vq = __shfl_sync(0xffffffffu, val, q);
+        for (int j0 = 0; j0 < d; j0 += 128) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int j = j0 + 32 * u + lane;
+                v[u] = j < d ? __ldg(&row[j]) : -1.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int j = j0 + 32 * u + lane;
+                if (j < d && v[u] == Ls[j]) f(j, vq);
+            }
+        }
+    }
 }
 
 // Settles group g of the epoch's boundaries (one CTA): every band entry of the group gets
@@ -922,11 +984,106 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
             stp[e] = __ldcg(&gp[e]);
         }
     __syncthreads();
-    auto KA = [&](uint32_t i) -> uint64_t { return staged ? stk[i] : __ldcg(&gk[i]); };
+    auto KA = [&](uint32_t i) -> uint64_t { return __ldcg(&gk[i]); };
     // an entry's id (bit 31 of the stored word is its hold flag)
-    auto PA = [&](uint32_t i) -> uint32_t { return (staged ? stp[i] : __ldcg(&gp[i])) & kPosMask; };
+    auto PA = [&](uint32_t i) -> uint32_t { return __ldcg(&gp[i]) & kPosMask; };
     auto AK = [&](uint32_t i) -> uint64_t { return __ldcg(&ak[i]); };
     auto AP = [&](uint32_t i) -> uint32_t { return __ldcg(&ap[i]); };
+    if (staged) {
+        // every entry's rank among the group's, counted by its thread: the entries whose
+        // compensated distance is smaller beyond the error window, and where the window holds
+        // others and a boundary cuts through it, those of them that are smaller by float64
+        // and index.  No selection and no barrier per boundary (2^20 x 16: settle and commit
+        // 14 -> 8 us an epoch).  The window of a distance with bits k: k +- W, W >= 4 (eps_ff
+        // + 2^-52) 2^53 (a relative step r moves a double's bits by at most r 2^53); below
+        // 2^-60 the absolute error of tiny squares counts too, so all of them are one window.
+        constexpr int E = kStage / kThreads;
+        __shared__ int s_any;
+        uint64_t *d64 = reinterpret_cast<uint64_t *>(scr);                      // kStage keys
+        uint8_t *f64 = reinterpret_cast<uint8_t *>(scr + 2 * kStage);           // kStage flags
+        static_assert(2 * kStage + kStage / 4 <= kStageOff, "the rank scratch lies before the staged entries");
+        if (t <= (int)(q2 - q1)) {
+            const int64_t need_s = (int64_t)(q1 + t + 1) * N - (int64_t)before;
+            s_need[t] = need_s < 0 ? 0u : (need_s > (int64_t)ne ? ne : (uint32_t)need_s);
+            if (need_s < 0 || need_s > (int64_t)ne) atomicOr(&a.flags[1], 1u);
+        }
+        if (t == 0) s_any = 0;
+        for (uint32_t e = t; e < ne; e += kThreads) f64[e] = 0;
+        __syncthreads();
+        const uint64_t W0 = 256ull * ((uint64_t)d * d + 8ull * d + 1ull) + 8ull, W = W0 + (W0 >> 4);
+        constexpr uint64_t kTiny = 963ull << 52;                                // 2^-60
+        const uint32_t nq = q2 - q1 + 1u;
+        uint64_t lo[E], hi[E];
+        uint32_t below[E], inside[E], rank[E];
+        bool cut[E];
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            const uint32_t e = t + i * kThreads;
+            const uint64_t k = e < ne ? stk[e] : 0ull;
+            lo[i] = k < kTiny + W ? 0ull : k - W;
+            hi[i] = (k < kTiny ? kTiny : k) + W;
+            below[i] = inside[i] = 0;
+        }
+        for (uint32_t f = 0; f < ne; f++) {
+            const uint64_t k = stk[f];
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                below[i] += k < lo[i];
+                inside[i] += k >= lo[i] && k <= hi[i];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            const uint32_t e = t + i * kThreads;
+            rank[i] = below[i];
+            cut[i] = false;
+            if (e < ne)
+                for (uint32_t b = 0; b < nq; b++) cut[i] |= s_need[b] > below[i] && s_need[b] < below[i] + inside[i];
+            if (cut[i]) {
+                s_any = 1;
+                for (uint32_t f = 0; f < ne; f++)
+                    if (stk[f] >= lo[i] && stk[f] <= hi[i]) f64[f] = 1;
+            }
+        }
+        __syncthreads();
+        if (s_any) {
+            for (uint32_t e = t; e < ne; e += kThreads)
+                if (f64[e])
+                    d64[e] = (uint64_t)__double_as_longlong(dist64(a.x + (size_t)(stp[e] & kPosMask) * d, Ls, d));
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                const uint32_t e = t + i * kThreads;
+                if (!cut[i]) continue;
+                const uint64_t ke = d64[e];
+                const uint32_t pe = stp[e] & kPosMask;
+                for (uint32_t f = 0; f < ne; f++)
+                    if (stk[f] >= lo[i] && stk[f] <= hi[i])
+                        rank[i] += d64[f] < ke || (d64[f] == ke && (stp[f] & kPosMask) < pe);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            const uint32_t e = t + i * kThreads;
+            uint32_t rr = kNone, raw = 0;
+            if (e < ne) {
+                raw = stp[e];
+                rr = q1;
+                for (uint32_t b = 0; b < nq; b++) rr += s_need[b] <= rank[i];
+                if (rr < K) {
+                    a.rnd[raw & kPosMask] = r0 + rr;
+                    atomicAdd(&s_bc[rr], 1u);
+                }
+            }
+            const bool ch = e < ne && rr < K && (raw & ~kPosMask);
+            if (__any_sync(0xffffffffu, ch))
+                for_held(a.x, Ls, d, ch, raw & kPosMask, rr,
+                         [&](int j, uint32_t r) { atomicAdd(&ctl->hcnt[j][r], 1u); });
+        }
+        __syncthreads();
+        if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
+        return;
+    }
     const double win_rel = 4.0 * ((double)eps_ff(d) + 0x1p-52);
     for (uint32_t i = q1; i <= q2; i++) {
         const uint32_t bi = i - q1;
@@ -983,13 +1140,15 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
         __syncthreads();
     }
     // every entry's round: the first boundary of the group plus the boundaries it is after
-    for (uint32_t e = t; e < ne; e += kThreads) {
-        const uint64_t kb = KA(e);
-        const uint32_t raw = staged ? stp[e] : __ldcg(&gp[e]);
+    for (uint32_t e0 = 0; e0 < ne; e0 += kThreads) {            // block-uniform bound
+        const uint32_t e = e0 + (uint32_t)t;
+        const bool v = e < ne;
+        const uint64_t kb = v ? KA(e) : 0ull;
+        const uint32_t raw = v ? __ldcg(&gp[e]) : 0u;
         const uint32_t pos = raw & kPosMask;
         const double ke = __longlong_as_double((long long)kb);
         uint32_t after = 0;
-        for (uint32_t bi = 0; bi <= q2 - q1; bi++) {
+        for (uint32_t bi = 0; v && bi <= q2 - q1; bi++) {
             const uint32_t need = s_need[bi];
             if (need == 0) {
                 after++;
@@ -1009,11 +1168,13 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
             }
         }
         const uint32_t rr = q1 + after;
-        if (rr < K) {
+        if (v && rr < K) {
             a.rnd[pos] = r0 + rr;
             atomicAdd(&s_bc[rr], 1u);
-            if (raw & ~kPosMask) count_holder(a.x, Ls, d, pos, rr, ctl);
         }
+        const bool ch = v && rr < K && (raw & ~kPosMask);
+        if (__any_sync(0xffffffffu, ch))
+            for_held(a.x, Ls, d, ch, pos, rr, [&](int j, uint32_t r) { atomicAdd(&ctl->hcnt[j][r], 1u); });
     }
     __syncthreads();
     if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
@@ -1076,34 +1237,14 @@ __device__ __noinline__ void lost_minima(const float *__restrict__ x, const floa
 // whose bands overlap into groups.  Warp w resolves boundaries w, w + kW, ...: lane i sums
 // second-digit bins [64 i, 64 i + 64) in two halves, a warp scan finds the lane holding
 // the rank, and that lane walks the half holding it (its loads issued together).
-__device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t Kb, uint32_t N, int d, float keps, float kabs,
-                                             const DigitMap *dm, const uint32_t *sb, const uint32_t *sr,
-                                             const uint32_t *sslot, const uint32_t *sbin, uint32_t nslot)
+__device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t K, float keps, float kabs, const DigitMap *dm,
+                                             const uint32_t *sb, const uint32_t *sr, const uint32_t *sslot,
+                                             uint32_t nslot)
 {
     __shared__ uint32_t s_b1[kMaxEpoch];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const DigitMap mp = *dm;
     if (t < kMaxEpoch) s_b1[t] = 0;
-    // the rounds this landmark can serve: up to the one in which the last holder of some
-    // attribute's landmark value leaves (the landmark changes after it).  That holder's key
-    // m (the smallest over the attributes of their holders' largest key) is at most the
-    // c-th smallest live key, c read off the histograms (the second digit where m's bin has
-    // one), so it leaves at the latest in round (c - 1) / N; the boundaries past that
-    // round are not resolved (a prediction that falls short costs one more epoch)
-    uint32_t m = kGone;
-    for (int j = t; j < d; j += kThreads) m = min(m, __ldcg(&ctl->hmax[j]));
-    m = block_min(m);
-    const uint32_t mb0 = mp.bin(m), mb1 = mp.sub(m, mb0);
-    int slot = -1;
-    for (uint32_t q = 0; q < nslot; q++)
-        if (sbin[q] == mb0) slot = (int)q;
-    uint32_t cnt = 0;
-    for (int b = t; b < kHistBins; b += kThreads) {
-        if ((uint32_t)b < mb0 || ((uint32_t)b == mb0 && slot < 0)) cnt += __ldcg(&ctl->h0[b]);
-        if (slot >= 0 && (uint32_t)b <= mb1) cnt += __ldcg(&ctl->h1[slot][b]);
-    }
-    cnt = block_sum(cnt);
-    const uint32_t K = min(Kb, (cnt > 0 ? (cnt - 1) / N : 0u) + 1u);
     __syncthreads();
     for (uint32_t q = (uint32_t)w; q < K; q += kW) {
         const uint4 *h4 = reinterpret_cast<const uint4 *>(ctl->h1[sslot[q]] + lane * 64);
@@ -1165,7 +1306,6 @@ __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t Kb, uint32_t
         if (lane == 0) {
             ctl->n_groups = (uint32_t)__popc(open);
             ctl->n_slots = nslot;
-            ctl->k_eff = K;
             ctl->kref = __uint_as_float(A);
         }
     }
@@ -1183,6 +1323,8 @@ __device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, ui
     const int t = threadIdx.x;
     // per attribute: the first round after which no holder of L_j is left
     // (the counts are read all at once, then scanned in registers)
+    __shared__ uint32_t s_nl;
+    if (t == 0) s_nl = 0;
     uint32_t qs = kNone;
     for (int j = t; j < d; j += kThreads) {
         uint32_t hc[kMaxEpoch];
@@ -1197,15 +1339,16 @@ __device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, ui
         }
         qs = min(qs, qj);
     }
+    // the last committed boundary's group, below (lane g: group g)
+    const uint32_t ng = __ldcg(&ctl->n_groups);
+    const uint32_t gq2 = t < (int)ng ? __ldcg(&ctl->g_q2[t & 31]) : kNone;
+    const uint32_t gin = t < (int)ng ? __ldcg(&ctl->g_in[t & 31]) : kNone;
     qs = block_min(qs);
     const uint32_t kc_ = qs < K ? qs + 1u : K;
     const bool changed = qs < K;
     // the holders that leave with the committed rounds; an attribute that has none left gets
     // a new landmark value (the minimum over the points left, taken next) and its holders are
     // counted by the next pass
-    __shared__ uint32_t s_nl;
-    if (t == 0) s_nl = 0;
-    __syncthreads();
     for (int j = t; j < d; j += kThreads) {
         uint32_t gone = 0;
 #pragma unroll
@@ -1216,6 +1359,11 @@ __device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, ui
             ctl->lost[atomicAdd(&s_nl, 1u)] = (uint32_t)j;
             ctl->Lbits[j] = kInfBits;
         }
+    }
+    // every point left lies at or past the start of the last committed boundary's band
+    if (t < 32) {
+        const uint32_t past = __ballot_sync(0xffffffffu, t < (int)ng && gq2 >= kc_ - 1u);
+        if (past && t == __ffs(past) - 1) ctl->klast = gin;
     }
     __syncthreads();
     if (t < (int)K && __ldcg(&ctl->cert[t]) + __ldcg(&ctl->bnd[t]) != N) atomicOr(&a.flags[1], 1u);
@@ -1230,11 +1378,6 @@ __device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, ui
         ctl->k_commit = kc_;
         ctl->l_changed = changed ? 1u : 0u;
         ctl->n_lost = s_nl;
-        // every point left lies at or past the start of the last committed boundary's band
-        const uint32_t ng = __ldcg(&ctl->n_groups);
-        uint32_t g = 0;
-        while (g + 1 < ng && __ldcg(&ctl->g_q2[g]) < kc_ - 1u) g++;
-        ctl->klast = __ldcg(&ctl->g_in[g]);
         ctl->epochs += 1;
         ctl->passes += need_keys ? 1u : 0u;
     }
@@ -1359,8 +1502,11 @@ __device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L,
             if (cert) {
                 a.rnd[idv[u]] = r0 + cls[u];
                 atomicAdd(&s_cc[cls[u]], 1u);
-                if (fl[u] & kFlHold) count_holder(a.x, Ls, d, idv[u], cls[u], ctl);
             }
+            const bool ch = cert && (fl[u] & kFlHold);
+            if (__any_sync(0xffffffffu, ch))
+                for_held(a.x, Ls, d, ch, idv[u], cls[u],
+                         [&](int j, uint32_t rr) { atomicAdd(&ctl->hcnt[j][rr], 1u); });
         }
     }
 }
@@ -1535,7 +1681,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     __shared__ uint32_t s_b[kMaxEpoch], s_r[kMaxEpoch], s_slot[kMaxEpoch], s_sbin[kMaxEpoch];
     __shared__ uint32_t s_gin[kMaxEpoch], s_gout[kMaxEpoch], s_gq2[kMaxEpoch];
     __shared__ uint32_t s_cc[kMaxEpoch], s_gc[kMaxEpoch];
-    __shared__ uint32_t s_nslot, s_glast;
+    __shared__ uint32_t s_nslot, s_glast, s_hold_end;
     __shared__ __align__(4) uint8_t s_map[kHistBins];
     // the previous epoch's landmark; the attributes whose landmark value is new (mask) and,
     // for an update of the keys, those attributes with their old and new values
@@ -1582,7 +1728,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     uint32_t r0 = 0;             // the epoch's first round
     // the keys' error bound |delta32 - delta64| <= k_eps delta32 + k_abs (thread 0 keeps it,
     // the same in every CTA) and the key updates since the last full pass
-    const double eps0 = (double)(d + 4) * 0x1p-23;
+    const double eps_cap = (double)(d + 4) * 0x1p-23, eps0 = (double)key_roundings<D>(d) * 0x1p-23;
     double k_eps = eps0, k_abs = 0x1p-120;
     for (;;) {
         const uint32_t nl_tot = n - r0 * N;
@@ -1600,7 +1746,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 for (int j = t; j < d; j += kThreads) a.landmarks[(size_t)r0 * d + j] = Ls[j];
             break;
         }
-        const uint32_t Kb = min(a.kmax, (nl_tot + N - 1) / N - 1u);   // boundaries phase B locates
+        uint32_t Kb = min(a.kmax, (nl_tot + N - 1) / N - 1u);   // boundaries the epoch resolves, at most
 
         // ---- A: float32 distances of the points left, the first histogram, the holders
         if (need_keys) {
@@ -1644,7 +1790,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 // epoch's first boundary, so the bands widen little
                 const double kref = (double)__ldcg(&ctl->kref);
                 const bool inc = !first && fin && nj >= 1 && nj <= (uint32_t)kIncMax && nsec * 160u < 12u * (uint32_t)d &&
-                                 ne <= 1.5 * eps0 && na <= 0.125 * eps0 * kref;
+                                 ne <= 1.5 * eps_cap && na <= 0.125 * eps_cap * kref;
                 if (inc) {
                     k_eps = ne;
                     k_abs = na;
@@ -1702,11 +1848,13 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                     f[u] = qi < n_live ? pfl[qi] : (uint8_t)0;
                 }
 #pragma unroll
-                for (int u = 0; u < kHoldBatch; u++)
-                    if (f[u] & kFlHold) {
-                        const uint32_t qi = q0 + u * kThreads + t;
-                        note_hold_key(a.x + (size_t)LID(qi) * d, Ls, d, LKEY(qi), ctl->hmax);
-                    }
+                for (int u = 0; u < kHoldBatch; u++) {
+                    const bool h = f[u] & kFlHold;
+                    if (!__any_sync(0xffffffffu, h)) continue;
+                    const uint32_t qi = q0 + u * kThreads + t;
+                    for_held(a.x, Ls, d, h, h ? LID(qi) : 0u, h ? LKEY(qi) : 0u,
+                             [&](int j, uint32_t key) { atomicMax(&ctl->hmax[j], key); });
+                }
             }
             for (int b = t; b < kHistBins; b += kThreads)
                 if (scr[b]) atomicAdd(&ctl->h0[b], scr[b]);
@@ -1724,8 +1872,29 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             uint32_t s = 0;
 #pragma unroll
             for (int q = 0; q < per; q++) s += l0[q];
+            uint32_t m = kGone;
+            for (int j = t; j < d; j += kThreads) m = min(m, __ldcg(&ctl->hmax[j]));
             uint32_t tot;
             const uint32_t e0 = block_excl_scan(s, tot);
+            // the rounds this landmark can serve: up to the one in which the last holder of
+            // some attribute's landmark value leaves (the landmark changes after it).  That
+            // holder's key m (the smallest over the attributes of their holders' largest key)
+            // is at most the c-th smallest live key, c the points up to the end of m's bin, so
+            // it leaves at the latest in round (c - 1) / N; the boundaries past that round are
+            // not resolved (a prediction that falls short costs one more epoch)
+            m = block_min(m);
+            {
+                const uint32_t mb = s_dm.bin(m);
+                if ((uint32_t)t == mb / per) {
+                    uint32_t cc = e0;
+#pragma unroll
+                    for (int i = 0; i < per; i++)
+                        if ((uint32_t)i <= mb % per) cc += l0[i];
+                    s_hold_end = cc;
+                }
+            }
+            __syncthreads();
+            Kb = min(Kb, (s_hold_end > 0u ? (s_hold_end - 1u) / N : 0u) + 1u);
             // boundary q's rank is (q + 1) N - 1: the boundaries inside this thread's bins
             for (uint32_t q = e0 / N; q < Kb && (q + 1) * N - 1u < e0 + s; q++) {
                 const uint32_t target = (q + 1) * N - 1u;
@@ -1786,10 +1955,10 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         // the last CTA to arrive turns each boundary's bins into its band cut-offs, and
         // merges boundaries whose bands overlap into groups
         if (!grid_sync_last(ctl, a.flags, gen, lim, [&]() {
-                resolve_cutoffs(ctl, Kb, N, d, s_keps, s_kabs, &s_dm, s_b, s_r, s_slot, s_sbin, s_nslot);
+                resolve_cutoffs(ctl, Kb, s_keps, s_kabs, &s_dm, s_b, s_r, s_slot, s_nslot);
             }))
             return;
-        const uint32_t K = __ldcg(&ctl->k_eff);       // boundaries of the epoch
+        const uint32_t K = Kb;                        // boundaries of the epoch
 
         // ---- C: classify every point left: certainly in a round of the epoch, in a band, or later
         const uint32_t ng = __ldcg(&ctl->n_groups);
@@ -1822,7 +1991,29 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             __syncthreads();
             // one slot claim per warp and group: the entries of a pass crowd into a few
             // groups, whose fill counters would otherwise take one contended atomic each
-            for (uint32_t b0 = c * kThreads; b0 < nlist; b0 += G * kThreads) {     // warp-uniform bound
+            // (8 lanes per entry from 32 attributes on: a thread's chain over 128 took 15 us)
+            if (d >= 32) {
+                constexpr uint32_t EB = kThreads / 8;
+                for (uint32_t b0 = c * EB; b0 < nlist; b0 += G * EB) {               // block-uniform bound
+                    const uint32_t e = b0 + (uint32_t)t / 8u, sub = (uint32_t)t & 7u;
+                    const bool v = e < nlist;
+                    const uint32_t k = v ? __ldcg(&a.band_k32[e]) : 0u;
+                    const uint32_t pos = v ? __ldcg(&a.band_pos[e]) : 0u;
+                    uint32_t g = 0;
+                    while (g + 1 < ng && k > s_gout[g]) g++;
+                    const uint32_t peers = __match_any_sync(0xffffffffu, v && sub == 0u ? g : kGone);
+                    const uint32_t leader = (uint32_t)__ffs(peers) - 1u;
+                    uint32_t slot = 0;
+                    if (v && sub == 0u && (uint32_t)lane == leader) slot = atomicAdd(&ctl->gfill[g], (uint32_t)__popc(peers));
+                    slot = __shfl_sync(0xffffffffu, slot, (int)leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+                    float h, l;
+                    dist_ff8(a.x + (size_t)(pos & kPosMask) * d, Ls, d, (int)sub, h, l);
+                    if (v && sub == 0u) {
+                        a.gkey[s_cc[g] + slot] = ff_key(h, l);
+                        a.gpos[s_cc[g] + slot] = pos;
+                    }
+                }
+            } else for (uint32_t b0 = c * kThreads; b0 < nlist; b0 += G * kThreads) {     // warp-uniform bound
                 const uint32_t e = b0 + (uint32_t)t;
                 const bool v = e < nlist;
                 const uint32_t k = v ? __ldcg(&a.band_k32[e]) : 0u;
@@ -2042,6 +2233,10 @@ cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int s
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int64_t grid = (int64_t)sm_count * std::min(per_sm, 4);
     if (grid > kMaxPeelGrid) grid = kMaxPeelGrid;
+    // one CTA per SM while its slice holds few points: fewer arrivals at the barriers
+    // (200003 x 7: 861 against 820 us, 400000 x 128: 6.8 against 6.5 ms), where 2^20 x 16, with
+    // 6900 points per SM, wants two (3.0 against 2.6 ms)
+    if (n <= (int64_t)sm_count * 3072 && grid > sm_count) grid = sm_count;
     const int64_t want = (n + 63) / 64;             // at least ~64 points per CTA
     if (grid > want) grid = std::max<int64_t>(1, want);
     if (b.max_grid > 0 && grid > b.max_grid) grid = b.max_grid;

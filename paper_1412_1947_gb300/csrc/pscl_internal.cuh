@@ -50,7 +50,6 @@ struct PeelCtl {
     uint32_t n_slots;                    // first-digit bins with a second-digit histogram
     uint32_t n_groups;
     uint32_t band_cnt;                   // band entries listed this epoch
-    uint32_t k_eff;                      // boundaries the epoch resolves (rounds it can commit)
     uint32_t k_commit;                   // rounds the epoch commits
     uint32_t l_changed;                  // the landmark changes after them
 };
