@@ -64,7 +64,8 @@ struct Owner {
 
 // One Lloyd launch plan: tables on the device and their host copies.
 struct LloydPlan {
-    int n_seg = 0, n_units = 0, kmax = 0, d = 0, max_unit = 0;
+    int n_seg = 0, n_units = 0, kmax = 0, d = 0, max_unit = 0, max_seg = 0;
+    double evals = 0.0;             // sum over the sets of rows x centers
     int64_t rows = 0, P = 0;
     std::vector<int64_t> seg_start;
     std::vector<int32_t> seg_size, cen_off, k_eff, unit_seg, unit_start, unit_count, seg_unit0;
@@ -457,13 +458,16 @@ static int build_lloyd_plan(Owner *j, LloydPlan &p, const std::vector<int64_t> &
     p.seg_size = sizes;
     p.k_eff = keff;
     p.cen_off.assign(p.n_seg, 0);
-    p.kmax = 0;
+    p.kmax = p.max_seg = 0;
+    p.evals = 0.0;
     int64_t P = 0, rows = 0;
     for (int s = 0; s < p.n_seg; s++) {
         p.cen_off[s] = (int32_t)P;
         P += keff[s];
         rows += sizes[s];
         p.kmax = std::max(p.kmax, keff[s]);
+        p.max_seg = std::max(p.max_seg, sizes[s]);
+        p.evals += (double)sizes[s] * keff[s];
     }
     p.P = P;
     p.rows = rows;
@@ -840,7 +844,9 @@ static int run_lloyd(pscl_job *j, const LloydPlan &p, const float *pts, float *c
     b.wait_limit = j->wait_limit;
     b.tc_stall = j->test_stall == 2;
     CU(launch_lloyd_init(b, t, j->d, p.P, seed, stage, j->first_k, p.kmax, st, &j->kt));
-    if (!plain) {
+    if (!plain && !j->rpt && sets_supported(t, j->d, p.max_seg, p.kmax, p.evals, prec, b, j->ctx->sm_count)) {
+        CU(launch_lloyd_sets(b, t, j->d, p.P, p.max_seg, p.kmax, iters, st, &j->kt));
+    } else if (!plain) {
         for (int it = 0; it < iters; it++) {
             b.count = cnt2 + (size_t)(it & 1) * p.P;
             CU(launch_lloyd_iter(b, cnt2 + (size_t)((it + 1) & 1) * p.P, t, j->d, it, 0, p.n_units, 0, p.P,
@@ -1453,7 +1459,10 @@ static int batch_enqueue(pscl_batch *b, int iters, uint64_t seed, int prec, bool
     const int64_t P = b->plan.P;
     CU(launch_lloyd_init(lb, t, b->d, P, seed, 0u, 0, b->plan.kmax, st, &b->kt));
     if (events) CU(cudaEventRecord(b->ev[0], st));
-    if (!b->plain) {
+    if (!b->plain && !b->rpt &&
+        sets_supported(t, b->d, b->plan.max_seg, b->plan.kmax, b->plan.evals, prec, lb, b->ctx->sm_count)) {
+        CU(launch_lloyd_sets(lb, t, b->d, P, b->plan.max_seg, b->plan.kmax, iters, st, &b->kt));
+    } else if (!b->plain) {
         for (int it = 0; it < iters; it++) {
             lb.count = b->cnt + (size_t)(it & 1) * P;
             CU(launch_lloyd_iter(lb, b->cnt + (size_t)((it + 1) & 1) * P, t, b->d, it, 0, b->plan.n_units, 0, P,

@@ -41,6 +41,7 @@
 #include <algorithm>
 
 #include "pscl_internal.cuh"
+#include "sse.cuh"
 
 namespace pscl {
 namespace {
@@ -1244,54 +1245,46 @@ __global__ void __launch_bounds__(256) k_tc_rescore_ties(const float *__restrict
 }
 
 // The SSE from the labels: each point's float32 direct distance to its center, added in
-// double per thread, per block in a fixed tree and over blocks in block order -- the rows of
-// a thread, the tree and the block order of the float32 SSE pass (same grid, 256 threads),
-// so the value is the same bit for bit.
+// double per thread and in the fixed tree -- the rows of a thread and the order of the float32
+// SSE pass (same grid, 256 threads), so the value is the same bit for bit.  A block's 256 rows
+// come in whole through shared memory (a thread reading its own row attribute by attribute
+// touched 32 sectors an instruction: 0.62 of 6.8 TB/s at 2^24 x 64).
 template <int D>
-__global__ void __launch_bounds__(256) k_sse_from_labels(const float *__restrict__ x, int64_t n,
-                                                         const float *__restrict__ centers, int k,
-                                                         const int32_t *__restrict__ labels, double *blk_sse,
-                                                         double *sse, uint32_t *ticket)
+__global__ void __launch_bounds__(kSseThreads) k_sse_from_labels(const float *__restrict__ x, int64_t n,
+                                                                 const float *__restrict__ centers, int k,
+                                                                 const int32_t *__restrict__ labels, double *blk_sse,
+                                                                 double *sse, uint32_t *ticket)
 {
-    constexpr int NT = 256;
+    extern __shared__ __align__(16) float4 xs[];
+    constexpr int LD4 = tile_ld4(D);
     double part = 0.0;
-    const int64_t stride = (int64_t)gridDim.x * NT;
-    const int64_t nround = (n + stride - 1) / stride;
-    for (int64_t it = 0; it < nround; it++) {
-        const int64_t i = it * stride + (int64_t)blockIdx.x * NT + threadIdx.x;
-        if (i < n) {
-            int32_t l = labels[i];
-            if ((uint32_t)l >= (uint32_t)k) l = 0;          // only after a search that gave up
-            const float *xr = x + i * D, *cr = centers + (size_t)l * D;
+    const int64_t stride = (int64_t)gridDim.x * kSseThreads;
+    for (int64_t i0 = (int64_t)blockIdx.x * kSseThreads; i0 < n; i0 += stride) {
+        const int rows = (int)min((int64_t)kSseThreads, n - i0);
+        __syncthreads();
+        tile_load(xs, x + i0 * D, rows, rows, D, LD4);
+        int32_t l = (int)threadIdx.x < rows ? labels[i0 + threadIdx.x] : 0;
+        if ((uint32_t)l >= (uint32_t)k) l = 0;              // only after a search that gave up
+        const float4 *cr = reinterpret_cast<const float4 *>(centers + (size_t)l * D);
+        __syncthreads();
+        if ((int)threadIdx.x < rows) {
             float acc = 0.0f;
-#pragma unroll
-            for (int a = 0; a < D; a++) {
-                const float t = __fsub_rn(__ldg(&xr[a]), __ldg(&cr[a]));
+#pragma unroll 8
+            for (int q = 0; q < D / 4; q++) {
+                const float4 v = xs[threadIdx.x * LD4 + q], c = __ldg(&cr[q]);
+                float t = __fsub_rn(v.x, c.x);
+                acc = __fmaf_rn(t, t, acc);
+                t = __fsub_rn(v.y, c.y);
+                acc = __fmaf_rn(t, t, acc);
+                t = __fsub_rn(v.z, c.z);
+                acc = __fmaf_rn(t, t, acc);
+                t = __fsub_rn(v.w, c.w);
                 acc = __fmaf_rn(t, t, acc);
             }
             part = __dadd_rn(part, (double)acc);
         }
     }
-    for (int o = 16; o; o >>= 1) part = __dadd_rn(part, __shfl_down_sync(0xffffffffu, part, o));
-    __shared__ double ws[NT / 32];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double b = ws[0];
-        for (int w = 1; w < NT / 32; w++) b = __dadd_rn(b, ws[w]);
-        blk_sse[blockIdx.x] = b;
-    }
-    __shared__ bool is_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!is_last || threadIdx.x != 0) return;
-    __threadfence();
-    double tot = 0.0;
-    for (unsigned b = 0; b < gridDim.x; b++) tot = __dadd_rn(tot, __ldcg(&blk_sse[b]));
-    *sse = tot;
-    *ticket = 0;
+    sse_reduce(part, blk_sse, sse, ticket);
 }
 
 // ---------------------------------------------------------------- host side
@@ -1523,8 +1516,10 @@ cudaError_t sse_tc_dispatch(const float *x, int64_t n, const float *centers, int
     cudaError_t e = chunk_search<D, MODE>(x, n, centers, k, t256, trem, scratch, labels, flags, wait_limit, sm_count,
                                           st, kt, PSCL_K_FINAL_SSE);
     if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)kSseThreads * tile_ld4(D) * 16;
+    if ((e = cudaFuncSetAttribute(k_sse_from_labels<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     kt->begin(st);
-    k_sse_from_labels<D><<<sse_grid(n, sm_count), 256, 0, st>>>(x, n, centers, k, labels, blk_sse, sse, ticket);
+    k_sse_from_labels<D><<<sse_grid(n, sm_count), kSseThreads, smem, st>>>(x, n, centers, k, labels, blk_sse, sse, ticket);
     kt->end(PSCL_K_FINAL_SSE, st);
     return cudaGetLastError();
 }

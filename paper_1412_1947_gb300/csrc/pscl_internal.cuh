@@ -232,6 +232,12 @@ cudaError_t launch_lloyd_iter(const LloydBuffers &b, int32_t *count_next, const 
                               int d, int iter, int unit_lo, int unit_hi, int64_t cen_lo,
                               int64_t cen_hi, int kmax, int prec, uint32_t *flags, int sm_count,
                               cudaStream_t st, KTimer *kt, int rows_per_thread = 0);
+// All iterations of every set in one launch, for small sets (b.count: both parities; evals:
+// sum over the sets of rows x centers).
+bool sets_supported(const SegTable &t, int d, int max_rows, int kmax, double evals, int prec, const LloydBuffers &b,
+                    int sm_count);
+cudaError_t launch_lloyd_sets(const LloydBuffers &b, const SegTable &t, int d, int64_t P, int max_rows, int kmax,
+                              int iters, cudaStream_t st, KTimer *kt);
 // Independent sets: nearest center of every row within its set, per-set sums of the
 // squared distances (unit_sse: n_units doubles, seg_sse: n_seg doubles).
 cudaError_t launch_seg_sse(const float *pts, const SegTable &t, const int32_t *seg_unit0, int d,
