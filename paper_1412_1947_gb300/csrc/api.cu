@@ -439,6 +439,11 @@ static int64_t unit_target(int64_t rows, int sm_count, int64_t unit_rows)
     return std::max<int64_t>(unit_rows > 0 ? 32 : 128, std::min<int64_t>(1024, target));
 }
 
+// A row's fixed cost in the tensor-core assignment, in centers (see build_lloyd_plan): with
+// rows alone as weights, the ranges of the sets with most centers ended last (the uneven batch,
+// k = 8 .. 255: 2.45 ms an iteration; weights 16 3.07, 64 2.20, 160 2.00, 256 and 600 1.8-1.9).
+constexpr int64_t kRowWeight = 256;
+
 // rows per unit of a set of m rows (a multiple of 32)
 static int64_t unit_size(int64_t m, int64_t target)
 {
@@ -508,21 +513,26 @@ static int build_lloyd_plan(Owner *j, LloydPlan &p, const std::vector<int64_t> &
     CU(cudaMemcpyAsync(p.d_seg_start, p.seg_start.data(), p.n_seg * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(p.d_i32, packed.data(), packed.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     // Contiguous unit ranges of near-equal weight for persistent launches of G = m * SMs
-    // CTAs (rows, plus a set-up allowance wherever a range has to start a new set).
+    // CTAs.  m = 1..3 (the tensor-core assignment): a row costs its conversion and the work
+    // over its set's centers (kRowWeight centers' worth and k), a set its set-up.  m = 4 and
+    // kSplitMany (the sums): rows alone.
     const int sm = j->ctx->sm_count;
-    std::vector<int64_t> wpre(p.n_units + 1, 0);
+    std::vector<int64_t> wk(p.n_units + 1, 0), wr(p.n_units + 1, 0);
     for (int u = 0; u < p.n_units; u++) {
         const bool first = u == 0 || p.unit_seg[u] != p.unit_seg[u - 1];
-        wpre[u + 1] = wpre[u] + p.unit_count[u] + (first ? 256 : 0);
+        const int64_t rows_u = p.unit_count[u] + (first ? 256 : 0);
+        wr[u + 1] = wr[u] + rows_u;
+        wk[u + 1] = wk[u] + rows_u * (kRowWeight + keff[p.unit_seg[u]]);
     }
     std::vector<int32_t> split;
-    for (int m = 1; m <= 4; m++) {
+    for (int m : {1, 2, 3, 4, kSplitMany}) {
         const int G = m * sm;
-        p.split_off[m] = (int)split.size();
+        const std::vector<int64_t> &w = m < 4 ? wk : wr;
+        p.split_off[m < 5 ? m : 0] = (int)split.size();
         int u = 0;
         for (int c = 0; c <= G; c++) {
-            const int64_t target = wpre[p.n_units] * c / G;
-            while (u < p.n_units && wpre[u] < target) u++;
+            const int64_t target = w[p.n_units] / G * c + w[p.n_units] % G * c / G;
+            while (u < p.n_units && w[u] < target) u++;
             split.push_back(c == G ? p.n_units : u);
         }
     }
@@ -753,7 +763,7 @@ static size_t job_footprint(int64_t n, int d, int64_t N, int local_k, int final_
         units += (m + unit_size(m, tl) - 1) / unit_size(m, tl);
         P += std::min<int64_t>(local_k, m);
     }
-    const size_t split = (size_t)10 * sm + 4;
+    const size_t split = split_words(sm);
     b += r256((size_t)S * 8) + r256((4 * (size_t)S + 3 * (size_t)units + 1) * 4) + r256(split * 4);
     b += r256((size_t)P * d * 4) + r256((size_t)P * d * 8) + r256(2 * (size_t)P * 4);
     if (trace) b += r256((size_t)iters * n * 4);

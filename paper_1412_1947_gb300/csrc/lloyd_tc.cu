@@ -23,9 +23,9 @@
 //   * producer warp: one thread streams 128-row tiles of the float32 points into shared
 //     memory with cp.async.bulk.tensor (a tensor map over the packed points, rows of d
 //     floats, boxes of 128 rows x min(d, 32) attributes with the bank swizzle that fits);
-//   * converter warps (128 threads, a row each): centre the row, split it into the mode's
-//     parts and write operand A in the canonical K-major layout (8-row x 16-byte core
-//     matrices, no swizzle), with ||x~|| for the epilogue; at the start of each set they
+//   * converter warps (a thread per row, or two from d = 32 on): centre the row, split it into
+//     the mode's parts and write operand A in the canonical K-major layout (8-row x 16-byte
+//     core matrices, no swizzle), with ||x~|| for the epilogue; at the start of each set they
 //     build operand B from the set's centers;
 //   * MMA warp: one thread issues the tcgen05.mma of a tile into one of two TMEM
 //     accumulators and commits them to mbarriers (operand A free, accumulator full);
@@ -47,10 +47,7 @@ namespace pscl {
 namespace {
 
 constexpr int kTileRows = 128;            // MMA M, rows per tile
-constexpr int kCvtWarp0 = 8;              // converter warps 8..11
-constexpr int kProdWarp = 12;
-constexpr int kMmaWarp = 13;
-constexpr int kTcThreads = 14 * 32;
+constexpr int kCvtWarp0 = 8;              // the first converter warp
 constexpr int kXMax = 4;                  // slots of the point ring, at most
 constexpr int kAMax = 2;                  // operand A buffers, at most
 constexpr int kMeta = 8;                  // per-tile metadata ring (tiles in flight < kMeta)
@@ -70,12 +67,29 @@ __device__ __forceinline__ float min3f(float a, float b, float c)
     return m;
 }
 
-// all ones if v <= thr, else 0
-__device__ __forceinline__ uint32_t le_mask(float v, float thr)
+// The signs of v_q - thr as a mask: bit q is set iff v_q < thr (a float32 difference has the
+// sign of the exact one).  The differences go two at a time through the otherwise idle FMA
+// pipe, and a funnel shift takes each sign, in four chains of eight: one ALU instruction per
+// value, where a comparison and a select-and-merge took two (the half-rate ALU pipe 63 % busy
+// at 2^24 x 64, k = 256) in one chain of 32.
+__device__ __forceinline__ uint32_t less_mask(const uint32_t (&v)[32], float thr)
 {
-    uint32_t s;
-    asm("set.le.u32.f32 %0, %1, %2;" : "=r"(s) : "f"(v), "f"(thr));
-    return s;
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    uint64_t nt;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(nt) : "f"(-thr));
+#pragma unroll
+    for (int q = 6; q >= 0; q -= 2) {
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            uint32_t lo, hi;
+            asm("{\n .reg .b64 a;\n mov.b64 a, {%2, %3};\n add.rn.f32x2 a, a, %4;\n mov.b64 {%0, %1}, a;\n}\n"
+                : "=r"(lo), "=r"(hi)
+                : "r"(v[8 * e + q]), "r"(v[8 * e + q + 1]), "l"(nt));
+            w[e] = __funnelshift_l(hi, w[e], 1);
+            w[e] = __funnelshift_l(lo, w[e], 1);
+        }
+    }
+    return __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
 }
 
 // ---------------------------------------------------------------- mbarriers
@@ -127,24 +141,56 @@ __device__ __forceinline__ void mbar_drain(uint32_t a, uint32_t parity, unsigned
         if (mbar_try(a, parity)) return;
 }
 
-// The converter warps' named barrier (id 1, 128 threads), returning the AND of `ok` over them.
+// Converter warps.  The conversion of a tile (a chain of shared-memory loads, roundings and
+// stores per row) took longer than its MMAs and its epilogue: where one CTA fits an SM, two
+// threads share a row (500009 x 32, k = 32: 29 -> 25 us an iteration; the uneven batch 1.93 ->
+// 1.82 ms).  d = 16 fits two CTAs, whose converters overlap anyway.
+template <int D>
+__host__ __device__ constexpr int cvt_warps()
+{
+    return D <= 16 ? 4 : 8;
+}
+
+// Warps 0..7 are the epilogue's, then the converters, the producer and the MMA warp.
+template <int D>
+__host__ __device__ constexpr int tc_threads()
+{
+    return (kCvtWarp0 + cvt_warps<D>() + 2) * 32;
+}
+
+// The converter warps' named barrier (id 1), returning the AND of `ok` over them.
+template <int D>
 __device__ __forceinline__ bool cvt_bar_and(bool ok)
 {
     uint32_t r;
-    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.and.pred q, 1, 128, p;\n"
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.and.pred q, 1, %2, p;\n"
                  " selp.u32 %0, 1, 0, q;\n}\n"
                  : "=r"(r)
-                 : "r"((uint32_t)ok)
+                 : "r"((uint32_t)ok), "n"(cvt_warps<D>() * 32)
                  : "memory");
     return r != 0;
 }
 
-// CTAs of the assignment kernel per SM the register budget is set for: two for narrow
-// points, whose per-tile work is short and whose pipeline latency a second CTA hides
+template <int D>
+__device__ __forceinline__ void cvt_bar()
+{
+    asm volatile("bar.sync 1, %0;" ::"n"(cvt_warps<D>() * 32) : "memory");
+}
+
+// CTAs of the assignment kernel per SM the register budget is set for.
 template <int D>
 __host__ __device__ constexpr int tc_min_blocks()
 {
-    return D <= 32 ? 2 : 1;
+    return D <= 16 ? 2 : 1;
+}
+
+// Threads the register budget is set for: registers are allotted per sub-partition of an SM,
+// which takes every fourth warp, so a CTA's warps count rounded up to a multiple of four (two
+// CTAs of 14 warps put 8 in one sub-partition: 64 registers a thread).
+template <int D>
+__host__ __device__ constexpr int tc_bound_threads()
+{
+    return (tc_threads<D>() + 127) / 128 * 128;
 }
 
 // ---------------------------------------------------------------- TMA
@@ -356,7 +402,7 @@ __device__ __forceinline__ bool next_run(const SegTable &t, int &u, int ue, Run 
 }
 
 template <int D, int MODE>
-__global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(const __grid_constant__ CUtensorMap xmap, const TcArgs p)
+__global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_tc_assign(const __grid_constant__ CUtensorMap xmap, const TcArgs p)
 {
     using O = Op<MODE>;
     using L = TcLayout<D, MODE>;
@@ -373,7 +419,8 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     __shared__ float s_ref[D];
-    __shared__ float s_part[128];
+    constexpr int CW = cvt_warps<D>(), CT = CW * 32;
+    __shared__ float s_part[CT];
     __shared__ float s_cmax2;
     __shared__ uint32_t s_stat[2];
     const uint32_t b0 = smem_u32(bars);
@@ -398,10 +445,10 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
         s_stat[1] = 0u;
         for (int s = 0; s < kXMax; s++) {
             mbar_init(XFULL(s), 1);
-            mbar_init(XEMPTY(s), 4);
+            mbar_init(XEMPTY(s), CW);
         }
         for (int s = 0; s < kAMax; s++) {
-            mbar_init(AFULL(s), 4);
+            mbar_init(AFULL(s), CW);
             mbar_init(AEMPTY(s), 1);
         }
         for (int s = 0; s < 2; s++) {
@@ -409,7 +456,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
             mbar_init(TEMPTY(s), 4);
         }
         for (int s = 0; s < kMeta; s++) {
-            mbar_init(MFULL(s), 4);
+            mbar_init(MFULL(s), CW);
             mbar_init(MEMPTY(s), 4);
         }
         mbar_init(STALL, 1);
@@ -430,7 +477,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
     __syncthreads();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == kProdWarp) {
+    if (warp == kCvtWarp0 + CW) {
         // ---- producer: point tiles by TMA
         uint32_t issued = 0;
         if (lane == 0 && !*abort) {
@@ -460,7 +507,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                 for (uint32_t q = issued > XS ? issued - XS : 0u; q < issued; q++)
                     mbar_drain(XFULL((int)(q % XS)), (q / XS) & 1u, lim);
         }
-    } else if (warp == kMmaWarp) {
+    } else if (warp == kCvtWarp0 + CW + 1) {
         // ---- MMA issue: one thread
         if (lane == 0 && !*abort) {
             int u = ub;
@@ -519,7 +566,11 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
         }
     } else if (warp >= kCvtWarp0) {
         // ---- converters: operand B per set, operand A and ||x~|| per tile
-        const int r = tid - kCvtWarp0 * 32;                 // 0..127: the tile row of this thread
+        // ct: the converter thread; r: its tile row; with eight warps a warp takes 16 rows and
+        // its lanes 16.. the second half of the attributes
+        constexpr int H = CW / 4;
+        const int ct = tid - kCvtWarp0 * 32;
+        const int r = H == 1 ? ct : (ct >> 5) * 16 + (lane & 15), half = H == 1 ? 0 : lane >> 4;
         int u = ub;
         Run run;
         uint32_t i = 0;
@@ -530,7 +581,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
             // the earlier tiles' MMAs must be done before operand B and s_ref change
             for (uint32_t j = i > AS ? i - AS : 0u; ok && j < i; j++)
                 ok = mbar_wait(AEMPTY((int)(j % AS)), (j / AS) & 1u, lim, abort);
-            ok = cvt_bar_and(ok && !*abort);
+            ok = cvt_bar_and<D>(ok && !*abort);
             if (!ok) {
                 i += (uint32_t)run.ntiles;
                 continue;
@@ -542,23 +593,25 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
             const float *rcen = p.ref_centers ? p.ref_centers : cen;
             const int rk = p.ref_centers ? p.ref_k : k;
             {   // reference point: the mean of those centers
-                constexpr int G = 128 / D;
-                const int at = r % D, g = r / D;
+                constexpr int G = CT / D;
+                const int at = ct % D, g = ct / D;
                 float m = 0.0f;
-                if (g < G)
+                if (g < G) {
+#pragma unroll 8
                     for (int j = g; j < rk; j += G) m = __fadd_rn(m, __ldg(&rcen[(size_t)j * D + at]));
-                s_part[r] = m;
-                if (r == 0) s_cmax2 = 0.0f;
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (r < D) {
-                    float tot = 0.0f;
-                    for (int q = 0; q < G; q++) tot = __fadd_rn(tot, s_part[q * D + r]);
-                    s_ref[r] = __fdiv_rn(tot, (float)rk);
                 }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                s_part[ct] = m;
+                if (ct == 0) s_cmax2 = 0.0f;
+                cvt_bar<D>();
+                if (ct < D) {
+                    float tot = 0.0f;
+                    for (int q = 0; q < G; q++) tot = __fadd_rn(tot, s_part[q * D + ct]);
+                    s_ref[ct] = __fdiv_rn(tot, (float)rk);
+                }
+                cvt_bar<D>();
             }
             if (p.ref_centers)       // the bound's center norm over the whole set
-                for (int j = r; j < rk; j += 128) {
+                for (int j = ct; j < rk; j += CT) {
                     float n2 = 0.0f;
                     for (int a = 0; a < D; a++) {
                         const float c = __fsub_rn(__ldg(&rcen[(size_t)j * D + a]), s_ref[a]);
@@ -567,7 +620,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                     atomicMax(reinterpret_cast<int *>(&s_cmax2), __float_as_int(n2));
                 }
             // operand B: row j = [H | L | norm parts] of -2 c~_j (zero rows past k)
-            for (int j = r; j < np; j += 128) {
+            for (int j = ct; j < np; j += CT) {
                 float n2 = 0.0f;
 #pragma unroll 4
                 for (int a4 = 0; a4 < D / 4; a4++) {
@@ -600,7 +653,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                 if (j < k) atomicMax(reinterpret_cast<int *>(&s_cmax2), __float_as_int(n2));   // non-negative
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            cvt_bar<D>();
             const float cmax = sqrtf(s_cmax2);
             for (int tt = 0; tt < run.ntiles; tt++, i++) {
                 const int a = (int)(i % AS), m = (int)(i % kMeta);
@@ -617,8 +670,10 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     const unsigned char *xt = sx + (size_t)xs * L::kXBytes;
+                    constexpr int NB = L::kXPer * L::kXBoxCols / 4;
 #pragma unroll 4
-                    for (int b4 = 0; b4 < L::kXPer * L::kXBoxCols / 4; b4++) {
+                    for (int q4 = 0; q4 < NB / H; q4++) {
+                        const int b4 = half * (NB / H) + q4;
                         const int a4 = part * (L::kXPer * L::kXBoxCols / 4) + b4;
                         const int bx = (4 * b4) / L::kXBoxCols, c = ((4 * b4) % L::kXBoxCols) / 4;
                         const float4 v = *reinterpret_cast<const float4 *>(xt + (size_t)bx * L::kXBoxBytes +
@@ -655,12 +710,17 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                     if (lane == 0) mbar_arrive(XEMPTY(xs));
                 }
                 if (!ok) continue;
+                if (H == 2) xn2 = __fadd_rn(xn2, __shfl_xor_sync(0xffffffffu, xn2, 16));
                 const float one = live ? 1.0f : 0.0f;
-                put4<D, MODE>(at, r, L::kParts * D, one, one, O::kNormParts > 2 ? one : 0.0f, 0.0f);
+                if (half == 0) {
+                    put4<D, MODE>(at, r, L::kParts * D, one, one, O::kNormParts > 2 ? one : 0.0f, 0.0f);
+                    meta[m].xn[r] = sqrtf(xn2);
+                }
+                if (half == H - 1) {
 #pragma unroll
-                for (int e = 4; e < O::kMmaK; e += 4) put4<D, MODE>(at, r, L::kParts * D + e, 0.f, 0.f, 0.f, 0.f);
-                meta[m].xn[r] = sqrtf(xn2);
-                if (r == 0) {
+                    for (int e = 4; e < O::kMmaK; e += 4) put4<D, MODE>(at, r, L::kParts * D + e, 0.f, 0.f, 0.f, 0.f);
+                }
+                if (ct == 0) {
                     meta[m].cmax = cmax;
                     meta[m].k = run.k;
                     meta[m].nvalid = min(kTileRows, run.R - tt * kTileRows);
@@ -690,6 +750,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
         uint32_t i = 0;
         bool ok = !*abort;
         while (ok && next_run(p.t, u, ue, run)) {
+            const int k = run.k;
             for (int tt = 0; tt < run.ntiles; tt++, i++) {
                 if ((int)(i & 1u) != g) continue;
                 const int m = (int)(i % kMeta);
@@ -699,12 +760,11 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int k = meta[m].k;
                 const float cmax = meta[m].cmax, xn = meta[m].xn[r];
                 const bool live = r < meta[m].nvalid;
                 const int64_t row = meta[m].row0 + r;
                 const uint32_t taddr = tmem + (uint32_t)g * p.ncols + ((uint32_t)(q4 * 32) << 16);
-                // pass 1: the smallest of the k values (four independent chains; two 32-column
+                // pass 1: the smallest of the values (four independent chains; two 32-column
                 // loads in flight per wait)
                 float m4[4] = {kInf, kInf, kInf, kInf};
                 constexpr bool kLean = tc_min_blocks<D>() > 1;     // one load in flight: fewer registers
@@ -742,19 +802,19 @@ __global__ void __launch_bounds__(kTcThreads, tc_min_blocks<D>()) k_tc_assign(co
                 // center left out could win the float32 direct comparison
                 const float E = alpha * xn * cmax + beta * cmax * cmax +
                                 (float)(2 * (D + 3)) * 0x1p-24f * (xn + cmax) * (xn + cmax) + 0x1p-100f;
-                const float thr = b1 + 2.0f * E;
-                // pass 2: the centers with v_j <= thr as a bit mask (word c: centers 32c .. 32c+31);
+                // (the next float up, for a strict comparison; b1 and E are finite)
+                const float thr = __fadd_ru(b1 + 2.0f * E, 0x1p-149f);
+                // pass 2: the centers with v_j < thr as a bit mask (word c: centers 32c .. 32c+31);
                 // one bit is the label, more a near tie
                 uint32_t w[8];
 #pragma unroll
                 for (int c = 0; c < 8; c++) {
                     w[c] = 0u;
                     if (32 * c < k) {
-                        uint32_t v[32], acc = 0u;
+                        uint32_t v[32];
                         tmem_ld32_nowait(taddr + (uint32_t)(32 * c), v);
                         tmem_wait();
-#pragma unroll
-                        for (int q = 0; q < 32; q++) acc |= le_mask(__uint_as_float(v[q]), thr) & (1u << q);
+                        const uint32_t acc = less_mask(v, thr);
                         const int rem = k - 32 * c;          // columns past k hold no center
                         w[c] = rem >= 32 ? acc : acc & ((1u << rem) - 1u);
                     }
@@ -1384,27 +1444,31 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     // as many CTAs per SM as registers, shared memory and the 512 TMEM columns allow (<= 4):
     // every resident CTA must get its TMEM at once
     int occ = 1;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ka, kTcThreads, smem)) != cudaSuccess) return e;
-    // d <= 32 is built for two CTAs per SM (at most 64 registers, under 80 KB of shared
-    // memory each); the query answers one for it, but two CTAs' unit ranges run faster
-    // (2^20 x 16: 1.70 -> 1.62 ms per job); no CTA waits on another, so the count is safe
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ka, tc_threads<D>(), smem)) != cudaSuccess) return e;
+    // d <= 16 is built for two CTAs per SM (64 registers a thread); the query answers one for
+    // it, but two CTAs' unit ranges run faster (2^20 x 16: 30 -> 25 us an iteration); no CTA
+    // waits on another, so the count is safe
     if (tc_min_blocks<D>() > 1) occ = std::max(occ, tc_min_blocks<D>());
     const int ma = std::max(1, std::min(std::min(occ, (int)(512u / (2u * a.ncols))), 4));
     a.split = t.split + t.split_off[ma];
     kt->begin(st);
-    ka<<<ma * sm_count, kTcThreads, smem, st>>>(map, a);
+    ka<<<ma * sm_count, tc_threads<D>(), smem, st>>>(map, a);
     kt->end(PSCL_K_LLOYD_ASSIGN, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // sums: four CTAs' unit ranges per SM whatever fits at once, so that the block scheduler
     // evens out ranges whose near ties cost more; the first iteration adds every row, the
     // later ones (raw labels kept apart) only the rows that moved
+    // (2^24 x 64: ties concentrate in some sets, with four ranges per SM half of the SMs idled
+    // at the end; sixteen 0.90 -> 0.55 ms; at 2^20 x 16, with 430 rows a range, 9 -> 13 us)
     const int m = 4;
     if (b.raw && iter > 0) {
+        const int md = b.rows >= (int64_t)kSplitMany * sm_count * 2048 ? kSplitMany : 4;
         const size_t sd = delta_smem<D>(kmax);
         auto kd = k_tc_delta<D>;
         if ((e = cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sd)) != cudaSuccess) return e;
         kt->begin(st);
-        kd<<<m * sm_count, delta_threads<D>(), sd, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], b.raw, b.labels,
+        kd<<<md * sm_count, delta_threads<D>(), sd, st>>>(b.pts, b.centers, t, t.split + t.split_off[md == 4 ? 4 : 0], b.raw,
+                                                          b.labels,
                                                          b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count,
                                                          kmax);
         kt->end(PSCL_K_LLOYD_SUMS, st);
@@ -1465,11 +1529,11 @@ cudaError_t chunk_search(const float *x, int64_t n, const float *centers, int k,
         if ((e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
             return e;
         int occ = 1;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ka, kTcThreads, smem)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ka, tc_threads<D>(), smem)) != cudaSuccess) return e;
         const int ma = std::max(1, std::min(std::min(occ, (int)(512u / (2u * a.ncols))), 4));
         a.split = t.split + t.split_off[ma];
         kt->begin(st);
-        ka<<<ma * sm_count, kTcThreads, smem, st>>>(map, a);
+        ka<<<ma * sm_count, tc_threads<D>(), smem, st>>>(map, a);
         kt->end(ktag, st);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -81,6 +81,10 @@ __device__ __forceinline__ unsigned long long fix_of(float v)
 //   [3] rows the tensor-core assignment assigned
 constexpr int kFlagWords = 4;
 
+constexpr int kSplitMany = 16;
+// Words of the split tables (build_lloyd_plan): m sm + 1 for each m.
+constexpr size_t split_words(int sm) { return (size_t)(1 + 2 + 3 + 4 + kSplitMany) * sm + 5; }
+
 // Segment table of one batched Lloyd launch (device arrays).
 struct SegTable {
     const int64_t *seg_start;        // first row of each segment in the packed points
@@ -93,7 +97,9 @@ struct SegTable {
     int n_seg;
     int n_units;
     // Persistent launches over all units with m CTAs per SM (m = 1..4): CTA c serves the
-    // units [split[split_off[m] + c], split[split_off[m] + c + 1]) (NULL: no split).
+    // units [split[split_off[m] + c], split[split_off[m] + c + 1]) (NULL: no split).  m = 1..3
+    // weigh rows by their set's centers too, m = 4 by rows alone; split_off[0]: kSplitMany
+    // ranges per SM by rows alone.
     const int32_t *split;
     int split_off[5];
 };
