@@ -162,8 +162,10 @@ struct pscl_job : Owner {
     int32_t *u_group = nullptr;
     uint32_t *u_cnt = nullptr, *u_total = nullptr;
     double *u_lo = nullptr, *u_hi = nullptr;
-    // serving: the peel goes to a stream shared by all jobs (cooperative launches one at a time)
-    cudaStream_t coop = nullptr;
+    // serving: the peel goes to a stream shared with other jobs' (coop); coop_all: the streams
+    // of all peels, if it has to run alone
+    cudaStream_t coop = nullptr, coop_all[4] = {};
+    int coop_n = 0;
     cudaEvent_t coop_ev[2] = {};
 };
 
@@ -793,11 +795,14 @@ static size_t job_footprint(int64_t n, int d, int64_t N, int local_k, int final_
 cudaStream_t pscl::ctx_stream(const pscl_ctx *c) { return c->stream; }
 int pscl::ctx_device(const pscl_ctx *c) { return c->device; }
 
-int pscl::job_set_coop_stream(pscl_job *j, cudaStream_t s)
+int pscl::job_set_coop_stream(pscl_job *j, const cudaStream_t *s, int n, int at, bool alone)
 {
     for (int i = 0; i < 2; i++)
         if (!j->coop_ev[i]) CU(cudaEventCreateWithFlags(&j->coop_ev[i], cudaEventDisableTiming));
-    j->coop = s;
+    j->coop = s[at];
+    j->coop_n = 0;
+    for (int i = 0; alone && i < n; i++)
+        if (i != at) j->coop_all[j->coop_n++] = s[i];
     drop_graph(j);
     return PSCL_OK;
 }
@@ -898,9 +903,14 @@ static int enqueue_subcluster(pscl_job *j, bool events)
     if (j->coop) {
         CU(cudaEventRecord(j->coop_ev[0], st));
         CU(cudaStreamWaitEvent(j->coop, j->coop_ev[0], 0));
+        for (int i = 0; i < j->coop_n; i++) {
+            CU(cudaEventRecord(j->coop_ev[1], j->coop_all[i]));
+            CU(cudaStreamWaitEvent(j->coop, j->coop_ev[1], 0));
+        }
         CU(launch_peel(j->pb, j->n, j->d, j->N, j->ctx->sm_count, j->coop, &j->kt));
         CU(cudaEventRecord(j->coop_ev[1], j->coop));
         CU(cudaStreamWaitEvent(st, j->coop_ev[1], 0));
+        for (int i = 0; i < j->coop_n; i++) CU(cudaStreamWaitEvent(j->coop_all[i], j->coop_ev[1], 0));
     } else {
         CU(launch_peel(j->pb, j->n, j->d, j->N, j->ctx->sm_count, st, &j->kt));
     }

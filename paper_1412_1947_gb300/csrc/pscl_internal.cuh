@@ -192,9 +192,10 @@ size_t group_cnt_words(int64_t n, int m);
 cudaError_t launch_group_unequal(const float *x, int64_t n, int d, const double *lo, const double *hi, int m,
                                  float *lm, int32_t *group, uint32_t *cnt, uint32_t *total, uint32_t *perm,
                                  cudaStream_t st, KTimer *kt);
-// api.cu: route a job's peel through stream s (ordered with the job's own stream);
-// a context's stream and device.
-int job_set_coop_stream(pscl_job *j, cudaStream_t s);
+// api.cu: route a job's peel through stream s[at] of the n (<= 4) that peels of other jobs use
+// (ordered with the job's own stream; with `alone` after all peels queued on any of them and
+// before all later ones); a context's stream and device.
+int job_set_coop_stream(pscl_job *j, const cudaStream_t *s, int n, int at, bool alone);
 cudaStream_t ctx_stream(const pscl_ctx *c);
 int ctx_device(const pscl_ctx *c);
 
