@@ -293,7 +293,8 @@ int pscl_measure_grid_barrier(int device, double *us);
  * The paper has no counterpart: this is a service for callers that cannot allocate
  * device memory (a framework whose allocator owns the device, a real-time host that
  * forbids allocation after start-up, code where an allocation would synchronise).  It
- * runs the kernel of the SSE step of pscl_cluster: labels[i] = the nearest of the k
+ * runs the SSE step of pscl_cluster (large calls with d = 16, 32 or 64, up to 512 centers and
+ * both arrays on 16-byte boundaries on the tensor cores, with the same results): labels[i] = the nearest of the k
  * centers to points[i] (float32 squared distance, lowest index on ties) and *sse = the
  * sum over points of that distance, added in double in a fixed order.
  *   points   n x d float32 row-major, device memory of the current device

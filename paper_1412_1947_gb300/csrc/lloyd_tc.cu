@@ -55,6 +55,8 @@ constexpr unsigned kDefaultWait = 1u << 26;
 constexpr size_t kTcSmemMax = 220 * 1024;
 constexpr uint32_t kTieBit = 0x80000000u; // label of a row left to the float32 re-scoring
 
+constexpr uint32_t kFlatAll = 0x40000000u; // FLAT: every center is a candidate
+
 enum TcMode { kModeTf32 = 0, kModeBf16 = 1, kModeTf32x3 = 2, kModeBf16x3 = 3 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -242,6 +244,20 @@ __device__ __forceinline__ float tf32_rna(float x)
 
 __device__ __forceinline__ float bf16_rn(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
+// One MMA of the tile's 128 rows: kind::f16 on bfloat16 operands, or kind::tf32.
+template <bool BF16>
+__device__ __forceinline__ void mma(uint32_t dcol, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t accum)
+{
+    if (BF16)
+        asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %4, 0;\n"
+                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n}\n"
+                     ::"r"(dcol), "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+    else
+        asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %4, 0;\n"
+                     " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, q;\n}\n"
+                     ::"r"(dcol), "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+}
+
 // ---------------------------------------------------------------- operand modes
 template <int MODE>
 struct Op {
@@ -376,6 +392,11 @@ struct TcArgs {
     float *st_m1 = nullptr, *st_m2 = nullptr;
     int32_t *st_c1 = nullptr;
     uint32_t *ties = nullptr;
+    // FLAT launches: one set of flat_rows rows and flat_k centers (up to 512), CTA c the tiles
+    // [c T / G, (c + 1) T / G); undecided rows are only marked.  tbufs: accumulators (one of
+    // up to 512 columns when k > 256).
+    int64_t flat_rows = 0;
+    int flat_k = 0, tbufs = 2;
 };
 
 // A run: consecutive units of one set in a CTA's range, streamed as 128-row tiles.
@@ -401,7 +422,23 @@ __device__ __forceinline__ bool next_run(const SegTable &t, int &u, int ue, Run 
     return true;
 }
 
-template <int D, int MODE>
+// The next run of a FLAT launch's CTA (its only one).
+__device__ __forceinline__ bool flat_run(const TcArgs &p, int &u, int ue, Run &run)
+{
+    if (u >= ue) return false;
+    u = ue;
+    const int64_t tiles = (p.flat_rows + kTileRows - 1) / kTileRows;
+    const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
+    run.s = 0;
+    run.k = p.flat_k;
+    run.c0 = 0;
+    run.row0 = t0 * kTileRows;
+    run.R = (int)(min(p.flat_rows, t1 * kTileRows) - run.row0);
+    run.ntiles = (int)(t1 - t0);
+    return run.ntiles > 0;
+}
+
+template <int D, int MODE, bool FLAT = false>
 __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_tc_assign(const __grid_constant__ CUtensorMap xmap, const TcArgs p)
 {
     using O = Op<MODE>;
@@ -411,7 +448,9 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
     // boundary (the bank swizzle of the point boxes repeats every 8 rows of 128 bytes)
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     unsigned char *sx = smem;
-    const uint32_t XS = D == 128 ? (uint32_t)p.xslots : 2u, AS = D == 128 ? (uint32_t)p.astages : 2u;
+    constexpr bool kVar = FLAT || D == 128;                 // ring sizes set by the launch
+    const uint32_t XS = kVar ? (uint32_t)p.xslots : 2u, AS = kVar ? (uint32_t)p.astages : 2u;
+    const uint32_t TB = FLAT ? (uint32_t)p.tbufs : 2u;       // accumulators
     unsigned char *sa = sx + (size_t)XS * L::kXBytes;
     unsigned char *sb = sa + (size_t)AS * L::kABytes;
     TileMeta *meta = reinterpret_cast<TileMeta *>(sb + (size_t)(p.npmax / 8) * L::kGroup);
@@ -435,7 +474,8 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
     const uint32_t STALL = b0 + 8u * (uint32_t)(2 * kXMax + 2 * kAMax + 4 + 2 * kMeta);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ub = p.split[blockIdx.x], ue = p.split[blockIdx.x + 1];
+    const int ub = FLAT ? 0 : p.split[blockIdx.x], ue = FLAT ? 1 : p.split[blockIdx.x + 1];
+    auto next = [&](int &u, Run &run) { return FLAT ? flat_run(p, u, ue, run) : next_run(p.t, u, ue, run); };
     const unsigned lim = p.wait_limit;
     volatile int *abort = &s_abort;
 
@@ -464,7 +504,7 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
     }
     if (warp == 0 && ub < ue) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&tmem_slot)), "r"(2u * p.ncols));
+                     ::"r"(smem_u32(&tmem_slot)), "r"(TB * p.ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -485,7 +525,7 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
             Run run;
             uint32_t j = 0;                              // slots filled so far
             bool ok = true;
-            while (ok && next_run(p.t, u, ue, run)) {
+            while (ok && next(u, run)) {
                 for (int tt = 0; tt < run.ntiles && ok; tt++) {
                     for (int part = 0; part < L::kXTile; part++, j++) {
                         const int s = (int)(j % XS);
@@ -514,13 +554,16 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
             Run run;
             uint32_t i = 0, issued = 0;
             bool ok = true;
-            while (ok && next_run(p.t, u, ue, run)) {
+            while (ok && next(u, run)) {
                 const int np = (run.k + 15) & ~15;
-                const uint32_t idesc = O::idesc(np);
+                // more than 256 columns (FLAT): two instructions per step, the second on the
+                // operand B rows and accumulator columns from 256 on
+                const int n2 = FLAT && np > 256 ? np - 256 : 0;
+                const uint32_t idesc = O::idesc(np - n2), idesc2 = O::idesc(n2);
                 for (int tt = 0; tt < run.ntiles; tt++, i++) {
-                    const int a = (int)(i % AS), bfr = (int)(i & 1u);
+                    const int a = (int)(i % AS), bfr = (int)(TB == 2u ? i & 1u : 0u);
                     if (!mbar_wait(AFULL(a), (i / AS) & 1u, lim, abort) ||
-                        (i >= 2 && !mbar_wait(TEMPTY(bfr), ((i >> 1) - 1) & 1u, lim, abort))) {
+                        (i >= TB && !mbar_wait(TEMPTY(bfr), (i / TB - 1) & 1u, lim, abort))) {
                         ok = false;
                         break;
                     }
@@ -542,14 +585,8 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
                             const uint32_t cb = (uint32_t)((pb * D) / O::kPerChunk + 2 * kb) * 128u;
                             const uint64_t ad = smem_desc(abase + ca, 128, L::kGroup);
                             const uint64_t bd = smem_desc(bbase + cb, 128, L::kGroup);
-                            if (O::kBf16)
-                                asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %4, 0;\n"
-                                             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n}\n"
-                                             ::"r"(dcol), "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
-                            else
-                                asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %4, 0;\n"
-                                             " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, q;\n}\n"
-                                             ::"r"(dcol), "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+                            mma<O::kBf16>(dcol, ad, bd, idesc, accum);
+                            if (FLAT && n2) mma<O::kBf16>(dcol + 256u, ad, smem_desc(bbase + 32u * L::kGroup + cb, 128, L::kGroup), idesc2, accum);
                             accum = 1;
                         }
                     }
@@ -561,8 +598,8 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
                 }
             }
             if (*abort)   // MMAs still in flight finish before TMEM is released
-                for (uint32_t j = issued > 2 ? issued - 2 : 0u; j < issued; j++)
-                    mbar_drain(TFULL((int)(j & 1u)), (j >> 1) & 1u, lim);
+                for (uint32_t j = issued > TB ? issued - TB : 0u; j < issued; j++)
+                    mbar_drain(TFULL((int)(j % TB)), (j / TB) & 1u, lim);
         }
     } else if (warp >= kCvtWarp0) {
         // ---- converters: operand B per set, operand A and ||x~|| per tile
@@ -577,7 +614,7 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
         bool ok = !*abort;
         // every converter thread passes the same named barriers: the set loop runs to the
         // end, and after a failed wait only the bookkeeping goes on
-        while (next_run(p.t, u, ue, run)) {
+        while (next(u, run)) {
             // the earlier tiles' MMAs must be done before operand B and s_ref change
             for (uint32_t j = i > AS ? i - AS : 0u; ok && j < i; j++)
                 ok = mbar_wait(AEMPTY((int)(j % AS)), (j / AS) & 1u, lim, abort);
@@ -735,7 +772,8 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
             }
         }
     } else {
-        // ---- epilogue warpgroup g = warp / 4 takes the tiles i with i % 2 == g
+        // ---- epilogue warpgroup g = warp / 4 takes the tiles i with i % 2 == g (with a single
+        // accumulator group 0 takes them all)
         const int g = warp >> 2, q4 = warp & 3, r = q4 * 32 + lane;
         const float kInf = __int_as_float(0x7f800000);
         constexpr int kTerms = (O::kSplit ? 3 : 1) * D + O::kMmaK;   // products accumulated per v_j
@@ -749,12 +787,12 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
         Run run;
         uint32_t i = 0;
         bool ok = !*abort;
-        while (ok && next_run(p.t, u, ue, run)) {
+        while (ok && next(u, run)) {
             const int k = run.k;
             for (int tt = 0; tt < run.ntiles; tt++, i++) {
-                if ((int)(i & 1u) != g) continue;
+                if ((int)(TB == 2u ? i & 1u : 0u) != g) continue;
                 const int m = (int)(i % kMeta);
-                ok = mbar_wait(TFULL(g), (i >> 1) & 1u, lim, abort) && mbar_wait(MFULL(m), (i / kMeta) & 1u, lim, abort);
+                ok = mbar_wait(TFULL(g), (i / TB) & 1u, lim, abort) && mbar_wait(MFULL(m), (i / kMeta) & 1u, lim, abort);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
                     break;
@@ -807,6 +845,19 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
                 // pass 2: the centers with v_j < thr as a bit mask (word c: centers 32c .. 32c+31);
                 // one bit is the label, more a near tie
                 uint32_t w[8];
+                int nc = 0, first = 0;
+                if constexpr (FLAT) {        // the candidates, if they are few
+                    for (int c = 0; 32 * c < k; c++) {
+                        uint32_t v[32];
+                        tmem_ld32_nowait(taddr + (uint32_t)(32 * c), v);
+                        tmem_wait();
+                        const int rem = k - 32 * c;
+                        uint32_t acc = less_mask(v, thr) & (rem >= 32 ? 0xffffffffu : (1u << rem) - 1u);
+                        // up to three candidates, nine bits each in ascending order
+                        for (; acc; acc &= acc - 1u, nc++)
+                            if (nc < 3) first |= (32 * c + __ffs(acc) - 1) << (9 * nc);
+                    }
+                } else
 #pragma unroll
                 for (int c = 0; c < 8; c++) {
                     w[c] = 0u;
@@ -822,13 +873,19 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(TEMPTY(g));
-                int nc = 0, first = 0;
+                if constexpr (!FLAT) {
 #pragma unroll
-                for (int c = 7; c >= 0; c--) {
-                    nc += __popc(w[c]);
-                    if (w[c]) first = 32 * c + __ffs(w[c]) - 1;
+                    for (int c = 7; c >= 0; c--) {
+                        nc += __popc(w[c]);
+                        if (w[c]) first = 32 * c + __ffs(w[c]) - 1;
+                    }
                 }
-                if (p.ref_centers) {
+                if constexpr (FLAT) {
+                    // one candidate: the label; two or three: their indices (two: the second
+                    // twice); more, or none (values that are not finite): every center
+                    if (nc == 2) first |= (first >> 9) << 18;
+                    if (live) p.labels[row] = nc == 1 ? first : (int32_t)(kTieBit | (nc == 2 || nc == 3 ? (uint32_t)first : kFlatAll));
+                } else if (p.ref_centers) {
                     // a chunk of a whole-set search: fold this chunk into the row's state
                     bool tie_row = false;
                     if (live) {
@@ -893,7 +950,7 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
         if (s_stat[1]) atomicAdd(&p.flags[3], s_stat[1]);
         if (s_abort) atomicOr(&p.flags[1], 4u);
     }
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2u * p.ncols));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TB * p.ncols));
 }
 
 // ---------------------------------------------------------------- sums and near ties
@@ -1399,14 +1456,14 @@ cudaError_t make_xmap(const float *pts, int64_t rows, CUtensorMap *map)
 // two A buffers before four slots (the conversion of a tile then overlaps the MMAs of the
 // one before; with one buffer they alternate).
 template <int D, int MODE>
-size_t assign_smem(int kmax, int *xslots = nullptr, int *astages = nullptr)
+size_t assign_smem(int kmax, int *xslots = nullptr, int *astages = nullptr, bool flat = false)
 {
     using L = TcLayout<D, MODE>;
     const int np = (kmax + 15) & ~15;
     const size_t fixed = 1024 + (size_t)(np / 8) * L::kGroup + (size_t)kMeta * sizeof(TileMeta);
-    static const int opt[4][2] = {{4, 2}, {2, 2}, {4, 1}, {2, 1}};
+    static const int opt[5][2] = {{4, 2}, {2, 2}, {4, 1}, {2, 1}, {1, 1}};
     size_t b = 0;
-    for (int o = D == 128 ? 0 : 1; o < (D == 128 ? 4 : 2); o++) {
+    for (int o = D == 128 ? 0 : 1; o < (flat ? 5 : D == 128 ? 4 : 2); o++) {
         b = fixed + (size_t)opt[o][0] * L::kXBytes + (size_t)opt[o][1] * L::kABytes;
         if (xslots) *xslots = opt[o][0];
         if (astages) *astages = opt[o][1];
@@ -1606,6 +1663,152 @@ cudaError_t lloyd_chunks_dispatch(const LloydBuffers &b, int iter, int k, uint32
     return cudaGetLastError();
 }
 
+// float32 direct distance of a row in shared memory to a center in global memory.
+template <int D>
+__device__ __forceinline__ float tile_dist(const float4 *xr, const float *__restrict__ center)
+{
+    const float4 *cr = reinterpret_cast<const float4 *>(center);
+    float acc = 0.0f;
+#pragma unroll 8
+    for (int a = 0; a < D / 4; a++) {
+        const float4 v = xr[a], c = __ldg(&cr[a]);
+        float e;
+        e = __fsub_rn(v.x, c.x); acc = __fmaf_rn(e, e, acc);
+        e = __fsub_rn(v.y, c.y); acc = __fmaf_rn(e, e, acc);
+        e = __fsub_rn(v.z, c.z); acc = __fmaf_rn(e, e, acc);
+        e = __fsub_rn(v.w, c.w); acc = __fmaf_rn(e, e, acc);
+    }
+    return acc;
+}
+
+// Labels and SSE after a FLAT assignment: a row with two or three candidates is scored against
+// them in float32 by its thread; the rows with more (all rows if the assignment gave up)
+// against every center, a warp per row and lane l the centers l, l + 32, ... (the lowest index
+// among equal sums).  The distances are summed as k_sse_from_labels does it, from the same
+// tile in shared memory.
+template <int D>
+__global__ void __launch_bounds__(kSseThreads) k_flat_resolve(const float *__restrict__ x, int64_t n,
+                                                              const float *__restrict__ centers, int k, int32_t *labels,
+                                                              const uint32_t *flags, double *blk_sse, double *sse,
+                                                              uint32_t *ticket)
+{
+    extern __shared__ __align__(16) float4 xs[];
+    constexpr int LD4 = tile_ld4(D), NW = kSseThreads / 32;
+    __shared__ int s_lab[kSseThreads], s_list[kSseThreads];
+    __shared__ int s_n;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const bool gave_up = flags[1] != 0u;
+    double part = 0.0;
+    const int64_t stride = (int64_t)gridDim.x * kSseThreads;
+    for (int64_t i0 = (int64_t)blockIdx.x * kSseThreads; i0 < n; i0 += stride) {
+        const int rows = (int)min((int64_t)kSseThreads, n - i0);
+        __syncthreads();
+        if (t == 0) s_n = 0;
+        tile_load(xs, x + i0 * D, rows, rows, D, LD4);
+        const int32_t l0 = t < rows ? labels[i0 + t] : 0;
+        const bool known = t < rows && !gave_up && (uint32_t)l0 < (uint32_t)k;
+        const bool few = t < rows && !gave_up && !known && !((uint32_t)l0 & kFlatAll);
+        const bool open = t < rows && !known && !few;
+        __syncthreads();
+        if (open) s_list[atomicAdd(&s_n, 1)] = t;
+        __syncthreads();
+        const int no = s_n;
+        for (int q = w; q < no; q += NW) {
+            const int r = s_list[q];
+            float bd = __int_as_float(0x7f800000);
+            int bj = 0x7fffffff;
+            for (int j = lane; j < k; j += 64) {           // two centers at a time
+                const int j2 = j + 32 < k ? j + 32 : j;
+                const float4 *c0 = reinterpret_cast<const float4 *>(centers + (size_t)j * D);
+                const float4 *c1 = reinterpret_cast<const float4 *>(centers + (size_t)j2 * D);
+                float d0 = 0.0f, d1 = 0.0f;
+#pragma unroll 4
+                for (int a = 0; a < D / 4; a++) {
+                    const float4 v = xs[r * LD4 + a], u = __ldg(&c0[a]), y = __ldg(&c1[a]);
+                    float e;
+                    e = __fsub_rn(v.x, u.x); d0 = __fmaf_rn(e, e, d0);
+                    e = __fsub_rn(v.x, y.x); d1 = __fmaf_rn(e, e, d1);
+                    e = __fsub_rn(v.y, u.y); d0 = __fmaf_rn(e, e, d0);
+                    e = __fsub_rn(v.y, y.y); d1 = __fmaf_rn(e, e, d1);
+                    e = __fsub_rn(v.z, u.z); d0 = __fmaf_rn(e, e, d0);
+                    e = __fsub_rn(v.z, y.z); d1 = __fmaf_rn(e, e, d1);
+                    e = __fsub_rn(v.w, u.w); d0 = __fmaf_rn(e, e, d0);
+                    e = __fsub_rn(v.w, y.w); d1 = __fmaf_rn(e, e, d1);
+                }
+                if (d0 < bd) { bd = d0; bj = j; }
+                if (j2 != j && d1 < bd) { bd = d1; bj = j2; }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                const float od = __shfl_xor_sync(0xffffffffu, bd, o);
+                const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+                if (od < bd || (od == bd && oj < bj)) {
+                    bd = od;
+                    bj = oj;
+                }
+            }
+            if (lane == 0) s_lab[r] = bj < k ? bj : 0;     // (no distance below infinity: center 0)
+        }
+        __syncthreads();
+        if (t < rows) {
+            const float4 *xr = xs + t * LD4;
+            int l = known ? l0 : open ? s_lab[t] : min(l0 & 511, k - 1);
+            float acc = tile_dist<D>(xr, centers + (size_t)l * D);
+            if (few) {
+#pragma unroll
+                for (int c = 1; c < 3; c++) {
+                    const int j = min((l0 >> (9 * c)) & 511, k - 1);
+                    const float v = tile_dist<D>(xr, centers + (size_t)j * D);
+                    if (v < acc) {
+                        acc = v;
+                        l = j;
+                    }
+                }
+            }
+            if (!known) labels[i0 + t] = l;
+            // the float32 pass adds its smallest distance, infinity where none is smaller
+            part = __dadd_rn(part, acc < __int_as_float(0x7f800000) ? (double)acc : (double)__int_as_float(0x7f800000));
+        }
+    }
+    sse_reduce(part, blk_sse, sse, ticket);
+}
+
+template <int D, int MODE>
+cudaError_t flat_dispatch(const float *x, int64_t n, const float *centers, int k, int32_t *labels, double *blk_sse,
+                          double *sse, uint32_t *ticket, uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt)
+{
+    CUtensorMap map;
+    cudaError_t e = make_xmap<D, MODE>(x, n, &map);
+    if (e != cudaSuccess) return e;
+    TcArgs a;
+    a.centers = centers;
+    a.labels = labels;
+    a.tmask = nullptr;
+    a.t = SegTable{};
+    a.split = nullptr;
+    a.flags = flags;
+    a.wait_limit = kDefaultWait;
+    a.stall = 0;
+    a.npmax = (k + 15) & ~15;
+    a.tbufs = a.npmax > 256 ? 1 : 2;
+    a.ncols = a.npmax > 256 ? 512u : tmem_cols(a.npmax);
+    a.flat_rows = n;
+    a.flat_k = k;
+    const size_t smem = assign_smem<D, MODE>(k, &a.xslots, &a.astages, true);
+    auto ka = k_tc_assign<D, MODE, true>;
+    if ((e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    const size_t sr = (size_t)kSseThreads * tile_ld4(D) * 16;
+    auto kr = k_flat_resolve<D>;
+    if ((e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr)) != cudaSuccess) return e;
+    // one CTA per SM, two where the kernel is built for it and the accumulators leave room
+    const int m = tc_min_blocks<D>() > 1 && a.tbufs * a.ncols <= 256u && smem <= kTcSmemMax / 2 ? 2 : 1;
+    kt->begin(st);
+    ka<<<m * sm_count, tc_threads<D>(), smem, st>>>(map, a);
+    kr<<<sse_grid(n, sm_count), kSseThreads, sr, st>>>(x, n, centers, k, labels, flags, blk_sse, sse, ticket);
+    kt->end(PSCL_K_FINAL_SSE, st);
+    return cudaGetLastError();
+}
+
 template <int MODE>
 cudaError_t lloyd_chunks_by_d(int d, const LloydBuffers &b, int iter, int k, uint32_t *flags, int sm_count,
                               cudaStream_t st, KTimer *kt)
@@ -1653,6 +1856,9 @@ cudaError_t tc_by_d(const LloydBuffers &b, const SegTable &t, int d, int iter, i
 // k = 64 180 against 75; 300000 rows, k = 64, 365 against 138); TF32X3's 135 KB of operand A
 // per tile would leave one buffer and no overlap.
 constexpr int64_t kWideRows = 160 * kTileRows;
+constexpr int64_t kFlatRows = 160 * kTileRows;     // see flat_sse_supported
+constexpr int kFlatCenters = 32;
+constexpr double kFlatWork = 8e7;
 
 template <int MODE>
 bool fits_by_d(int d, int kmax, int64_t rows)
@@ -1707,6 +1913,38 @@ bool tc_supported(int d, int kmax, int prec, int64_t rows)
 bool tc_sse_supported(int d, int k, int prec, int64_t rows)
 {
     return k >= 1 && tc_supported(d, std::min(k, tc_chunk(d)), prec, rows);
+}
+
+// The nearest-center pass of one set without scratch per row: at most two chunks of columns,
+// points and centers on 16-byte boundaries (the tensor map's and operand B's reads), rows for
+// a tile per SM, and enough work.  Float32 kernel against this pass, us: 20480 x 16 k = 64
+// 14.5, 18.5, k = 256 33, 21; 20480 x 64 k = 64 23.7, 27.3, k = 128 35.9, 28.7; 10^6 x 16
+// k = 32 80, 71; 10^6 x 32 k = 64 273, 157; 10^6 x 64 k = 32 275, 248, k = 300 1508, 404; so the
+// line lies at rows x centers x attributes = 8e7 and 32 centers.
+bool flat_sse_supported(const float *x, int64_t n, int d, const float *centers, int k)
+{
+    if (n < kFlatRows || n >= ((int64_t)1 << 31) || k < kFlatCenters || k > 512 || (double)n * k * d < kFlatWork ||
+        !encode_tiled())
+        return false;
+    if ((((uintptr_t)x | (uintptr_t)centers) & 15u) != 0) return false;
+    switch (d) {
+    case 16: return assign_smem<16, kModeTf32x3>(k, nullptr, nullptr, true) <= kTcSmemMax;
+    case 32: return assign_smem<32, kModeTf32x3>(k, nullptr, nullptr, true) <= kTcSmemMax;
+    case 64: return assign_smem<64, kModeBf16x3>(k, nullptr, nullptr, true) <= kTcSmemMax;
+    default: return false;
+    }
+}
+
+cudaError_t launch_flat_sse(const float *x, int64_t n, int d, const float *centers, int k, int32_t *labels,
+                            double *blk_sse, double *sse, uint32_t *ticket, uint32_t *flags, int sm_count,
+                            cudaStream_t st, KTimer *kt)
+{
+    switch (d) {
+    case 16: return flat_dispatch<16, kModeTf32x3>(x, n, centers, k, labels, blk_sse, sse, ticket, flags, sm_count, st, kt);
+    case 32: return flat_dispatch<32, kModeTf32x3>(x, n, centers, k, labels, blk_sse, sse, ticket, flags, sm_count, st, kt);
+    case 64: return flat_dispatch<64, kModeBf16x3>(x, n, centers, k, labels, blk_sse, sse, ticket, flags, sm_count, st, kt);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_lloyd_chunks_tc(const LloydBuffers &b, int d, int iter, int k, int prec, uint32_t *flags,

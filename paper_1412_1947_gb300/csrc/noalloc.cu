@@ -4,8 +4,8 @@
 // Some callers may not call cudaMalloc at all: code that runs under an allocator that
 // owns the whole device (a framework's caching allocator, a fixed memory plan), real-time
 // or embedded hosts that forbid allocation after start-up, or code paths where an
-// allocation would synchronise the device.  This entry point runs the same kernel as the
-// SSE step of pscl_cluster, but its scratch (one float64 partial sum per thread block and a
+// allocation would synchronise the device.  This entry point runs the
+// SSE step of pscl_cluster, on the tensor cores where the shape pays, but its scratch (one float64 partial sum per thread block and a
 // completion ticket) lives in the file-scope array below instead of memory the library
 // allocates.  The caller supplies the points, the centers and the two outputs.
 #include <cuda.h>
@@ -22,7 +22,8 @@ constexpr int kNoAllocMaxBlocks = 4096;               // partial sums the scratc
 constexpr size_t kNoAllocBytes = kNoAllocMaxBlocks * sizeof(double) + 256;
 constexpr int kMaxDevices = 64;
 
-// Scratch shared by every call on a device: [partials (kNoAllocMaxBlocks doubles) | ticket].
+// Scratch shared by every call on a device: [partials (kNoAllocMaxBlocks doubles) | ticket, 3
+// words, the tensor-core kernel's 4 flag words].
 // In host code this name is only a stand-in for the device array; the device address is
 // obtained with cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char g_sse_scratch[kNoAllocBytes];
@@ -119,13 +120,16 @@ extern "C" int pscl_assign_sse_noalloc(const float *points, int64_t n, int32_t d
     uint32_t *ticket = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(scratch) +
                                                     kNoAllocMaxBlocks * sizeof(double));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the ticket counts finished blocks and must start at zero (the partials are overwritten)
-    if (cudaMemsetAsync(ticket, 0, sizeof(uint32_t), st) != cudaSuccess) {
+    // the ticket counts finished blocks and must start at zero, as must the flags (the partials
+    // are overwritten)
+    if (cudaMemsetAsync(ticket, 0, 8 * sizeof(uint32_t), st) != cudaSuccess) {
         cudaGetLastError();
         return fail(PSCL_ECUDA, "pscl_assign_sse_noalloc: clearing the scratch failed");
     }
     KTimer kt;
-    cudaError_t e = launch_final_sse(points, n, d, centers, k, labels, partials, sse, ticket, sms, st, &kt);
+    cudaError_t e = flat_sse_supported(points, n, d, centers, k)
+                        ? launch_flat_sse(points, n, d, centers, k, labels, partials, sse, ticket, ticket + 4, sms, st, &kt)
+                        : launch_final_sse(points, n, d, centers, k, labels, partials, sse, ticket, sms, st, &kt);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(PSCL_ECUDA, cudaGetErrorString(e));

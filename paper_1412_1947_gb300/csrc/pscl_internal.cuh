@@ -268,6 +268,12 @@ cudaError_t launch_final_sse_tc(const float *x, int64_t n, int d, const float *c
                                 const SegTable &trem, uint32_t *scratch, int32_t *labels, double *blk_sse,
                                 double *sse, uint32_t *ticket, int prec, uint32_t *flags, unsigned wait_limit,
                                 int sm_count, cudaStream_t st, KTimer *kt);
+// The SSE pass of launch_final_sse for a caller's arrays, on the tensor cores (flags: 4 words,
+// cleared; the same labels and sum).
+bool flat_sse_supported(const float *x, int64_t n, int d, const float *centers, int k);
+cudaError_t launch_flat_sse(const float *x, int64_t n, int d, const float *centers, int k, int32_t *labels,
+                            double *blk_sse, double *sse, uint32_t *ticket, uint32_t *flags, int sm_count,
+                            cudaStream_t st, KTimer *kt);
 // Assignment on the tensor cores and the exact sums of the iteration (two persistent
 // launches over all units; needs t.split).
 cudaError_t launch_lloyd_assign_tc(const LloydBuffers &b, const SegTable &t, int d, int iter, int kmax, int prec,
