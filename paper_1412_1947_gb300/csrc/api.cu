@@ -1501,8 +1501,8 @@ static int batch_enqueue(pscl_batch *b, int iters, uint64_t seed, int prec, bool
         }
     }
     if (events) CU(cudaEventRecord(b->ev[1], st));
-    CU(launch_seg_sse(b->x, t, u0, b->d, b->centers, b->plan.kmax, b->out_labels, b->unit_sse, b->seg_sse, st,
-                      &b->kt));
+    CU(launch_seg_sse(lb, t, u0, b->d, b->plan.kmax, prec, b->out_labels, b->unit_sse, b->seg_sse, b->flags,
+                      b->ctx->sm_count, st, &b->kt));
     return PSCL_OK;
 }
 

@@ -1071,12 +1071,15 @@ cudaError_t launch_lloyd_iter(const LloydBuffers &b, int32_t *count_next, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_seg_sse(const float *pts, const SegTable &t, const int32_t *seg_unit0, int d,
-                           const float *centers, int kmax, int32_t *labels, double *unit_sse, double *seg_sse,
-                           cudaStream_t st, KTimer *kt)
+cudaError_t launch_seg_sse(const LloydBuffers &b, const SegTable &t, const int32_t *seg_unit0, int d, int kmax,
+                           int prec, int32_t *labels, double *unit_sse, double *seg_sse, uint32_t *flags,
+                           int sm_count, cudaStream_t st, KTimer *kt)
 {
+    const float *pts = b.pts, *centers = b.centers;
     cudaError_t e;
-    if (d >= kTiledMin && d <= kTiledMax && kmax >= kTiledCenters) {
+    if (seg_sse_tc_supported(b, t, d, kmax, prec)) {
+        e = launch_seg_sse_tc(b, t, d, kmax, prec, labels, unit_sse, flags, sm_count, st, kt);
+    } else if (d >= kTiledMin && d <= kTiledMax && kmax >= kTiledCenters) {
         const size_t smem = tile_smem(d);
         if (const cudaError_t ea = cudaFuncSetAttribute(k_seg_sse_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return ea;
         kt->begin(st);

@@ -1479,8 +1479,8 @@ size_t sums_smem(int kmax)
 }
 
 template <int D, int MODE>
-cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int kmax, uint32_t *flags, int sm_count,
-                        cudaStream_t st, KTimer *kt)
+cudaError_t assign_only(const LloydBuffers &b, const SegTable &t, int kmax, uint32_t *flags, int sm_count,
+                        cudaStream_t st, KTimer *kt, int ktag)
 {
     CUtensorMap map;
     cudaError_t e = make_xmap<D, MODE>(b.pts, b.rows, &map);
@@ -1510,8 +1510,17 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     a.split = t.split + t.split_off[ma];
     kt->begin(st);
     ka<<<ma * sm_count, tc_threads<D>(), smem, st>>>(map, a);
-    kt->end(PSCL_K_LLOYD_ASSIGN, st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    kt->end(ktag, st);
+    return cudaGetLastError();
+}
+
+template <int D, int MODE>
+cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int kmax, uint32_t *flags, int sm_count,
+                        cudaStream_t st, KTimer *kt)
+{
+    cudaError_t e = assign_only<D, MODE>(b, t, kmax, flags, sm_count, st, kt, PSCL_K_LLOYD_ASSIGN);
+    if (e != cudaSuccess) return e;
+    const int32_t *raw = b.raw ? b.raw : b.labels;
     // sums: four CTAs' unit ranges per SM whatever fits at once, so that the block scheduler
     // evens out ranges whose near ties cost more; the first iteration adds every row, the
     // later ones (raw labels kept apart) only the rows that moved
@@ -1535,7 +1544,7 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
     auto ks = k_tc_sums<D>;
     if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss)) != cudaSuccess) return e;
     kt->begin(st);
-    ks<<<m * sm_count, sum_threads<D>(), ss, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], a.labels, b.labels,
+    ks<<<m * sm_count, sum_threads<D>(), ss, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], raw, b.labels,
                                                    b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count, kmax);
     kt->end(PSCL_K_LLOYD_SUMS, st);
     return cudaGetLastError();
@@ -1809,6 +1818,91 @@ cudaError_t flat_dispatch(const float *x, int64_t n, const float *centers, int k
     return cudaGetLastError();
 }
 
+// Labels and SSE of independent sets after an assignment against their final centers, a CTA per
+// work unit: the near ties scored in float32 against their candidates (rescore_row, the centers
+// in shared memory), every row's distance to its center summed as the float32 pass does it (a
+// thread's rows in order, the block's fixed tree).  A unit's rows come in 256 at a time through
+// shared memory.
+template <int D>
+__global__ void __launch_bounds__(kSseThreads) k_seg_sse_ties(const float *__restrict__ pts, SegTable t,
+                                                              const float *__restrict__ centers,
+                                                              const int32_t *__restrict__ raw,
+                                                              const uint32_t *__restrict__ tmask, int32_t *labels,
+                                                              double *unit_sse, int kmax)
+{
+    extern __shared__ __align__(16) float4 xs[];               // [256 rows | centers]
+    constexpr int LD4 = tile_ld4(D), DC = D + 4;
+    float *scen = reinterpret_cast<float *>(xs + kSseThreads * LD4);
+    const int u = blockIdx.x, s = t.unit_seg[u], k = t.k_eff[s], rows = t.unit_count[u];
+    const float *cen = centers + (int64_t)t.cen_off[s] * D;
+    const int64_t row0 = t.seg_start[s] + t.unit_start[u];
+    for (int e = threadIdx.x; e < k * (D / 4); e += kSseThreads)
+        *reinterpret_cast<float4 *>(scen + (e / (D / 4)) * DC + 4 * (e % (D / 4))) =
+            __ldg(reinterpret_cast<const float4 *>(cen) + e);
+    double part = 0.0;
+    for (int p0 = 0; p0 < rows; p0 += kSseThreads) {
+        const int nr = min(kSseThreads, rows - p0);
+        __syncthreads();
+        tile_load(xs, pts + (row0 + p0) * D, nr, nr, D, LD4);
+        const int64_t row = row0 + p0 + threadIdx.x;
+        int32_t l = (int)threadIdx.x < nr ? raw[row] : 0;
+        __syncthreads();
+        if ((int)threadIdx.x < nr) {
+            if ((uint32_t)l & kTieBit) l = rescore_row<D>(pts, tmask, scen, k, row);
+            if ((uint32_t)l >= (uint32_t)k) l = 0;              // only after an assignment that gave up
+            labels[row] = l;
+            const float4 *cr = reinterpret_cast<const float4 *>(scen + (size_t)l * DC);
+            float acc = 0.0f;
+#pragma unroll 8
+            for (int q = 0; q < D / 4; q++) {
+                const float4 v = xs[threadIdx.x * LD4 + q], c = cr[q];
+                float e;
+                e = __fsub_rn(v.x, c.x); acc = __fmaf_rn(e, e, acc);
+                e = __fsub_rn(v.y, c.y); acc = __fmaf_rn(e, e, acc);
+                e = __fsub_rn(v.z, c.z); acc = __fmaf_rn(e, e, acc);
+                e = __fsub_rn(v.w, c.w); acc = __fmaf_rn(e, e, acc);
+            }
+            part = __dadd_rn(part, (double)acc);
+        }
+    }
+    const double b = block_tree_sum(part);
+    if (threadIdx.x == 0) unit_sse[u] = b;
+}
+
+template <int D>
+size_t seg_ties_smem(int kmax)
+{
+    return (size_t)kSseThreads * tile_ld4(D) * 16 + (size_t)kmax * (D + 4) * 4;
+}
+
+template <int D, int MODE>
+cudaError_t seg_sse_tc_dispatch(const LloydBuffers &b, const SegTable &t, int kmax, int32_t *labels, double *unit_sse,
+                                uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt)
+{
+    cudaError_t e = assign_only<D, MODE>(b, t, kmax, flags, sm_count, st, kt, PSCL_K_FINAL_SSE);
+    if (e != cudaSuccess) return e;
+    const size_t smem = seg_ties_smem<D>(kmax);
+    auto kern = k_seg_sse_ties<D>;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    kt->begin(st);
+    kern<<<t.n_units, kSseThreads, smem, st>>>(b.pts, t, b.centers, b.raw, b.tmask, labels, unit_sse, kmax);
+    kt->end(PSCL_K_FINAL_SSE, st);
+    return cudaGetLastError();
+}
+
+template <int MODE>
+cudaError_t seg_sse_tc_by_d(int d, const LloydBuffers &b, const SegTable &t, int kmax, int32_t *labels,
+                            double *unit_sse, uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt)
+{
+    switch (d) {
+    case 16: return seg_sse_tc_dispatch<16, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    case 32: return seg_sse_tc_dispatch<32, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    case 64: return seg_sse_tc_dispatch<64, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    case 128: return seg_sse_tc_dispatch<128, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 template <int MODE>
 cudaError_t lloyd_chunks_by_d(int d, const LloydBuffers &b, int iter, int k, uint32_t *flags, int sm_count,
                               cudaStream_t st, KTimer *kt)
@@ -1913,6 +2007,25 @@ bool tc_supported(int d, int kmax, int prec, int64_t rows)
 bool tc_sse_supported(int d, int k, int prec, int64_t rows)
 {
     return k >= 1 && tc_supported(d, std::min(k, tc_chunk(d)), prec, rows);
+}
+
+// Independent sets' SSE on the tensor cores: where their Lloyd iterations run there, with rows
+// for a few tiles per SM (below, the float32 pass's one launch is as fast).
+bool seg_sse_tc_supported(const LloydBuffers &b, const SegTable &t, int d, int kmax, int prec)
+{
+    return prec != PSCL_PREC_FP32 && b.raw && b.tmask && t.split && b.rows >= 8 * kWideRows &&
+           tc_supported(d, kmax, prec, b.rows) && (d < 128 || seg_ties_smem<128>(kmax) <= kTcSmemMax);
+}
+
+cudaError_t launch_seg_sse_tc(const LloydBuffers &b, const SegTable &t, int d, int kmax, int prec, int32_t *labels,
+                              double *unit_sse, uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt)
+{
+    switch (mode_of(resolve_prec(d, kmax, prec, b.rows))) {
+    case kModeBf16: return seg_sse_tc_by_d<kModeBf16>(d, b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    case kModeTf32x3: return seg_sse_tc_by_d<kModeTf32x3>(d, b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    case kModeBf16x3: return seg_sse_tc_by_d<kModeBf16x3>(d, b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    default: return seg_sse_tc_by_d<kModeTf32>(d, b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
+    }
 }
 
 // The nearest-center pass of one set without scratch per row: at most two chunks of columns,

@@ -246,10 +246,11 @@ bool sets_supported(const SegTable &t, int d, int max_rows, int kmax, double eva
 cudaError_t launch_lloyd_sets(const LloydBuffers &b, const SegTable &t, int d, int64_t P, int max_rows, int kmax,
                               int iters, cudaStream_t st, KTimer *kt);
 // Independent sets: nearest center of every row within its set, per-set sums of the
-// squared distances (unit_sse: n_units doubles, seg_sse: n_seg doubles).
-cudaError_t launch_seg_sse(const float *pts, const SegTable &t, const int32_t *seg_unit0, int d,
-                           const float *centers, int kmax, int32_t *labels, double *unit_sse, double *seg_sse,
-                           cudaStream_t st, KTimer *kt);
+// squared distances (unit_sse: n_units doubles, seg_sse: n_seg doubles); b as the iterations
+// used it, prec a pscl_prec.
+cudaError_t launch_seg_sse(const LloydBuffers &b, const SegTable &t, const int32_t *seg_unit0, int d, int kmax,
+                           int prec, int32_t *labels, double *unit_sse, double *seg_sse, uint32_t *flags,
+                           int sm_count, cudaStream_t st, KTimer *kt);
 
 // lloyd_tc.cu
 bool tc_supported(int d, int kmax, int prec, int64_t rows);
@@ -268,6 +269,10 @@ cudaError_t launch_final_sse_tc(const float *x, int64_t n, int d, const float *c
                                 const SegTable &trem, uint32_t *scratch, int32_t *labels, double *blk_sse,
                                 double *sse, uint32_t *ticket, int prec, uint32_t *flags, unsigned wait_limit,
                                 int sm_count, cudaStream_t st, KTimer *kt);
+// The same on the tensor cores: labels and per-unit sums.
+bool seg_sse_tc_supported(const LloydBuffers &b, const SegTable &t, int d, int kmax, int prec);
+cudaError_t launch_seg_sse_tc(const LloydBuffers &b, const SegTable &t, int d, int kmax, int prec, int32_t *labels,
+                              double *unit_sse, uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt);
 // The SSE pass of launch_final_sse for a caller's arrays, on the tensor cores (flags: 4 words,
 // cleared; the same labels and sum).
 bool flat_sse_supported(const float *x, int64_t n, int d, const float *centers, int k);
