@@ -94,7 +94,7 @@ constexpr int kScrWords = kStageOff + 3 * kStage;
 static_assert(kScrWords >= kHistBins, "phase A's histogram fits the scratch");
 static_assert(kStageOff % 2 == 0, "staged 64-bit keys are 8-byte aligned");
 constexpr int kPeelDynWords = kScrWords + 2 * kKeyCache + kKeyCache / 4;
-constexpr int kQT = 8;                        // tiles of kThreads items per compaction scan
+constexpr int kQT = 4;                        // tiles of kThreads items per compaction scan
 constexpr int kCB = 8;                        // keys per thread in flight when classifying
 constexpr int kHoldBatch = 8;                 // state bytes per thread in flight when finding holders
 // State byte of each list position: bit 7 set once the point has held some attribute's
@@ -105,6 +105,7 @@ constexpr uint8_t kFlBand = 0x7E;
 constexpr uint8_t kFlNone = 0x7F;
 constexpr uint32_t kPosMask = 0x7FFFFFFFu;    // a band entry's id; bit 31 carries its hold flag
 constexpr int kDefaultRounds = 32;            // rounds per distance pass by default
+constexpr uint32_t kAllResolve = 6;           // boundaries up to which every CTA resolves them itself
 constexpr unsigned kDefaultSpin = 1u << 25;   // ~1-2 s of polling per barrier at most
 
 // ------------------------------------------------------------------ block helpers
@@ -193,10 +194,9 @@ __device__ bool bar_wait(PeelCtl *ctl, uint32_t *flags, unsigned target, unsigne
 // Grid-wide barrier with a bounded wait: a monotonic arrival counter (release on arrival,
 // acquire while polling), so no reset is needed within a launch.  `extra` arrivals more
 // than the grid gives are awaited (a test of the give-up path; 0 otherwise).
-__device__ bool grid_sync(PeelCtl *ctl, uint32_t *flags, unsigned &target, unsigned limit, unsigned extra = 0)
+__device__ __noinline__ bool grid_wait(PeelCtl *ctl, uint32_t *flags, unsigned target, unsigned limit, unsigned extra)
 {
     __shared__ int ok;
-    target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
         if (blockIdx.x == 0) ctl->barriers += 1;     // statistics (one writer)
@@ -205,6 +205,13 @@ __device__ bool grid_sync(PeelCtl *ctl, uint32_t *flags, unsigned &target, unsig
     }
     __syncthreads();
     return ok != 0;
+}
+
+__device__ __forceinline__ bool grid_sync(PeelCtl *ctl, uint32_t *flags, unsigned &target, unsigned limit,
+                                          unsigned extra = 0)
+{
+    target += gridDim.x;
+    return grid_wait(ctl, flags, target, limit, extra);
 }
 
 // A grid barrier whose last arriving CTA runs work() (all its threads) before any CTA
@@ -274,9 +281,10 @@ __device__ __forceinline__ float dist32(const float *__restrict__ row, const flo
 }
 
 // float64 distance exactly as defined: diff, square, add, each rounded, no fusion.
-__device__ double dist64(const float *__restrict__ row, const float *Ls, int d)
+__device__ __noinline__ double dist64(const float *__restrict__ row, const float *Ls, int d)
 {
     double s = 0.0;
+#pragma unroll 4
     for (int j = 0; j < d; j++) {
         double diff = __dsub_rn((double)__ldg(&row[j]), (double)Ls[j]);
         s = __dadd_rn(s, __dmul_rn(diff, diff));
@@ -602,10 +610,12 @@ __device__ bool select_fast(KeyAt key_at, PosAt pos_at, uint32_t nb, uint32_t ne
     return true;
 }
 
-template <class KeyAt, class PosAt>
-__device__ void select_kth(KeyAt key_at, PosAt pos_at, uint32_t nb, uint32_t need, uint32_t *scratch, uint64_t &K,
-                           uint32_t &Pp)
+// Of entries in global memory: keys gk, ids gp (bit 31 is no part of an id).
+__device__ __noinline__ void select_kth(const uint64_t *gk, const uint32_t *gp, uint32_t nb, uint32_t need,
+                                        uint32_t *scratch, uint64_t &K, uint32_t &Pp)
 {
+    auto key_at = [&](uint32_t i) -> uint64_t { return __ldcg(&gk[i]); };
+    auto pos_at = [&](uint32_t i) -> uint32_t { return __ldcg(&gp[i]) & kPosMask; };
     if (!select_fast(key_at, pos_at, nb, need, scratch, K, Pp)) select_radix(key_at, pos_at, nb, need, K, Pp);
 }
 
@@ -708,7 +718,7 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
 {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const DigitMap mp = *dm;
-    auto LID = [&](uint32_t q) -> uint32_t { return first ? s0 + q : kc ? sid[q] : __ldcg(&glin[q]); };
+    auto LID = [&](uint32_t q) -> uint32_t { return kc ? sid[q] : __ldcg(&glin[q]); };
     auto key_out = [&](bool live, uint32_t pos, uint32_t k) {
         if (live) {
             if (kc) skey[pos] = k;
@@ -740,6 +750,8 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
                 const uint32_t pos = base + q * kThreads + w * 32 + lane;
                 myid[q] = pos < n_live ? LID(pos) : s0;
             }
+            static_assert(BC * P <= 32, "a mask bit per row");
+            uint32_t hzs = 0;                              // rows with a landmark value
             float4 v[BC][P][F];
 #pragma unroll
             for (int q = 0; q < BC; q++)
@@ -787,33 +799,34 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
                         ps[i] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, m));
                     }
                 }
-                if (__any_sync(0xffffffffu, hz != 0u)) {
-                    // rare: some row of the chunk holds a landmark value (warp-uniform branch)
-#pragma unroll 1
-                    for (int u = 0; u < P; u++) {
-                        const uint32_t id = __shfl_sync(0xffffffffu, myid[q], u * RW + g);
-                        const uint32_t rpos = base + q * kThreads + w * 32 + u * RW + g;
-                        if (((hz >> u) & 1u) && rpos < n_live) {
-                            const float4 *r4 = reinterpret_cast<const float4 *>(x + (size_t)id * D) + sl;
-                            for (int f = 0; f < F; f++) {
-                                const float4 vv = __ldg(r4 + P * f);
-                                const int j = 4 * (sl + P * f);
-                                if (vv.x == Ls[j + 0] && in_mask(jm, j + 0)) atomicAdd(&chold[j + 0], 1u);
-                                if (vv.y == Ls[j + 1] && in_mask(jm, j + 1)) atomicAdd(&chold[j + 1], 1u);
-                                if (vv.z == Ls[j + 2] && in_mask(jm, j + 2)) atomicAdd(&chold[j + 2], 1u);
-                                if (vv.w == Ls[j + 3] && in_mask(jm, j + 3)) atomicAdd(&chold[j + 3], 1u);
-                            }
-                            pfl[rpos] |= kFlHold;
-                        }
-                    }
-                }
+                hzs |= hz << (q * P);
                 const uint32_t src = (uint32_t)(sl * RW + g);
                 const uint32_t pos = base + q * kThreads + w * 32 + src;
                 key_out(pos < n_live, pos, __float_as_uint(ps[0]));
             }
+            // rare: rows holding a landmark value in this lane's attributes
+#pragma unroll 1
+            while (hzs) {
+                const int b = __ffs(hzs) - 1;
+                hzs &= hzs - 1u;
+                const uint32_t rpos = base + (uint32_t)(b / P) * kThreads + w * 32 + (uint32_t)(b % P) * RW + g;
+                if (rpos >= n_live) continue;
+                const float4 *r4 = reinterpret_cast<const float4 *>(x + (size_t)LID(rpos) * D) + sl;
+#pragma unroll 1
+                for (int f = 0; f < F; f++) {
+                    const float4 vv = __ldg(r4 + P * f);
+                    const int j = 4 * (sl + P * f);
+                    if (vv.x == Ls[j + 0] && in_mask(jm, j + 0)) atomicAdd(&chold[j + 0], 1u);
+                    if (vv.y == Ls[j + 1] && in_mask(jm, j + 1)) atomicAdd(&chold[j + 1], 1u);
+                    if (vv.z == Ls[j + 2] && in_mask(jm, j + 2)) atomicAdd(&chold[j + 2], 1u);
+                    if (vv.w == Ls[j + 3] && in_mask(jm, j + 3)) atomicAdd(&chold[j + 3], 1u);
+                }
+                pfl[rpos] |= kFlHold;
+            }
         }
     } else {
         constexpr int B = kPeelBatch<D>();
+#pragma unroll 1
         for (uint32_t base = 0; base < n_live; base += B * kThreads) {
             bool lv[B];
             uint32_t ids[B];
@@ -829,11 +842,17 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
             bool hz[B];
 #pragma unroll
             for (int q = 0; q < B; q++) dl[q] = dist32<D>(x + (size_t)ids[q] * d, Ls, d, hz[q]);
+            uint32_t hzs = 0;
 #pragma unroll
             for (int q = 0; q < B; q++) {
-                if (lv[q] && hz[q])
-                    note_holder(x + (size_t)ids[q] * d, Ls, d, &pfl[base + q * kThreads + t], chold, jm);
+                hzs |= (uint32_t)(lv[q] && hz[q]) << q;
                 key_out(lv[q], base + q * kThreads + t, __float_as_uint(dl[q]));
+            }
+#pragma unroll 1
+            while (hzs) {
+                const uint32_t pos = base + (uint32_t)(__ffs(hzs) - 1) * kThreads + t;
+                hzs &= hzs - 1u;
+                note_holder(x + (size_t)LID(pos) * d, Ls, d, &pfl[pos], chold, jm);
             }
         }
     }
@@ -859,6 +878,7 @@ __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float 
     // launch may have written the copy
     const float *src = xt ? xt : x;
     const size_t ps = xt ? 1 : (size_t)(D > 0 ? D : d), as = xt ? (size_t)n : 1;
+#pragma unroll 1
     for (uint32_t q0 = 0; q0 < n_live; q0 += U * kThreads) {          // block-uniform bound
         uint32_t id[U], key[U], hold = 0;
         float acc[U];
@@ -911,11 +931,13 @@ __device__ __forceinline__ void for_held(const float *__restrict__ x, const floa
 {
     const int lane = threadIdx.x & 31;
     uint32_t m = __ballot_sync(0xffffffffu, hold);
+#pragma unroll 1
     while (m) {
         const int q = __ffs(m) - 1;
         m &= m - 1u;
         const float *row = x + (size_t)__shfl_sync(0xffffffffu, id, q) * d;
         const uint32_t vq = __shfl_sync(0xffffffffu, val, q);
+#pragma unroll 1
         for (int j0 = 0; j0 < d; j0 += 128) {
             float v[4];
 #pragma unroll
@@ -932,12 +954,18 @@ __device__ __forceinline__ void for_held(const float *__restrict__ x, const floa
     }
 }
 
-// Settles group g of the epoch's boundaries (one CTA): every band entry of the group gets
-// its round, exactly by (delta64, index).  Entries are ranked by their compensated
-// distance; at each boundary only the entries within that distance's error of the cut are
-// ranked again by float64.  r0: the epoch's first round; K: its boundaries.
-__device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, uint32_t g, uint32_t r0, uint32_t K,
-                                          uint32_t *scr)
+// The holders counted per attribute and round (out of line: rare, and three callers)
+__device__ __noinline__ void count_held(const float *__restrict__ x, const float *Ls, int d, bool hold, uint32_t id,
+                                        uint32_t round, uint32_t (*hcnt)[kMaxEpoch])
+{
+    for_held(x, Ls, d, hold, id, round, [&](int j, uint32_t r) { atomicAdd(&hcnt[j][r], 1u); });
+}
+
+// A group of more entries than fit in shared memory: each of its boundaries' cut by selection,
+// then the entries within the cut's error ranked by float64 and index (see settle_group).
+__device__ __noinline__ void settle_large(const PeelArgs &a, const float *Ls, uint32_t q1, uint32_t q2, uint32_t off,
+                                          uint32_t ne, uint32_t before, uint32_t r0, uint32_t K,
+                                          uint32_t (*hcnt)[kMaxEpoch], uint32_t *scr)
 {
     PeelCtl *ctl = a.ctl;
     const int d = a.d;
@@ -948,142 +976,15 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
     __shared__ uint32_t s_need[kMaxEpoch], s_need3[kMaxEpoch], s_na3[kMaxEpoch], s_p3[kMaxEpoch];
     __shared__ unsigned long long s_k3[kMaxEpoch];
     __shared__ uint32_t s_bc[kMaxEpoch];
-    const uint32_t q1 = __ldcg(&ctl->g_q1[g]), q2 = __ldcg(&ctl->g_q2[g]);
-    const uint32_t ne = __ldcg(&ctl->gcnt[g]);
-    // points certainly before the group: certain points of rounds up to q1 and the
-    // entries of the groups before it, whose regions precede the group's (q1, g < 32:
-    // lane i of warp 0 loads round i's and group i's counts)
-    __shared__ uint32_t s_before, s_off;
-    if (t < 32) {
-        uint32_t cb = (uint32_t)t <= q1 ? __ldcg(&ctl->cert[t]) : 0u;
-        uint32_t go = (uint32_t)t < g ? __ldcg(&ctl->gcnt[t]) : 0u;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            cb += __shfl_xor_sync(0xffffffffu, cb, o);
-            go += __shfl_xor_sync(0xffffffffu, go, o);
-        }
-        if (t == 0) {
-            s_before = cb + go;
-            s_off = go;
-        }
-    }
-    __syncthreads();
-    const uint32_t before = s_before, off = s_off;
-    const bool staged = ne <= (uint32_t)kStage;
-    uint64_t *stk = reinterpret_cast<uint64_t *>(scr + kStageOff);
-    uint32_t *stp = scr + kStageOff + 2 * kStage;
     const uint64_t *gk = a.gkey + off;
     const uint32_t *gp = a.gpos + off;
     uint64_t *ak = a.akey + off;
     uint32_t *ap = a.apos + off;
     if (t < kMaxEpoch) s_bc[t] = 0;
-    if (t == 0 && __ldcg(&ctl->gfill[g]) != ne) atomicOr(&a.flags[1], 1u);
-    if (staged)
-        for (uint32_t e = t; e < ne; e += kThreads) {
-            stk[e] = __ldcg(&gk[e]);
-            stp[e] = __ldcg(&gp[e]);
-        }
     __syncthreads();
     auto KA = [&](uint32_t i) -> uint64_t { return __ldcg(&gk[i]); };
     // an entry's id (bit 31 of the stored word is its hold flag)
     auto PA = [&](uint32_t i) -> uint32_t { return __ldcg(&gp[i]) & kPosMask; };
-    auto AK = [&](uint32_t i) -> uint64_t { return __ldcg(&ak[i]); };
-    auto AP = [&](uint32_t i) -> uint32_t { return __ldcg(&ap[i]); };
-    if (staged) {
-        // every entry's rank among the group's, counted by its thread: the entries whose
-        // compensated distance is smaller beyond the error window, and where the window holds
-        // others and a boundary cuts through it, those of them that are smaller by float64
-        // and index.  No selection and no barrier per boundary (2^20 x 16: settle and commit
-        // 14 -> 8 us an epoch).  The window of a distance with bits k: k +- W, W >= 4 (eps_ff
-        // + 2^-52) 2^53 (a relative step r moves a double's bits by at most r 2^53); below
-        // 2^-60 the absolute error of tiny squares counts too, so all of them are one window.
-        constexpr int E = kStage / kThreads;
-        __shared__ int s_any;
-        uint64_t *d64 = reinterpret_cast<uint64_t *>(scr);                      // kStage keys
-        uint8_t *f64 = reinterpret_cast<uint8_t *>(scr + 2 * kStage);           // kStage flags
-        static_assert(2 * kStage + kStage / 4 <= kStageOff, "the rank scratch lies before the staged entries");
-        if (t <= (int)(q2 - q1)) {
-            const int64_t need_s = (int64_t)(q1 + t + 1) * N - (int64_t)before;
-            s_need[t] = need_s < 0 ? 0u : (need_s > (int64_t)ne ? ne : (uint32_t)need_s);
-            if (need_s < 0 || need_s > (int64_t)ne) atomicOr(&a.flags[1], 1u);
-        }
-        if (t == 0) s_any = 0;
-        for (uint32_t e = t; e < ne; e += kThreads) f64[e] = 0;
-        __syncthreads();
-        const uint64_t W0 = 256ull * ((uint64_t)d * d + 8ull * d + 1ull) + 8ull, W = W0 + (W0 >> 4);
-        constexpr uint64_t kTiny = 963ull << 52;                                // 2^-60
-        const uint32_t nq = q2 - q1 + 1u;
-        uint64_t lo[E], hi[E];
-        uint32_t below[E], inside[E], rank[E];
-        bool cut[E];
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            const uint32_t e = t + i * kThreads;
-            const uint64_t k = e < ne ? stk[e] : 0ull;
-            lo[i] = k < kTiny + W ? 0ull : k - W;
-            hi[i] = (k < kTiny ? kTiny : k) + W;
-            below[i] = inside[i] = 0;
-        }
-        for (uint32_t f = 0; f < ne; f++) {
-            const uint64_t k = stk[f];
-#pragma unroll
-            for (int i = 0; i < E; i++) {
-                below[i] += k < lo[i];
-                inside[i] += k >= lo[i] && k <= hi[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            const uint32_t e = t + i * kThreads;
-            rank[i] = below[i];
-            cut[i] = false;
-            if (e < ne)
-                for (uint32_t b = 0; b < nq; b++) cut[i] |= s_need[b] > below[i] && s_need[b] < below[i] + inside[i];
-            if (cut[i]) {
-                s_any = 1;
-                for (uint32_t f = 0; f < ne; f++)
-                    if (stk[f] >= lo[i] && stk[f] <= hi[i]) f64[f] = 1;
-            }
-        }
-        __syncthreads();
-        if (s_any) {
-            for (uint32_t e = t; e < ne; e += kThreads)
-                if (f64[e])
-                    d64[e] = (uint64_t)__double_as_longlong(dist64(a.x + (size_t)(stp[e] & kPosMask) * d, Ls, d));
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < E; i++) {
-                const uint32_t e = t + i * kThreads;
-                if (!cut[i]) continue;
-                const uint64_t ke = d64[e];
-                const uint32_t pe = stp[e] & kPosMask;
-                for (uint32_t f = 0; f < ne; f++)
-                    if (stk[f] >= lo[i] && stk[f] <= hi[i])
-                        rank[i] += d64[f] < ke || (d64[f] == ke && (stp[f] & kPosMask) < pe);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            const uint32_t e = t + i * kThreads;
-            uint32_t rr = kNone, raw = 0;
-            if (e < ne) {
-                raw = stp[e];
-                rr = q1;
-                for (uint32_t b = 0; b < nq; b++) rr += s_need[b] <= rank[i];
-                if (rr < K) {
-                    a.rnd[raw & kPosMask] = r0 + rr;
-                    atomicAdd(&s_bc[rr], 1u);
-                }
-            }
-            const bool ch = e < ne && rr < K && (raw & ~kPosMask);
-            if (__any_sync(0xffffffffu, ch))
-                for_held(a.x, Ls, d, ch, raw & kPosMask, rr,
-                         [&](int j, uint32_t r) { atomicAdd(&ctl->hcnt[j][r], 1u); });
-        }
-        __syncthreads();
-        if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
-        return;
-    }
     const double win_rel = 4.0 * ((double)eps_ff(d) + 0x1p-52);
     for (uint32_t i = q1; i <= q2; i++) {
         const uint32_t bi = i - q1;
@@ -1097,7 +998,7 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
         }
         uint64_t V;
         uint32_t Pv;
-        select_kth(KA, PA, ne, need, scr, V, Pv);
+        select_kth(gk, gp, ne, need, scr, V, Pv);
         const double v = __longlong_as_double((long long)V);
         const double win = win_rel * v + 0x1p-110;
         const double lo = v - win, hi = v + win;
@@ -1126,7 +1027,7 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
                 ak[e] = (uint64_t)__double_as_longlong(dist64(a.x + (size_t)pos * d, Ls, d));
             }
             __syncthreads();
-            select_kth(AK, AP, na, need3, scr, K3, P3);
+            select_kth(ak, ap, na, need3, scr, K3, P3);
         }
         if (t == 0) {
             s_need[bi] = need;
@@ -1173,14 +1074,153 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
             atomicAdd(&s_bc[rr], 1u);
         }
         const bool ch = v && rr < K && (raw & ~kPosMask);
-        if (__any_sync(0xffffffffu, ch))
-            for_held(a.x, Ls, d, ch, pos, rr, [&](int j, uint32_t r) { atomicAdd(&ctl->hcnt[j][r], 1u); });
+        if (__any_sync(0xffffffffu, ch)) count_held(a.x, Ls, d, ch, pos, rr, hcnt);
     }
     __syncthreads();
     if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
 }
 
-// The next landmark: in each attribute that lost its last holder (lost[0 .. nl)), the smallest
+// Settles group g of the epoch's boundaries (one CTA): every band entry of the group gets
+// its round, exactly by (delta64, index).  Entries are ranked by their compensated
+// distance; at each boundary only the entries within that distance's error of the cut are
+// ranked again by float64.  r0: the epoch's first round; K: its boundaries.
+// q1 .. q2: the group's boundaries; off, ne: its region of the regrouped entries; certs: the
+// points certainly in rounds 0 .. q1.
+__device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, uint32_t g, uint32_t q1, uint32_t q2,
+                                          uint32_t off, uint32_t ne, uint32_t certs, uint32_t r0, uint32_t K,
+                                          uint32_t (*hcnt)[kMaxEpoch], uint32_t *scr)
+{
+    PeelCtl *ctl = a.ctl;
+    const int d = a.d;
+    const uint32_t N = (uint32_t)a.N;
+    const int t = threadIdx.x;
+    __shared__ uint32_t s_need[kMaxEpoch], s_bc[kMaxEpoch];
+    // points before the group: the certain ones and the entries of the groups before it
+    const uint32_t before = certs + off, filled = __ldcg(&ctl->gfill[g]);
+    uint64_t *stk = reinterpret_cast<uint64_t *>(scr + kStageOff);
+    uint32_t *stp = scr + kStageOff + 2 * kStage;
+    const uint64_t *gk = a.gkey + off;
+    const uint32_t *gp = a.gpos + off;
+    if (t < kMaxEpoch) s_bc[t] = 0;
+    if (t == 0 && filled != ne) atomicOr(&a.flags[1], 1u);
+    if (ne > (uint32_t)kStage) {
+        settle_large(a, Ls, q1, q2, off, ne, before, r0, K, hcnt, scr);
+        return;
+    }
+    for (uint32_t e = t; e < ne; e += kThreads) {
+        stk[e] = __ldcg(&gk[e]);
+        stp[e] = __ldcg(&gp[e]);
+    }
+    __syncthreads();
+    // every entry's rank among the group's, counted by eight lanes: the entries whose
+    // compensated distance is smaller beyond the error window, and where the window holds
+    // others and a boundary cuts through it, those of them that are smaller by float64
+    // and index.  No selection and no barrier per boundary (2^20 x 16: settle and commit
+    // 14 -> 8 us an epoch).  The window of a distance with bits k: k +- W, W >= 4 (eps_ff
+    // + 2^-52) 2^53 (a relative step r moves a double's bits by at most r 2^53); below
+    // 2^-60 the absolute error of tiny squares counts too, so all of them are one window.
+    // Short rolled loops throughout: the CTA that settles a group is the only one that
+    // fetches this code, and the others wait for it.
+    __shared__ int s_any;
+    uint64_t *d64 = reinterpret_cast<uint64_t *>(scr);                      // kStage keys
+    uint32_t *rk = scr + 2 * kStage;                                        // kStage ranks, bit 31: cut
+    uint8_t *f64 = reinterpret_cast<uint8_t *>(scr + 3 * kStage);           // kStage flags
+    static_assert(3 * kStage + kStage / 4 <= kStageOff, "the rank scratch lies before the staged entries");
+    constexpr uint32_t EB = kThreads / 8;
+    constexpr uint32_t kCut = 0x80000000u;
+    const uint32_t sub = (uint32_t)t & 7u;
+    if (t <= (int)(q2 - q1)) {
+        const int64_t need_s = (int64_t)(q1 + t + 1) * N - (int64_t)before;
+        s_need[t] = need_s < 0 ? 0u : (need_s > (int64_t)ne ? ne : (uint32_t)need_s);
+        if (need_s < 0 || need_s > (int64_t)ne) atomicOr(&a.flags[1], 1u);
+    }
+    if (t == 0) s_any = 0;
+    for (uint32_t e = t; e < ne; e += kThreads) f64[e] = 0;
+    __syncthreads();
+    const uint64_t W0 = 256ull * ((uint64_t)d * d + 8ull * d + 1ull) + 8ull, W = W0 + (W0 >> 4);
+    constexpr uint64_t kTiny = 963ull << 52;                                // 2^-60
+    const uint32_t nq = q2 - q1 + 1u;
+    // the window of the staged distance k
+    auto win_lo = [&](uint64_t k) { return k < kTiny + W ? 0ull : k - W; };
+    auto win_hi = [&](uint64_t k) { return (k < kTiny ? kTiny : k) + W; };
+#pragma unroll 1
+    for (uint32_t e0 = 0; e0 < ne; e0 += EB) {                              // block-uniform bound
+        const uint32_t e = e0 + (uint32_t)t / 8u;
+        const uint64_t k = e < ne ? stk[e] : 0ull, lo = win_lo(k), hi = win_hi(k);
+        uint32_t below = 0, upto = 0;
+#pragma unroll 4
+        for (uint32_t f = sub; f < ne; f += 8) {
+            const uint64_t kf = stk[f];
+            below += kf < lo;
+            upto += kf <= hi;
+        }
+#pragma unroll
+        for (int o = 4; o; o >>= 1) {
+            below += __shfl_xor_sync(0xffffffffu, below, o);
+            upto += __shfl_xor_sync(0xffffffffu, upto, o);
+        }
+        if (e < ne) {
+            bool cut = false;
+#pragma unroll 1
+            for (uint32_t b = 0; b < nq; b++) cut |= s_need[b] > below && s_need[b] < upto;
+            if (sub == 0) rk[e] = below | (cut ? kCut : 0u);
+            if (cut) {
+                s_any = 1;
+#pragma unroll 1
+                for (uint32_t f = sub; f < ne; f += 8)
+                    if (stk[f] >= lo && stk[f] <= hi) f64[f] = 1;
+            }
+        }
+    }
+    __syncthreads();
+    if (s_any) {
+#pragma unroll 1
+        for (uint32_t e = t; e < ne; e += kThreads)
+            if (f64[e])
+                d64[e] = (uint64_t)__double_as_longlong(dist64(a.x + (size_t)(stp[e] & kPosMask) * d, Ls, d));
+        __syncthreads();
+#pragma unroll 1
+        for (uint32_t e0 = 0; e0 < ne; e0 += EB) {
+            const uint32_t e = e0 + (uint32_t)t / 8u;
+            const bool cut = e < ne && (rk[e] & kCut);
+            uint32_t more = 0;
+            if (cut) {
+                const uint64_t k = stk[e], lo = win_lo(k), hi = win_hi(k), ke = d64[e];
+                const uint32_t pe = stp[e] & kPosMask;
+#pragma unroll 1
+                for (uint32_t f = sub; f < ne; f += 8)
+                    if (stk[f] >= lo && stk[f] <= hi)
+                        more += d64[f] < ke || (d64[f] == ke && (stp[f] & kPosMask) < pe);
+            }
+#pragma unroll
+            for (int o = 4; o; o >>= 1) more += __shfl_xor_sync(0xffffffffu, more, o);
+            if (cut && sub == 0) rk[e] += more;
+        }
+        __syncthreads();
+    }
+#pragma unroll 1
+    for (uint32_t e0 = 0; e0 < ne; e0 += kThreads) {                        // block-uniform bound
+        const uint32_t e = e0 + (uint32_t)t;
+        uint32_t rr = kNone, raw = 0;
+        if (e < ne) {
+            raw = stp[e];
+            rr = q1;
+            const uint32_t rank = rk[e] & ~kCut;
+#pragma unroll 1
+            for (uint32_t b = 0; b < nq; b++) rr += s_need[b] <= rank;
+            if (rr < K) {
+                a.rnd[raw & kPosMask] = r0 + rr;
+                atomicAdd(&s_bc[rr], 1u);
+            }
+        }
+        const bool ch = e < ne && rr < K && (raw & ~kPosMask);
+        if (__any_sync(0xffffffffu, ch)) count_held(a.x, Ls, d, ch, raw & kPosMask, rr, hcnt);
+    }
+    __syncthreads();
+    if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
+}
+
+// The next landmark: in each attribute that lost its last holder (lost[0 .. nl), shared), the smallest
 // value among the points left, here those of one CTA's list, kMinAttrs attributes and
 // kMinBatch points per thread at a time (their loads issued together), added to the grid's
 // minimum (values lie in [0, 1], so their bits order like them).
@@ -1189,24 +1229,26 @@ constexpr int kMinBatch = 4;
 
 __device__ __noinline__ void lost_minima(const float *__restrict__ x, const float *__restrict__ xt, uint32_t n, int d,
                                          uint32_t n_live, bool kc, const uint32_t *sid, const uint32_t *glist,
-                                         const uint32_t *lost, uint32_t nl, uint32_t *Lbits)
+                                         const uint16_t *lost, uint32_t nl, uint32_t *Lbits)
 {
     __shared__ uint32_t s_min[kMinAttrs];
     const int t = threadIdx.x, lane = t & 31;
     const float *src = xt ? xt : x;
     const size_t ps = xt ? 1 : (size_t)d, as = xt ? (size_t)n : 1;
+#pragma unroll 1
     for (uint32_t l0 = 0; l0 < nl; l0 += kMinAttrs) {
         const float *col[kMinAttrs];
         uint32_t mn[kMinAttrs];
 #pragma unroll
         for (int i = 0; i < kMinAttrs; i++) {       // past the last one, the first of the group again
-            const uint32_t j = __ldcg(&lost[l0 + i < nl ? l0 + i : l0]);
+            const uint32_t j = lost[l0 + i < nl ? l0 + i : l0];
             col[i] = src + (size_t)j * as;
             mn[i] = kInfBits;
         }
         if (t < kMinAttrs) s_min[t] = kInfBits;
         __syncthreads();
         const uint32_t na = min((uint32_t)kMinAttrs, nl - l0);
+#pragma unroll 1
         for (uint32_t q0 = 0; q0 < n_live; q0 += kMinBatch * kThreads) {
             uint32_t id[kMinBatch];
 #pragma unroll
@@ -1228,56 +1270,59 @@ __device__ __noinline__ void lost_minima(const float *__restrict__ x, const floa
             if (lane == 0 && i < (int)na) atomicMin(&s_min[i], m);
         }
         __syncthreads();
-        if (t < (int)na && s_min[t] != kInfBits) atomicMin(&Lbits[__ldcg(&lost[l0 + t])], s_min[t]);
+        if (t < (int)na && s_min[t] != kInfBits) atomicMin(&Lbits[lost[l0 + t]], s_min[t]);
     }
 }
 
-// The last CTA of phase B turns each boundary's first-digit bin and rank inside it into
-// its band cut-offs (second digit from the boundary's histogram), and merges boundaries
-// whose bands overlap into groups.  Warp w resolves boundaries w, w + kW, ...: lane i sums
-// second-digit bins [64 i, 64 i + 64) in two halves, a warp scan finds the lane holding
-// the rank, and that lane walks the half holding it (its loads issued together).
+// The epoch's groups of boundaries: group g's band holds the keys in [in, out], its last
+// boundary is q2 (its first the one after group g - 1's).
+struct GroupTab {
+    uint32_t in[kMaxEpoch], out[kMaxEpoch], q2[kMaxEpoch], ng;
+    float kref;                  // lower end of the first boundary's key range
+};
+
+// After phase B: each boundary's first-digit bin and rank inside it become its band cut-offs
+// (second digit from the boundary's histogram), and boundaries whose bands overlap merge into
+// groups (tab, in shared memory).  Every CTA does this for itself when the boundaries are
+// few; otherwise the last CTA to arrive does it for all.  Warp w resolves boundaries w, w + kW, ...: lane i holds
+// second-digit bins [64 i, 64 i + 64), a warp scan finds the lane holding the rank, and that
+// lane counts its bins before it.
 __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t K, float keps, float kabs, const DigitMap *dm,
                                              const uint32_t *sb, const uint32_t *sr, const uint32_t *sslot,
-                                             uint32_t nslot)
+                                             GroupTab &tab)
 {
     __shared__ uint32_t s_b1[kMaxEpoch];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const DigitMap mp = *dm;
     if (t < kMaxEpoch) s_b1[t] = 0;
     __syncthreads();
+#pragma unroll 1
     for (uint32_t q = (uint32_t)w; q < K; q += kW) {
         const uint4 *h4 = reinterpret_cast<const uint4 *>(ctl->h1[sslot[q]] + lane * 64);
-        uint32_t lo = 0, hi = 0;
+        uint4 h[16];
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            const uint4 u = __ldcg(h4 + i), v = __ldcg(h4 + 8 + i);
-            lo += u.x + u.y + u.z + u.w;
-            hi += v.x + v.y + v.z + v.w;
-        }
-        const uint32_t ls = lo + hi;
+        for (int i = 0; i < 16; i++) h[i] = __ldcg(h4 + i);
+        uint32_t ls = 0, hs[16];
+#pragma unroll
+        for (int i = 0; i < 16; i++) hs[i] = ls += h[i].x + h[i].y + h[i].z + h[i].w;
         const uint32_t ex = warp_incl_scan(ls) - ls;
         const uint32_t r = sr[q];
         if (r >= ex && r < ex + ls) {
-            const int half = r >= ex + lo ? 1 : 0;
-            uint4 u[8];
+            // the four bins that hold the rank, then the one of them
+            uint32_t cc = ex, found = 0;
+            uint4 at = h[0];
 #pragma unroll
-            for (int i = 0; i < 8; i++) u[i] = __ldcg(h4 + 8 * half + i);
-            uint32_t cc = ex + (half ? lo : 0u), found = 0;
-            bool done = false;
-#pragma unroll
-            for (int i = 0; i < 8; i++) {
-                const uint32_t v4[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    if (!done && r < cc + v4[k]) {
-                        found = (uint32_t)(lane * 64 + 32 * half + 4 * i + k);
-                        done = true;
-                    }
-                    cc += v4[k];
+            for (int i = 0; i < 16; i++) {
+                const uint32_t end = ex + hs[i];      // past the i-th four
+                if (end <= r) {
+                    found = 4u * (uint32_t)i + 4u;
+                    cc = end;
+                } else if (found == 4u * (uint32_t)i) {
+                    at = h[i];
                 }
             }
-            s_b1[q] = found;
+            found += (cc + at.x <= r) + (cc + at.x + at.y <= r) + (cc + at.x + at.y + at.z <= r);
+            s_b1[q] = found + (uint32_t)lane * 64u;
         }
     }
     __syncthreads();
@@ -1294,93 +1339,84 @@ __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t K, float kep
         const uint32_t open = __ballot_sync(0xffffffffu, lane < (int)K && (lane == 0 || ik > pk));
         if (lane < (int)K) {
             const uint32_t g = (uint32_t)__popc(open & ((2u << lane) - 1u)) - 1u;
-            if ((open >> lane) & 1u) {
-                ctl->g_in[g] = ik;
-                ctl->g_q1[g] = (uint32_t)lane;
-            }
+            if ((open >> lane) & 1u) tab.in[g] = ik;
             if (lane == (int)K - 1 || ((open >> (lane + 1)) & 1u)) {
-                ctl->g_out[g] = ok;
-                ctl->g_q2[g] = (uint32_t)lane;
+                tab.out[g] = ok;
+                tab.q2[g] = (uint32_t)lane;
             }
         }
         if (lane == 0) {
-            ctl->n_groups = (uint32_t)__popc(open);
-            ctl->n_slots = nslot;
-            ctl->kref = __uint_as_float(A);
+            tab.ng = (uint32_t)__popc(open);
+            tab.kref = __uint_as_float(A);
         }
     }
+    __syncthreads();
 }
 
-// The last CTA of phase D finds how many rounds the epoch commits: up to the first round
-// after which some attribute has no holder of its landmark value left (the landmark then
-// changes).  It updates the live holder counts, checks that every round of the epoch got
-// exactly N points, records the epoch's landmarks and publishes k_commit and l_changed.
-__device__ __noinline__ void commit_count(const PeelArgs &a, const float *Ls, uint32_t K, uint32_t r0, bool need_keys)
+// After phase D, in every CTA: how many rounds the epoch commits, up to the first round after
+// which some attribute has no holder of its landmark value left (the landmark then changes);
+// which attributes those are (s_lost); and the smallest key that a point left can have.  Each
+// CTA forms them from the grid's counts (an L2 round trip; one CTA doing it for all would
+// add another for its answer).  chold, the holders per attribute, is read here and its
+// successor chold2 written by CTA 0; CTA 0 also checks that every round got exactly N points.
+__device__ __noinline__ void commit_count(const PeelArgs &a, uint32_t K, const GroupTab &tab, const uint32_t *chold,
+                                          uint32_t *chold2, const uint32_t (*hcnt)[kMaxEpoch], uint32_t &s_kcm,
+                                          uint32_t &s_nl, uint32_t &s_klast, uint16_t *s_lost)
 {
     PeelCtl *ctl = a.ctl;
     const int d = a.d;
-    const uint32_t N = (uint32_t)a.N;
     const int t = threadIdx.x;
-    // per attribute: the first round after which no holder of L_j is left
-    // (the counts are read all at once, then scanned in registers)
-    __shared__ uint32_t s_nl;
+    const bool own = blockIdx.x == 0;
     if (t == 0) s_nl = 0;
-    uint32_t qs = kNone;
-    for (int j = t; j < d; j += kThreads) {
-        uint32_t hc[kMaxEpoch];
-#pragma unroll
-        for (int r = 0; r < kMaxEpoch; r++) hc[r] = r < (int)K ? __ldcg(&ctl->hcnt[j][r]) : 0u;
-        const uint32_t ch = __ldcg(&ctl->chold[j]);
+    if (own && t < (int)K && __ldcg(&ctl->cert[t]) + __ldcg(&ctl->bnd[t]) != (uint32_t)a.N) atomicOr(&a.flags[1], 1u);
+    // per attribute: the first round after which no holder of L_j is left
+    // (the counts are read all at once, then scanned in registers; those of a thread's first
+    // attribute stay there for the second use)
+    constexpr int RB = 8;
+    uint32_t qs = kNone, hc[RB], ch = 0;
+    for (int j0 = (d - 1) / kThreads * kThreads; j0 >= 0; j0 -= kThreads) {
+        const int j = j0 + t;
+        ch = j < d ? __ldcg(&chold[j]) : 0u;
         uint32_t acc = 0, qj = kNone;
+#pragma unroll 1
+        for (uint32_t q0 = 0; q0 < K; q0 += RB) {
 #pragma unroll
-        for (int r = 0; r < kMaxEpoch; r++) {
-            acc += hc[r];
-            if (qj == kNone && r < (int)K && acc >= ch) qj = (uint32_t)r;
+            for (int r = 0; r < RB; r++) hc[r] = q0 + r < K && j < d ? __ldcg(&hcnt[j][q0 + r]) : 0u;
+#pragma unroll
+            for (int r = 0; r < RB; r++) {
+                acc += hc[r];
+                if (qj == kNone && q0 + r < K && j < d && acc >= ch) qj = q0 + (uint32_t)r;
+            }
         }
         qs = min(qs, qj);
     }
-    // the last committed boundary's group, below (lane g: group g)
-    const uint32_t ng = __ldcg(&ctl->n_groups);
-    const uint32_t gq2 = t < (int)ng ? __ldcg(&ctl->g_q2[t & 31]) : kNone;
-    const uint32_t gin = t < (int)ng ? __ldcg(&ctl->g_in[t & 31]) : kNone;
     qs = block_min(qs);
     const uint32_t kc_ = qs < K ? qs + 1u : K;
-    const bool changed = qs < K;
     // the holders that leave with the committed rounds; an attribute that has none left gets
     // a new landmark value (the minimum over the points left, taken next) and its holders are
     // counted by the next pass
     for (int j = t; j < d; j += kThreads) {
         uint32_t gone = 0;
+#pragma unroll 1
+        for (uint32_t q0 = 0; q0 < kc_; q0 += RB) {
+            if (j >= kThreads || K > (uint32_t)RB) {
 #pragma unroll
-        for (int r = 0; r < kMaxEpoch; r++) gone += r < (int)kc_ ? __ldcg(&ctl->hcnt[j][r]) : 0u;
-        const uint32_t left = __ldcg(&ctl->chold[j]) - gone;
-        ctl->chold[j] = left;
-        if (left == 0u) {
-            ctl->lost[atomicAdd(&s_nl, 1u)] = (uint32_t)j;
-            ctl->Lbits[j] = kInfBits;
+                for (int r = 0; r < RB; r++) hc[r] = q0 + r < kc_ ? __ldcg(&hcnt[j][q0 + r]) : 0u;
+            }
+#pragma unroll
+            for (int r = 0; r < RB; r++) gone += q0 + r < kc_ ? hc[r] : 0u;
         }
+        const uint32_t left = (j >= kThreads ? __ldcg(&chold[j]) : ch) - gone;
+        if (own) chold2[j] = left;
+        if (left == 0u) s_lost[atomicAdd(&s_nl, 1u)] = (uint16_t)j;
     }
     // every point left lies at or past the start of the last committed boundary's band
     if (t < 32) {
-        const uint32_t past = __ballot_sync(0xffffffffu, t < (int)ng && gq2 >= kc_ - 1u);
-        if (past && t == __ffs(past) - 1) ctl->klast = gin;
+        const uint32_t past = __ballot_sync(0xffffffffu, t < (int)tab.ng && tab.q2[t] >= kc_ - 1u);
+        if (past && t == __ffs(past) - 1) s_klast = tab.in[t];
     }
+    if (t == 0) s_kcm = kc_;
     __syncthreads();
-    if (t < (int)K && __ldcg(&ctl->cert[t]) + __ldcg(&ctl->bnd[t]) != N) atomicOr(&a.flags[1], 1u);
-    if (changed) {
-        for (int b = t; b < kHistBins; b += kThreads) ctl->h0[b] = 0;
-        for (int j = t; j < d; j += kThreads) ctl->hmax[j] = 0;    // recomputed by the next pass
-    }
-    if (a.landmarks)
-        for (uint32_t e = t; e < kc_ * (uint32_t)d; e += kThreads)
-            a.landmarks[(size_t)(r0 + e / d) * d + e % d] = Ls[e % d];
-    if (t == 0) {
-        ctl->k_commit = kc_;
-        ctl->l_changed = changed ? 1u : 0u;
-        ctl->n_lost = s_nl;
-        ctl->epochs += 1;
-        ctl->passes += need_keys ? 1u : 0u;
-    }
 }
 
 // ------------------------------------------------------------------ the points by attribute
@@ -1424,15 +1460,14 @@ __global__ void __launch_bounds__(kThreads) k_transpose(const float *__restrict_
 // A CTA's list of points left, by list position: ids, float32 keys and state bytes; in
 // shared memory when the slice fits the key cache (kc), else in one of two global lists.
 struct ListView {
-    bool first, kc;
-    uint32_t s0;
+    bool kc;
     const uint32_t *sid, *skey;
     uint8_t *sfl;
     const uint32_t *gid, *gkp;
     uint8_t *gfl;
     uint32_t *gid2, *gkp2;       // the other global list (compaction target)
     uint8_t *gfl2;
-    __device__ __forceinline__ uint32_t id(uint32_t q) const { return first ? s0 + q : kc ? sid[q] : __ldcg(&gid[q]); }
+    __device__ __forceinline__ uint32_t id(uint32_t q) const { return kc ? sid[q] : __ldcg(&gid[q]); }
     __device__ __forceinline__ uint32_t key(uint32_t q) const { return kc ? skey[q] : __ldcg(&gkp[q]); }
     __device__ __forceinline__ uint8_t *fl() const { return kc ? sfl : gfl; }
 };
@@ -1443,7 +1478,7 @@ struct ListView {
 __device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L, uint32_t n_live, const float *Ls,
                                           uint32_t r0, uint32_t K, uint32_t ng, const uint32_t *s_gin,
                                           const uint32_t *s_gout, const uint32_t *s_gq2, uint32_t s_glast,
-                                          uint32_t *s_cc, uint32_t *s_gc)
+                                          uint32_t *s_cc, uint32_t *s_gc, uint32_t (*hcnt)[kMaxEpoch])
 {
     PeelCtl *ctl = a.ctl;
     const int d = a.d;
@@ -1451,41 +1486,50 @@ __device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L,
     const uint32_t lt = (1u << lane) - 1u;
     uint8_t *pfl = L.fl();
     // a key's class: kNone (after the epoch, or past the end of the list), its round r < K
-    // (certainly), or kBandTag | g (in group g's band).  The keys, ids and state bytes of
-    // kCB positions are loaded before any is used; the class goes to the state byte and is
-    // counted in shared memory (the points of the epoch are spread over the list, so few
-    // lanes of a warp meet on one counter).
+    // (certainly), or kBandTag | g (in group g's band).  Only the keys of all points are read,
+    // kCB per thread in flight; the few in the epoch then load their state byte and id, write
+    // the class to the state byte and are counted in shared memory (the points of the epoch are
+    // spread over the list, so few lanes of a warp meet on one counter).  Those are handled
+    // one batch index at a time in a rolled loop: unrolled, the phase was 48 KB of code, and
+    // its fetch bound it (2^24 x 64: 41 us an epoch).
     constexpr uint32_t kBandTag = 0x100u;
+#pragma unroll 1
     for (uint32_t q0 = 0; q0 < n_live; q0 += kCB * kThreads) {
-        uint32_t kk[kCB], cls[kCB], idv[kCB], fl[kCB];
+        uint32_t kk[kCB];
+        uint32_t in = 0;                           // the batch indexes in the epoch
 #pragma unroll
         for (int u = 0; u < kCB; u++) {
             const uint32_t qi = q0 + u * kThreads + t;
-            const bool v = qi < n_live;
-            kk[u] = v ? L.key(qi) : kGone;
-            idv[u] = v ? L.id(qi) : 0u;
-            fl[u] = v ? pfl[qi] : 0u;
+            kk[u] = qi < n_live ? L.key(qi) : kGone;
         }
 #pragma unroll
-        for (int u = 0; u < kCB; u++) {
-            cls[u] = kNone;
-            if (kk[u] <= s_glast) {
+        for (int u = 0; u < kCB; u++) in |= (uint32_t)(kk[u] <= s_glast) << u;
+        uint32_t todo = __reduce_or_sync(0xffffffffu, in);
+#pragma unroll 1
+        while (todo) {
+            const int u = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            uint32_t k = kk[0];
+#pragma unroll
+            for (int v = 1; v < kCB; v++) k = u == v ? kk[v] : k;
+            const uint32_t qi = q0 + u * kThreads + t;
+            uint32_t cls = kNone, id = 0, fl = 0;
+            if ((in >> u) & 1u) {
+                id = L.id(qi);
+                fl = pfl[qi];
                 uint32_t g = 0, cum = 0;
-                while (g < ng && kk[u] > s_gout[g]) {
+#pragma unroll 1
+                while (g < ng && k > s_gout[g]) {
                     cum = s_gq2[g] + 1u;
                     g++;
                 }
-                if (g < ng && kk[u] >= s_gin[g]) cls[u] = kBandTag | g;
-                else if (cum < K) cls[u] = cum;
+                if (g < ng && k >= s_gin[g]) cls = kBandTag | g;
+                else if (cum < K) cls = cum;
+                // a point outside the epoch keeps its state byte (kFlNone since the last commit)
+                if (cls != kNone) pfl[qi] = (uint8_t)((fl & kFlHold) | (cls >= kBandTag ? kFlBand : cls));
             }
-            // a point outside the epoch keeps its state byte (kFlNone since the last commit)
-            if (cls[u] != kNone)
-                pfl[q0 + u * kThreads + t] = (uint8_t)((fl[u] & kFlHold) | (cls[u] >= kBandTag ? kFlBand : cls[u]));
-        }
-#pragma unroll
-        for (int u = 0; u < kCB; u++) {
-            const bool band = cls[u] != kNone && cls[u] >= kBandTag;
-            const bool cert = cls[u] < kBandTag;
+            const bool band = cls != kNone && cls >= kBandTag;
+            const bool cert = cls < kBandTag;
             const uint32_t bm = __ballot_sync(0xffffffffu, band);
             if (bm) {
                 uint32_t base = 0;
@@ -1494,19 +1538,17 @@ __device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L,
                 base = __shfl_sync(0xffffffffu, base, leader);
                 if (band) {
                     const uint32_t slot = base + (uint32_t)__popc(bm & lt);
-                    a.band_k32[slot] = kk[u];
-                    a.band_pos[slot] = idv[u] | ((fl[u] & kFlHold) ? ~kPosMask : 0u);
-                    atomicAdd(&s_gc[cls[u] - kBandTag], 1u);
+                    a.band_k32[slot] = k;
+                    a.band_pos[slot] = id | ((fl & kFlHold) ? ~kPosMask : 0u);
+                    atomicAdd(&s_gc[cls - kBandTag], 1u);
                 }
             }
             if (cert) {
-                a.rnd[idv[u]] = r0 + cls[u];
-                atomicAdd(&s_cc[cls[u]], 1u);
+                a.rnd[id] = r0 + cls;
+                atomicAdd(&s_cc[cls], 1u);
             }
-            const bool ch = cert && (fl[u] & kFlHold);
-            if (__any_sync(0xffffffffu, ch))
-                for_held(a.x, Ls, d, ch, idv[u], cls[u],
-                         [&](int j, uint32_t rr) { atomicAdd(&ctl->hcnt[j][rr], 1u); });
+            const bool ch = cert && (fl & kFlHold);
+            if (__any_sync(0xffffffffu, ch)) count_held(a.x, Ls, d, ch, id, cls, hcnt);
         }
     }
 }
@@ -1534,28 +1576,53 @@ __device__ __noinline__ uint32_t compact_shared(const PeelArgs &a, const ListVie
     // is written, and those land at or below the tile's own positions.  A position's
     // state byte tells its round in the epoch; only band entries read their round
     // (settled by another CTA) from rnd[].
+#pragma unroll 1
     for (uint32_t cb = 0; cb < n_live; cb += kQT * kThreads) {
-        uint32_t ids[kQT], keys[kQT], fls[kQT], rv[kQT], vl = 0, kp = 0;
+        // the positions kept, and of those the ones whose assignment is dropped
+        uint32_t kp = 0, dropped = 0, out = 0, rv[kQT];
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
             const uint32_t qi = cb + q * kThreads + t;
-            const bool v = qi < n_live;
-            ids[q] = v ? L.id(qi) : 0u;
-            keys[q] = v ? L.key(qi) : kGone;
-            fls[q] = v ? pfl[qi] : (uint32_t)kFlNone;
-            vl |= (uint32_t)v << q;
+            rv[q] = 0;                                       // past the end: leaves the list
+            if (qi < n_live) {
+                const uint32_t st = pfl[qi] & 0x7Fu;
+                rv[q] = st == kFlBand ? __ldcg(&a.rnd[kid[qi]]) : st == kFlNone ? kNone : r0 + st;
+                out |= 1u << q;
+            }
         }
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
-            const uint32_t st = fls[q] & 0x7Fu;
-            rv[q] = st == kFlBand ? __ldcg(&a.rnd[ids[q]]) : st == kFlNone ? kNone : r0 + st;
-            kp |= (uint32_t)(((vl >> q) & 1u) && rv[q] >= live_from) << q;
+            const bool keep = ((out >> q) & 1u) && rv[q] >= live_from;
+            kp |= (uint32_t)keep << q;
+            dropped |= (uint32_t)(keep && rv[q] != kNone) << q;
         }
-        uint32_t bk[kQT];
+        out &= ~kp;
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
-            bk[q] = __ballot_sync(0xffffffffu, (kp >> q) & 1u);
-            if (lane == 0) woff[q * kW + w] = __popc(bk[q]);
+            const uint32_t b = __ballot_sync(0xffffffffu, (kp >> q) & 1u);
+            if (lane == 0) woff[q * kW + w] = __popc(b);
+        }
+        // few: in rolled loops (the phase's time was the fetch of 19 KB of unrolled code)
+#pragma unroll 1
+        while (dropped) {                                    // an assignment dropped
+            a.rnd[kid[cb + (__ffs(dropped) - 1) * kThreads + t]] = kNone;
+            dropped &= dropped - 1u;
+        }
+#pragma unroll 1
+        while (out && !changed) {
+            // the next epoch keeps these keys: the committed ones leave the histogram
+            atomicAdd(&scr[dm.bin(kkey[cb + (__ffs(out) - 1) * kThreads + t])], 1u);
+            out &= out - 1u;
+        }
+        uint32_t ids[kQT], keys[kQT], fls[kQT];
+#pragma unroll
+        for (int q = 0; q < kQT; q++) {
+            const uint32_t qi = cb + q * kThreads + t;
+            if ((kp >> q) & 1u) {
+                ids[q] = kid[qi];
+                keys[q] = kkey[qi];
+                fls[q] = pfl[qi];
+            }
         }
         __syncthreads();
         if (w == 0) {
@@ -1577,17 +1644,13 @@ __device__ __noinline__ uint32_t compact_shared(const PeelArgs &a, const ListVie
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
-            const bool valid = (vl >> q) & 1u;
             const bool keep = (kp >> q) & 1u;
+            const uint32_t b = __ballot_sync(0xffffffffu, keep);
             if (keep) {
-                const uint32_t o = done + woff[q * kW + w] + __popc(bk[q] & lt);
+                const uint32_t o = done + woff[q * kW + w] + __popc(b & lt);
                 kid[o] = ids[q];
                 kkey[o] = keys[q];
                 pfl[o] = (uint8_t)((fls[q] & kFlHold) | kFlNone);
-                if (rv[q] != kNone) a.rnd[ids[q]] = kNone;       // an assignment dropped
-            } else if (valid && !changed) {
-                // the next epoch keeps these keys: the committed ones leave the histogram
-                atomicAdd(&scr[dm.bin(keys[q])], 1u);
             }
         }
         done += woff[kQT * kW];
@@ -1619,6 +1682,7 @@ __device__ __noinline__ uint32_t compact_global(const PeelArgs &a, const ListVie
         for (int b = t; b < kHistBins; b += kThreads) scr[b] = 0;
     if (t == 0) s_out = 0;
     __syncthreads();
+#pragma unroll 1
     for (uint32_t cb = (uint32_t)w * 32 * kQT; cb < n_live; cb += kW * 32 * kQT) {
         uint32_t ids[kQT], keys[kQT], fls[kQT];
 #pragma unroll
@@ -1629,32 +1693,47 @@ __device__ __noinline__ uint32_t compact_global(const PeelArgs &a, const ListVie
             keys[q] = v ? __ldcg(&L.gkp[qi]) : kGone;
             fls[q] = v ? L.gfl[qi] : (uint32_t)kFlNone;
         }
-        uint32_t bk[kQT], rvs[kQT], tot = 0;
+        uint32_t rvs[kQT], tot = 0, kp = 0, dropped = 0, out = 0;
+#pragma unroll
+        for (int q = 0; q < kQT; q++) {
+            const uint32_t st = fls[q] & 0x7Fu;
+            rvs[q] = st == kFlBand ? __ldcg(&a.rnd[ids[q]]) : st == kFlNone ? kNone : r0 + st;
+        }
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
             const bool valid = cb + q * 32 + lane < n_live;
-            const uint32_t st = fls[q] & 0x7Fu;
-            rvs[q] = st == kFlBand ? __ldcg(&a.rnd[ids[q]]) : st == kFlNone ? kNone : r0 + st;
-            bk[q] = __ballot_sync(0xffffffffu, valid && rvs[q] >= live_from);
-            tot += __popc(bk[q]);
+            const bool keep = valid && rvs[q] >= live_from;
+            kp |= (uint32_t)keep << q;
+            out |= (uint32_t)(valid && !keep) << q;
+            dropped |= (uint32_t)(keep && rvs[q] != kNone) << q;
+            tot += __popc(__ballot_sync(0xffffffffu, keep));
         }
         // one slot claim per warp and chunk
         uint32_t ob = 0;
         if (lane == 0 && tot) ob = atomicAdd(&s_out, tot);
+        // few of them: in rolled loops, which read the entry again
+#pragma unroll 1
+        while (dropped) {                                    // an assignment dropped
+            a.rnd[L.id(cb + (__ffs(dropped) - 1) * 32 + lane)] = kNone;
+            dropped &= dropped - 1u;
+        }
+#pragma unroll 1
+        while (out && !changed) {
+            atomicAdd(&scr[dm.bin(__ldcg(&L.gkp[cb + (__ffs(out) - 1) * 32 + lane]))], 1u);
+            out &= out - 1u;
+        }
         ob = __shfl_sync(0xffffffffu, ob, 0);
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
-            const bool valid = cb + q * 32 + lane < n_live;
-            if ((bk[q] >> lane) & 1u) {
-                const uint32_t o = ob + __popc(bk[q] & lt);
+            const bool keep = (kp >> q) & 1u;
+            const uint32_t b = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const uint32_t o = ob + __popc(b & lt);
                 L.gid2[o] = ids[q];
                 L.gkp2[o] = keys[q];
                 L.gfl2[o] = (uint8_t)((fls[q] & kFlHold) | kFlNone);
-                if (rvs[q] != kNone) a.rnd[ids[q]] = kNone;          // an assignment dropped
-            } else if (valid && !changed) {
-                atomicAdd(&scr[dm.bin(keys[q])], 1u);
             }
-            ob += __popc(bk[q]);
+            ob += __popc(b);
         }
     }
     __syncthreads();
@@ -1679,9 +1758,11 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     uint8_t *sfl = reinterpret_cast<uint8_t *>(sid + kKeyCache);     // state bytes by list position (kc)
     __shared__ float Ls[D > 0 ? D : kMaxD];
     __shared__ uint32_t s_b[kMaxEpoch], s_r[kMaxEpoch], s_slot[kMaxEpoch], s_sbin[kMaxEpoch];
-    __shared__ uint32_t s_gin[kMaxEpoch], s_gout[kMaxEpoch], s_gq2[kMaxEpoch];
+    __shared__ GroupTab s_tab;
+    __shared__ uint32_t s_kcm, s_nl, s_klast, s_off[kMaxEpoch + 1], s_cert[kMaxEpoch];
+    __shared__ uint16_t s_lost[D > 0 ? D : kMaxD];
     __shared__ uint32_t s_cc[kMaxEpoch], s_gc[kMaxEpoch];
-    __shared__ uint32_t s_nslot, s_glast, s_hold_end;
+    __shared__ uint32_t s_nslot, s_hold_end;
     __shared__ __align__(4) uint8_t s_map[kHistBins];
     // the previous epoch's landmark; the attributes whose landmark value is new (mask) and,
     // for an update of the keys, those attributes with their old and new values
@@ -1713,36 +1794,55 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     // host) and the slice's state; then the points by attribute where the launch makes them
     {
         uint32_t *cw = &ctl->h0[0];
-        constexpr uint32_t words = (uint32_t)(sizeof(PeelCtl) - offsetof(PeelCtl, h0)) / 4u;
+        constexpr uint32_t words = (uint32_t)(offsetof(PeelCtl, Lbits) - offsetof(PeelCtl, h0)) / 4u;
+#pragma unroll 1
         for (uint32_t b = c * kThreads + t; b < words; b += G * kThreads) cw[b] = 0;
+#pragma unroll 1
+        for (uint32_t j = c * kThreads + t; j < (uint32_t)kMaxD; j += G * kThreads) {
+            ctl->Lbits[0][j] = 0u;
+            ctl->Lbits[1][j] = kInfBits;
+        }
+#pragma unroll 1
         for (uint32_t q = t; q < s1 - s0; q += kThreads) {
             a.rnd[s0 + q] = kNone;
             pfl[q] = kFlNone;
+            if (kc) sid[q] = s0 + q;
+            else gid[q] = s0 + q;
         }
     }
     if (!grid_sync(ctl, a.flags, gen, lim, a.stall)) return;
     if (a.transpose) transpose_tiles(a.x, a.n, d, a.xt_out, reinterpret_cast<float(*)[33]>(scr));
     if (!grid_sync(ctl, a.flags, gen, lim)) return;
-    bool first = true;           // the first epoch: a slice's list is the slice itself
+    bool first = true;           // the first epoch
     bool need_keys = true;       // the landmark changed: the keys must be computed
     uint32_t r0 = 0;             // the epoch's first round
+    int lpar = 0, hpar = 0;      // the landmark's and the holder counts' current arrays
     // the keys' error bound |delta32 - delta64| <= k_eps delta32 + k_abs (thread 0 keeps it,
     // the same in every CTA) and the key updates since the last full pass
-    const double eps_cap = (double)(d + 4) * 0x1p-23, eps0 = (double)key_roundings<D>(d) * 0x1p-23;
-    double k_eps = eps0, k_abs = 0x1p-120;
+    const float eps_cap = (float)(d + 4) * 0x1p-23f, eps0 = (float)key_roundings<D>(d) * 0x1p-23f;
+    float k_eps = eps0, k_abs = 0x1p-120f;
     for (;;) {
         const uint32_t nl_tot = n - r0 * N;
-        auto LID = [&](uint32_t q) -> uint32_t { return first ? s0 + q : kc ? sid[q] : __ldcg(&gid[q]); };
+        auto LID = [&](uint32_t q) -> uint32_t { return kc ? sid[q] : __ldcg(&gid[q]); };
         auto LKEY = [&](uint32_t q) -> uint32_t { return kc ? skey[q] : __ldcg(&gkp[q]); };
-        const ListView LV{first, kc, s0, sid, skey, sfl, gid, gkp, gfl, gid2, gkp2, gfl2};
+        const ListView LV{kc, sid, skey, sfl, gid, gkp, gfl, gid2, gkp2, gfl2};
+        // the landmark and the holder counts alternate between two arrays, so that no CTA
+        // overwrites what a slower one still reads
+        const uint32_t *Lcur = ctl->Lbits[lpar];
+        uint32_t *chold = ctl->chold[hpar];
+        uint32_t (*hcnt)[kMaxEpoch] = ctl->hcnt[hpar];
+        const uint32_t e_kmax = __ldcg(&ctl->kmax);
+#pragma unroll 1
         for (int j = t; j < d; j += kThreads) {
             Lold[j] = Ls[j];
-            Ls[j] = __uint_as_float(__ldcg(&ctl->Lbits[j]));
+            Ls[j] = __uint_as_float(__ldcg(&Lcur[j]));
         }
         __syncthreads();
         if (nl_tot <= N) {                            // the last subcluster: all that is left
+#pragma unroll 1
             for (uint32_t q = t; q < n_live; q += kThreads) a.rnd[LID(q)] = r0;
             if (c == 0 && a.landmarks)
+#pragma unroll 1
                 for (int j = t; j < d; j += kThreads) a.landmarks[(size_t)r0 * d + j] = Ls[j];
             break;
         }
@@ -1751,18 +1851,21 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         // ---- A: float32 distances of the points left, the first histogram, the holders
         if (need_keys) {
             // the attributes whose landmark value is new (all of them at first)
+#pragma unroll 1
             for (int j0 = w * 32; j0 < d; j0 += kW * 32) {
                 const int j = j0 + lane;
                 const bool mv = j < d && (first || __float_as_uint(Ls[j]) != __float_as_uint(Lold[j]));
                 const uint32_t m = __ballot_sync(0xffffffffu, mv);
                 if (lane == 0) s_jm[j0 >> 5] = m;
             }
+#pragma unroll 1
             for (int b = t; b < kHistBins; b += kThreads) scr[b] = 0;
             __syncthreads();
             if (t == 0) {
                 // an update of the keys, or a full pass (the same choice in every CTA)
+                // (float32 rounded up throughout: a float64 chain here held up every CTA)
                 uint32_t nj = 0, nsec = 0, last_sec = kGone;
-                double cs = 0.0;
+                float cs = 0.0f;
                 bool fin = true;
                 for (int wd = 0; wd < (d + 31) / 32; wd++) {
                     uint32_t m = s_jm[wd];
@@ -1775,7 +1878,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                             s_il[nj] = Ls[j];
                             const float c = __fsub_rn(Ls[j], Lold[j]);
                             fin = fin && c >= 0.0f && c <= 1.0f;
-                            cs += (double)c;
+                            cs = __fadd_ru(cs, c);
                         }
                         nj++;
                         if ((uint32_t)(j >> 3) != last_sec) {
@@ -1784,44 +1887,46 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                         }
                     }
                 }
-                const double ne = k_eps + 0x1p-23;
-                const double na = k_abs + (5.0 * k_eps + (16.0 + 4.0 * nj) * 0x1p-24) * cs * (1.0 + 0x1p-20);
+                cs = __fmul_ru(cs, 1.0f + 0x1p-20f);
+                const float ne = __fadd_ru(k_eps, 0x1p-23f);
+                const float na = __fadd_ru(
+                    k_abs, __fmul_ru(__fadd_ru(__fmul_ru(5.0f, k_eps), (16.0f + 4.0f * (float)nj) * 0x1p-24f), cs));
                 // the absolute term stays below an eighth of the relative one at the last
                 // epoch's first boundary, so the bands widen little
-                const double kref = (double)__ldcg(&ctl->kref);
                 const bool inc = !first && fin && nj >= 1 && nj <= (uint32_t)kIncMax && nsec * 160u < 12u * (uint32_t)d &&
-                                 ne <= 1.5 * eps_cap && na <= 0.125 * eps_cap * kref;
+                                 ne <= 1.5f * eps_cap && na <= 0.125f * eps_cap * s_tab.kref;
                 if (inc) {
                     k_eps = ne;
                     k_abs = na;
                 } else {
                     k_eps = eps0;
-                    k_abs = 0x1p-120;
+                    k_abs = 0x1p-120f;
                 }
                 s_nj = inc ? nj : 0u;
                 s_inc = inc ? 1 : 0;
                 if (inc && c == 0) ctl->key_updates += 1;
-                s_keps = __double2float_ru(k_eps);
-                s_kabs = __double2float_ru(k_abs);
+                s_keps = k_eps;
+                s_kabs = k_abs;
                 // the range of the new keys: none was below klast, the landmark's move takes
                 // at most 2 cs off a distance (c (2 x - l - o) <= 2 c per attribute, x <= 1) and
                 // adds nothing (x >= l for every point left), so none is above the first
                 // epoch's largest; a margin of 2^-12 for the roundings
                 if (!first) {
-                    const float lo = __uint_as_float(__ldcg(&ctl->klast)) * (1.0f - 0x1p-12f) - (float)cs * (2.0f + 0x1p-12f);
-                    s_dm = digit_map(lo > 0.0f ? __float_as_uint(lo) : 0u, __ldcg(&ctl->kmax) + 4096u);
+                    const float lo = __uint_as_float(s_klast) * (1.0f - 0x1p-12f) - cs * (2.0f + 0x1p-12f);
+                    s_dm = digit_map(lo > 0.0f ? __float_as_uint(lo) : 0u, e_kmax + 4096u);
                 }
             }
             __syncthreads();
             if (s_inc)
-                phase_inc<D>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, ctl->chold, s_nj, s_ij,
+                phase_inc<D>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, chold, s_nj, s_ij,
                              s_io, s_il);
             else
-                phase_keys<D>(a.x, Ls, d, n_live, s0, first, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, ctl->chold, s_jm);
+                phase_keys<D>(a.x, Ls, d, n_live, s0, first, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, chold, s_jm);
             __syncthreads();
             if (first) {
                 // the first epoch's bins, from its own keys
                 uint32_t mn = kGone, mx = 0;
+#pragma unroll 4
                 for (uint32_t q = t; q < n_live; q += kThreads) {
                     const uint32_t k = LKEY(q);
                     mn = min(mn, k);
@@ -1836,26 +1941,31 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 if (!grid_sync(ctl, a.flags, gen, lim)) return;
                 if (t == 0) s_dm = digit_map(~__ldcg(&ctl->kmin), __ldcg(&ctl->kmax) + 4096u);
                 __syncthreads();
+#pragma unroll 4
                 for (uint32_t q = t; q < n_live; q += kThreads) atomicAdd(&scr[s_dm.bin(LKEY(q))], 1u);
                 __syncthreads();
             }
             // each attribute's largest holder key (the holders are the flagged points left)
+#pragma unroll 1
             for (uint32_t q0 = 0; q0 < n_live; q0 += kHoldBatch * kThreads) {
-                uint8_t f[kHoldBatch];
+                uint32_t held = 0;
 #pragma unroll
                 for (int u = 0; u < kHoldBatch; u++) {
                     const uint32_t qi = q0 + u * kThreads + t;
-                    f[u] = qi < n_live ? pfl[qi] : (uint8_t)0;
+                    held |= (uint32_t)(qi < n_live && (pfl[qi] & kFlHold)) << u;
                 }
-#pragma unroll
-                for (int u = 0; u < kHoldBatch; u++) {
-                    const bool h = f[u] & kFlHold;
-                    if (!__any_sync(0xffffffffu, h)) continue;
+                uint32_t todo = __reduce_or_sync(0xffffffffu, held);
+#pragma unroll 1
+                while (todo) {
+                    const int u = __ffs(todo) - 1;
+                    todo &= todo - 1u;
+                    const bool h = (held >> u) & 1u;
                     const uint32_t qi = q0 + u * kThreads + t;
                     for_held(a.x, Ls, d, h, h ? LID(qi) : 0u, h ? LKEY(qi) : 0u,
                              [&](int j, uint32_t key) { atomicMax(&ctl->hmax[j], key); });
                 }
             }
+#pragma unroll 1
             for (int b = t; b < kHistBins; b += kThreads)
                 if (scr[b]) atomicAdd(&ctl->h0[b], scr[b]);
             if (!grid_sync(ctl, a.flags, gen, lim)) return;
@@ -1873,6 +1983,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
 #pragma unroll
             for (int q = 0; q < per; q++) s += l0[q];
             uint32_t m = kGone;
+#pragma unroll 1
             for (int j = t; j < d; j += kThreads) m = min(m, __ldcg(&ctl->hmax[j]));
             uint32_t tot;
             const uint32_t e0 = block_excl_scan(s, tot);
@@ -1908,6 +2019,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                     cc += l0[i];
                 }
             }
+#pragma unroll 1
             for (int b = t; b < kHistBins / 4; b += kThreads) reinterpret_cast<uint32_t *>(s_map)[b] = 0xFFFFFFFFu;
             __syncthreads();
             if (w == 0) {
@@ -1932,6 +2044,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             // the keys in those bins, straight to the grid's histograms: few of them, but one
             // atomic per warp for the equal ones (tied data crowds them into one)
             const DigitMap mp = s_dm;
+#pragma unroll 1
             for (uint32_t q0 = t - lane; q0 < n_live; q0 += 4 * kThreads) {       // warp-uniform bound
                 uint32_t k4[4];
 #pragma unroll
@@ -1952,28 +2065,34 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 }
             }
         }
-        // the last CTA to arrive turns each boundary's bins into its band cut-offs, and
-        // merges boundaries whose bands overlap into groups
-        if (!grid_sync_last(ctl, a.flags, gen, lim, [&]() {
-                resolve_cutoffs(ctl, Kb, s_keps, s_kabs, &s_dm, s_b, s_r, s_slot, s_nslot);
-            }))
-            return;
+        // each boundary's bins become its band cut-offs, and boundaries whose bands overlap
+        // merge into groups
         const uint32_t K = Kb;                        // boundaries of the epoch
+        if (K <= kAllResolve) {
+            if (!grid_sync(ctl, a.flags, gen, lim)) return;
+            resolve_cutoffs(ctl, K, s_keps, s_kabs, &s_dm, s_b, s_r, s_slot, s_tab);
+        } else {
+            if (!grid_sync_last(ctl, a.flags, gen, lim, [&]() {
+                    resolve_cutoffs(ctl, K, s_keps, s_kabs, &s_dm, s_b, s_r, s_slot, s_tab);
+#pragma unroll 1
+                    for (uint32_t e = t; e < sizeof(GroupTab) / 4u; e += kThreads)
+                        ctl->tab[e] = reinterpret_cast<const uint32_t *>(&s_tab)[e];
+                }))
+                return;
+#pragma unroll 1
+            for (uint32_t e = t; e < sizeof(GroupTab) / 4u; e += kThreads)
+                reinterpret_cast<uint32_t *>(&s_tab)[e] = __ldcg(&ctl->tab[e]);
+            __syncthreads();
+        }
 
         // ---- C: classify every point left: certainly in a round of the epoch, in a band, or later
-        const uint32_t ng = __ldcg(&ctl->n_groups);
-        if (t < (int)ng) {
-            s_gin[t] = __ldcg(&ctl->g_in[t]);
-            s_gout[t] = __ldcg(&ctl->g_out[t]);
-            s_gq2[t] = __ldcg(&ctl->g_q2[t]);
-        }
+        const uint32_t ng = s_tab.ng;
         if (t < kMaxEpoch) {
             s_cc[t] = 0;
             s_gc[t] = 0;
         }
-        if (t == 0) s_glast = __ldcg(&ctl->g_out[ng - 1]);
         __syncthreads();
-        classify_live(a, LV, n_live, Ls, r0, K, ng, s_gin, s_gout, s_gq2, s_glast, s_cc, s_gc);
+        classify_live(a, LV, n_live, Ls, r0, K, ng, s_tab.in, s_tab.out, s_tab.q2, s_tab.out[ng - 1], s_cc, s_gc, hcnt);
         __syncthreads();
         if (t < (int)K && s_cc[t]) atomicAdd(&ctl->cert[t], s_cc[t]);
         if (t < (int)ng && s_gc[t]) atomicAdd(&ctl->gcnt[t], s_gc[t]);
@@ -1983,10 +2102,12 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         // (across the grid), then each group's band settled (CTA c takes groups c, c + G, ...)
         {
             const uint32_t nlist = __ldcg(&ctl->band_cnt);
-            if (t < (int)ng) {
-                uint32_t off = 0;
-                for (uint32_t h = 0; h < (uint32_t)t; h++) off += __ldcg(&ctl->gcnt[h]);
-                s_cc[t] = off;                       // the group's region in gkey / gpos
+            // each group's region in gkey / gpos, and the certain points up to each round
+            if (t < 32) {
+                const uint32_t v = __ldcg(&ctl->gcnt[t]), cv = __ldcg(&ctl->cert[t]);
+                s_off[t + 1] = warp_incl_scan(v);
+                s_cert[t] = warp_incl_scan(cv);
+                if (t == 0) s_off[0] = 0;
             }
             __syncthreads();
             // one slot claim per warp and group: the entries of a pass crowd into a few
@@ -1994,23 +2115,24 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             // (8 lanes per entry from 32 attributes on: a thread's chain over 128 took 15 us)
             if (d >= 32) {
                 constexpr uint32_t EB = kThreads / 8;
+#pragma unroll 1
                 for (uint32_t b0 = c * EB; b0 < nlist; b0 += G * EB) {               // block-uniform bound
                     const uint32_t e = b0 + (uint32_t)t / 8u, sub = (uint32_t)t & 7u;
                     const bool v = e < nlist;
                     const uint32_t k = v ? __ldcg(&a.band_k32[e]) : 0u;
                     const uint32_t pos = v ? __ldcg(&a.band_pos[e]) : 0u;
                     uint32_t g = 0;
-                    while (g + 1 < ng && k > s_gout[g]) g++;
+                    while (g + 1 < ng && k > s_tab.out[g]) g++;
                     const uint32_t peers = __match_any_sync(0xffffffffu, v && sub == 0u ? g : kGone);
                     const uint32_t leader = (uint32_t)__ffs(peers) - 1u;
                     uint32_t slot = 0;
                     if (v && sub == 0u && (uint32_t)lane == leader) slot = atomicAdd(&ctl->gfill[g], (uint32_t)__popc(peers));
-                    slot = __shfl_sync(0xffffffffu, slot, (int)leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
                     float h, l;
                     dist_ff8(a.x + (size_t)(pos & kPosMask) * d, Ls, d, (int)sub, h, l);
+                    slot = __shfl_sync(0xffffffffu, slot, (int)leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
                     if (v && sub == 0u) {
-                        a.gkey[s_cc[g] + slot] = ff_key(h, l);
-                        a.gpos[s_cc[g] + slot] = pos;
+                        a.gkey[s_off[g] + slot] = ff_key(h, l);
+                        a.gpos[s_off[g] + slot] = pos;
                     }
                 }
             } else for (uint32_t b0 = c * kThreads; b0 < nlist; b0 += G * kThreads) {     // warp-uniform bound
@@ -2019,34 +2141,44 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 const uint32_t k = v ? __ldcg(&a.band_k32[e]) : 0u;
                 const uint32_t pos = v ? __ldcg(&a.band_pos[e]) : 0u;
                 uint32_t g = 0;
-                while (g + 1 < ng && k > s_gout[g]) g++;
+                while (g + 1 < ng && k > s_tab.out[g]) g++;
                 const uint32_t lane = (uint32_t)t & 31u;
                 const uint32_t peers = __match_any_sync(0xffffffffu, v ? g : 0xFFFFFFFFu);
                 const uint32_t leader = (uint32_t)__ffs(peers) - 1u;
                 uint32_t slot = 0;
                 if (v && lane == leader) slot = atomicAdd(&ctl->gfill[g], (uint32_t)__popc(peers));
+                const uint64_t key = v ? dff_key(a.x + (size_t)(pos & kPosMask) * d, Ls, d) : 0ull;
                 slot = __shfl_sync(0xffffffffu, slot, (int)leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
                 if (v) {
-                    a.gkey[s_cc[g] + slot] = dff_key(a.x + (size_t)(pos & kPosMask) * d, Ls, d);
-                    a.gpos[s_cc[g] + slot] = pos;
+                    a.gkey[s_off[g] + slot] = key;
+                    a.gpos[s_off[g] + slot] = pos;
                 }
             }
             if (!grid_sync(ctl, a.flags, gen, lim)) return;
-            for (uint32_t g = c; g < ng; g += G) settle_group(a, Ls, g, r0, K, scr);
+#pragma unroll 1
+            for (uint32_t g = c; g < ng; g += G) {
+                const uint32_t q1 = g ? s_tab.q2[g - 1] + 1u : 0u;
+                settle_group(a, Ls, g, q1, s_tab.q2[g], s_off[g], s_off[g + 1] - s_off[g], s_cert[q1], r0, K, hcnt, scr);
+            }
         }
-        // the last CTA to arrive finds how many rounds the epoch commits: up to the first
-        // round after which some attribute has no holder of its landmark value left
-        if (!grid_sync_last(ctl, a.flags, gen, lim, [&]() { commit_count(a, Ls, K, r0, need_keys); }))
-            return;
+        // how many rounds the epoch commits: up to the first round after which some attribute
+        // has no holder of its landmark value left
+        if (!grid_sync(ctl, a.flags, gen, lim)) return;
+        commit_count(a, K, s_tab, chold, ctl->chold[hpar ^ 1], hcnt, s_kcm, s_nl, s_klast, s_lost);
 
         // ---- E: commit: the epoch's first k_commit rounds leave the lists; the other
         // assignments are dropped; the next landmark if it changes
-        uint32_t kcm = __ldcg(&ctl->k_commit);
+        const uint32_t n_lost = s_nl;
+        uint32_t kcm = s_kcm;
         if (kcm < 1u || kcm > K) {                    // cannot happen; keeps the loop finite
             if (c == 0 && t == 0) atomicOr(&a.flags[1], 1u);
             kcm = 1u;
         }
-        const bool changed = __ldcg(&ctl->l_changed) != 0;
+        const bool changed = n_lost != 0u;
+        if (c == 0 && t == 0) {
+            ctl->epochs += 1;
+            ctl->passes += need_keys ? 1u : 0u;
+        }
         const uint32_t live_from = r0 + kcm;
         n_live = kc ? compact_shared(a, LV, n_live, r0, live_from, changed, &s_dm, scr)
                     : compact_global(a, LV, n_live, r0, live_from, changed, &s_dm, scr);
@@ -2058,10 +2190,30 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         }
         // the epoch's scratch, cleared across the grid for the next one
         {
-            const uint32_t ns = __ldcg(&ctl->n_slots);
+            if (changed) {                            // recomputed by the next pass
+#pragma unroll 1
+                for (uint32_t b = c * kThreads + t; b < (uint32_t)kHistBins; b += G * kThreads) ctl->h0[b] = 0;
+                // the next landmark: the attributes that keep theirs here, the others' minima
+                // below; this one's array becomes the one after's
+                uint32_t *Lnext = ctl->Lbits[lpar ^ 1];
+#pragma unroll 1
+                for (uint32_t j = c * kThreads + t; j < (uint32_t)d; j += G * kThreads) {
+                    ctl->hmax[j] = 0;
+                    ctl->Lbits[lpar][j] = kInfBits;
+                    bool keep = true;
+                    for (uint32_t e = 0; e < n_lost; e++) keep = keep && s_lost[e] != (uint16_t)j;
+                    if (keep) Lnext[j] = __float_as_uint(Ls[j]);
+                }
+            }
+            if (a.landmarks)
+#pragma unroll 1
+                for (uint32_t e = c * kThreads + t; e < kcm * (uint32_t)d; e += G * kThreads)
+                    a.landmarks[(size_t)(r0 + e / d) * d + e % d] = Ls[e % d];
             uint32_t *h1 = &ctl->h1[0][0];
-            for (uint32_t b = c * kThreads + t; b < ns * (uint32_t)kHistBins; b += G * kThreads) h1[b] = 0;
-            uint32_t *hc = &ctl->hcnt[0][0];
+#pragma unroll 1
+            for (uint32_t b = c * kThreads + t; b < s_nslot * (uint32_t)kHistBins; b += G * kThreads) h1[b] = 0;
+            uint32_t *hc = &ctl->hcnt[hpar ^ 1][0][0];        // the next epoch's
+#pragma unroll 1
             for (uint32_t b = c * kThreads + t; b < (uint32_t)d * kMaxEpoch; b += G * kThreads) hc[b] = 0;
             if (c == 0 && t < kMaxEpoch) {
                 ctl->cert[t] = 0;
@@ -2072,8 +2224,10 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             if (c == 0 && t == 0) ctl->band_cnt = 0;
         }
         if (changed && n_live)
-            lost_minima(a.x, a.xt, n, d, n_live, kc, sid, gid, ctl->lost, __ldcg(&ctl->n_lost), ctl->Lbits);
+            lost_minima(a.x, a.xt, n, d, n_live, kc, sid, gid, s_lost, n_lost, ctl->Lbits[lpar ^ 1]);
         first = false;
+        hpar ^= 1;
+        if (changed) lpar ^= 1;
         need_keys = changed;
         r0 += kcm;
         if (!grid_sync(ctl, a.flags, gen, lim)) return;

@@ -33,25 +33,16 @@ struct PeelCtl {
     uint32_t kmin, kmax;                 // smallest and largest key of the first epoch (kmin: ~key)
     uint32_t h0[kHistBins];              // first digit of the live keys
     uint32_t h1[kMaxEpoch][kHistBins];   // second digit inside each boundary's bin
-    uint32_t Lbits[kMaxD];               // landmark of the current epoch (float bits)
-    uint32_t lost[kMaxD];                // attributes whose last holder left with the last commit
-    uint32_t chold[kMaxD];               // live points whose attribute j equals L_j
+    uint32_t chold[2][kMaxD];            // live points whose attribute j equals L_j (alternating)
     uint32_t hmax[kMaxD];                // the largest key among them (since the last pass)
-    uint32_t hcnt[kMaxD][kMaxEpoch];     // of those, the ones assigned to each round of the epoch
+    uint32_t hcnt[2][kMaxD][kMaxEpoch];  // of those, the ones assigned to each round of the epoch
     uint32_t cert[kMaxEpoch];            // points certainly in each round of the epoch
     uint32_t bnd[kMaxEpoch];             // band points settled into each round of the epoch
     uint32_t gcnt[kMaxEpoch];            // band entries of each group of boundaries
     uint32_t gfill[kMaxEpoch];           // of those, regrouped into the group's region so far
-    uint32_t g_in[kMaxEpoch], g_out[kMaxEpoch];   // a group's band: keys in [g_in, g_out]
-    uint32_t g_q1[kMaxEpoch], g_q2[kMaxEpoch];    // a group's first and last boundary
-    float kref;                          // lower end of the first boundary's key range, last epoch
-    uint32_t klast;                      // no point left has a smaller key (before the landmark moved)
-    uint32_t n_lost;
-    uint32_t n_slots;                    // first-digit bins with a second-digit histogram
-    uint32_t n_groups;
+    uint32_t tab[3 * kMaxEpoch + 2];     // the epoch's groups, when one CTA forms them for all
     uint32_t band_cnt;                   // band entries listed this epoch
-    uint32_t k_commit;                   // rounds the epoch commits
-    uint32_t l_changed;                  // the landmark changes after them
+    uint32_t Lbits[2][kMaxD];            // landmark of the current epoch (float bits), and the next one's
 };
 
 // v (a scaled coordinate, in [0, 1]) times 2^32 rounded to the nearest integer, ties to
