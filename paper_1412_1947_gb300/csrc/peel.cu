@@ -88,14 +88,23 @@ constexpr int kKeyCache = 4096;               // keys and ids of a slice kept in
 constexpr int kSelBins = 2048;
 constexpr int kSelList = 1024;
 constexpr int kSelBatch = 8;
-constexpr int kStage = 1024;                  // band entries of one group staged in shared memory
-constexpr int kStageOff = kSelBins + 3 * kSelList;
-constexpr int kScrWords = kStageOff + 3 * kStage;
+constexpr int kScrWords = 8192;
 static_assert(kScrWords >= kHistBins, "phase A's histogram fits the scratch");
-static_assert(kStageOff % 2 == 0, "staged 64-bit keys are 8-byte aligned");
+static_assert(kScrWords >= kSelBins + 3 * kSelList, "a selection's scratch fits");
 constexpr int kPeelDynWords = kScrWords + 2 * kKeyCache + kKeyCache / 4;
+// Settling a group in shared memory: the histogram of its distances, the bins marked, and the
+// entries near a boundary (distance, id, float64 distance, two bytes of state); in place of a
+// slice's key cache, where there is none, all entries' distances and ids.
+constexpr int kRankBins = 2048;
+constexpr int kNear = 1024;
+constexpr int kStage = (2 * kKeyCache + kKeyCache / 4) / 3;
+static_assert(kRankBins + kRankBins / 32 + 5 * kNear + kNear / 2 <= kScrWords, "settling fits the scratch");
 constexpr int kQT = 4;                        // tiles of kThreads items per compaction scan
 constexpr int kCB = 8;                        // keys per thread in flight when classifying
+// list positions a thread has in flight in the passes that read attributes by id: a slice in
+// shared memory has 16 a thread at most, and wants little code; one in global memory is bound by
+// the loads in flight (2^24 x 64: landmark 63 -> 41 us, key update 77 -> 68 us an epoch)
+constexpr int kLoadKc = 4, kLoadGlobal = 8;
 constexpr int kHoldBatch = 8;                 // state bytes per thread in flight when finding holders
 // State byte of each list position: bit 7 set once the point has held some attribute's
 // landmark value (it then holds it while it is left); bits 0..6 its place in the current
@@ -743,12 +752,14 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
         for (uint32_t base = 0; base < n_live; base += BC * kThreads) {
             // chunk q of this warp: list positions cb + [0, 32); lane i fetches the id of
             // position cb + i, and row u of its group is position cb + u*RW + g.  Past the
-            // end the id is the slice's first row (read again, an L1 hit).
-            uint32_t myid[BC];
+            // end and at gaps the id is the slice's first row (read again, an L1 hit).
+            uint32_t myid[BC], live[BC];
 #pragma unroll
             for (int q = 0; q < BC; q++) {
                 const uint32_t pos = base + q * kThreads + w * 32 + lane;
-                myid[q] = pos < n_live ? LID(pos) : s0;
+                myid[q] = pos < n_live ? LID(pos) : kGone;
+                live[q] = __ballot_sync(0xffffffffu, myid[q] != kGone);
+                if (myid[q] == kGone) myid[q] = s0;
             }
             static_assert(BC * P <= 32, "a mask bit per row");
             uint32_t hzs = 0;                              // rows with a landmark value
@@ -801,8 +812,7 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
                 }
                 hzs |= hz << (q * P);
                 const uint32_t src = (uint32_t)(sl * RW + g);
-                const uint32_t pos = base + q * kThreads + w * 32 + src;
-                key_out(pos < n_live, pos, __float_as_uint(ps[0]));
+                key_out((live[q] >> src) & 1u, base + q * kThreads + w * 32 + src, __float_as_uint(ps[0]));
             }
             // rare: rows holding a landmark value in this lane's attributes
 #pragma unroll 1
@@ -810,8 +820,9 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
                 const int b = __ffs(hzs) - 1;
                 hzs &= hzs - 1u;
                 const uint32_t rpos = base + (uint32_t)(b / P) * kThreads + w * 32 + (uint32_t)(b % P) * RW + g;
-                if (rpos >= n_live) continue;
-                const float4 *r4 = reinterpret_cast<const float4 *>(x + (size_t)LID(rpos) * D) + sl;
+                const uint32_t id = rpos < n_live ? LID(rpos) : kGone;
+                if (id == kGone) continue;
+                const float4 *r4 = reinterpret_cast<const float4 *>(x + (size_t)id * D) + sl;
 #pragma unroll 1
                 for (int f = 0; f < F; f++) {
                     const float4 vv = __ldg(r4 + P * f);
@@ -833,10 +844,11 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
 #pragma unroll
             for (int q = 0; q < B; q++) {
                 const uint32_t qi = base + q * kThreads + t;
-                lv[q] = qi < n_live;
-                ids[q] = lv[q] ? LID(qi) : s0;
+                ids[q] = qi < n_live ? LID(qi) : kGone;
+                lv[q] = ids[q] != kGone;
+                if (!lv[q]) ids[q] = s0;
             }
-            // past the end a thread reads the slice's first row again (an L1 hit), so every
+            // past the end and at gaps a thread reads the slice's first row (an L1 hit), so every
             // thread keeps B rows in flight without branching
             float dl[B];
             bool hz[B];
@@ -863,14 +875,14 @@ __device__ __noinline__ void phase_keys(const float *__restrict__ x, const float
 // sum_i (jl_i - jo_i)(jl_i + jo_i - 2 x_{jj_i}) (FMA chain in float32), read from those
 // attributes only; the result is clamped at 0, stored in place and counted in sh, and the
 // holders of the new values are counted and flagged as in phase_keys.
-template <int D>
+// U: list positions per thread in flight (kLoadKc, kLoadGlobal).
+template <int D, int U>
 __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float *__restrict__ xt, uint32_t n, int d,
                                        uint32_t n_live, bool kc, const uint32_t *sid, const uint32_t *glin,
                                        uint32_t *skey, uint32_t *kpos, uint32_t *sh, const DigitMap *dm,
                                        uint8_t *pfl, uint32_t *chold, uint32_t nj, const int *jj, const float *jo,
                                        const float *jl)
 {
-    constexpr int U = 4;                                   // list positions per thread in flight
     const int t = threadIdx.x;
     const DigitMap mp = *dm;
     // attribute j of point i at src[i * ps + j * as]: the by-attribute copy (a CTA's ids
@@ -1081,141 +1093,260 @@ __device__ __noinline__ void settle_large(const PeelArgs &a, const float *Ls, ui
 }
 
 // Settles group g of the epoch's boundaries (one CTA): every band entry of the group gets
-// its round, exactly by (delta64, index).  Entries are ranked by their compensated
-// distance; at each boundary only the entries within that distance's error of the cut are
-// ranked again by float64.  r0: the epoch's first round; K: its boundaries.
-// q1 .. q2: the group's boundaries; off, ne: its region of the regrouped entries; certs: the
-// points certainly in rounds 0 .. q1.
+// its round, exactly by (delta64, index).  q1 .. q2: the group's boundaries; off, ne: its region
+// of the regrouped entries; certs: the points certainly in rounds 0 .. q1; r0: the epoch's first
+// round; K: its boundaries; stage: the entries that fit past the scratch (0: none).
+//
+// An entry's round follows from its rank among the group's by their compensated distances:
+// the entries whose distance is smaller beyond the error window come before it, and where the
+// window holds others and a boundary cuts through it, those of them that are smaller by float64
+// and index.  The window of a distance with bits k: k +- W, W >= 4 (eps_ff + 2^-52) 2^53 (a
+// relative step r moves a double's bits by at most r 2^53); below 2^-60 the absolute error of
+// tiny squares counts too, so all of them are one window.  A histogram of the distances tells
+// most entries' sides of every boundary; only those close to one (all, of a small group) are
+// ranked one by one, a warp each, against the entries of the bins their windows touch: no
+// selection, and few barriers.  Short rolled loops throughout: the CTA that settles a group is
+// the only one that fetches this code, and the others wait for it.  (Every entry ranked against
+// every other: 25 us for 1000 entries; the selection of larger groups: 130 to 170 us.)
 __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, uint32_t g, uint32_t q1, uint32_t q2,
                                           uint32_t off, uint32_t ne, uint32_t certs, uint32_t r0, uint32_t K,
-                                          uint32_t (*hcnt)[kMaxEpoch], uint32_t *scr)
+                                          uint32_t (*hcnt)[kMaxEpoch], uint32_t *scr, uint32_t stage)
 {
     PeelCtl *ctl = a.ctl;
     const int d = a.d;
     const uint32_t N = (uint32_t)a.N;
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ uint32_t s_need[kMaxEpoch], s_bc[kMaxEpoch];
+    __shared__ unsigned long long s_mn[kW], s_mx[kW];
+    __shared__ uint32_t s_near, s_any;
     // points before the group: the certain ones and the entries of the groups before it
     const uint32_t before = certs + off, filled = __ldcg(&ctl->gfill[g]);
-    uint64_t *stk = reinterpret_cast<uint64_t *>(scr + kStageOff);
-    uint32_t *stp = scr + kStageOff + 2 * kStage;
+    uint32_t *hist = scr, *mark = hist + kRankBins;                         // entries before a bin; bins marked
+    uint64_t *nk = reinterpret_cast<uint64_t *>(mark + kRankBins / 32);     // near entries: distance,
+    uint64_t *d64 = nk + kNear;                                             // by float64,
+    uint32_t *np = reinterpret_cast<uint32_t *>(d64 + kNear);               // id and hold flag,
+    uint8_t *nst = reinterpret_cast<uint8_t *>(np + kNear), *e64 = nst + kNear;   // state, in a cut window
+    // state: the entry's round is its rank's to find; a boundary cuts its window; else neither
+    constexpr uint8_t kClose = 1, kCut = 2;
+    uint64_t *stk = reinterpret_cast<uint64_t *>(scr + kScrWords);
+    uint32_t *stp = reinterpret_cast<uint32_t *>(stk + kStage);
     const uint64_t *gk = a.gkey + off;
     const uint32_t *gp = a.gpos + off;
+    const bool all = ne <= 64u, st = ne <= stage && !all;
+    const uint32_t nq = q2 - q1 + 1u;
     if (t < kMaxEpoch) s_bc[t] = 0;
     if (t == 0 && filled != ne) atomicOr(&a.flags[1], 1u);
-    if (ne > (uint32_t)kStage) {
-        settle_large(a, Ls, q1, q2, off, ne, before, r0, K, hcnt, scr);
-        return;
-    }
-    for (uint32_t e = t; e < ne; e += kThreads) {
-        stk[e] = __ldcg(&gk[e]);
-        stp[e] = __ldcg(&gp[e]);
-    }
-    __syncthreads();
-    // every entry's rank among the group's, counted by eight lanes: the entries whose
-    // compensated distance is smaller beyond the error window, and where the window holds
-    // others and a boundary cuts through it, those of them that are smaller by float64
-    // and index.  No selection and no barrier per boundary (2^20 x 16: settle and commit
-    // 14 -> 8 us an epoch).  The window of a distance with bits k: k +- W, W >= 4 (eps_ff
-    // + 2^-52) 2^53 (a relative step r moves a double's bits by at most r 2^53); below
-    // 2^-60 the absolute error of tiny squares counts too, so all of them are one window.
-    // Short rolled loops throughout: the CTA that settles a group is the only one that
-    // fetches this code, and the others wait for it.
-    __shared__ int s_any;
-    uint64_t *d64 = reinterpret_cast<uint64_t *>(scr);                      // kStage keys
-    uint32_t *rk = scr + 2 * kStage;                                        // kStage ranks, bit 31: cut
-    uint8_t *f64 = reinterpret_cast<uint8_t *>(scr + 3 * kStage);           // kStage flags
-    static_assert(3 * kStage + kStage / 4 <= kStageOff, "the rank scratch lies before the staged entries");
-    constexpr uint32_t EB = kThreads / 8;
-    constexpr uint32_t kCut = 0x80000000u;
-    const uint32_t sub = (uint32_t)t & 7u;
-    if (t <= (int)(q2 - q1)) {
+    if (t < (int)nq) {
         const int64_t need_s = (int64_t)(q1 + t + 1) * N - (int64_t)before;
         s_need[t] = need_s < 0 ? 0u : (need_s > (int64_t)ne ? ne : (uint32_t)need_s);
         if (need_s < 0 || need_s > (int64_t)ne) atomicOr(&a.flags[1], 1u);
     }
-    if (t == 0) s_any = 0;
-    for (uint32_t e = t; e < ne; e += kThreads) f64[e] = 0;
-    __syncthreads();
+    if (t == 0) {
+        s_any = 0;
+        s_near = all ? ne : 0u;
+    }
     const uint64_t W0 = 256ull * ((uint64_t)d * d + 8ull * d + 1ull) + 8ull, W = W0 + (W0 >> 4);
     constexpr uint64_t kTiny = 963ull << 52;                                // 2^-60
-    const uint32_t nq = q2 - q1 + 1u;
-    // the window of the staged distance k
+    // the window of the distance k
     auto win_lo = [&](uint64_t k) { return k < kTiny + W ? 0ull : k - W; };
     auto win_hi = [&](uint64_t k) { return (k < kTiny ? kTiny : k) + W; };
-#pragma unroll 1
-    for (uint32_t e0 = 0; e0 < ne; e0 += EB) {                              // block-uniform bound
-        const uint32_t e = e0 + (uint32_t)t / 8u;
-        const uint64_t k = e < ne ? stk[e] : 0ull, lo = win_lo(k), hi = win_hi(k);
-        uint32_t below = 0, upto = 0;
-#pragma unroll 4
-        for (uint32_t f = sub; f < ne; f += 8) {
-            const uint64_t kf = stk[f];
-            below += kf < lo;
-            upto += kf <= hi;
+    auto KEY = [&](uint32_t e) -> uint64_t { return st ? stk[e] : __ldcg(&gk[e]); };
+    auto RAW = [&](uint32_t e) -> uint32_t { return st ? stp[e] : __ldcg(&gp[e]); };
+    auto settle = [&](bool v, uint32_t raw, uint32_t rr) {                  // a warp's entries with v set
+        if (v && rr < K) {
+            a.rnd[raw & kPosMask] = r0 + rr;
+            atomicAdd(&s_bc[rr], 1u);
         }
+        const bool ch = v && rr < K && (raw & ~kPosMask);
+        if (__any_sync(0xffffffffu, ch)) count_held(a.x, Ls, d, ch, raw & kPosMask, rr, hcnt);
+    };
+    unsigned long long mn = ~0ull, mx = 0ull;
+    int sh = 0;
+    auto bin = [&](uint64_t k) { return k <= mn ? 0u : (uint32_t)(min(k, (uint64_t)mx) - mn >> sh); };
+    // an entry's round from the bins alone; true if a boundary lies among those of its window
+    auto close_to = [&](uint64_t k, uint32_t &rr, uint32_t &bl, uint32_t &bh) {
+        bl = bin(win_lo(k));
+        bh = bin(win_hi(k));
+        const uint32_t least = hist[bl], most = bh + 1u < (uint32_t)kRankBins ? hist[bh + 1u] : ne;
+        rr = q1;
+        bool close = false;                                                 // the rank lies in [least, most)
+#pragma unroll 1
+        for (uint32_t b = 0; b < nq; b++) {
+            rr += s_need[b] <= least;
+            close |= s_need[b] > least && s_need[b] < most;
+        }
+        return close;
+    };
+    // f(e, key, whether e < ne) for every entry, by whole warps: the keys of four loaded at once
+    auto each = [&](auto f) {
+#pragma unroll 1
+        for (uint32_t e0 = 0; e0 < ne; e0 += 4 * kThreads) {
+            uint64_t k4[4];
 #pragma unroll
-        for (int o = 4; o; o >>= 1) {
-            below += __shfl_xor_sync(0xffffffffu, below, o);
-            upto += __shfl_xor_sync(0xffffffffu, upto, o);
-        }
-        if (e < ne) {
-            bool cut = false;
+            for (int u = 0; u < 4; u++) {
+                const uint32_t e = e0 + u * kThreads + t;
+                k4[u] = e < ne ? KEY(e) : 0ull;
+            }
 #pragma unroll 1
-            for (uint32_t b = 0; b < nq; b++) cut |= s_need[b] > below && s_need[b] < upto;
-            if (sub == 0) rk[e] = below | (cut ? kCut : 0u);
-            if (cut) {
-                s_any = 1;
-#pragma unroll 1
-                for (uint32_t f = sub; f < ne; f += 8)
-                    if (stk[f] >= lo && stk[f] <= hi) f64[f] = 1;
+            for (uint32_t u = 0; u < 4 && e0 + u * kThreads < ne; u++) {
+                const uint32_t e = e0 + u * kThreads + t;
+                f(e, u < 2 ? (u ? k4[1] : k4[0]) : (u == 2 ? k4[2] : k4[3]), e < ne);
             }
         }
+    };
+    if (all) {
+        if (t < (int)ne) {
+            nk[t] = __ldcg(&gk[t]);
+            np[t] = __ldcg(&gp[t]);
+            nst[t] = kClose;
+            e64[t] = 0;
+        }
+    } else {
+#pragma unroll 4
+        for (uint32_t e = t; e < ne; e += kThreads) {
+            const unsigned long long k = __ldcg(&gk[e]);
+            if (st) {
+                stk[e] = k;
+                stp[e] = __ldcg(&gp[e]);
+            }
+            mn = min(mn, k);
+            mx = max(mx, k);
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        }
+        if (lane == 0) {
+            s_mn[w] = mn;
+            s_mx[w] = mx;
+        }
+#pragma unroll 1
+        for (int b = t; b < kRankBins + kRankBins / 32; b += kThreads) hist[b] = 0;
+        __syncthreads();
+#pragma unroll 1
+        for (int q = 0; q < kW; q++) {
+            mn = min(mn, s_mn[q]);
+            mx = max(mx, s_mx[q]);
+        }
+        sh = max(0, 53 - __clzll((long long)((mx - mn) | 1ull)));           // (mx - mn) >> sh < kRankBins
+        each([&](uint32_t, uint64_t k, bool v) {
+            if (v) atomicAdd(&hist[bin(k)], 1u);
+        });
+        __syncthreads();
+        {
+            constexpr int per = kRankBins / kThreads;
+            uint32_t c[per], sum = 0, tot;
+#pragma unroll
+            for (int q = 0; q < per; q++) {
+                c[q] = hist[t * per + q];
+                sum += c[q];
+            }
+            uint32_t ex = block_excl_scan(sum, tot);
+#pragma unroll
+            for (int q = 0; q < per; q++) {
+                hist[t * per + q] = ex;
+                ex += c[q];
+            }
+        }
+        __syncthreads();
+        // the bins of the close entries' windows, and the entries in those
+        each([&](uint32_t, uint64_t k, bool v) {
+            uint32_t rr, bl, bh;
+            if (v && close_to(k, rr, bl, bh))
+#pragma unroll 1
+                for (uint32_t b = bl; b <= bh; b++)
+                    if (!((mark[b >> 5] >> (b & 31u)) & 1u)) atomicOr(&mark[b >> 5], 1u << (b & 31u));
+        });
+        __syncthreads();
+        each([&](uint32_t e, uint64_t k, bool v) {
+            const uint32_t b = bin(k);
+            if (v && ((mark[b >> 5] >> (b & 31u)) & 1u)) {
+                const uint32_t slot = atomicAdd(&s_near, 1u);
+                if (slot < (uint32_t)kNear) {
+                    uint32_t rr, bl, bh;
+                    nk[slot] = k;
+                    np[slot] = RAW(e);
+                    nst[slot] = close_to(k, rr, bl, bh) ? kClose : (uint8_t)0;
+                    e64[slot] = 0;
+                }
+            }
+        });
+    }
+    __syncthreads();
+    const uint32_t nn = s_near;
+    if (nn > (uint32_t)kNear) {                                             // heavily tied
+        settle_large(a, Ls, q1, q2, off, ne, before, r0, K, hcnt, scr);
+        return;
+    }
+    // the close entries' ranks, among the near ones: every entry of the bins that a close one's
+    // window touches is near
+    __shared__ uint32_t s_rank[kNear];
+#pragma unroll 1
+    for (uint32_t u = (uint32_t)w; u < nn; u += kW) {
+        if (!(nst[u] & kClose)) continue;                                   // the warp's
+        const uint64_t k = nk[u], lo = win_lo(k), hi = win_hi(k);
+        const uint32_t bl = all ? 0u : bin(lo), base = all ? 0u : hist[bl];
+        uint32_t below = 0, upto = 0;
+#pragma unroll 2
+        for (uint32_t f = (uint32_t)lane; f < nn; f += 32) {
+            const uint64_t kf = nk[f];
+            const bool in = all || bin(kf) >= bl;
+            below += in && kf < lo;
+            upto += in && kf <= hi;
+        }
+        below = base + __reduce_add_sync(0xffffffffu, below);
+        upto = base + __reduce_add_sync(0xffffffffu, upto);
+        // lane q: the group's boundary q
+        const bool cut = __any_sync(0xffffffffu, (uint32_t)lane < nq && s_need[lane] > below && s_need[lane] < upto);
+        if (lane == 0) {
+            s_rank[u] = below;
+            if (cut) nst[u] = kClose | kCut;
+            if (cut) s_any = 1;
+        }
+        // the entries of a window that a boundary cuts are ranked by float64
+        if (cut)
+#pragma unroll 2
+            for (uint32_t f = (uint32_t)lane; f < nn; f += 32)
+                if (nk[f] >= lo && nk[f] <= hi) e64[f] = 1;
     }
     __syncthreads();
     if (s_any) {
 #pragma unroll 1
-        for (uint32_t e = t; e < ne; e += kThreads)
-            if (f64[e])
-                d64[e] = (uint64_t)__double_as_longlong(dist64(a.x + (size_t)(stp[e] & kPosMask) * d, Ls, d));
+        for (uint32_t f = t; f < nn; f += kThreads)
+            if (e64[f]) d64[f] = (uint64_t)__double_as_longlong(dist64(a.x + (size_t)(np[f] & kPosMask) * d, Ls, d));
         __syncthreads();
 #pragma unroll 1
-        for (uint32_t e0 = 0; e0 < ne; e0 += EB) {
-            const uint32_t e = e0 + (uint32_t)t / 8u;
-            const bool cut = e < ne && (rk[e] & kCut);
+        for (uint32_t u = (uint32_t)w; u < nn; u += kW) {
+            if (!(nst[u] & kCut)) continue;                                 // the warp's
+            const uint32_t pu = np[u] & kPosMask;
+            const uint64_t k = nk[u], lo = win_lo(k), hi = win_hi(k), ku = d64[u];
             uint32_t more = 0;
-            if (cut) {
-                const uint64_t k = stk[e], lo = win_lo(k), hi = win_hi(k), ke = d64[e];
-                const uint32_t pe = stp[e] & kPosMask;
-#pragma unroll 1
-                for (uint32_t f = sub; f < ne; f += 8)
-                    if (stk[f] >= lo && stk[f] <= hi)
-                        more += d64[f] < ke || (d64[f] == ke && (stp[f] & kPosMask) < pe);
-            }
-#pragma unroll
-            for (int o = 4; o; o >>= 1) more += __shfl_xor_sync(0xffffffffu, more, o);
-            if (cut && sub == 0) rk[e] += more;
+#pragma unroll 2
+            for (uint32_t f = (uint32_t)lane; f < nn; f += 32)
+                if (nk[f] >= lo && nk[f] <= hi)
+                    more += d64[f] < ku || (d64[f] == ku && (np[f] & kPosMask) < pu);
+            more = __reduce_add_sync(0xffffffffu, more);
+            if (lane == 0) s_rank[u] += more;
         }
         __syncthreads();
     }
+    // the rounds: of the close entries by rank, of the others by their bins
 #pragma unroll 1
-    for (uint32_t e0 = 0; e0 < ne; e0 += kThreads) {                        // block-uniform bound
-        const uint32_t e = e0 + (uint32_t)t;
-        uint32_t rr = kNone, raw = 0;
-        if (e < ne) {
-            raw = stp[e];
-            rr = q1;
-            const uint32_t rank = rk[e] & ~kCut;
+    for (uint32_t u0 = 0; u0 < nn; u0 += kThreads) {                        // block-uniform bounds
+        const uint32_t u = u0 + (uint32_t)t;
+        const bool v = u < nn && (nst[u] & kClose);
+        uint32_t rr = q1;
 #pragma unroll 1
-            for (uint32_t b = 0; b < nq; b++) rr += s_need[b] <= rank;
-            if (rr < K) {
-                a.rnd[raw & kPosMask] = r0 + rr;
-                atomicAdd(&s_bc[rr], 1u);
-            }
-        }
-        const bool ch = e < ne && rr < K && (raw & ~kPosMask);
-        if (__any_sync(0xffffffffu, ch)) count_held(a.x, Ls, d, ch, raw & kPosMask, rr, hcnt);
+        for (uint32_t b = 0; v && b < nq; b++) rr += s_need[b] <= s_rank[u];
+        settle(v, v ? np[u] : 0u, rr);
     }
+    if (!all)
+        each([&](uint32_t e, uint64_t k, bool in) {
+            uint32_t rr = 0, bl, bh;
+            const bool v = in && !close_to(k, rr, bl, bh);
+            settle(v, v ? RAW(e) : 0u, rr);
+        });
     __syncthreads();
     if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
 }
@@ -1225,8 +1356,8 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
 // kMinBatch points per thread at a time (their loads issued together), added to the grid's
 // minimum (values lie in [0, 1], so their bits order like them).
 constexpr int kMinAttrs = 4;
-constexpr int kMinBatch = 4;
 
+template <int kMinBatch>
 __device__ __noinline__ void lost_minima(const float *__restrict__ x, const float *__restrict__ xt, uint32_t n, int d,
                                          uint32_t n_live, bool kc, const uint32_t *sid, const uint32_t *glist,
                                          const uint16_t *lost, uint32_t nl, uint32_t *Lbits)
@@ -1253,15 +1384,15 @@ __device__ __noinline__ void lost_minima(const float *__restrict__ x, const floa
             uint32_t id[kMinBatch];
 #pragma unroll
             for (int u = 0; u < kMinBatch; u++) {
-                const uint32_t qi = min(q0 + u * kThreads + t, n_live - 1u);
-                id[u] = kc ? sid[qi] : __ldcg(&glist[qi]);
+                const uint32_t qi = q0 + u * kThreads + t;
+                id[u] = qi < n_live ? (kc ? sid[qi] : __ldcg(&glist[qi])) : kGone;
             }
 #pragma unroll
             for (int i = 0; i < kMinAttrs; i++)
                 if (i < (int)na) {
 #pragma unroll
                     for (int u = 0; u < kMinBatch; u++)
-                        mn[i] = min(mn[i], __float_as_uint(__ldcg(&col[i][(size_t)id[u] * ps])));
+                        mn[i] = min(mn[i], id[u] != kGone ? __float_as_uint(__ldcg(&col[i][(size_t)id[u] * ps])) : kInfBits);
                 }
         }
 #pragma unroll
@@ -1474,59 +1605,82 @@ struct ListView {
 
 // Phase C for one CTA's list: every live key classified against the epoch's groups (see
 // the kernel); certain points get their round in rnd[] and counted in s_cc, band entries
-// are listed (with their hold flag in bit 31 of the id) and counted per group in s_gc.
-__device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L, uint32_t n_live, const float *Ls,
-                                          uint32_t r0, uint32_t K, uint32_t ng, const uint32_t *s_gin,
-                                          const uint32_t *s_gout, const uint32_t *s_gq2, uint32_t s_glast,
-                                          uint32_t *s_cc, uint32_t *s_gc, uint32_t (*hcnt)[kMaxEpoch])
+// are listed (with their hold flag in bit 31 of the id) and counted per group in s_gc.  Only the
+// keys of all points are read, kCB per thread in flight; each warp queues its few points of the
+// epoch in shared memory and takes them 32 at a time, with full lanes and one round trip for
+// their ids and state bytes.  For a list in global memory their positions are noted in gid2 (the
+// other list, idle until a compaction) for the commit; returned: how many.  (Handled where they
+// were found, unrolled, the phase was 48 KB of code, and fetching it bound the smaller jobs; in
+// a rolled loop, a round trip for every few points bound 2^24 x 64: 38 us an epoch.)
+constexpr int kQueue = 32 * (kCB + 1);        // a warp's queue: less than 32 left over, and a batch
+static_assert(2 * kQueue * kW <= kScrWords, "the warps' queues fit the scratch");
+
+__device__ __noinline__ uint32_t classify_live(const PeelArgs &a, const ListView &L, uint32_t n_live, const float *Ls,
+                                              uint32_t r0, uint32_t K, const GroupTab &tab, uint32_t *s_cc,
+                                              uint32_t *s_gc, uint32_t (*hcnt)[kMaxEpoch], uint32_t *scr)
 {
+    __shared__ uint32_t s_hits;
     PeelCtl *ctl = a.ctl;
     const int d = a.d;
-    const int t = threadIdx.x, lane = t & 31;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t ng = tab.ng, last = tab.out[ng - 1];
     uint8_t *pfl = L.fl();
-    // a key's class: kNone (after the epoch, or past the end of the list), its round r < K
-    // (certainly), or kBandTag | g (in group g's band).  Only the keys of all points are read,
-    // kCB per thread in flight; the few in the epoch then load their state byte and id, write
-    // the class to the state byte and are counted in shared memory (the points of the epoch are
-    // spread over the list, so few lanes of a warp meet on one counter).  Those are handled
-    // one batch index at a time in a rolled loop: unrolled, the phase was 48 KB of code, and
-    // its fetch bound it (2^24 x 64: 41 us an epoch).
+    uint32_t *qk = scr + w * 2 * kQueue, *qp = qk + kQueue;      // the warp's queue: keys, positions
+    if (t == 0) s_hits = 0;
+    __syncthreads();
     constexpr uint32_t kBandTag = 0x100u;
+    uint32_t cnt = 0;
 #pragma unroll 1
-    for (uint32_t q0 = 0; q0 < n_live; q0 += kCB * kThreads) {
+    for (uint32_t q0 = (uint32_t)w * 32; q0 < n_live; q0 += kCB * kThreads) {
         uint32_t kk[kCB];
-        uint32_t in = 0;                           // the batch indexes in the epoch
 #pragma unroll
         for (int u = 0; u < kCB; u++) {
-            const uint32_t qi = q0 + u * kThreads + t;
+            const uint32_t qi = q0 + u * kThreads + lane;
             kk[u] = qi < n_live ? L.key(qi) : kGone;
         }
 #pragma unroll
-        for (int u = 0; u < kCB; u++) in |= (uint32_t)(kk[u] <= s_glast) << u;
-        uint32_t todo = __reduce_or_sync(0xffffffffu, in);
+        for (int u = 0; u < kCB; u++) {
+            const bool in = kk[u] <= last;
+            const uint32_t m = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const uint32_t o = cnt + __popc(m & lt);
+                qk[o] = kk[u];
+                qp[o] = q0 + u * kThreads + lane;
+            }
+            cnt += __popc(m);
+        }
+        __syncwarp();
+        const bool end = q0 + kCB * kThreads >= n_live;           // what is left in the queue, too
 #pragma unroll 1
-        while (todo) {
-            const int u = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            uint32_t k = kk[0];
-#pragma unroll
-            for (int v = 1; v < kCB; v++) k = u == v ? kk[v] : k;
-            const uint32_t qi = q0 + u * kThreads + t;
-            uint32_t cls = kNone, id = 0, fl = 0;
-            if ((in >> u) & 1u) {
+        while (cnt >= 32u || (end && cnt)) {
+            const uint32_t m = min(cnt, 32u);
+            cnt -= m;
+            // a key's class: its round r < K (certainly), kBandTag | g (in group g's band), or
+            // kNone (after the epoch: the point keeps its state byte, kFlNone since the last commit)
+            uint32_t cls = kNone, id = 0, fl = 0, k = 0;
+            if ((uint32_t)lane < m) {
+                k = qk[cnt + lane];
+                const uint32_t qi = qp[cnt + lane];
                 id = L.id(qi);
                 fl = pfl[qi];
                 uint32_t g = 0, cum = 0;
 #pragma unroll 1
-                while (g < ng && k > s_gout[g]) {
-                    cum = s_gq2[g] + 1u;
+                while (g < ng && k > tab.out[g]) {
+                    cum = tab.q2[g] + 1u;
                     g++;
                 }
-                if (g < ng && k >= s_gin[g]) cls = kBandTag | g;
+                if (g < ng && k >= tab.in[g]) cls = kBandTag | g;
                 else if (cum < K) cls = cum;
-                // a point outside the epoch keeps its state byte (kFlNone since the last commit)
                 if (cls != kNone) pfl[qi] = (uint8_t)((fl & kFlHold) | (cls >= kBandTag ? kFlBand : cls));
+            }
+            __syncwarp();
+            if (!L.kc) {
+                const uint32_t hm = __ballot_sync(0xffffffffu, cls != kNone);
+                uint32_t base = 0;
+                if (lane == 0 && hm) base = atomicAdd(&s_hits, (uint32_t)__popc(hm));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (cls != kNone) L.gid2[base + __popc(hm & lt)] = qp[cnt + lane];
             }
             const bool band = cls != kNone && cls >= kBandTag;
             const bool cert = cls < kBandTag;
@@ -1551,6 +1705,8 @@ __device__ __noinline__ void classify_live(const PeelArgs &a, const ListView &L,
             if (__any_sync(0xffffffffu, ch)) count_held(a.x, Ls, d, ch, id, cls, hcnt);
         }
     }
+    __syncthreads();
+    return s_hits;
 }
 
 // Phase E for a list in shared memory (kc), compacted in place: the points whose round
@@ -1666,84 +1822,109 @@ __device__ __noinline__ uint32_t compact_shared(const PeelArgs &a, const ListVie
     return done;
 }
 
-// Phase E for a list in global memory: each warp takes chunks of 32 kQT positions and
-// appends the points it keeps to the other list (their order does not matter: the
-// subclusters are packed by a counting sort over rnd afterwards), claiming slots with one
-// shared atomic per 32 positions; no block barrier inside.  Returns the points left.
-__device__ __noinline__ uint32_t compact_global(const PeelArgs &a, const ListView &L, uint32_t n_live, uint32_t r0,
-                                                uint32_t live_from, bool changed, const DigitMap *dmp, uint32_t *scr)
+// Phase E for a list in global memory.  The epoch's points (n_hit positions noted in gid2 by
+// the classification) are taken out in place: those that leave get kGone for their id and key,
+// which every pass skips; dropped assignments are reset; with the landmark kept, the committed
+// keys leave the first-digit histogram.  Once a quarter of the list is gone, each warp takes
+// chunks of 32 kQT positions and appends what is left to the other list (the order does not
+// matter: the subclusters are packed by a counting sort over rnd afterwards), claiming slots with
+// one shared atomic per chunk.  (Copying the list every epoch moved 18 bytes a point: 44 us an
+// epoch at 2^24 x 64.)  gone: the list's gaps, kept by the caller; returns whether the lists
+// changed places.
+__device__ __noinline__ bool commit_global(const PeelArgs &a, const ListView &L, uint32_t &n_live, uint32_t &gone,
+                                           uint32_t n_hit, uint32_t r0, uint32_t live_from, bool changed,
+                                           const DigitMap *dmp, uint32_t *scr)
 {
     PeelCtl *ctl = a.ctl;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const DigitMap dm = *dmp;
+    uint32_t *gid = const_cast<uint32_t *>(L.gid), *gkp = const_cast<uint32_t *>(L.gkp);
     __shared__ uint32_t s_out;
     if (!changed)
+#pragma unroll 1
         for (int b = t; b < kHistBins; b += kThreads) scr[b] = 0;
+    if (t == 0) s_out = 0;
+    __syncthreads();
+    uint32_t left = 0;
+#pragma unroll 1
+    for (uint32_t h0 = 0; h0 < n_hit; h0 += kQT * kThreads) {
+        uint32_t pos[kQT], ids[kQT], keys[kQT], fls[kQT];
+#pragma unroll
+        for (int q = 0; q < kQT; q++) {
+            const uint32_t h = h0 + q * kThreads + t;
+            pos[q] = h < n_hit ? __ldcg(&L.gid2[h]) : kGone;
+        }
+#pragma unroll
+        for (int q = 0; q < kQT; q++)
+            if (pos[q] != kGone) {
+                ids[q] = __ldcg(&gid[pos[q]]);
+                keys[q] = __ldcg(&gkp[pos[q]]);
+                fls[q] = L.gfl[pos[q]];
+            }
+#pragma unroll
+        for (int q = 0; q < kQT; q++)
+            if (pos[q] != kGone) {
+                const uint32_t st = fls[q] & 0x7Fu;
+                const uint32_t rv = st == kFlBand ? __ldcg(&a.rnd[ids[q]]) : r0 + st;
+                if (rv < live_from) {
+                    gid[pos[q]] = kGone;
+                    gkp[pos[q]] = kGone;
+                    L.gfl[pos[q]] = kFlNone;
+                    left++;
+                    if (!changed) atomicAdd(&scr[dm.bin(keys[q])], 1u);
+                } else {
+                    L.gfl[pos[q]] = (uint8_t)((fls[q] & kFlHold) | kFlNone);
+                    if (rv != kNone) a.rnd[ids[q]] = kNone;              // an assignment dropped
+                }
+            }
+    }
+    left = __reduce_add_sync(0xffffffffu, left);
+    if (lane == 0 && left) atomicAdd(&s_out, left);
+    __syncthreads();
+    if (!changed) {
+        // the next epoch keeps these keys: the committed ones leave the histogram
+#pragma unroll 1
+        for (int b = t; b < kHistBins; b += kThreads)
+            if (scr[b]) atomicSub(&ctl->h0[b], scr[b]);
+    }
+    gone += s_out;
+    if (gone < (n_live + 3u) / 4u) return false;
+    __syncthreads();
     if (t == 0) s_out = 0;
     __syncthreads();
 #pragma unroll 1
     for (uint32_t cb = (uint32_t)w * 32 * kQT; cb < n_live; cb += kW * 32 * kQT) {
-        uint32_t ids[kQT], keys[kQT], fls[kQT];
+        uint32_t ids[kQT], keys[kQT], fls[kQT], tot = 0;
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
             const uint32_t qi = cb + q * 32 + lane;
             const bool v = qi < n_live;
-            ids[q] = v ? L.id(qi) : 0u;
-            keys[q] = v ? __ldcg(&L.gkp[qi]) : kGone;
+            ids[q] = v ? __ldcg(&gid[qi]) : kGone;
+            keys[q] = v ? __ldcg(&gkp[qi]) : kGone;
             fls[q] = v ? L.gfl[qi] : (uint32_t)kFlNone;
         }
-        uint32_t rvs[kQT], tot = 0, kp = 0, dropped = 0, out = 0;
 #pragma unroll
-        for (int q = 0; q < kQT; q++) {
-            const uint32_t st = fls[q] & 0x7Fu;
-            rvs[q] = st == kFlBand ? __ldcg(&a.rnd[ids[q]]) : st == kFlNone ? kNone : r0 + st;
-        }
-#pragma unroll
-        for (int q = 0; q < kQT; q++) {
-            const bool valid = cb + q * 32 + lane < n_live;
-            const bool keep = valid && rvs[q] >= live_from;
-            kp |= (uint32_t)keep << q;
-            out |= (uint32_t)(valid && !keep) << q;
-            dropped |= (uint32_t)(keep && rvs[q] != kNone) << q;
-            tot += __popc(__ballot_sync(0xffffffffu, keep));
-        }
-        // one slot claim per warp and chunk
+        for (int q = 0; q < kQT; q++) tot += __popc(__ballot_sync(0xffffffffu, ids[q] != kGone));
         uint32_t ob = 0;
         if (lane == 0 && tot) ob = atomicAdd(&s_out, tot);
-        // few of them: in rolled loops, which read the entry again
-#pragma unroll 1
-        while (dropped) {                                    // an assignment dropped
-            a.rnd[L.id(cb + (__ffs(dropped) - 1) * 32 + lane)] = kNone;
-            dropped &= dropped - 1u;
-        }
-#pragma unroll 1
-        while (out && !changed) {
-            atomicAdd(&scr[dm.bin(__ldcg(&L.gkp[cb + (__ffs(out) - 1) * 32 + lane]))], 1u);
-            out &= out - 1u;
-        }
         ob = __shfl_sync(0xffffffffu, ob, 0);
 #pragma unroll
         for (int q = 0; q < kQT; q++) {
-            const bool keep = (kp >> q) & 1u;
-            const uint32_t b = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
+            const uint32_t b = __ballot_sync(0xffffffffu, ids[q] != kGone);
+            if (ids[q] != kGone) {
                 const uint32_t o = ob + __popc(b & lt);
                 L.gid2[o] = ids[q];
                 L.gkp2[o] = keys[q];
-                L.gfl2[o] = (uint8_t)((fls[q] & kFlHold) | kFlNone);
+                L.gfl2[o] = (uint8_t)fls[q];
             }
             ob += __popc(b);
         }
     }
     __syncthreads();
-    if (!changed) {
-        // the next epoch keeps these keys: the committed ones leave the histogram
-        __syncthreads();
-        for (int b = t; b < kHistBins; b += kThreads)
-            if (scr[b]) atomicSub(&ctl->h0[b], scr[b]);
-    }
-    return s_out;
+    n_live = s_out;
+    gone = 0;
+    return true;
 }
 
 template <int D>
@@ -1782,7 +1963,8 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
     const unsigned lim = a.spin;
     const uint32_t s0 = (uint32_t)((uint64_t)c * n / G);
     const uint32_t s1 = (uint32_t)((uint64_t)(c + 1) * n / G);
-    uint32_t n_live = s1 - s0;           // points of the slice left
+    uint32_t n_live = s1 - s0;           // its list's length: the points of the slice left
+    uint32_t gone = 0;                   // and (not kc) the gaps among them
     const bool kc = s1 - s0 <= (uint32_t)kKeyCache;   // the list and its keys stay in shared memory
     // slices beyond the key cache alternate between two lists in global memory
     uint32_t *gid = a.lidx + s0, *gid2 = a.lidx + n + s0;
@@ -1840,7 +2022,10 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         __syncthreads();
         if (nl_tot <= N) {                            // the last subcluster: all that is left
 #pragma unroll 1
-            for (uint32_t q = t; q < n_live; q += kThreads) a.rnd[LID(q)] = r0;
+            for (uint32_t q = t; q < n_live; q += kThreads) {
+                const uint32_t id = LID(q);
+                if (id != kGone) a.rnd[id] = r0;
+            }
             if (c == 0 && a.landmarks)
 #pragma unroll 1
                 for (int j = t; j < d; j += kThreads) a.landmarks[(size_t)r0 * d + j] = Ls[j];
@@ -1917,9 +2102,12 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                 }
             }
             __syncthreads();
-            if (s_inc)
-                phase_inc<D>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, chold, s_nj, s_ij,
-                             s_io, s_il);
+            if (s_inc && kc)
+                phase_inc<D, kLoadKc>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, chold, s_nj,
+                                      s_ij, s_io, s_il);
+            else if (s_inc)
+                phase_inc<D, kLoadGlobal>(a.x, a.xt, n, d, n_live, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, chold, s_nj,
+                                          s_ij, s_io, s_il);
             else
                 phase_keys<D>(a.x, Ls, d, n_live, s0, first, kc, sid, gid, skey, gkp, scr, &s_dm, pfl, chold, s_jm);
             __syncthreads();
@@ -2092,8 +2280,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             s_gc[t] = 0;
         }
         __syncthreads();
-        classify_live(a, LV, n_live, Ls, r0, K, ng, s_tab.in, s_tab.out, s_tab.q2, s_tab.out[ng - 1], s_cc, s_gc, hcnt);
-        __syncthreads();
+        const uint32_t n_hit = classify_live(a, LV, n_live, Ls, r0, K, s_tab, s_cc, s_gc, hcnt, scr);
         if (t < (int)K && s_cc[t]) atomicAdd(&ctl->cert[t], s_cc[t]);
         if (t < (int)ng && s_gc[t]) atomicAdd(&ctl->gcnt[t], s_gc[t]);
         if (!grid_sync(ctl, a.flags, gen, lim)) return;
@@ -2158,7 +2345,8 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
 #pragma unroll 1
             for (uint32_t g = c; g < ng; g += G) {
                 const uint32_t q1 = g ? s_tab.q2[g - 1] + 1u : 0u;
-                settle_group(a, Ls, g, q1, s_tab.q2[g], s_off[g], s_off[g + 1] - s_off[g], s_cert[q1], r0, K, hcnt, scr);
+                settle_group(a, Ls, g, q1, s_tab.q2[g], s_off[g], s_off[g + 1] - s_off[g], s_cert[q1], r0, K, hcnt, scr,
+                             kc ? 0u : (uint32_t)kStage);
             }
         }
         // how many rounds the epoch commits: up to the first round after which some attribute
@@ -2180,9 +2368,9 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             ctl->passes += need_keys ? 1u : 0u;
         }
         const uint32_t live_from = r0 + kcm;
-        n_live = kc ? compact_shared(a, LV, n_live, r0, live_from, changed, &s_dm, scr)
-                    : compact_global(a, LV, n_live, r0, live_from, changed, &s_dm, scr);
-        if (!kc) {
+        if (kc) {
+            n_live = compact_shared(a, LV, n_live, r0, live_from, changed, &s_dm, scr);
+        } else if (commit_global(a, LV, n_live, gone, n_hit, r0, live_from, changed, &s_dm, scr)) {
             uint32_t *ti = gid; gid = gid2; gid2 = ti;
             uint32_t *tk = gkp; gkp = gkp2; gkp2 = tk;
             uint8_t *tf = gfl; gfl = gfl2; gfl2 = tf;
@@ -2223,8 +2411,10 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             }
             if (c == 0 && t == 0) ctl->band_cnt = 0;
         }
-        if (changed && n_live)
-            lost_minima(a.x, a.xt, n, d, n_live, kc, sid, gid, s_lost, n_lost, ctl->Lbits[lpar ^ 1]);
+        if (changed && n_live && kc)
+            lost_minima<kLoadKc>(a.x, a.xt, n, d, n_live, kc, sid, gid, s_lost, n_lost, ctl->Lbits[lpar ^ 1]);
+        else if (changed && n_live)
+            lost_minima<kLoadGlobal>(a.x, a.xt, n, d, n_live, kc, sid, gid, s_lost, n_lost, ctl->Lbits[lpar ^ 1]);
         first = false;
         hpar ^= 1;
         if (changed) lpar ^= 1;
