@@ -406,12 +406,18 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
 constexpr int kSetThreads = 1024;
 constexpr size_t kSetSmemMax = 100 * 1024;
 
-// rows per thread: 32 floats of rows at most (MAXT is 1024 only for sets that need as many
-// threads: at 64 registers a thread the wider of them spill)
+// rows per thread: 32 floats of rows at most, or one wider row (MAXT is 1024 only for sets that
+// need as many threads: at 64 registers a thread the wider of them spill)
 template <int D>
 __host__ __device__ constexpr int kSetRows()
 {
-    return 32 / D > 4 ? 4 : 32 / D;
+    return D >= 32 ? 1 : (32 / D > 4 ? 4 : 32 / D);
+}
+
+// the rows of a set that one CTA's registers hold
+inline int set_rows(int D)
+{
+    return D <= 32 ? kSetThreads * (32 / D > 4 ? 4 : 32 / D) : D <= 64 ? 512 : 256;
 }
 
 // [centers k x D | high, low sums k x (d | 1) | reciprocals k (double) | counts k | touched k]
@@ -474,18 +480,24 @@ k_lloyd_sets(const float *__restrict__ pts, SegTable t, int d, float *centers, i
                 atomicSub(&scnt[o], 1);
                 stouch[o] = it + 1;
             }
-#pragma unroll
-            for (int a = 0; a < D; a++) {
-                if (a < d) {
-                    uint32_t hi, lo;
-                    fix_parts(xv[q][a], hi, lo);
-                    atomicAdd(&shi[bj[q] * ds + a], hi);
-                    atomicAdd(&slo[bj[q] * ds + a], lo);
-                    if (o >= 0) {
-                        atomicSub(&shi[o * ds + a], hi);
-                        atomicSub(&slo[o * ds + a], lo);
-                    }
+            auto move = [&](float v, int a) {
+                uint32_t hi, lo;
+                fix_parts(v, hi, lo);
+                atomicAdd(&shi[bj[q] * ds + a], hi);
+                atomicAdd(&slo[bj[q] * ds + a], lo);
+                if (o >= 0) {
+                    atomicSub(&shi[o * ds + a], hi);
+                    atomicSub(&slo[o * ds + a], lo);
                 }
+            };
+            if constexpr (D <= 32) {
+#pragma unroll
+                for (int a = 0; a < D; a++)
+                    if (a < d) move(xv[q][a], a);
+            } else {                            // a wide row read again: unrolled, its sums spill
+                const float *x = pts + (row0 + r) * d;
+#pragma unroll 4
+                for (int a = 0; a < d; a++) move(__ldg(&x[a]), a);
             }
             lab[q] = bj[q];
         }
@@ -940,8 +952,10 @@ cudaError_t sets_dispatch(const LloydBuffers &b, const SegTable &t, int d, int64
     // many as the registers hold (each center read from shared memory serves them all)
     constexpr int R = kSetRows<D>();
     if (max_rows <= 256) return sets_launch<D, 1, 256>(b, t, d, P, max_rows, kmax, iters, st, kt);
-    if (max_rows <= 512 * R) return sets_launch<D, R, 512>(b, t, d, P, max_rows, kmax, iters, st, kt);
-    return sets_launch<D, R, 1024>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    if constexpr (D <= 64)
+        if (max_rows <= 512 * R) return sets_launch<D, R, 512>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    if constexpr (D <= 32) return sets_launch<D, R, 1024>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    return cudaErrorInvalidValue;
 }
 
 // rows_per_thread: 0 = kRowsPerThread<D>(), 1 = one row per thread, 2 = eight rows per
@@ -1002,18 +1016,16 @@ cudaError_t launch_lloyd_init(const LloydBuffers &b, const SegTable &t, int d, i
 // Whether small sets run all their iterations in one launch (k_lloyd_sets) rather than two
 // launches an iteration.  Both score the same distances; per iteration the launches add about
 // 11000 cycles on an idle GPU (2.5-3 us each) where the one launch's barriers add 1500, but a
-// set then has one SM alone: rows k (2 D + 3) instructions at 60 % of 128 lanes.  The launch
-// pays while the largest set's time stays below the whole work spread over the SMs plus the
+// set then has one SM alone: rows k (2 D + 3) instructions at 60 % of 128 lanes (half of that
+// with one wide row per thread, bound by reading the centers).  The launch pays while the largest set's time stays below the whole work spread over the SMs plus the
 // difference.
 bool sets_supported(const SegTable &t, int d, int max_rows, int kmax, double evals, int prec, const LloydBuffers &b,
                     int sm_count)
 {
     const int D = pad_width(d);
-    if (b.weights || D == 0 || D > 32 || max_rows > kSetThreads * (32 / D > 4 ? 4 : 32 / D) ||
-        set_smem(D, d, kmax) > kSetSmemMax)
-        return false;
+    if (b.weights || D == 0 || max_rows > set_rows(D) || set_smem(D, d, kmax) > kSetSmemMax) return false;
     if (prec != PSCL_PREC_FP32 && b.tmask && t.split && tc_supported(d, kmax, prec, b.rows)) return false;
-    const double per = (2.0 * D + 3.0) / (128.0 * 0.6);
+    const double per = (2.0 * D + 3.0) / (128.0 * (D <= 32 ? 0.6 : 0.3));
     return (double)max_rows * kmax * per <= evals * per / sm_count + 9500.0;
 }
 
@@ -1028,6 +1040,10 @@ cudaError_t launch_lloyd_sets(const LloydBuffers &b, const SegTable &t, int d, i
     case 16: return sets_dispatch<16>(b, t, d, P, max_rows, kmax, iters, st, kt);
     case 24: return sets_dispatch<24>(b, t, d, P, max_rows, kmax, iters, st, kt);
     case 32: return sets_dispatch<32>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    case 48: return sets_dispatch<48>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    case 64: return sets_dispatch<64>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    case 96: return sets_dispatch<96>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    case 128: return sets_dispatch<128>(b, t, d, P, max_rows, kmax, iters, st, kt);
     default: return cudaErrorInvalidValue;
     }
 }

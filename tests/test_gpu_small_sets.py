@@ -27,6 +27,8 @@ def _run(raw, N, lk, fk, T, plain):
     (16384, 8, 4096, 12, 4, 5), (16388, 5, 4095, 7, 4, 5),    # the largest sets of 8 attributes
     (8194, 16, 2048, 20, 3, 4), (4099, 12, 1025, 40, 6, 4),   # 2 rows per thread
     (3000, 32, 1000, 33, 5, 4), (3000, 17, 1024, 9, 5, 4),    # one
+    (1024, 64, 512, 5, 3, 4), (770, 33, 257, 8, 3, 4),        # one wide row per thread
+    (500, 128, 250, 4, 2, 4), (600, 100, 200, 6, 2, 4), (400, 65, 190, 9, 2, 4),
     (600, 3, 20, 20, 1, 3),                                   # every row a center: over at once
     (500, 4, 100, 1, 1, 30),                                  # a fixed point after two iterations
     (900, 6, 90, 8, 3, 1), (900, 6, 90, 8, 3, 0),
