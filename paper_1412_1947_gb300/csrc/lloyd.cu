@@ -971,6 +971,24 @@ cudaError_t assign_dispatch(const LloydBuffers &b, const SegTable &t, int d, int
     return assign_launch<D, kRowsPerThread<D>()>(b, t, d, iter, unit_lo, unit_hi, kmax, st, kt);
 }
 
+// An SSE kernel; its blocks as one cluster where no ticket is given (see sse_reduce).
+template <class... P, class... A>
+cudaError_t sse_launch(void (*kern)(P...), int grid, size_t smem, bool cluster, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)grid;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(kThreads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = cluster ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
 template <int D>
 cudaError_t sse_dispatch(const float *x, int64_t n, int d, const float *centers, int k, int32_t *labels,
                          double *blk_sse, double *sse, uint32_t *ticket, int sm_count, cudaStream_t st,
@@ -985,12 +1003,15 @@ cudaError_t sse_dispatch(const float *x, int64_t n, int d, const float *centers,
     auto kern = n > (int64_t)grid * kThreads ? k_final_sse<D, kRowsPerThread<D>()> : k_final_sse<D, 1>;
     if (const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return ea;
     kt->begin(st);
-    kern<<<grid, kThreads, smem, st>>>(x, n, d, centers, k, chunk, labels, blk_sse, sse, ticket);
+    const cudaError_t e = sse_launch(kern, grid, smem, ticket == nullptr, st, x, n, d, centers, k, chunk, labels, blk_sse,
+                                     sse, ticket);
     kt->end(PSCL_K_FINAL_SSE, st);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace
+
+bool small_sse(int64_t n) { return n <= (int64_t)kClusterSse * kThreads; }
 
 int sse_grid(int64_t n, int sm_count)
 {
@@ -1129,10 +1150,10 @@ cudaError_t launch_final_sse(const float *x, int64_t n, int d, const float *cent
         const size_t smem = tile_smem(d);
         if (const cudaError_t ea = cudaFuncSetAttribute(k_final_sse_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return ea;
         kt->begin(st);
-        k_final_sse_tiled<<<std::max(1, sse_grid(n, sm_count)), kThreads, smem, st>>>(x, n, d, centers, k, labels, blk_sse,
-                                                                                      sse, ticket);
+        const cudaError_t e = sse_launch(k_final_sse_tiled, std::max(1, sse_grid(n, sm_count)), smem, ticket == nullptr, st,
+                                         x, n, d, centers, k, labels, blk_sse, sse, ticket);
         kt->end(PSCL_K_FINAL_SSE, st);
-        return cudaGetLastError();
+        return e;
     }
     switch (pad_width(d)) {
     case 2: return sse_dispatch<2>(x, n, d, centers, k, labels, blk_sse, sse, ticket, sm_count, st, kt);

@@ -120,16 +120,21 @@ extern "C" int pscl_assign_sse_noalloc(const float *points, int64_t n, int32_t d
     uint32_t *ticket = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(scratch) +
                                                     kNoAllocMaxBlocks * sizeof(double));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the ticket counts finished blocks and must start at zero, as must the flags (the partials
-    // are overwritten)
-    if (cudaMemsetAsync(ticket, 0, 8 * sizeof(uint32_t), st) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(PSCL_ECUDA, "pscl_assign_sse_noalloc: clearing the scratch failed");
-    }
     KTimer kt;
-    cudaError_t e = flat_sse_supported(points, n, d, centers, k)
-                        ? launch_flat_sse(points, n, d, centers, k, labels, partials, sse, ticket, ticket + 4, sms, st, &kt)
-                        : launch_final_sse(points, n, d, centers, k, labels, partials, sse, ticket, sms, st, &kt);
+    cudaError_t e;
+    if (small_sse(n)) {
+        e = launch_final_sse(points, n, d, centers, k, labels, partials, sse, nullptr, sms, st, &kt);
+    } else {
+        // the ticket counts finished blocks and must start at zero, as must the flags (the partials
+        // are overwritten)
+        if (cudaMemsetAsync(ticket, 0, 8 * sizeof(uint32_t), st) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(PSCL_ECUDA, "pscl_assign_sse_noalloc: clearing the scratch failed");
+        }
+        e = flat_sse_supported(points, n, d, centers, k)
+                ? launch_flat_sse(points, n, d, centers, k, labels, partials, sse, ticket, ticket + 4, sms, st, &kt)
+                : launch_final_sse(points, n, d, centers, k, labels, partials, sse, ticket, sms, st, &kt);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(PSCL_ECUDA, cudaGetErrorString(e));

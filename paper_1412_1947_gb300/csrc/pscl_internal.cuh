@@ -274,6 +274,8 @@ cudaError_t launch_flat_sse(const float *x, int64_t n, int d, const float *cente
 // launches over all units; needs t.split).
 cudaError_t launch_lloyd_assign_tc(const LloydBuffers &b, const SegTable &t, int d, int iter, int kmax, int prec,
                                    uint32_t *flags, int sm_count, cudaStream_t st, KTimer *kt);
+// (without a ticket where small_sse(n): one launch that needs nothing cleared)
+bool small_sse(int64_t n);
 cudaError_t launch_final_sse(const float *x, int64_t n, int d, const float *centers, int k,
                              int32_t *labels, double *blk_sse, double *sse, uint32_t *ticket,
                              int sm_count, cudaStream_t st, KTimer *kt);

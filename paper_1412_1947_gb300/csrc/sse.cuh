@@ -55,9 +55,27 @@ __device__ __forceinline__ double block_tree_sum(double part)
 // The blocks' sums, added by the last block to finish: thread t those of blocks t, t + 256,
 // ... in that order, then the same tree.  (One thread adding 1216 blocks' sums in order was a
 // chain of as many float64 additions, 40-60 us behind every SSE pass.)
+// Without a ticket the blocks (kClusterSse at most) are one cluster and hand their sums to its
+// first through shared memory, in the same order: one launch, where the ticket takes a clearing
+// before it (1000 x 16: 10.2 -> 7.9 us a call).
+constexpr int kClusterSse = 8;
+
 __device__ __forceinline__ void sse_reduce(double part, double *blk_sse, double *sse, uint32_t *ticket)
 {
     const double b = block_tree_sum(part);
+    if (!ticket) {
+        __shared__ double all[kClusterSse];
+        if (threadIdx.x == 0) {
+            uint32_t at = (uint32_t)__cvta_generic_to_shared(&all[blockIdx.x]);
+            asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(at));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(b) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (blockIdx.x != 0) return;
+        const double tot = block_tree_sum(threadIdx.x < gridDim.x ? __dadd_rn(0.0, all[threadIdx.x]) : 0.0);
+        if (threadIdx.x == 0) *sse = tot;
+        return;
+    }
     if (threadIdx.x == 0) blk_sse[blockIdx.x] = b;
     __shared__ bool is_last;
     __threadfence();
