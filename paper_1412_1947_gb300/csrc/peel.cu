@@ -2440,7 +2440,8 @@ __global__ void __launch_bounds__(kThreads) k_barrier_bench(PeelCtl *ctl, uint32
 // ------------------------------------------------------------------ packing by round
 // Stable counting sort of the points by round (8 bits of it per pass): the subclusters,
 // each in ascending point index.  Chunk c of the items is [c m/G, (c+1) m/G).
-constexpr int kPermThreads = 256;
+constexpr int kPermThreads = kThreads;        // 256, a digit's values: block_excl_scan's block
+static_assert(kPermThreads == 256, "a thread per digit value");
 
 __global__ void __launch_bounds__(kPermThreads) k_perm_count(const uint32_t *__restrict__ rnd,
                                                              const uint32_t *__restrict__ src, uint32_t m, int sh,
@@ -2460,41 +2461,29 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_count(const uint32_t *__r
     cnt[(size_t)t * G + c] = h[t];
 }
 
-// Exclusive scan of the 256 x G counts in place (digit-major): one block of 1024 threads,
-// each taking a run of consecutive counts (a multiple of 4, read and written as uint4 with
-// several loads in flight: the scan is a chain of L2 round trips, not a bandwidth cost).
-__global__ void __launch_bounds__(1024) k_perm_scan(uint32_t *cnt, uint32_t total)
+// Inclusive scan of each digit's G counts over the chunks, in place: a block per digit, whose
+// last value is the digit's total (the scatter adds the digits before).  One block for all 256 G
+// was a chain of L2 round trips (2^20 points: 59 us).
+__global__ void __launch_bounds__(kPermThreads) k_perm_scan(uint32_t *cnt, uint32_t G)
 {
-    __shared__ uint32_t ws[32];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const uint32_t per = (((total + 1023u) / 1024u) + 3u) & ~3u;        // total = 256 G, a multiple of 4
-    const uint32_t b = min(total, (uint32_t)t * per), e = min(total, b + per);
-    uint4 *c4 = reinterpret_cast<uint4 *>(cnt);
-    uint32_t s = 0;
-#pragma unroll 8
-    for (uint32_t i = b; i < e; i += 4) {
-        const uint4 v = c4[i / 4];
-        s += v.x + v.y + v.z + v.w;
-    }
-    const uint32_t inc = warp_incl_scan(s);
-    if (lane == 31) ws[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        const uint32_t v = ws[lane];
-        ws[lane] = warp_incl_scan(v) - v;
-    }
-    __syncthreads();
-    uint32_t run = ws[w] + inc - s;
-#pragma unroll 8
-    for (uint32_t i = b; i < e; i += 4) {
-        const uint4 v = c4[i / 4];
-        uint4 o;
-        o.x = run;
-        o.y = run + v.x;
-        o.z = o.y + v.y;
-        o.w = o.z + v.z;
-        run = o.w + v.w;
-        c4[i / 4] = o;
+    uint32_t *c = cnt + (size_t)blockIdx.x * G;
+    uint32_t run = 0;
+    for (uint32_t b = 0; b < G; b += 4 * kPermThreads) {
+        uint32_t v[4], s = 0, tot;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t e = b + 4 * threadIdx.x + q;
+            v[q] = e < G ? c[e] : 0u;
+            s += v[q];
+        }
+        uint32_t at = run + block_excl_scan(s, tot);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t e = b + 4 * threadIdx.x + q;
+            at += v[q];
+            if (e < G) c[e] = at;
+        }
+        run += tot;
     }
 }
 
@@ -2509,7 +2498,11 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(const uint32_t *_
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const uint32_t G = gridDim.x, c = blockIdx.x;
     const uint32_t lt = (1u << lane) - 1u;
-    base[t] = cnt[(size_t)t * G + c];
+    {
+        uint32_t all;
+        const uint32_t before = block_excl_scan(__ldg(&cnt[(size_t)t * G + G - 1]), all);
+        base[t] = before + (c ? __ldg(&cnt[(size_t)t * G + c - 1]) : 0u);
+    }
     const uint32_t lo = (uint32_t)((uint64_t)c * m / G), hi = (uint32_t)((uint64_t)(c + 1) * m / G);
     for (uint32_t i0 = lo; i0 < hi; i0 += kPermThreads) {
         const uint32_t i = i0 + t;
@@ -2640,7 +2633,7 @@ cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int s
         uint32_t *dst = ((passes - 1 - p) & 1) ? b.gpos : b.perm;
         kt->begin(st);
         k_perm_count<<<pg, kPermThreads, 0, st>>>(b.rnd, src, m, 8 * p, b.pcnt);
-        k_perm_scan<<<1, 1024, 0, st>>>(b.pcnt, (uint32_t)(256 * pg));
+        k_perm_scan<<<256, kPermThreads, 0, st>>>(b.pcnt, (uint32_t)pg);
         k_perm_scatter<<<pg, kPermThreads, 0, st>>>(b.rnd, src, m, 8 * p, b.pcnt, dst);
         kt->end(PSCL_K_GATHER, st);
         src = dst;
