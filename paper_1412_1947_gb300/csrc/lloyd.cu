@@ -293,6 +293,7 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
         }
         for (int j = threadIdx.x; j < k; j += kThreads) scnt[j] = 0;
     }
+    chain_wait();
     const bool one_chunk = chunk_k >= k;
     if (one_chunk) load_centers<D>(sc, centers + c0 * d, k, d);
     __syncthreads();
@@ -545,6 +546,7 @@ template <int EPT, typename I>
 __global__ void k_lloyd_finalize(float *centers, unsigned long long *acc, const int32_t *count,
                                  int32_t *count_next, int64_t cen_lo, int64_t cen_hi, int d, bool keep)
 {
+    chain_wait();
     const I g0 = (I)(cen_lo * d / EPT), g1 = (I)(cen_hi * d / EPT), dd = (I)d;
     for (I g = g0 + (I)blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += (I)gridDim.x * blockDim.x) {
         const I e = g * EPT;
@@ -567,7 +569,7 @@ __global__ void k_lloyd_finalize(float *centers, unsigned long long *acc, const 
 }
 
 template <int EPT>
-void finalize_launch(const LloydBuffers &b, int32_t *count_next, int64_t cen_lo, int64_t cen_hi, int d,
+cudaError_t finalize_launch(const LloydBuffers &b, int32_t *count_next, int64_t cen_lo, int64_t cen_hi, int d,
                      int sm_count, bool keep, cudaStream_t st)
 {
     const int64_t work = (cen_hi - cen_lo) * d / EPT;
@@ -575,9 +577,10 @@ void finalize_launch(const LloydBuffers &b, int32_t *count_next, int64_t cen_lo,
     if (g > (int64_t)sm_count * 8) g = (int64_t)sm_count * 8;
     if (g < 1) g = 1;
     if (cen_hi * d < ((int64_t)1 << 31))
-        k_lloyd_finalize<EPT, uint32_t><<<(int)g, 256, 0, st>>>(b.centers, b.acc, b.count, count_next, cen_lo, cen_hi, d, keep);
-    else
-        k_lloyd_finalize<EPT, int64_t><<<(int)g, 256, 0, st>>>(b.centers, b.acc, b.count, count_next, cen_lo, cen_hi, d, keep);
+        return launch_chained(b.chain, k_lloyd_finalize<EPT, uint32_t>, g, 256, 0, st, b.centers, b.acc, b.count, count_next, cen_lo,
+                              cen_hi, d, keep);
+    return launch_chained(b.chain, k_lloyd_finalize<EPT, int64_t>, g, 256, 0, st, b.centers, b.acc, b.count, count_next, cen_lo, cen_hi,
+                          d, keep);
 }
 
 // The nearest of a set's centers to R rows of one thread: float32 direct distances, two centers
@@ -912,22 +915,23 @@ cudaError_t assign_launch(const LloydBuffers &b, const SegTable &t, int d, int i
     const size_t smem = (smem_acc ? acc_bytes : 0) + c_bytes;
     const int grid = unit_hi - unit_lo;
     if (grid <= 0) return cudaSuccess;
+    cudaError_t e;
     if (smem_acc) {
         auto kern = k_lloyd_assign<D, R, true>;
         if (const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return ea;
         kt->begin(st);
-        kern<<<grid, kThreads, smem, st>>>(b.pts, t, d, b.centers, b.acc, b.count, b.labels, b.trace,
-                                           (int64_t)iter * b.rows, unit_lo, chunk, b.weights);
+        e = launch_chained(b.chain, kern, grid, kThreads, smem, st, b.pts, t, d, b.centers, b.acc, b.count, b.labels, b.trace,
+                           (int64_t)iter * b.rows, unit_lo, chunk, b.weights);
         kt->end(PSCL_K_LLOYD_ASSIGN, st);
     } else {
         auto kern = k_lloyd_assign<D, R, false>;
         if (const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return ea;
         kt->begin(st);
-        kern<<<grid, kThreads, smem, st>>>(b.pts, t, d, b.centers, b.acc, b.count, b.labels, b.trace,
-                                           (int64_t)iter * b.rows, unit_lo, chunk, b.weights);
+        e = launch_chained(b.chain, kern, grid, kThreads, smem, st, b.pts, t, d, b.centers, b.acc, b.count, b.labels, b.trace,
+                           (int64_t)iter * b.rows, unit_lo, chunk, b.weights);
         kt->end(PSCL_K_LLOYD_ASSIGN, st);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 template <int D, int R, int MAXT>
@@ -1101,11 +1105,11 @@ cudaError_t launch_lloyd_iter(const LloydBuffers &b, int32_t *count_next, const 
     }
     if (e != cudaSuccess) return e;
     kt->begin(st);
-    if (d % 4 == 0) finalize_launch<4>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
-    else if (d % 2 == 0) finalize_launch<2>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
-    else finalize_launch<1>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
+    if (d % 4 == 0) e = finalize_launch<4>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
+    else if (d % 2 == 0) e = finalize_launch<2>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
+    else e = finalize_launch<1>(b, count_next, cen_lo, cen_hi, d, sm_count, keep, st);
     kt->end(PSCL_K_LLOYD_FINALIZE, st);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_seg_sse(const LloydBuffers &b, const SegTable &t, const int32_t *seg_unit0, int d, int kmax,

@@ -510,6 +510,7 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    chain_wait();
     if (ub >= ue) return;
     // test hook: a wait on a barrier that nothing completes runs out before any copy or
     // MMA is issued, and the CTA leaves through the abort path
@@ -1075,6 +1076,7 @@ __global__ void __launch_bounds__(sum_threads<D>(), D <= 32 ? 2 : 1) k_tc_sums(c
                                                              int32_t *trace, int64_t trace_off,
                                                              unsigned long long *acc, int32_t *count, int kmax)
 {
+    chain_wait();
     constexpr int NT = sum_threads<D>();
     constexpr int DS = D | 1;            // odd stride: lanes adding one attribute of different centers spread over banks
     extern __shared__ uint32_t sm[];
@@ -1207,6 +1209,7 @@ k_tc_delta(const float *__restrict__ pts, const float *__restrict__ centers, Seg
            const int32_t *__restrict__ raw, int32_t *labels, const uint32_t *__restrict__ tmask, int32_t *trace,
            int64_t trace_off, unsigned long long *acc, int32_t *count, int kmax)
 {
+    chain_wait();
     constexpr int NT = delta_threads<D>(), NW = NT / 32, WR = delta_rows<D>(), Q = WR / 32;
     constexpr int DC = D + 4;
     constexpr int RPI = D < 32 ? 32 / D : 1;           // moved rows per atomic instruction
@@ -1509,9 +1512,9 @@ cudaError_t assign_only(const LloydBuffers &b, const SegTable &t, int kmax, uint
     const int ma = std::max(1, std::min(std::min(occ, (int)(512u / (2u * a.ncols))), 4));
     a.split = t.split + t.split_off[ma];
     kt->begin(st);
-    ka<<<ma * sm_count, tc_threads<D>(), smem, st>>>(map, a);
+    e = launch_chained(b.chain, ka, ma * sm_count, tc_threads<D>(), smem, st, map, a);
     kt->end(ktag, st);
-    return cudaGetLastError();
+    return e;
 }
 
 template <int D, int MODE>
@@ -1533,21 +1536,20 @@ cudaError_t tc_dispatch(const LloydBuffers &b, const SegTable &t, int iter, int 
         auto kd = k_tc_delta<D>;
         if ((e = cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sd)) != cudaSuccess) return e;
         kt->begin(st);
-        kd<<<md * sm_count, delta_threads<D>(), sd, st>>>(b.pts, b.centers, t, t.split + t.split_off[md == 4 ? 4 : 0], b.raw,
-                                                          b.labels,
-                                                         b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count,
-                                                         kmax);
+        e = launch_chained(b.chain, kd, md * sm_count, delta_threads<D>(), sd, st, b.pts, b.centers, t,
+                           t.split + t.split_off[md == 4 ? 4 : 0], b.raw, b.labels, b.tmask, b.trace,
+                           (int64_t)iter * b.rows, b.acc, b.count, kmax);
         kt->end(PSCL_K_LLOYD_SUMS, st);
-        return cudaGetLastError();
+        return e;
     }
     const size_t ss = sums_smem<D>(kmax);
     auto ks = k_tc_sums<D>;
     if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss)) != cudaSuccess) return e;
     kt->begin(st);
-    ks<<<m * sm_count, sum_threads<D>(), ss, st>>>(b.pts, b.centers, t, t.split + t.split_off[m], raw, b.labels,
-                                                   b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count, kmax);
+    e = launch_chained(b.chain, ks, m * sm_count, sum_threads<D>(), ss, st, b.pts, b.centers, t, t.split + t.split_off[m], raw,
+                       b.labels, b.tmask, b.trace, (int64_t)iter * b.rows, b.acc, b.count, kmax);
     kt->end(PSCL_K_LLOYD_SUMS, st);
-    return cudaGetLastError();
+    return e;
 }
 
 // A whole-set search on the tensor cores: the k centers in chunks of up to tc_chunk(D), one

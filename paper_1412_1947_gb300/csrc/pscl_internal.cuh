@@ -219,6 +219,7 @@ struct LloydBuffers {
     bool has_chunks = false;
     uint32_t *chunk_scratch = nullptr;
     uint32_t wait_limit = 0;         // polls of the tensor-core kernel's bounded waits (0: default)
+    bool chain = false;              // the iterations' kernels overlap (launch_chained)
     int tc_stall = 0;                // test hook: the tensor-core kernel waits once on a barrier nothing completes
 };
 cudaError_t launch_lloyd_init(const LloydBuffers &b, const SegTable &t, int d, int64_t P,
@@ -242,6 +243,41 @@ cudaError_t launch_lloyd_sets(const LloydBuffers &b, const SegTable &t, int d, i
 cudaError_t launch_seg_sse(const LloydBuffers &b, const SegTable &t, const int32_t *seg_unit0, int d, int kmax,
                            int prec, int32_t *labels, double *unit_sse, double *seg_sse, uint32_t *flags,
                            int sm_count, cudaStream_t st, KTimer *kt);
+
+// Kernels of Lloyd's iterations follow each other a few microseconds long, so that launching and
+// draining took a good part of them: one launched by launch_chained starts while the kernel before
+// it drains, sets its shared memory up and waits in chain_wait() for that kernel's results.  Every
+// thread of such a kernel passes chain_wait() before it touches global memory that a kernel
+// writes and before it returns; the next one is let start only then, so no more than two overlap.
+// (500009 x 32 in 128 sets: 2800 -> 2496 us.)  A graph's kernels follow each other closely as it
+// is, and such edges slow it down (2^20 x 16: 4328 against 4455 us): a capture takes plain ones.  Nor do a
+// server's jobs chain: a kernel's blocks that wait early hold room that another job's could use
+// (the mixed jobs: 93 against 97 ms).
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+cudaError_t launch_chained(bool chain, void (*kern)(P...), int64_t grid, int block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (chain)
+        if (const cudaError_t e = cudaStreamIsCapturing(st, &cap)) return e;
+    c.numAttrs = chain && cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
 
 // lloyd_tc.cu
 bool tc_supported(int d, int kmax, int prec, int64_t rows);
