@@ -1309,59 +1309,97 @@ k_tc_delta(const float *__restrict__ pts, const float *__restrict__ centers, Seg
 }
 
 // ---------------------------------------------------------------- whole-set search: ties, SSE
-// The rows a whole-set search (the SSE pass) could not decide: a warp per row, lane l the
-// centers l, l + 32, ..., with PSCL_PREC_FP32's arithmetic (t = RN(x_a - c_a), acc =
-// RN(t t + acc) in ascending a; the lowest index among equal sums), so the label is the
-// float32 direct winner.
+// centers in shared memory at a time while tie rows are re-scored (48 KB with the rows)
+__host__ __device__ constexpr int tie_chunk(int D) { return D <= 64 ? 128 : 32; }
+
+// The rows a whole-set search (the SSE pass) could not decide, with PSCL_PREC_FP32's arithmetic
+// (t = RN(x_a - c_a), acc = RN(t t + acc) in ascending a; the lowest index among equal sums), so
+// the label is the float32 direct winner.  A warp takes R rows, lane l the centers l, l + 32, ...;
+// both come through shared memory, the centers in chunks for the block, so that a center's
+// 16 bytes serve R rows and a row's 16 bytes 32 centers: four rows take eight shared-memory
+// cycles for eight of arithmetic.  (Each lane reading its own center from L1 took a cycle per
+// lane and load, 16000 for a row of 64 attributes among
+// 1024 centers: 6500 of 65536 rows 364 -> 57 us; 128 attributes 49 -> 16 us.)
+template <int D, int R>
+__device__ __forceinline__ void rescore_list(const float *__restrict__ x, const float *__restrict__ centers, int k,
+                                             int32_t *labels, const uint32_t *ties, uint32_t nt, float4 *sc, float4 *sr)
+{
+    constexpr int D4 = D / 4, DC4 = D4 + 1, CH = tie_chunk(D), W = 256 / 32;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    for (uint32_t q0 = blockIdx.x * (W * R); q0 < nt; q0 += gridDim.x * (W * R)) {
+        __syncthreads();
+        for (int e = tid; e < W * R * D4; e += 256) {
+            const uint32_t q = q0 + (uint32_t)(e / D4);
+            const int64_t row = __ldcg(&ties[1 + (q < nt ? q : q0)]);
+            sr[e] = __ldg(reinterpret_cast<const float4 *>(x + row * D) + e % D4);
+        }
+        float best[R];
+        int bj[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+            best[r] = __int_as_float(0x7f800000);
+            bj[r] = 0x7fffffff;
+        }
+        const float4 *rw = sr + w * R * D4;
+        for (int cb = 0; cb < k; cb += CH) {
+            const int n = min(CH, k - cb);
+            __syncthreads();
+            for (int e = tid; e < n * D4; e += 256)
+                sc[e / D4 * DC4 + e % D4] = __ldg(reinterpret_cast<const float4 *>(centers + (size_t)cb * D) + e);
+            __syncthreads();
+            for (int j0 = 0; j0 < n; j0 += 32) {
+                const int j = j0 + lane;
+                const float4 *c = sc + (j < n ? j : 0) * DC4;
+                float acc[R];
+#pragma unroll
+                for (int r = 0; r < R; r++) acc[r] = 0.0f;
+#pragma unroll 8
+                for (int a = 0; a < D4; a++) {
+                    const float4 u = c[a];
+#pragma unroll
+                    for (int r = 0; r < R; r++) {
+                        const float4 v = rw[r * D4 + a];
+                        float t;
+                        t = __fsub_rn(v.x, u.x); acc[r] = __fmaf_rn(t, t, acc[r]);
+                        t = __fsub_rn(v.y, u.y); acc[r] = __fmaf_rn(t, t, acc[r]);
+                        t = __fsub_rn(v.z, u.z); acc[r] = __fmaf_rn(t, t, acc[r]);
+                        t = __fsub_rn(v.w, u.w); acc[r] = __fmaf_rn(t, t, acc[r]);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; r++)
+                    if (j < n && acc[r] < best[r]) {       // ascending j in the lane
+                        best[r] = acc[r];
+                        bj[r] = cb + j;
+                    }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                const float od = __shfl_xor_sync(0xffffffffu, best[r], o);
+                const int oj = __shfl_xor_sync(0xffffffffu, bj[r], o);
+                if (od < best[r] || (od == best[r] && oj < bj[r])) {
+                    best[r] = od;
+                    bj[r] = oj;
+                }
+            }
+            const uint32_t q = q0 + (uint32_t)(w * R + r);
+            if (lane == 0 && q < nt) labels[__ldcg(&ties[1 + q])] = (uint32_t)bj[r] < (uint32_t)k ? bj[r] : 0;
+        }
+    }
+}
+
 template <int D>
 __global__ void __launch_bounds__(256) k_tc_rescore_ties(const float *__restrict__ x, const float *__restrict__ centers,
                                                          int k, int32_t *labels, const uint32_t *ties)
 {
+    __shared__ float4 sc[tie_chunk(D) * (D / 4 + 1)], sr[32 * (D / 4)];
     const uint32_t nt = __ldcg(&ties[0]);
-    const int lane = threadIdx.x & 31;
-    const uint32_t nw = gridDim.x * (blockDim.x / 32);
-    for (uint32_t q = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; q < nt; q += nw) {
-        const int64_t row = __ldcg(&ties[1 + q]);
-        float xr[D];
-        const float4 *x4 = reinterpret_cast<const float4 *>(x + row * D);
-#pragma unroll
-        for (int a4 = 0; a4 < D / 4; a4++) {
-            const float4 v = __ldg(&x4[a4]);               // the same address in every lane
-            xr[4 * a4 + 0] = v.x;
-            xr[4 * a4 + 1] = v.y;
-            xr[4 * a4 + 2] = v.z;
-            xr[4 * a4 + 3] = v.w;
-        }
-        float bd = __int_as_float(0x7f800000);
-        int bj = 0x7fffffff;
-        for (int j = lane; j < k; j += 32) {
-            const float4 *c4 = reinterpret_cast<const float4 *>(centers + (size_t)j * D);
-            float acc = 0.0f;
-#pragma unroll
-            for (int a4 = 0; a4 < D / 4; a4++) {
-                const float4 u = __ldg(&c4[a4]);
-                float t;
-                t = __fsub_rn(xr[4 * a4 + 0], u.x); acc = __fmaf_rn(t, t, acc);
-                t = __fsub_rn(xr[4 * a4 + 1], u.y); acc = __fmaf_rn(t, t, acc);
-                t = __fsub_rn(xr[4 * a4 + 2], u.z); acc = __fmaf_rn(t, t, acc);
-                t = __fsub_rn(xr[4 * a4 + 3], u.w); acc = __fmaf_rn(t, t, acc);
-            }
-            if (acc < bd) {                                // ascending j in the lane
-                bd = acc;
-                bj = j;
-            }
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            const float od = __shfl_xor_sync(0xffffffffu, bd, o);
-            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-            if (od < bd || (od == bd && oj < bj)) {
-                bd = od;
-                bj = oj;
-            }
-        }
-        if (lane == 0) labels[row] = (uint32_t)bj < (uint32_t)k ? bj : 0;
-    }
+    // few rows: one a warp, so that they spread over the SMs
+    if (nt <= 2 * gridDim.x) rescore_list<D, 1>(x, centers, k, labels, ties, nt, sc, sr);
+    else rescore_list<D, 4>(x, centers, k, labels, ties, nt, sc, sr);
 }
 
 // The SSE from the labels: each point's float32 direct distance to its center, added in
