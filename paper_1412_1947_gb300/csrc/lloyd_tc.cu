@@ -1406,7 +1406,8 @@ __global__ void __launch_bounds__(256) k_tc_rescore_ties(const float *__restrict
 // double per thread and in the fixed tree -- the rows of a thread and the order of the float32
 // SSE pass (same grid, 256 threads), so the value is the same bit for bit.  A block's 256 rows
 // come in whole through shared memory (a thread reading its own row attribute by attribute
-// touched 32 sectors an instruction: 0.62 of 6.8 TB/s at 2^24 x 64).
+// touched 32 sectors an instruction: 0.62 of 6.8 TB/s at 2^24 x 64), as differences from the
+// rows' centers: a thread reading its own center then bound it (2^24 x 64: 2.72 -> 1.49 ms).
 template <int D>
 __global__ void __launch_bounds__(kSseThreads) k_sse_from_labels(const float *__restrict__ x, int64_t n,
                                                                  const float *__restrict__ centers, int k,
@@ -1414,30 +1415,34 @@ __global__ void __launch_bounds__(kSseThreads) k_sse_from_labels(const float *__
                                                                  double *sse, uint32_t *ticket)
 {
     extern __shared__ __align__(16) float4 xs[];
+    __shared__ int32_t sl[kSseThreads];
     constexpr int LD4 = tile_ld4(D);
     double part = 0.0;
     const int64_t stride = (int64_t)gridDim.x * kSseThreads;
     for (int64_t i0 = (int64_t)blockIdx.x * kSseThreads; i0 < n; i0 += stride) {
         const int rows = (int)min((int64_t)kSseThreads, n - i0);
-        __syncthreads();
-        tile_load(xs, x + i0 * D, rows, rows, D, LD4);
         int32_t l = (int)threadIdx.x < rows ? labels[i0 + threadIdx.x] : 0;
         if ((uint32_t)l >= (uint32_t)k) l = 0;              // only after a search that gave up
-        const float4 *cr = reinterpret_cast<const float4 *>(centers + (size_t)l * D);
+        sl[threadIdx.x] = l;
+        __syncthreads();
+        // the differences, a row and its center both read whole by neighbouring lanes
+        const float4 *x4 = reinterpret_cast<const float4 *>(x + i0 * D), *c4 = reinterpret_cast<const float4 *>(centers);
+#pragma unroll 8
+        for (int e = threadIdx.x; e < rows * (D / 4); e += kSseThreads) {
+            const int r = e / (D / 4), q = e % (D / 4);
+            const float4 v = __ldg(&x4[e]), c = __ldg(&c4[(size_t)sl[r] * (D / 4) + q]);
+            xs[r * LD4 + q] = make_float4(__fsub_rn(v.x, c.x), __fsub_rn(v.y, c.y), __fsub_rn(v.z, c.z), __fsub_rn(v.w, c.w));
+        }
         __syncthreads();
         if ((int)threadIdx.x < rows) {
             float acc = 0.0f;
 #pragma unroll 8
             for (int q = 0; q < D / 4; q++) {
-                const float4 v = xs[threadIdx.x * LD4 + q], c = __ldg(&cr[q]);
-                float t = __fsub_rn(v.x, c.x);
-                acc = __fmaf_rn(t, t, acc);
-                t = __fsub_rn(v.y, c.y);
-                acc = __fmaf_rn(t, t, acc);
-                t = __fsub_rn(v.z, c.z);
-                acc = __fmaf_rn(t, t, acc);
-                t = __fsub_rn(v.w, c.w);
-                acc = __fmaf_rn(t, t, acc);
+                const float4 t = xs[threadIdx.x * LD4 + q];
+                acc = __fmaf_rn(t.x, t.x, acc);
+                acc = __fmaf_rn(t.y, t.y, acc);
+                acc = __fmaf_rn(t.z, t.z, acc);
+                acc = __fmaf_rn(t.w, t.w, acc);
             }
             part = __dadd_rn(part, (double)acc);
         }
