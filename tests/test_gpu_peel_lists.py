@@ -21,6 +21,8 @@ pytestmark = pytest.mark.gpu
     ("mixture", 70000, 4, 69999, 16), ("mixture", 90000, 64, 45, 16),
     ("levels", 4000, 2, 500, 304), ("levels", 6000, 3, 1500, 304),       # groups of 65 entries and more
     ("levels", 9000, 12, 2000, 304), ("equal", 1400, 2, 70, 304),
+    ("mixture", 30000, 20, 700, 304), ("mixture", 30001, 12, 900, 304),  # copies by attribute: odd tiles
+    ("chain", 9001, 48, 400, 304),
 ])
 def test_partition_equals_the_oracle(kind, n, d, N, cap):
     with B.Job(_points(kind, n, d, 5500 + n + d)) as job:
