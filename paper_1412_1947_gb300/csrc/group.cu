@@ -77,7 +77,8 @@ __global__ void __launch_bounds__(256) k_group(const float *__restrict__ x, int6
     // [counts m | c, v: d each | the landmarks, d | 1 floats apart (table): lanes read several]
     extern __shared__ uint32_t hist[];
     __shared__ float s_vv[8], s_mm[8], s_scale;
-    __shared__ int s_w;
+    __shared__ int s_w, s_close;
+    __shared__ uint16_t s_list[kTile];
     const int dd = D > 0 ? D : d, t = threadIdx.x, ds = dd | 1;
     float *sc = reinterpret_cast<float *>(hist + m), *sv = sc + dd, *sl = sv + dd;
     for (int g = t; g < m; g += blockDim.x) hist[g] = 0;
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(256) k_group(const float *__restrict__ x, int6
             w = 1;
             while (w < m && !((float)(w + 1) * ((float)w - q2) >= need)) w++;
         }
+        s_close = 0;
         s_w = w;
         s_scale = (float)(m - 1) / vv;
     }
@@ -125,9 +127,10 @@ __global__ void __launch_bounds__(256) k_group(const float *__restrict__ x, int6
     const float scale = s_scale;
     const float eps = (float)(d + 4) * 0x1p-23f;
     const int64_t i0 = (int64_t)blockIdx.x * kTile;
-    for (int q = t; q < kTile; q += blockDim.x) {
+    // point q of the tile; one whose best two the float32 bound cannot separate is put off
+    // (exact: decided)
+    auto place = [&](int q, bool exact) {
         const int64_t i = i0 + q;
-        if (i >= n) break;
         const float *xi = x + i * dd;
         float xv[D > 0 ? D : 1];
         if constexpr (D > 0 && D % 4 == 0) {
@@ -170,6 +173,10 @@ __global__ void __launch_bounds__(256) k_group(const float *__restrict__ x, int6
         // for those
         const float top = __fadd_ru(__fmul_ru(best, 1.0f + eps), 0x1p-120f);
         if (__fsub_rd(__fmul_rd(next, 1.0f - eps), 0x1p-120f) <= top) {
+            if (!exact) {
+                s_list[atomicAdd(&s_close, 1)] = (uint16_t)q;
+                return;
+            }
             double b64 = 0.0;
             int b = -1;
             for (int j = lo; j <= hi; j++) {
@@ -182,7 +189,13 @@ __global__ void __launch_bounds__(256) k_group(const float *__restrict__ x, int6
         }
         group[i] = bj;
         atomicAdd(&hist[bj], 1u);
-    }
+    };
+    const int rows = (int)min((int64_t)kTile, n - i0);
+    for (int q = t; q < rows; q += blockDim.x) place(q, false);
+    // those put off, side by side: found one at a time, the few of a tile took a float64 pass of
+    // most of its warps (500009 x 32, m = 128: 106 -> 53 us)
+    __syncthreads();
+    for (int q = t; q < s_close; q += blockDim.x) place(s_list[q], true);
     __syncthreads();
     for (int g = t; g < m; g += blockDim.x) cnt[(size_t)g * ntiles + blockIdx.x] = hist[g];
 }
