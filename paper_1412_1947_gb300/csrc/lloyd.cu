@@ -315,7 +315,10 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
             best[q] = __int_as_float(0x7f800000);
             bj[q] = 0;
         }
-        for (int cb = 0; cb < k; cb += chunk_k) {
+        // (a warp without a row left scores none: half of the warps of a unit of 128 rows; 25000 x 2,
+        // k = 500: 14.5 -> 11.6 us an iteration)
+        const int kw = one_chunk && p0 + (threadIdx.x & ~31) >= rows ? 0 : k;
+        for (int cb = 0; cb < kw; cb += chunk_k) {
             const int ce = min(k, cb + chunk_k);
             if (!one_chunk) {
                 __syncthreads();
