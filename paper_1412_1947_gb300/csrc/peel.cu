@@ -17,9 +17,8 @@
 // and the next epoch starts from the new landmark (a new pass of distances) or, when all
 // K rounds committed, from the same one (no pass at all).  K itself is read off the keys:
 // the holders' largest key per attribute bounds the round in which the landmark changes,
-// so an epoch resolves only the boundaries up to there (see resolve_cutoffs).  On the
-// headline workload (2^20 points, 16 attributes, 256 rounds) the landmark changes in 50
-// rounds, and the peel runs 50 epochs.
+// so an epoch resolves only the boundaries up to there (phase B).  On 2^20 points of 16
+// attributes in 256 rounds the landmark changes in 50 rounds or so, one epoch each.
 //
 // Each pass works in float32 and keeps exact arithmetic for thin bands around the
 // boundaries:
@@ -38,7 +37,12 @@
 //      form one group);
 //   D. each group is settled by one CTA: compensated float32 distances of its entries
 //      (within eps_ff of delta64) order all but the entries within that error of a cut,
-//      and those (in practice exact ties) are ranked by float64 and index.
+//      and those (in practice exact ties) are ranked by float64 and index;
+//   E. every CTA finds how many rounds the epoch commits from the grid's counts and takes
+//      their points out of its list.
+// A phase runs for a few microseconds once an epoch, so its code comes from beyond the
+// instruction cache every time: rare work sits in rolled loops or out of line, and loops are
+// unrolled only as far as their loads need (390 -> 240 KB in all; a fifth off an epoch).
 // The partition is therefore exactly the float64 definition's, whatever float32 does.
 //
 // Most landmark changes move one or two attributes (the others keep a holder).  The pass
@@ -57,7 +61,8 @@
 // are large and ea stays a small share of the bands' width).
 //
 // Points never move: CTA c owns the index slice [c n/G, (c+1) n/G) and keeps the ids of its
-// points left in a list, in ascending order, with their keys by list position.  Every
+// points left in a list with their keys by list position: in shared memory while the slice
+// fits (ascending), else in global memory, with gaps until a quarter of it is gone.  Every
 // point gets its round in rnd[]; after the launch a stable counting sort by round packs
 // the subclusters (ascending index inside each).  The next landmark differs from the last
 // one only in the attributes that lost their last holder (the commit knows them), usually
@@ -1415,7 +1420,8 @@ struct GroupTab {
 // After phase B: each boundary's first-digit bin and rank inside it become its band cut-offs
 // (second digit from the boundary's histogram), and boundaries whose bands overlap merge into
 // groups (tab, in shared memory).  Every CTA does this for itself when the boundaries are
-// few; otherwise the last CTA to arrive does it for all.  Warp w resolves boundaries w, w + kW, ...: lane i holds
+// few; otherwise the last CTA to arrive does it for all.  Warp w resolves boundaries w, w + kW,
+// ...: lane i holds
 // second-digit bins [64 i, 64 i + 64), a warp scan finds the lane holding the rank, and that
 // lane counts its bins before it.
 __device__ __noinline__ void resolve_cutoffs(PeelCtl *ctl, uint32_t K, float keps, float kabs, const DigitMap *dm,
@@ -2411,7 +2417,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
         if (!grid_sync(ctl, a.flags, gen, lim)) return;
         commit_count(a, K, s_tab, chold, ctl->chold[hpar ^ 1], hcnt, s_kcm, s_nl, s_klast, s_lost);
 
-        // ---- E: commit: the epoch's first k_commit rounds leave the lists; the other
+        // ---- E: commit: the epoch's first kcm rounds leave the lists; the other
         // assignments are dropped; the next landmark if it changes
         const uint32_t n_lost = s_nl;
         uint32_t kcm = s_kcm;
