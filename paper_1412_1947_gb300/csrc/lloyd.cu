@@ -406,7 +406,7 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
 // touched are formed again, and an iteration in which no row moved ends the set: its centers
 // are a fixed point, so every later iteration would repeat it.  Lloyd of 16 sets of 256 x 4
 // (k = 16, 20 iterations) 124 + 115 us of launches back to back -> 17 us; 300 sets of 40-600
-// rows x 5 222 -> 48 us; 250 sets of 1000 x 2 (k = 100) 640 -> 225 us.
+// rows x 5 222 -> 42 us; 250 sets of 1000 x 2 (k = 100) 640 -> 177 us.
 constexpr int kSetThreads = 1024;
 constexpr size_t kSetSmemMax = 100 * 1024;
 
@@ -955,12 +955,17 @@ template <int D>
 cudaError_t sets_dispatch(const LloydBuffers &b, const SegTable &t, int d, int64_t P, int max_rows, int kmax,
                           int iters, cudaStream_t st, KTimer *kt)
 {
-    // one row per thread for sets of up to 256 rows (more warps hide more latency), else as
-    // many as the registers hold (each center read from shared memory serves them all)
+    // one row per thread for sets of up to 256 rows (more warps hide more latency), two of up to 8
+    // attributes for sets of up to 2048 (300 sets of 40-600 rows x 5: the whole batch 126 -> 123
+    // us), else as many as the registers hold (each center read from shared memory serves them all)
     constexpr int R = kSetRows<D>();
     if (max_rows <= 256) return sets_launch<D, 1, 256>(b, t, d, P, max_rows, kmax, iters, st, kt);
-    if constexpr (D <= 64)
+    if constexpr (R >= 4) {
+        if (max_rows <= 1024) return sets_launch<D, 2, 512>(b, t, d, P, max_rows, kmax, iters, st, kt);
+        if (max_rows <= 2048) return sets_launch<D, 2, 1024>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    } else if constexpr (D <= 64) {
         if (max_rows <= 512 * R) return sets_launch<D, R, 512>(b, t, d, P, max_rows, kmax, iters, st, kt);
+    }
     if constexpr (D <= 32) return sets_launch<D, R, 1024>(b, t, d, P, max_rows, kmax, iters, st, kt);
     return cudaErrorInvalidValue;
 }

@@ -27,6 +27,7 @@ def _run(raw, N, lk, fk, T, plain):
     (16384, 8, 4096, 12, 4, 5), (16388, 5, 4095, 7, 4, 5),    # the largest sets of 8 attributes
     (8194, 16, 2048, 20, 3, 4), (4099, 12, 1025, 40, 6, 4),   # 2 rows per thread
     (3000, 32, 1000, 33, 5, 4), (3000, 17, 1024, 9, 5, 4),    # one
+    (4096, 8, 2048, 6, 3, 5), (3075, 4, 1025, 12, 3, 5), (4100, 2, 2050, 9, 3, 5),  # two rows, four
     (1024, 64, 512, 5, 3, 4), (770, 33, 257, 8, 3, 4),        # one wide row per thread
     (500, 128, 250, 4, 2, 4), (600, 100, 200, 6, 2, 4), (400, 65, 190, 9, 2, 4),
     (600, 3, 20, 20, 1, 3),                                   # every row a center: over at once
