@@ -858,7 +858,7 @@ static int run_lloyd(pscl_job *j, const LloydPlan &p, const float *pts, float *c
     }
     b.wait_limit = j->wait_limit;
     b.tc_stall = j->test_stall == 2;
-    b.chain = !j->coop;              // not a server's job
+    b.chain = !j->coop && j->ctx->own_stream;     // not a server's job, nor a caller's stream
     CU(launch_lloyd_init(b, t, j->d, p.P, seed, stage, j->first_k, p.kmax, st, &j->kt));
     if (!plain && !j->rpt && sets_supported(t, j->d, p.max_seg, p.kmax, p.evals, prec, b, j->ctx->sm_count)) {
         CU(launch_lloyd_sets(b, t, j->d, p.P, p.max_seg, p.kmax, iters, st, &j->kt));

@@ -252,7 +252,8 @@ cudaError_t launch_seg_sse(const LloydBuffers &b, const SegTable &t, const int32
 // (500009 x 32 in 128 sets: 2800 -> 2496 us.)  A graph's kernels follow each other closely as it
 // is, and such edges slow it down (2^20 x 16: 4328 against 4455 us): a capture takes plain ones.  Nor do a
 // server's jobs chain: a kernel's blocks that wait early hold room that another job's could use
-// (the mixed jobs: 93 against 97 ms).
+// (the mixed jobs: 93 against 97 ms).  A caller's stream, which may be of any kind, takes plain
+// launches too.
 __device__ __forceinline__ void chain_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
