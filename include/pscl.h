@@ -288,6 +288,12 @@ int pscl_measure_fp32_fma(int device, double *tflops);
  * PSCL_EINVAL if us is NULL, PSCL_ECUDA on a CUDA error, PSCL_ETIMEOUT if a wait gave up. */
 int pscl_measure_grid_barrier(int device, double *us);
 
+/* Beside the method as well: how many CTAs of the peel's kernel for d attributes one SM of
+ * `device` holds (an occupancy query, nothing is launched).  The peel's CTAs wait on one
+ * another, so peels that run side by side must all be resident (see pscl_server_peel_grid).
+ * PSCL_EINVAL if ctas is NULL or d outside 1..1024, PSCL_ECUDA on a CUDA error. */
+int pscl_peel_ctas_per_sm(int device, int32_t d, int32_t *ctas);
+
 /* Nearest center and sum of squared errors of n points, allocating nothing.
  *
  * The paper has no counterpart: this is a service for callers that cannot allocate
@@ -367,6 +373,11 @@ int pscl_fetch(pscl_server *s, uint64_t ticket, float *centers, int32_t *labels,
 /* out[8]: completed, failed, queued, running, bytes in use, peak bytes in use, most jobs
  * running at once, budget. */
 int pscl_server_stats(pscl_server *s, int64_t *out);
+/* The grid of a job's peel that shares the device with other jobs' peels of this server, and how
+ * many of them run at the same time: *ctas * *side_by_side CTAs of any mix of d fit the SMs
+ * (pscl_peel_ctas_per_sm), so each peel is resident as a whole.  (0, 1): every peel runs alone.
+ * Peels of other servers and of jobs run directly are not counted. */
+int pscl_server_peel_grid(pscl_server *s, int32_t *ctas, int32_t *side_by_side);
 /* Fails the queued jobs, waits for the running ones, releases everything. */
 int pscl_server_destroy(pscl_server *s);
 

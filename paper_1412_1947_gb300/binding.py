@@ -53,6 +53,7 @@ SIGNATURES = {
     "pscl_get_recheck_stats": (_I, [_P, _P, _P]),
     "pscl_get_peel_stats": (_I, [_P, _P, _P, _P, _P]),
     "pscl_measure_grid_barrier": (_I, [_I, _P]),
+    "pscl_peel_ctas_per_sm": (_I, [_I, _I32, _P]),
     "pscl_measure_fp32_fma": (_I, [_I, _P]),
     "pscl_assign_sse_noalloc": (_I, [_P, _I64, _I32, _P, _I32, _P, _P, _P]),
     "pscl_job_footprint": (_I, [_P, _I64, _I32, _I64, _I32, _I32, _I32, _I, _I, _I, _P]),
@@ -62,6 +63,7 @@ SIGNATURES = {
     "pscl_wait": (_I, [_P, _U64, _I64]),
     "pscl_fetch": (_I, [_P, _U64, _P, _P, _P, _P]),
     "pscl_server_stats": (_I, [_P, _P]),
+    "pscl_server_peel_grid": (_I, [_P, _P, _P]),
     "pscl_server_destroy": (_I, [_P]),
     "pscl_batch_create": (_I, [_P, _P, _I, _I32, _I32, _P, _P, _P]),
     "pscl_batch_load": (_I, [_P, _P, _I]),
@@ -284,6 +286,13 @@ def pscl_measure_grid_barrier(device=0):
     return t.value
 
 
+def pscl_peel_ctas_per_sm(d, device=0):
+    """CTAs of the peel's kernel for d attributes that an SM holds."""
+    c = C.c_int32()
+    _chk(lib().pscl_peel_ctas_per_sm(device, d, C.byref(c)))
+    return c.value
+
+
 def pscl_get_kernel_times(job):
     """{kernel name: (launches, total ms)} of the last run."""
     n = np.empty(len(KERNELS), np.int64)
@@ -347,6 +356,13 @@ def pscl_server_stats(server):
     _chk(lib().pscl_server_stats(server, _ptr(out)))
     keys = ["completed", "failed", "queued", "running", "bytes_in_use", "peak_bytes", "max_running", "budget"]
     return dict(zip(keys, (int(v) for v in out)))
+
+
+def pscl_server_peel_grid(server):
+    """(CTAs of a peel that shares the device, how many of them run side by side)."""
+    c, k = C.c_int32(), C.c_int32()
+    _chk(lib().pscl_server_peel_grid(server, C.byref(c), C.byref(k)))
+    return c.value, k.value
 
 
 def pscl_server_destroy(server):

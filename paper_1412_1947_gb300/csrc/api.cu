@@ -1266,6 +1266,17 @@ extern "C" int pscl_measure_grid_barrier(int device, double *us)
     return PSCL_OK;
 }
 
+extern "C" int pscl_peel_ctas_per_sm(int device, int32_t d, int32_t *ctas)
+{
+    if (!ctas) return fail(PSCL_EINVAL, "ctas is NULL");
+    if (d < 1 || d > kMaxD) return fail(PSCL_EINVAL, "d=%d outside 1..%d", d, kMaxD);
+    CU(cudaSetDevice(device));
+    int v = 0;
+    CU(peel_ctas_per_sm(d, &v));
+    *ctas = v;
+    return PSCL_OK;
+}
+
 extern "C" int pscl_get_phase_ms(pscl_job *j, float *ms)
 {
     TRY(pscl_job_sync(j));

@@ -1990,6 +1990,10 @@ __device__ __noinline__ bool commit_global(const PeelArgs &a, const ListView &L,
     return true;
 }
 
+// (No bound on the CTAs per SM: k_peel<128> takes 255 registers, so an SM holds one, the others
+// 128 and two.  Bounded to 128 it spills no more than they do and yet loses 8 us an epoch: 300000 x
+// 128 2.85 -> 3.36 ms.  Whoever runs peels side by side sizes their grids by
+// peel_least_ctas_per_sm.)
 template <int D>
 __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
 {
@@ -2615,6 +2619,16 @@ __global__ void k_gather_rows(const float *__restrict__ x, const uint32_t *__res
     }
 }
 
+// k_peel<D>'s CTAs per SM, its shared memory allowed.
+template <int D>
+cudaError_t peel_occupancy(int *per_sm)
+{
+    const size_t smem = kPeelDynWords * sizeof(uint32_t);
+    const cudaError_t e = cudaFuncSetAttribute(k_peel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_peel<D>, kThreads, smem);
+}
+
 template <int D>
 cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int sm_count,
                         cudaStream_t st, KTimer *kt)
@@ -2625,10 +2639,8 @@ cudaError_t peel_launch(const PeelBuffers &b, int64_t n, int d, int64_t N, int s
     cudaError_t e = cudaMemsetAsync(b.ctl, 0, offsetof(PeelCtl, h0), st);
     if (e != cudaSuccess) return e;
     const size_t smem = kPeelDynWords * sizeof(uint32_t);
-    e = cudaFuncSetAttribute(k_peel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel<D>, kThreads, smem);
+    e = peel_occupancy<D>(&per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int64_t grid = (int64_t)sm_count * std::min(per_sm, 4);
@@ -2730,10 +2742,8 @@ cudaError_t measure_grid_barrier(int sm_count, double *us, bool *timed_out)
     cudaError_t e = cudaFuncSetAttribute(k_barrier_bench, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // the peel's grid at full size: its CTAs per SM (capped at 4), as peel_launch sizes it
-    e = cudaFuncSetAttribute(k_peel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel<16>, kThreads, smem);
+    e = peel_occupancy<16>(&per_sm);
     if (e != cudaSuccess) return e;
     int bench_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bench_sm, k_barrier_bench, kThreads, smem);
@@ -2784,6 +2794,32 @@ int perm_grid(int64_t n, int sm_count)
     int64_t g = (n + 2047) / 2048;
     if (g > (int64_t)sm_count * 4) g = (int64_t)sm_count * 4;
     return (int)std::max<int64_t>(1, g);
+}
+
+cudaError_t peel_ctas_per_sm(int d, int *per_sm)
+{
+    switch (d) {
+    case 2: return peel_occupancy<2>(per_sm);
+    case 4: return peel_occupancy<4>(per_sm);
+    case 8: return peel_occupancy<8>(per_sm);
+    case 16: return peel_occupancy<16>(per_sm);
+    case 32: return peel_occupancy<32>(per_sm);
+    case 64: return peel_occupancy<64>(per_sm);
+    case 128: return peel_occupancy<128>(per_sm);
+    default: return peel_occupancy<0>(per_sm);
+    }
+}
+
+cudaError_t peel_least_ctas_per_sm(int *per_sm)
+{
+    int least = 0;
+    for (int d : {0, 2, 4, 8, 16, 32, 64, 128}) {           // launch_peel's widths
+        int v = 0;
+        if (const cudaError_t e = peel_ctas_per_sm(d, &v)) return e;
+        least = d == 0 ? v : std::min(least, v);
+    }
+    *per_sm = least;
+    return cudaSuccess;
 }
 
 cudaError_t launch_peel(const PeelBuffers &b, int64_t n, int d, int64_t N, int sm_count,

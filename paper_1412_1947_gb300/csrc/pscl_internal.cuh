@@ -168,6 +168,10 @@ struct PeelBuffers {
 // Time per grid-wide barrier of the peel's own implementation, in the peel's launch shape
 // (pscl_measure_grid_barrier).
 cudaError_t measure_grid_barrier(int sm_count, double *us, bool *timed_out);
+// CTAs of d attributes' peel kernel that an SM holds, and the fewest over all of its widths: a CTA
+// of any width takes at most that share of an SM, so as many of them fit it together.
+cudaError_t peel_ctas_per_sm(int d, int *per_sm);
+cudaError_t peel_least_ctas_per_sm(int *per_sm);
 // CTAs of the counting sort that packs the subclusters after the peel (pcnt: 256 x this).
 int perm_grid(int64_t n, int sm_count);
 // Rows of x in the order of perm, packed into xseg (the gather after any subclustering).

@@ -9,10 +9,13 @@
 // whole pipeline (scale, peel, local and final Lloyd, SSE) is queued on its slot's stream
 // at once, so the kernels of different jobs overlap on the device.  A peel is a cooperative
 // launch whose CTAs mostly wait on its grid barriers, so up to four run side by side, on
-// streams of their own with a grid of half an SM count each: together they fit the two CTAs
-// that an SM holds, so whatever order the CTAs are placed in every grid becomes resident.
-// Peels of more than kSharedPeelRows points take the whole grid and run alone.  Device memory is stream-ordered, so a finishing
-// job frees its memory without stalling the others.  When a job's last kernel has run,
+// streams of their own with a grid of a quarter of the CTAs that the SMs hold whatever the widths
+// (peel_least_ctas_per_sm).  Together they fit, so in whatever order the CTAs are placed every
+// grid becomes resident; a grid that waits at its barriers for a CTA without a place beside
+// another's would run out of its bounded waits and fail a good job.
+// Peels of more than kSharedPeelRows points take the whole grid and run alone.  Device memory is
+// stream-ordered, so a finishing job frees its memory without stalling the others.  When a job's
+// last kernel has run,
 // its results are copied to host memory, its device memory is released and its latency
 // (submission to completion, host clock) is recorded.
 #include <algorithm>
@@ -55,8 +58,9 @@ struct Ticket {
 
 // Peels side by side, and the largest that share the device (the serving mix of 20 jobs of
 // 10^4 .. 10^6 points, four slots: one stream 120 ms; two of 152 CTAs 105; four of 76 97; four
-// of 38 99).
-constexpr int kPeelStreams = 4;
+// of 38 99; later 85.9 for four of 38, where an SM holds one CTA of the widest rows' peel, against
+// 91.6 for four of 76 with that kernel held to two per SM).
+constexpr int kPeelStreams = 4, kPeelsPerSm = 2;
 constexpr int64_t kSharedPeelRows = int64_t(1) << 20;
 
 struct Slot {
@@ -68,7 +72,7 @@ struct Slot {
 
 struct pscl_server {
     int device = 0;
-    int sm_count = 0;
+    int shared_grid = 0;             // CTAs of a peel beside others (0: every peel alone)
     size_t budget = 0, in_use = 0, peak = 0;
     std::vector<Slot> slots;
     cudaStream_t coop[kPeelStreams] = {};
@@ -104,9 +108,9 @@ void start(pscl_server *s, Slot &sl, Ticket *t)
     t->t_start = Clock::now();
     int rc = pscl_job_create(sl.ctx, d.points, d.dtype, d.n, d.d, d.on_device, &t->job);
     if (!rc) {
-        const bool alone = d.n > kSharedPeelRows;
+        const bool alone = d.n > kSharedPeelRows || s->shared_grid < 1;
         rc = pscl::job_set_coop_stream(t->job, s->coop, kPeelStreams, alone ? 0 : s->next_peel++ % kPeelStreams, alone);
-        if (!rc && !alone) rc = pscl_job_set_option(t->job, PSCL_OPT_PEEL_GRID, std::max(1, s->sm_count / 2));
+        if (!rc && !alone) rc = pscl_job_set_option(t->job, PSCL_OPT_PEEL_GRID, s->shared_grid);
     }
     if (!rc) rc = pscl_run(t->job, d.N, d.local_k, d.final_k, d.iters, d.seed, d.prec);
     if (!rc && cudaEventRecord(t->done, pscl::ctx_stream(sl.ctx)) != cudaSuccess) {
@@ -249,8 +253,11 @@ extern "C" int pscl_server_create(pscl_ctx *ctx, int32_t slots, size_t hbm_budge
     // cooperative launch are placed before new CTAs of other jobs
     int lo_prio = 0, hi_prio = 0;
     cudaDeviceGetStreamPriorityRange(&lo_prio, &hi_prio);
+    int sm_count = 0, per_sm = 0;
     bool made = cudaSetDevice(s->device) == cudaSuccess &&
-                cudaDeviceGetAttribute(&s->sm_count, cudaDevAttrMultiProcessorCount, s->device) == cudaSuccess;
+                cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, s->device) == cudaSuccess &&
+                pscl::peel_least_ctas_per_sm(&per_sm) == cudaSuccess;
+    s->shared_grid = sm_count * std::min(per_sm, kPeelsPerSm) / kPeelStreams;
     for (cudaStream_t &c : s->coop)
         made = made && cudaStreamCreateWithPriority(&c, cudaStreamNonBlocking, hi_prio) == cudaSuccess;
     if (!made) {
@@ -398,6 +405,14 @@ extern "C" int pscl_server_stats(pscl_server *s, int64_t *out)
     out[5] = (int64_t)s->peak;
     out[6] = s->max_running;
     out[7] = (int64_t)s->budget;
+    return PSCL_OK;
+}
+
+extern "C" int pscl_server_peel_grid(pscl_server *s, int32_t *ctas, int32_t *side_by_side)
+{
+    if (!s || !ctas || !side_by_side) return set_err(PSCL_EINVAL, "server, ctas or side_by_side is NULL");
+    *ctas = s->shared_grid;
+    *side_by_side = s->shared_grid < 1 ? 1 : kPeelStreams;
     return PSCL_OK;
 }
 
