@@ -735,6 +735,7 @@ __global__ void __launch_bounds__(kThreads)
 k_final_sse(const float *__restrict__ x, int64_t n, int d, const float *__restrict__ centers,
             int k, int chunk_k, int32_t *labels, double *blk_sse, double *sse, uint32_t *ticket)
 {
+    sse_enter(ticket);
     extern __shared__ __align__(16) unsigned char smem[];
     float *sc = reinterpret_cast<float *>(smem);
     const bool one_chunk = chunk_k >= k;
@@ -774,6 +775,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 k_final_sse_tiled(const float *__restrict__ x, int64_t n, int d, const float *__restrict__ centers, int k,
                   int32_t *labels, double *blk_sse, double *sse, uint32_t *ticket)
 {
+    sse_enter(ticket);
     extern __shared__ __align__(16) float4 tiles[];
     const int ld4 = tile_ld4(d);
     float4 *xs = tiles, *cs = tiles + kThreads * ld4;

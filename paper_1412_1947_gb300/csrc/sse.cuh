@@ -57,20 +57,28 @@ __device__ __forceinline__ double block_tree_sum(double part)
 // chain of as many float64 additions, 40-60 us behind every SSE pass.)
 // Without a ticket the blocks (kClusterSse at most) are one cluster and hand their sums to its
 // first through shared memory, in the same order: one launch, where the ticket takes a clearing
-// before it (1000 x 16: 10.2 -> 7.9 us a call).
+// before it (1000 x 16: 10.2 -> 7.9 us a call).  A block may write to another's shared memory only
+// once that one has started: every thread of such a kernel passes sse_enter first, and the wait
+// for all of the cluster's arrivals there comes just before the write, behind the scoring.
 constexpr int kClusterSse = 8;
+
+__device__ __forceinline__ void sse_enter(const uint32_t *ticket)
+{
+    if (!ticket) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
 
 __device__ __forceinline__ void sse_reduce(double part, double *blk_sse, double *sse, uint32_t *ticket)
 {
     const double b = block_tree_sum(part);
     if (!ticket) {
         __shared__ double all[kClusterSse];
+        asm volatile("barrier.cluster.wait;" ::: "memory");
         if (threadIdx.x == 0) {
             uint32_t at = (uint32_t)__cvta_generic_to_shared(&all[blockIdx.x]);
             asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(at));
             asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(b) : "memory");
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
         if (blockIdx.x != 0) return;
         const double tot = block_tree_sum(threadIdx.x < gridDim.x ? __dadd_rn(0.0, all[threadIdx.x]) : 0.0);
         if (threadIdx.x == 0) *sse = tot;
