@@ -841,7 +841,8 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
                 // center left out could win the float32 direct comparison
                 const float E = alpha * xn * cmax + beta * cmax * cmax +
                                 (float)(2 * (D + 3)) * 0x1p-24f * (xn + cmax) * (xn + cmax) + 0x1p-100f;
-                // (the next float up, for a strict comparison; b1 and E are finite)
+                // (the next float up, for a strict comparison; b1 and E are finite but for a FLAT
+                // row that is left to float32 below)
                 const float thr = __fadd_ru(b1 + 2.0f * E, 0x1p-149f);
                 // pass 2: the centers with v_j < thr as a bit mask (word c: centers 32c .. 32c+31);
                 // one bit is the label, more a near tie
@@ -883,7 +884,11 @@ __global__ void __launch_bounds__(tc_bound_threads<D>(), tc_min_blocks<D>()) k_t
                 }
                 if constexpr (FLAT) {
                     // one candidate: the label; two or three: their indices (two: the second
-                    // twice); more, or none (values that are not finite): every center
+                    // twice); more, or none (values that are not finite): every center.  So too
+                    // where a distance might overflow, up to (||x~|| + cmax)^2 here: a center of
+                    // infinite norm is no candidate though the row lie next to it, and where
+                    // every distance is infinite the float32 kernel takes center 0
+                    if (!(xn + cmax < 0x1p63f)) nc = 0;
                     if (nc == 2) first |= (first >> 9) << 18;
                     if (live) p.labels[row] = nc == 1 ? first : (int32_t)(kTieBit | (nc == 2 || nc == 3 ? (uint32_t)first : kFlatAll));
                 } else if (p.ref_centers) {
