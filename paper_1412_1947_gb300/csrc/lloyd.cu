@@ -134,6 +134,40 @@ __device__ __forceinline__ void load_row(const float *__restrict__ xr, int d, fl
     }
 }
 
+// The float32 direct distance of a row of any width in global memory to a center in shared memory.
+// From its first 32-byte boundary on the row is read a sector at a time, so that the rows of a
+// block need not stay in L1 from one attribute to the next: read by attributes, rows of odd widths
+// took twice as long whenever they did not (60000 x 129, k = 33: 46 % of the sectors hit, 1.42 ms an
+// iteration, 75 % and 0.68 ms with other warps in the way; by sectors 0.6.  500 sets of 300 x 150
+// 46 -> 16 ms, 200000 x 256 in sets of 10000 26 -> 8.8).
+__device__ __forceinline__ float dist_any(const float *__restrict__ xr, const float *c, int d)
+{
+    float v = 0.0f;
+    auto add = [&](float x, int a) {
+        const float t = __fsub_rn(x, c[a]);
+        v = __fmaf_rn(t, t, v);
+    };
+    const int head = min(d, (int)(8u - ((uint32_t)((uintptr_t)xr >> 2) & 7u)) & 7);
+    int a = 0;
+#pragma unroll 1
+    for (; a < head; a++) add(__ldg(&xr[a]), a);
+#pragma unroll 2
+    for (; a + 8 <= d; a += 8) {
+        const float4 p = __ldg(reinterpret_cast<const float4 *>(xr + a)), q = __ldg(reinterpret_cast<const float4 *>(xr + a + 4));
+        add(p.x, a);
+        add(p.y, a + 1);
+        add(p.z, a + 2);
+        add(p.w, a + 3);
+        add(q.x, a + 4);
+        add(q.y, a + 5);
+        add(q.z, a + 6);
+        add(q.w, a + 7);
+    }
+#pragma unroll 1
+    for (; a < d; a++) add(__ldg(&xr[a]), a);
+    return v;
+}
+
 // n centers of d attributes into shared memory at a stride of D >= d (D = 0: d), zeros past d.
 template <int D>
 __device__ __forceinline__ void load_centers(float *sc, const float *__restrict__ c, int n, int d)
@@ -316,8 +350,10 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
             bj[q] = 0;
         }
         // (a warp without a row left scores none: half of the warps of a unit of 128 rows; 25000 x 2,
-        // k = 500: 14.5 -> 11.6 us an iteration)
-        const int kw = one_chunk && p0 + (threadIdx.x & ~31) >= rows ? 0 : k;
+        // k = 500: 14.5 -> 11.6 us an iteration.  Not where rows are walked in global memory: the
+        // others' rows then leave L1 sooner; 20000 x 256, k = 300: 5.8 ms an iteration with them,
+        // 6.5 without)
+        const int kw = D > 0 && one_chunk && p0 + (threadIdx.x & ~31) >= rows ? 0 : k;
         for (int cb = 0; cb < kw; cb += chunk_k) {
             const int ce = min(k, cb + chunk_k);
             if (!one_chunk) {
@@ -329,14 +365,9 @@ k_lloyd_assign(const float *__restrict__ pts, SegTable t, int d, const float *__
                 scan_centers<DR, R>(xv, one_chunk ? sc + (size_t)cb * dd : sc, ce - cb, cb, best, bj);
             } else {
                 const float *cbase = one_chunk ? sc + (size_t)cb * dd : sc;
+                const float *xr = pts + (row0 + (live[0] ? prow[0] : 0)) * d;
                 for (int j = cb; j < ce; j++) {
-                    const float *cj = cbase + (size_t)(j - cb) * dd;
-                    const float *xr = pts + (row0 + (live[0] ? prow[0] : 0)) * d;
-                    float v = 0.0f;
-                    for (int a = 0; a < d; a++) {
-                        const float tq = __fsub_rn(__ldg(&xr[a]), cj[a]);
-                        v = __fmaf_rn(tq, tq, v);
-                    }
+                    const float v = dist_any(xr, cbase + (size_t)(j - cb) * dd, d);
                     if (v < best[0]) { best[0] = v; bj[0] = j; }
                 }
             }
@@ -614,12 +645,7 @@ struct Nearest {
             scan_centers<D, R>(xv, sc, ce - cb, cb, best, bj);
         } else {
             for (int j = cb; j < ce; j++) {
-                float acc = 0.0f;
-                const float *c = sc + (size_t)(j - cb) * d;
-                for (int a = 0; a < d; a++) {
-                    const float t = __fsub_rn(__ldg(&xr[a]), c[a]);
-                    acc = __fmaf_rn(t, t, acc);
-                }
+                const float acc = dist_any(xr, sc + (size_t)(j - cb) * d, d);
                 if (acc < best[0]) { best[0] = acc; bj[0] = j; }
             }
         }
