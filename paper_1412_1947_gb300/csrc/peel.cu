@@ -103,6 +103,9 @@ constexpr int kPeelDynWords = kScrWords + 2 * kKeyCache + kKeyCache / 4;
 constexpr int kRankBins = 2048;
 constexpr int kNear = 1024;
 constexpr int kStage = (2 * kKeyCache + kKeyCache / 4) / 3;
+// Close entries ranked one by one, at most; more (tied data) are sorted.  Each of them against every
+// near one takes their product: 10^6 x 1 with 1000 points a value 73.5 ms of peel, sorted 8.3.
+constexpr int kRankOne = 128;
 static_assert(kRankBins + kRankBins / 32 + 5 * kNear + kNear / 2 <= kScrWords, "settling fits the scratch");
 constexpr int kQT = 4;                        // tiles of kThreads items per compaction scan
 constexpr int kCB = 8;                        // keys per thread in flight when classifying
@@ -1097,6 +1100,75 @@ __device__ __noinline__ void settle_large(const PeelArgs &a, const float *Ls, ui
     if (t < (int)K && s_bc[t]) atomicAdd(&ctl->bnd[t], s_bc[t]);
 }
 
+// The window k - W .. k + W of a distance k (bit patterns; see settle_group).
+constexpr uint64_t kTiny = 963ull << 52;                                    // 2^-60
+__device__ __forceinline__ uint64_t win_lo(uint64_t k, uint64_t W) { return k < kTiny + W ? 0ull : k - W; }
+__device__ __forceinline__ uint64_t win_hi(uint64_t k, uint64_t W) { return (k < kTiny ? kTiny : k) + W; }
+
+// The ranks of a group's nn (<= kNear) near entries by (float64 distance, id), where ties make most
+// of them close: a bitonic network over their indexes, padded to a power of two by indexes past the
+// last, then for each the entries before it: the near ones, and those of the bins below its window
+// that are not marked.  mn, sh, hist, mark: settle_group's bins; W: its window.
+__device__ __noinline__ void rank_many(const float *__restrict__ x, const float *Ls, int d, uint64_t mn, int sh,
+                                       uint32_t nn, const uint64_t *nk, uint64_t *d64, const uint32_t *np,
+                                       const uint32_t *hist, const uint32_t *mark, uint32_t *rank, uint64_t W)
+{
+    const uint32_t t = threadIdx.x, m = 1u << (32 - __clz((int)max(nn, 2u) - 1));
+    uint32_t *idx = rank;
+#pragma unroll 1
+    for (uint32_t f = t; f < nn; f += kThreads)
+        d64[f] = (uint64_t)__double_as_longlong(dist64(x + (size_t)(np[f] & kPosMask) * d, Ls, d));
+#pragma unroll 1
+    for (uint32_t i = t; i < m; i += kThreads) idx[i] = i;
+    __syncthreads();
+#pragma unroll 1
+    for (uint32_t k = 2; k <= m; k *= 2)
+#pragma unroll 1
+        for (uint32_t j = k / 2; j; j /= 2) {
+#pragma unroll 1
+            for (uint32_t q = t; q < m / 2; q += kThreads) {
+                const uint32_t lo = 2 * q - (q & (j - 1u)), hi = lo + j;
+                const uint32_t a = idx[lo], b = idx[hi];
+                bool less = b < nn;                       // b before a
+                if (less && a < nn) {
+                    const uint64_t ka = d64[a], kb = d64[b];
+                    less = kb < ka || (kb == ka && (np[b] & kPosMask) < (np[a] & kPosMask));
+                }
+                if (less == ((lo & k) == 0u)) {
+                    idx[lo] = b;
+                    idx[hi] = a;
+                }
+            }
+            __syncthreads();
+        }
+    uint32_t *rk = reinterpret_cast<uint32_t *>(d64);     // (done with)
+#pragma unroll 1
+    for (uint32_t p = t; p < nn; p += kThreads) {
+        const uint32_t u = idx[p];
+        const uint64_t lo = win_lo(nk[u], W);
+        const uint32_t bl = lo <= mn ? 0u : (uint32_t)((lo - mn) >> sh);
+        uint32_t before = p;
+#pragma unroll 1
+        for (uint32_t wd = 0; wd <= bl >> 5; wd++) {
+            uint32_t un = ~mark[wd];
+            if (wd == bl >> 5) un &= (1u << (bl & 31u)) - 1u;
+            if (un == ~0u) {
+                before += hist[32u * wd + 32u] - hist[32u * wd];
+                continue;
+            }
+#pragma unroll 1
+            for (; un; un &= un - 1u) {
+                const uint32_t b = 32u * wd + (uint32_t)__ffs(un) - 1u;
+                before += hist[b + 1u] - hist[b];
+            }
+        }
+        rk[u] = before;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (uint32_t u = t; u < nn; u += kThreads) rank[u] = rk[u];
+}
+
 // Settles group g of the epoch's boundaries (one CTA): every band entry of the group gets
 // its round, exactly by (delta64, index).  q1 .. q2: the group's boundaries; off, ne: its region
 // of the regrouped entries; certs: the points certainly in rounds 0 .. q1; r0: the epoch's first
@@ -1110,7 +1182,7 @@ __device__ __noinline__ void settle_large(const PeelArgs &a, const float *Ls, ui
 // tiny squares counts too, so all of them are one window.  A histogram of the distances tells
 // most entries' sides of every boundary; only those close to one (all, of a small group) are
 // ranked one by one, a warp each, against the entries of the bins their windows touch: no
-// selection, and few barriers.  Short rolled loops throughout: the CTA that settles a group is
+// selection, and few barriers (past kRankOne of them by rank_many).  Short rolled loops throughout: the CTA that settles a group is
 // the only one that fetches this code, and the others wait for it.  (Every entry ranked against
 // every other: 25 us for 1000 entries; the selection of larger groups: 130 to 170 us.)
 __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, uint32_t g, uint32_t q1, uint32_t q2,
@@ -1123,7 +1195,7 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ uint32_t s_need[kMaxEpoch], s_bc[kMaxEpoch];
     __shared__ unsigned long long s_mn[kW], s_mx[kW];
-    __shared__ uint32_t s_near, s_any;
+    __shared__ uint32_t s_near, s_close, s_any;
     // points before the group: the certain ones and the entries of the groups before it
     const uint32_t before = certs + off, filled = __ldcg(&ctl->gfill[g]);
     uint32_t *hist = scr, *mark = hist + kRankBins;                         // entries before a bin; bins marked
@@ -1147,14 +1219,10 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
         if (need_s < 0 || need_s > (int64_t)ne) atomicOr(&a.flags[1], 1u);
     }
     if (t == 0) {
-        s_any = 0;
+        s_any = s_close = 0;
         s_near = all ? ne : 0u;
     }
     const uint64_t W0 = 256ull * ((uint64_t)d * d + 8ull * d + 1ull) + 8ull, W = W0 + (W0 >> 4);
-    constexpr uint64_t kTiny = 963ull << 52;                                // 2^-60
-    // the window of the distance k
-    auto win_lo = [&](uint64_t k) { return k < kTiny + W ? 0ull : k - W; };
-    auto win_hi = [&](uint64_t k) { return (k < kTiny ? kTiny : k) + W; };
     auto KEY = [&](uint32_t e) -> uint64_t { return st ? stk[e] : __ldcg(&gk[e]); };
     auto RAW = [&](uint32_t e) -> uint32_t { return st ? stp[e] : __ldcg(&gp[e]); };
     auto settle = [&](bool v, uint32_t raw, uint32_t rr) {                  // a warp's entries with v set
@@ -1170,8 +1238,8 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
     auto bin = [&](uint64_t k) { return k <= mn ? 0u : (uint32_t)(min(k, (uint64_t)mx) - mn >> sh); };
     // an entry's round from the bins alone; true if a boundary lies among those of its window
     auto close_to = [&](uint64_t k, uint32_t &rr, uint32_t &bl, uint32_t &bh) {
-        bl = bin(win_lo(k));
-        bh = bin(win_hi(k));
+        bl = bin(win_lo(k, W));
+        bh = bin(win_hi(k, W));
         const uint32_t least = hist[bl], most = bh + 1u < (uint32_t)kRankBins ? hist[bh + 1u] : ne;
         rr = q1;
         bool close = false;                                                 // the rank lies in [least, most)
@@ -1270,10 +1338,12 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
                 const uint32_t slot = atomicAdd(&s_near, 1u);
                 if (slot < (uint32_t)kNear) {
                     uint32_t rr, bl, bh;
+                    const bool cl = close_to(k, rr, bl, bh);
                     nk[slot] = k;
                     np[slot] = RAW(e);
-                    nst[slot] = close_to(k, rr, bl, bh) ? kClose : (uint8_t)0;
+                    nst[slot] = cl ? kClose : (uint8_t)0;
                     e64[slot] = 0;
+                    if (cl) atomicAdd(&s_close, 1u);
                 }
             }
         });
@@ -1287,10 +1357,12 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
     // the close entries' ranks, among the near ones: every entry of the bins that a close one's
     // window touches is near
     __shared__ uint32_t s_rank[kNear];
+    const bool many = s_close > (uint32_t)kRankOne;
+    if (many) rank_many(a.x, Ls, d, mn, sh, nn, nk, d64, np, hist, mark, s_rank, W);
 #pragma unroll 1
-    for (uint32_t u = (uint32_t)w; u < nn; u += kW) {
+    for (uint32_t u = many ? nn : (uint32_t)w; u < nn; u += kW) {
         if (!(nst[u] & kClose)) continue;                                   // the warp's
-        const uint64_t k = nk[u], lo = win_lo(k), hi = win_hi(k);
+        const uint64_t k = nk[u], lo = win_lo(k, W), hi = win_hi(k, W);
         const uint32_t bl = all ? 0u : bin(lo), base = all ? 0u : hist[bl];
         uint32_t below = 0, upto = 0;
 #pragma unroll 2
@@ -1325,7 +1397,7 @@ __device__ __noinline__ void settle_group(const PeelArgs &a, const float *Ls, ui
         for (uint32_t u = (uint32_t)w; u < nn; u += kW) {
             if (!(nst[u] & kCut)) continue;                                 // the warp's
             const uint32_t pu = np[u] & kPosMask;
-            const uint64_t k = nk[u], lo = win_lo(k), hi = win_hi(k), ku = d64[u];
+            const uint64_t k = nk[u], lo = win_lo(k, W), hi = win_hi(k, W), ku = d64[u];
             uint32_t more = 0;
 #pragma unroll 2
             for (uint32_t f = (uint32_t)lane; f < nn; f += 32)
