@@ -941,16 +941,15 @@ __device__ __noinline__ void phase_inc(const float *__restrict__ x, const float 
     }
 }
 
-// The holders among a warp's 32 points (lanes with `hold` set; ids by lane), one at a time by
+// The holders among a warp's 32 points (the lanes of m; ids by lane), one at a time by
 // the whole warp: f(j, v) for every attribute j in which the point equals the landmark, v its
 // lane's val.  A row is read in one coalesced load per 32 attributes, where a thread walking
 // it alone held its warp for d loads (400000 x 128: 15 us of an epoch's key pass).
 template <class F>
-__device__ __forceinline__ void for_held(const float *__restrict__ x, const float *Ls, int d, bool hold, uint32_t id,
+__device__ __forceinline__ void for_held(const float *__restrict__ x, const float *Ls, int d, uint32_t m, uint32_t id,
                                          uint32_t val, F f)
 {
     const int lane = threadIdx.x & 31;
-    uint32_t m = __ballot_sync(0xffffffffu, hold);
 #pragma unroll 1
     while (m) {
         const int q = __ffs(m) - 1;
@@ -974,11 +973,33 @@ __device__ __forceinline__ void for_held(const float *__restrict__ x, const floa
     }
 }
 
+// Many holders among a warp's points, few attributes: the lanes walk their points side by side (10^6 x
+// 3 with 4 values an attribute, most of a band's 10^5 points holders and one CTA settling them: 9.0 ->
+// 5.1 ms of peel).
+__device__ __noinline__ void count_side(const float *__restrict__ x, const float *Ls, int d, bool hold, uint32_t id,
+                                        uint32_t round, uint32_t (*hcnt)[kMaxEpoch])
+{
+    if (!hold) return;
+    const float *row = x + (size_t)id * d;
+#pragma unroll 4
+    for (int j = 0; j < d; j++)
+        if (__ldg(&row[j]) == Ls[j]) atomicAdd(&hcnt[j][round], 1u);
+}
+
 // The holders counted per attribute and round (out of line: rare, and three callers)
 __device__ __noinline__ void count_held(const float *__restrict__ x, const float *Ls, int d, bool hold, uint32_t id,
                                         uint32_t round, uint32_t (*hcnt)[kMaxEpoch])
 {
-    for_held(x, Ls, d, hold, id, round, [&](int j, uint32_t r) { atomicAdd(&hcnt[j][r], 1u); });
+    const uint32_t m = __ballot_sync(0xffffffffu, hold);
+    if (__popc(m) > max(4, d / 2)) return count_side(x, Ls, d, hold, id, round, hcnt);
+    for_held(x, Ls, d, m, id, round, [&](int j, uint32_t r) { atomicAdd(&hcnt[j][r], 1u); });
+}
+
+// The largest key among the holders of each attribute
+__device__ __noinline__ void max_held(const float *__restrict__ x, const float *Ls, int d, bool hold, uint32_t id,
+                                      uint32_t key, uint32_t *hmax)
+{
+    for_held(x, Ls, d, __ballot_sync(0xffffffffu, hold), id, key, [&](int j, uint32_t k) { atomicMax(&hmax[j], k); });
 }
 
 // A group of more entries than fit in shared memory: each of its boundaries' cut by selection,
@@ -2288,8 +2309,7 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                     todo &= todo - 1u;
                     const bool h = (held >> u) & 1u;
                     const uint32_t qi = q0 + u * kThreads + t;
-                    for_held(a.x, Ls, d, h, h ? LID(qi) : 0u, h ? LKEY(qi) : 0u,
-                             [&](int j, uint32_t key) { atomicMax(&ctl->hmax[j], key); });
+                    max_held(a.x, Ls, d, h, h ? LID(qi) : 0u, h ? LKEY(qi) : 0u, ctl->hmax);
                 }
             }
 #pragma unroll 1
