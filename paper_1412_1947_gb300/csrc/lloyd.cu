@@ -672,7 +672,11 @@ struct Nearest {
 // index wins ties.  Rows and centers lie at an odd number of 16-byte words, so that 8
 // consecutive ones fall in different banks.
 constexpr int kTileC = 64;                                 // centers in shared memory at a time
-constexpr int kTiledMin = 33, kTiledMax = 128;             // widths that take the tiles (d = 32: two rows per thread are level)
+// Widths that take the tiles.  At d = 32 two rows per thread are faster for the units of independent
+// sets (the uneven batch 7.1 against 9.5 ms), and the tiles for one set, whose few rows leave a
+// thread one row and its two chains (6 x 32, k = 340: 62 us, tiles 40, one chain a thread 46; 400000 x
+// 32, k = 64: 134, 89 and 169).
+constexpr int kTiledMin = 32, kTiledMinUnits = 33, kTiledMax = 128;
 
 constexpr int kTiledCenters = 24;                          // fewer leave the tile's 32 mostly empty
 
@@ -1166,7 +1170,7 @@ cudaError_t launch_seg_sse(const LloydBuffers &b, const SegTable &t, const int32
     cudaError_t e;
     if (seg_sse_tc_supported(b, t, d, kmax, prec)) {
         e = launch_seg_sse_tc(b, t, d, kmax, prec, labels, unit_sse, flags, sm_count, st, kt);
-    } else if (d >= kTiledMin && d <= kTiledMax && kmax >= kTiledCenters) {
+    } else if (d >= kTiledMinUnits && d <= kTiledMax && kmax >= kTiledCenters) {
         const size_t smem = tile_smem(d);
         if (const cudaError_t ea = cudaFuncSetAttribute(k_seg_sse_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return ea;
         kt->begin(st);
