@@ -138,8 +138,8 @@ __device__ __forceinline__ void load_row(const float *__restrict__ xr, int d, fl
 // From its first 32-byte boundary on the row is read a sector at a time, so that the rows of a
 // block need not stay in L1 from one attribute to the next: read by attributes, rows of odd widths
 // took twice as long whenever they did not (60000 x 129, k = 33: 46 % of the sectors hit, 1.42 ms an
-// iteration, 75 % and 0.68 ms with other warps in the way; by sectors 0.6.  500 sets of 300 x 150
-// 46 -> 16 ms, 200000 x 256 in sets of 10000 26 -> 8.8).
+// iteration, 75 % and 0.68 ms with other warps in the way; by sectors 0.57.  500 sets of 300 x 150
+// 46 -> 13 ms, 200000 x 256 in sets of 10000 26 -> 8.8).
 __device__ __forceinline__ float dist_any(const float *__restrict__ xr, const float *c, int d)
 {
     float v = 0.0f;
@@ -148,9 +148,18 @@ __device__ __forceinline__ float dist_any(const float *__restrict__ xr, const fl
         v = __fmaf_rn(t, t, v);
     };
     const int head = min(d, (int)(8u - ((uint32_t)((uintptr_t)xr >> 2) & 7u)) & 7);
-    int a = 0;
-#pragma unroll 1
-    for (; a < head; a++) add(__ldg(&xr[a]), a);
+    // up to 7 attributes from a on, their loads together (one by one: one set of 20000 x 129, k = 300
+    // 20.2 ms of a batch's ten iterations, together 18.5)
+    auto part = [&](int a, int m) {
+        float x[7];
+#pragma unroll
+        for (int q = 0; q < 7; q++) x[q] = q < m ? __ldg(&xr[a + q]) : 0.0f;
+#pragma unroll
+        for (int q = 0; q < 7; q++)
+            if (q < m) add(x[q], a + q);
+    };
+    part(0, head);
+    int a = head;
 #pragma unroll 2
     for (; a + 8 <= d; a += 8) {
         const float4 p = __ldg(reinterpret_cast<const float4 *>(xr + a)), q = __ldg(reinterpret_cast<const float4 *>(xr + a + 4));
@@ -163,8 +172,7 @@ __device__ __forceinline__ float dist_any(const float *__restrict__ xr, const fl
         add(q.z, a + 6);
         add(q.w, a + 7);
     }
-#pragma unroll 1
-    for (; a < d; a++) add(__ldg(&xr[a]), a);
+    part(a, d - a);
     return v;
 }
 
