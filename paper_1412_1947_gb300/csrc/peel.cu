@@ -2253,7 +2253,10 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
             __syncthreads();
             if (t == 0) {
                 // an update of the keys, or a full pass (the same choice in every CTA)
-                // (float32 rounded up throughout: a float64 chain here held up every CTA)
+                // (float32 rounded up throughout: a float64 chain here held up every CTA; cs: the
+                // moves of all attributes, for the keys' range.  Those of the first kIncMax alone left
+                // keys below it, in one coarse bin, and a band of 10^5 points: 6 10^6 x 128 of 8
+                // blobs 75 -> 22 ms of peel)
                 uint32_t nj = 0, nsec = 0, last_sec = kGone;
                 float cs = 0.0f;
                 bool fin = true;
@@ -2262,13 +2265,13 @@ __global__ void __launch_bounds__(kThreads) k_peel(PeelArgs a)
                     while (m) {
                         const int j = wd * 32 + __ffs(m) - 1;
                         m &= m - 1u;
+                        const float c = __fsub_rn(Ls[j], Lold[j]);
+                        fin = fin && c >= 0.0f && c <= 1.0f;
+                        cs = __fadd_ru(cs, c);
                         if (nj < (uint32_t)kIncMax) {
                             s_ij[nj] = j;
                             s_io[nj] = Lold[j];
                             s_il[nj] = Ls[j];
-                            const float c = __fsub_rn(Ls[j], Lold[j]);
-                            fin = fin && c >= 0.0f && c <= 1.0f;
-                            cs = __fadd_ru(cs, c);
                         }
                         nj++;
                         if ((uint32_t)(j >> 3) != last_sec) {
