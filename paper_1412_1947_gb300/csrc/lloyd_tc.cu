@@ -2054,8 +2054,14 @@ bool tc_supported(int d, int kmax, int prec, int64_t rows)
     }
 }
 
+// Several chunks of 128 attributes need rows for a tile per SM, and more chunks more rows: each CTA of
+// each chunk's launch forms the norms of all k centers (us an iteration, float32 against chunks:
+// 1600 rows, k = 300 148, 183, k = 1024 467, 855; 19000 rows, k = 512 266, 309; 25600 rows, k = 300
+// 305, 223, k = 512 477, 329, k = 797 719, 722; 36000 rows, k = 1024 931, 965; 44800 rows, k = 1024
+// 1348, 1066).
 bool tc_sse_supported(int d, int k, int prec, int64_t rows)
 {
+    if (d == 128 && k > tc_chunk(d) && rows < kWideRows * (k > 6 * tc_chunk(d) ? 2 : 1)) return false;
     return k >= 1 && tc_supported(d, std::min(k, tc_chunk(d)), prec, rows);
 }
 
