@@ -227,14 +227,6 @@ __device__ __forceinline__ void dist_rows(const float (&xv)[R][D], const float *
     }
 }
 
-// min(a, b, c) in one instruction (sm_100 and later)
-__device__ __forceinline__ float min3f(float a, float b, float c)
-{
-    float m;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
-    return m;
-}
-
 // The nearest of the n centers at sc (stride D, indices from base on) to R rows, folded into
 // the best so far: strict comparisons in ascending order, so the lowest index wins equal
 // distances.  Narrow rows against many centers take four at a time and keep only the smallest

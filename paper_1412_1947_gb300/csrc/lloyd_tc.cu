@@ -61,14 +61,6 @@ enum TcMode { kModeTf32 = 0, kModeBf16 = 1, kModeTf32x3 = 2, kModeBf16x3 = 3 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// min(a, b, c) in one instruction (sm_100 and later)
-__device__ __forceinline__ float min3f(float a, float b, float c)
-{
-    float m;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
-    return m;
-}
-
 // The signs of v_q - thr as a mask: bit q is set iff v_q < thr (a float32 difference has the
 // sign of the exact one).  The differences go two at a time through the otherwise idle FMA
 // pipe, and a funnel shift takes each sign, in four chains of eight: one ALU instruction per
@@ -1704,7 +1696,7 @@ cudaError_t sse_tc_dispatch(const float *x, int64_t n, const float *centers, int
     return cudaGetLastError();
 }
 
-// One Lloyd iteration of a single set with more than 256 centers on the tensor cores: the
+// One Lloyd iteration of a single set with more than tc_chunk(d) centers on the tensor cores: the
 // chunked search, then the exact sums from the labels (the update follows separately).
 template <int D, int MODE>
 cudaError_t lloyd_chunks_dispatch(const LloydBuffers &b, int iter, int k, uint32_t *flags, int sm_count,
@@ -1878,7 +1870,7 @@ __global__ void __launch_bounds__(kSseThreads) k_seg_sse_ties(const float *__res
                                                               const float *__restrict__ centers,
                                                               const int32_t *__restrict__ raw,
                                                               const uint32_t *__restrict__ tmask, int32_t *labels,
-                                                              double *unit_sse, int kmax)
+                                                              double *unit_sse)
 {
     extern __shared__ __align__(16) float4 xs[];               // [256 rows | centers]
     constexpr int LD4 = tile_ld4(D), DC = D + 4;
@@ -1935,7 +1927,7 @@ cudaError_t seg_sse_tc_dispatch(const LloydBuffers &b, const SegTable &t, int km
     auto kern = k_seg_sse_ties<D>;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     kt->begin(st);
-    kern<<<t.n_units, kSseThreads, smem, st>>>(b.pts, t, b.centers, b.raw, b.tmask, labels, unit_sse, kmax);
+    kern<<<t.n_units, kSseThreads, smem, st>>>(b.pts, t, b.centers, b.raw, b.tmask, labels, unit_sse);
     kt->end(PSCL_K_FINAL_SSE, st);
     return cudaGetLastError();
 }
@@ -1948,9 +1940,10 @@ cudaError_t seg_sse_tc_by_d(int d, const LloydBuffers &b, const SegTable &t, int
     case 16: return seg_sse_tc_dispatch<16, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
     case 32: return seg_sse_tc_dispatch<32, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
     case 64: return seg_sse_tc_dispatch<64, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
-    case 128: return seg_sse_tc_dispatch<128, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
-    default: return cudaErrorInvalidValue;
+    case 128:
+        if constexpr (MODE != kModeTf32x3) return seg_sse_tc_dispatch<128, MODE>(b, t, kmax, labels, unit_sse, flags, sm_count, st, kt);
     }
+    return cudaErrorInvalidValue;
 }
 
 template <int MODE>
@@ -1961,9 +1954,10 @@ cudaError_t lloyd_chunks_by_d(int d, const LloydBuffers &b, int iter, int k, uin
     case 16: return lloyd_chunks_dispatch<16, MODE>(b, iter, k, flags, sm_count, st, kt);
     case 32: return lloyd_chunks_dispatch<32, MODE>(b, iter, k, flags, sm_count, st, kt);
     case 64: return lloyd_chunks_dispatch<64, MODE>(b, iter, k, flags, sm_count, st, kt);
-    case 128: return lloyd_chunks_dispatch<128, MODE>(b, iter, k, flags, sm_count, st, kt);
-    default: return cudaErrorInvalidValue;
+    case 128:
+        if constexpr (MODE != kModeTf32x3) return lloyd_chunks_dispatch<128, MODE>(b, iter, k, flags, sm_count, st, kt);
     }
+    return cudaErrorInvalidValue;
 }
 
 template <int MODE>
@@ -1976,9 +1970,10 @@ cudaError_t sse_tc_by_d(int d, const float *x, int64_t n, const float *centers, 
     case 16: return sse_tc_dispatch<16, MODE>(x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
     case 32: return sse_tc_dispatch<32, MODE>(x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
     case 64: return sse_tc_dispatch<64, MODE>(x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
-    case 128: return sse_tc_dispatch<128, MODE>(x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
-    default: return cudaErrorInvalidValue;
+    case 128:
+        if constexpr (MODE != kModeTf32x3) return sse_tc_dispatch<128, MODE>(x, n, centers, k, t256, trem, scratch, labels, blk_sse, sse, ticket, flags, wait_limit, sm_count, st, kt);
     }
+    return cudaErrorInvalidValue;
 }
 
 template <int MODE>
@@ -1989,9 +1984,10 @@ cudaError_t tc_by_d(const LloydBuffers &b, const SegTable &t, int d, int iter, i
     case 16: return tc_dispatch<16, MODE>(b, t, iter, kmax, flags, sm_count, st, kt);
     case 32: return tc_dispatch<32, MODE>(b, t, iter, kmax, flags, sm_count, st, kt);
     case 64: return tc_dispatch<64, MODE>(b, t, iter, kmax, flags, sm_count, st, kt);
-    case 128: return tc_dispatch<128, MODE>(b, t, iter, kmax, flags, sm_count, st, kt);
-    default: return cudaErrorInvalidValue;
+    case 128:
+        if constexpr (MODE != kModeTf32x3) return tc_dispatch<128, MODE>(b, t, iter, kmax, flags, sm_count, st, kt);
     }
+    return cudaErrorInvalidValue;
 }
 
 // d = 128: BF16 at any size that fits; TF32 and BF16X3 above 16 centers, or with rows for a
@@ -2007,14 +2003,16 @@ constexpr double kFlatWork = 8e7;
 template <int MODE>
 bool fits_by_d(int d, int kmax, int64_t rows)
 {
-    if (d == 128 && (MODE == kModeTf32x3 || (MODE != kModeBf16 && kmax <= 16 && rows < kWideRows))) return false;
+    if (d == 128 && MODE != kModeBf16 && kmax <= 16 && rows < kWideRows) return false;
     switch (d) {
     case 16: return assign_smem<16, MODE>(kmax) <= kTcSmemMax && sums_smem<16>(kmax) <= kTcSmemMax;
     case 32: return assign_smem<32, MODE>(kmax) <= kTcSmemMax && sums_smem<32>(kmax) <= kTcSmemMax;
     case 64: return assign_smem<64, MODE>(kmax) <= kTcSmemMax && sums_smem<64>(kmax) <= kTcSmemMax;
-    case 128: return assign_smem<128, MODE>(kmax) <= kTcSmemMax && sums_smem<128>(kmax) <= kTcSmemMax;
-    default: return false;
+    case 128:
+        if constexpr (MODE != kModeTf32x3)
+            return assign_smem<128, MODE>(kmax) <= kTcSmemMax && sums_smem<128>(kmax) <= kTcSmemMax;
     }
+    return false;
 }
 
 int mode_of(int prec)

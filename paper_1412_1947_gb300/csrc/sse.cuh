@@ -1,5 +1,5 @@
 // What the SSE passes of the float32 and the tensor-core path share: the fixed order of the
-// float64 sums (so that both give the same bits) and row tiles in shared memory.
+// float64 sums (so that both give the same bits), row tiles in shared memory and a minimum of three.
 #pragma once
 
 #include "pscl_internal.cuh"
@@ -8,6 +8,14 @@ namespace pscl {
 namespace {
 
 constexpr int kSseThreads = 256;
+
+// min(a, b, c) in one instruction (sm_100 and later)
+__device__ __forceinline__ float min3f(float a, float b, float c)
+{
+    float m;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+    return m;
+}
 
 // 16-byte words between rows of d floats in shared memory: an odd number, so that 8
 // consecutive rows fall in different banks.
