@@ -65,7 +65,9 @@ typedef enum { PSCL_F32 = 0, PSCL_BF16 = 1 } pscl_dtype;
  *  The contraction covers d in {16, 32, 64} with at most 256 centers per point set and
  *  d = 128 with at most 128, where the operand tiles fit one CTA's shared memory (d = 64
  *  in TF32X3 only with 16 centers; d = 128 not in TF32X3, and in TF32 and BF16X3 with 16
- *  centers or fewer only from 20480 rows on); other shapes use the float32 direct sum.
+ *  centers or fewer only from 20480 rows on); the pooled set and the SSE take more centers in
+ *  chunks of as many (d = 128 from 20480 rows on, 40960 for more than 768 centers); other
+ *  shapes use the float32 direct sum.
  *  The near-tie bound is rigorous, so every mode assigns exactly as PSCL_PREC_FP32 does.
  *  Every mode yields the same partition into subclusters; the update step is the same
  *  exact fixed-point mean in all modes. */
@@ -299,20 +301,23 @@ int pscl_peel_ctas_per_sm(int device, int32_t d, int32_t *ctas);
  * The paper has no counterpart: this is a service for callers that cannot allocate
  * device memory (a framework whose allocator owns the device, a real-time host that
  * forbids allocation after start-up, code where an allocation would synchronise).  It
- * runs the SSE step of pscl_cluster (large calls with d = 16, 32 or 64, up to 512 centers and
- * both arrays on 16-byte boundaries on the tensor cores, with the same results): labels[i] = the nearest of the k
- * centers to points[i] (float32 squared distance, lowest index on ties) and *sse = the
- * sum over points of that distance, added in double in a fixed order.
+ * runs the SSE step of pscl_cluster: labels[i] = the nearest of the k centers to points[i]
+ * (float32 squared distance, lowest index on ties; center 0 where no distance is below
+ * infinity) and *sse = the sum over points of that distance, added in double in a fixed order.
+ * Three routes give the same results: up to 2048 points one launch of one cluster of blocks;
+ * d = 16, 32 or 64 with 32 to 512 centers, 20480 points or more, n k d >= 8e7 and both arrays
+ * on 16-byte boundaries two launches on the tensor cores; all else one float32 launch.
  *   points   n x d float32 row-major, device memory of the current device
  *   centers  k x d float32 row-major, device memory
  *   labels   n int32, device memory (written)
  *   sse      one double, device memory (written)
  *   stream   cudaStream_t to run on, or NULL for the default stream
  * Limits: 1 <= n <= 2^31-1, 1 <= d <= 1024, 1 <= k <= 4096; PSCL_EINVAL beyond.
- * Scratch: a fixed array of 4096 float64 partial sums plus a counter (33 KB) that every
- * device loading the library holds until exit.  Every call on a device shares it and it
- * keeps the last call's contents (the counter is cleared at the start of each call), so
- * calls whose work overlaps on the GPU race: order them on one stream or synchronise.
+ * Scratch: a fixed array of 4096 float64 partial sums, a counter and four flag words (33 KB)
+ * that every device loading the library holds until exit.  Calls of up to 2048 points use
+ * none of it.  Every other call on a device shares it and it keeps the last call's contents
+ * (a clearing of the counter and the flags goes before the launches), so such calls whose
+ * work overlaps on the GPU race: order them on one stream or synchronise.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress);
  * make that first call before any stream capture.  The address is looked up again when
  * the current context is not the one it was found in (after cudaDeviceReset, say); that

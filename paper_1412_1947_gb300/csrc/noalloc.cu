@@ -4,10 +4,10 @@
 // Some callers may not call cudaMalloc at all: code that runs under an allocator that
 // owns the whole device (a framework's caching allocator, a fixed memory plan), real-time
 // or embedded hosts that forbid allocation after start-up, or code paths where an
-// allocation would synchronise the device.  This entry point runs the
-// SSE step of pscl_cluster, on the tensor cores where the shape pays, but its scratch (one float64 partial sum per thread block and a
-// completion ticket) lives in the file-scope array below instead of memory the library
-// allocates.  The caller supplies the points, the centers and the two outputs.
+// allocation would synchronise the device.  This entry point runs the SSE step of
+// pscl_cluster, on the tensor cores where the shape pays, but its scratch (one float64 partial
+// sum per thread block, a completion ticket and flags; none up to 2048 points) lives in the
+// file-scope array below instead of memory the library allocates.  The caller supplies the points, the centers and the two outputs.
 #include <cuda.h>
 #include <cuda_runtime.h>
 

@@ -59,7 +59,10 @@ struct Ticket {
 // Peels side by side, and the largest that share the device (the serving mix of 20 jobs of
 // 10^4 .. 10^6 points, four slots: one stream 120 ms; two of 152 CTAs 105; four of 76 97; four
 // of 38 99; later 85.9 for four of 38, where an SM holds one CTA of the widest rows' peel, against
-// 91.6 for four of 76 with that kernel held to two per SM).
+// 91.6 for four of 76 with that kernel held to two per SM).  The line for running alone: of 200 jobs
+// up to 10^6 points 342 a second with 2^18, 386 with 2^20 and above; of 120 jobs up to 10^7 points,
+// mostly bound by their Lloyd iterations, 10.8 a second with 2^18, 2^20 and 2^22 alike, and with all
+// of them shared 11.0, but half of them done after 5.6 s in place of 4.8.
 constexpr int kPeelStreams = 4, kPeelsPerSm = 2;
 constexpr int64_t kSharedPeelRows = int64_t(1) << 20;
 
